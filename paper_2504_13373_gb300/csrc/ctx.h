@@ -115,6 +115,11 @@ struct gasa_ctx {
   cudaGraphExec_t cg_exec[6] = {};
   long long cg_kernels[6] = {};
   int cg_max_iter[6] = {};
+  // one V-cycle per precision as an instantiated graph (host-driven callers,
+  // from their second V-cycle on); vc_calls < 0: the stream cannot be captured
+  cudaGraphExec_t vc_exec[3] = {};
+  int vc_calls[3] = {};
+  long long vc_kernels[3] = {};
   int *d_iters = nullptr;
   int *d_err = nullptr;          // set by kernels whose bounded waits time out
   // fused bottom of the V-cycle per precision (0: FP64, 1: FP32): levels

@@ -87,6 +87,12 @@ void free_graphs(gasa_ctx *ctx) {
     ctx->cg_graph[p] = nullptr;
     ctx->cg_kernels[p] = 0;
   }
+  for (int p = 0; p < 3; ++p) {
+    if (ctx->vc_exec[p]) cudaGraphExecDestroy(ctx->vc_exec[p]);
+    ctx->vc_exec[p] = nullptr;
+    ctx->vc_calls[p] = 0;
+    ctx->vc_kernels[p] = 0;
+  }
 }
 
 void free_all(gasa_ctx *ctx) {
@@ -655,9 +661,11 @@ struct FusedEnds {
   float *b32;
 };
 
+// first0: the caller has already launched level 0's first smoothing step
+//
 template <typename T>
 gasa_status vcycle_impl(gasa_ctx *ctx, const T *rhs, T *out, bool h16 = false,
-                        const FusedEnds *fe = nullptr) {
+                        const FusedEnds *fe = nullptr, bool first0 = false) {
   using P = Prec<T>;
   cudaStream_t s = ctx->stream;
   const int N = ctx->N;
@@ -725,8 +733,10 @@ gasa_status vcycle_impl(gasa_ctx *ctx, const T *rhs, T *out, bool h16 = false,
   std::vector<T *> xk(N + 1);
   bk[0] = rhs;
   for (int k = 1; k <= N; ++k) bk[k] = P::b(ctx->L[k]);
-  // levels whose first smoothing step the restriction of the level above took
+  // levels whose first smoothing step the restriction of the level above (level 0: the
+  // caller) took
   std::vector<char> first_done(N + 1, 0);
+  first_done[0] = first0 ? 1 : 0;
   for (int k = 0; k < kt; ++k) {
     Level &l = ctx->L[k];
     T *x = P::x(l), *x2 = P::x2(l);
@@ -840,12 +850,17 @@ gasa_status vcycle_impl(gasa_ctx *ctx, const T *rhs, T *out, bool h16 = false,
   return GASA_OK;
 }
 
+// the FP32 V-cycle's first level-0 step reads the FP64 residual itself
+bool first_step_reads_f64(const gasa_ctx *ctx, int precision) {
+  const Level &l0 = ctx->L[0];
+  return precision == GASA_PREC_MIXED32 && !l0.mf && l0.s <= 16 && ctx->opt.t_pre >= 1;
+}
+
 // FP32 V-cycle of the mixed precisions on the FP64 residual rr; z in FP32
 // is left in ctx->kf_out
 gasa_status vcycle_f32_out(gasa_ctx *ctx, const double *rr, int precision) {
-  Level &l0 = ctx->L[0];
-  const int64_t n = l0.ndof;
-  if (precision == GASA_PREC_MIXED32 && !l0.mf && l0.s <= 16 && ctx->opt.t_pre >= 1) {
+  const int64_t n = ctx->L[0].ndof;
+  if (first_step_reads_f64(ctx, precision)) {
     FusedEnds fe{rr, ctx->kf_in};
     return vcycle_impl<float>(ctx, ctx->kf_in, ctx->kf_out, false, &fe);
   }
@@ -857,6 +872,81 @@ gasa_status apply_M(gasa_ctx *ctx, const double *rr, double *z, int precision) {
   if (precision == GASA_PREC_FP64) return vcycle_impl<double>(ctx, rr, z);
   ST(vcycle_f32_out(ctx, rr, precision));
   CU(launch_convert<float, double>(ctx->L[0].ndof, ctx->kf_out, z, ctx->stream));
+  return GASA_OK;
+}
+
+// The launches of one V-cycle between its first and last use of the caller's
+// vectors: the FP32 cycles from kf_in (level 0's first step done when it reads
+// the FP64 residual) to kf_out, the FP64 cycle from kzold to kq.
+gasa_status vcycle_body(gasa_ctx *ctx, int precision) {
+  if (precision == GASA_PREC_FP64) return vcycle_impl<double>(ctx, ctx->kzold, ctx->kq);
+  return vcycle_impl<float>(ctx, ctx->kf_in, ctx->kf_out, precision == GASA_PREC_MIXED16, nullptr,
+                            first_step_reads_f64(ctx, precision));
+}
+
+// Capture vcycle_body into ctx->vc_exec[precision]; a stream that cannot be
+// captured leaves vc_calls negative and every V-cycle as separate launches.
+gasa_status build_vcycle_graph(gasa_ctx *ctx, int precision) {
+  cudaStream_t s = ctx->stream;
+  if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+    (void)cudaGetLastError();
+    ctx->vc_calls[precision] = -1;
+    return GASA_OK;
+  }
+  const long long k0 = launch_count();
+  const gasa_status st = vcycle_body(ctx, precision);
+  const long long captured = launch_count() - k0;
+  note_launches(-captured);   // recorded, not launched
+  cudaGraph_t g = nullptr;
+  const cudaError_t e = cudaStreamEndCapture(s, &g);
+  if (st != GASA_OK || e != cudaSuccess) {
+    if (g) cudaGraphDestroy(g);
+    ST(st);
+    CU(e);
+  }
+  const cudaError_t ei = cudaGraphInstantiate(&ctx->vc_exec[precision], g, 0);
+  cudaGraphDestroy(g);
+  if (ei != cudaSuccess) ctx->vc_exec[precision] = nullptr;
+  CU(ei);
+  ctx->vc_kernels[precision] = captured;
+  return GASA_OK;
+}
+
+// z = M r for host-driven callers (gasa_vcycle, GMRES).  A V-cycle is 30 to 40
+// launches of 2 to 40 us kernels, and launching them one by one from the host
+// costs more than half of them: from the second call of a precision on, one
+// graph launch replaces them (1.31M-dof P3 mixed V-cycle 559 -> 469 us,
+// 162k-dof FP16-block one 255 -> 180 us).  The caller's vectors are read and
+// written outside the graph, so it does not depend on their addresses: the
+// FP32 cycles convert at both ends anyway, the FP64 cycle takes two copies.
+// The first call launches directly: a hierarchy that is applied once pays for
+// no graph.
+gasa_status apply_M_host(gasa_ctx *ctx, const double *rr, double *z, int precision) {
+  int &calls = ctx->vc_calls[precision];
+  if (ctx->prof || calls < 1) {
+    if (!ctx->prof && calls == 0) calls = 1;
+    return apply_M(ctx, rr, z, precision);
+  }
+  if (!ctx->vc_exec[precision]) {
+    ST(build_vcycle_graph(ctx, precision));
+    if (!ctx->vc_exec[precision]) return apply_M(ctx, rr, z, precision);
+  }
+  cudaStream_t s = ctx->stream;
+  Level &l = ctx->L[0];
+  const int64_t n = l.ndof;
+  if (precision == GASA_PREC_FP64) {
+    CU(launch_copy(n, rr, ctx->kzold, s));
+  } else if (first_step_reads_f64(ctx, precision)) {
+    const bool fold0 = l.WA32 && !l.tma;
+    CU(launch_jacobi_first_conv(l.n, l.s, rr, ctx->kf_in, l.W32, l.xf, s,
+                                fold0 ? l.cf : nullptr));
+  } else {
+    CU(launch_convert<double, float>(n, rr, ctx->kf_in, s));
+  }
+  CU(cudaGraphLaunch(ctx->vc_exec[precision], s));
+  note_launches(ctx->vc_kernels[precision]);
+  if (precision == GASA_PREC_FP64) CU(launch_copy(n, ctx->kq, z, s));
+  else CU(launch_convert<float, double>(n, ctx->kf_out, z, s));
   return GASA_OK;
 }
 
@@ -874,11 +964,16 @@ gasa_status apply_M_cg(gasa_ctx *ctx, const double *rr, double *z, const double 
 
 // scalar slots in ctx->scal
 enum { S_RR = 0, S_ALPHA = 1, S_PQ = 2, S_RZ0 = 3, S_RZ1 = 4, S_BB = 5, S_TMP = 6, S_G = 7,
-       S_BETA = 8, S_BN = 9, S_TOL = 10, S_COUNT = 16 };
+       S_BETA = 8, S_BN = 9, S_TOL = 10, S_INTS = 12, S_COUNT = 16 };
 
 // GASA_ERR_TIMEOUT (flag cleared) when a bounded device-side wait of the
 // last launches ran out, else GASA_OK; synchronises the context stream
 gasa_status check_wait_flag(gasa_ctx *ctx) {
+  // only the bulk-copy staged step and the persistent coarse launch wait on the device
+  if (!ctx->L[0].tma && !ctx->grid_plan[0] && !ctx->grid_plan[1]) {
+    CU(cudaStreamSynchronize(ctx->stream));
+    return GASA_OK;
+  }
   int kerr = 0;
   CU(cudaMemcpyAsync(&kerr, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   CU(cudaStreamSynchronize(ctx->stream));
@@ -1149,10 +1244,12 @@ gasa_status pcg_graph(gasa_ctx *ctx, const double *b, double tol, int precision,
   const int max_iter = ctx->opt.max_iter;
   for (;;) {
     CU(cudaGraphLaunch(ctx->cg_exec[pi], s));
-    int it = 0, kerr = 0;
-    CU(cudaMemcpyAsync(&it, ctx->d_iters, sizeof(int), cudaMemcpyDeviceToHost, s));
-    CU(cudaMemcpyAsync(&kerr, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    // into the pinned mirror: copies to pageable memory would each wait on their own
+    int *hi = reinterpret_cast<int *>(ctx->hscal + S_INTS);
+    CU(cudaMemcpyAsync(hi, ctx->d_iters, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CU(cudaMemcpyAsync(hi + 1, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
     ST(read_scalars(ctx, 0, 3));
+    const int it = hi[0], kerr = hi[1];
     note_launches(ctx->cg_kernels[pi] * (long long)(it - done_iters));
     done_iters = it;
     *iters = it;
@@ -1244,7 +1341,7 @@ gasa_status gmres(gasa_ctx *ctx, const double *b, double tol, int precision, int
       return GASA_OK;
     }
     if (flex) CU(launch_copy(n, t, w, s));
-    else ST(apply_M(ctx, t, w, precision));
+    else ST(apply_M_host(ctx, t, w, precision));
     double beta2;
     ST(norm2(ctx, n, w, S_TMP, &beta2));
     const double beta = std::sqrt(beta2);
@@ -1258,11 +1355,11 @@ gasa_status gmres(gasa_ctx *ctx, const double *b, double tol, int precision, int
       double *vj = ctx->V + (size_t)j * n;
       if (flex) {
         double *zj = ctx->Z + (size_t)j * n;
-        ST(apply_M(ctx, vj, zj, precision));
+        ST(apply_M_host(ctx, vj, zj, precision));
         ST(spmv_outer(ctx, GASA_MV_ASSIGN, zj, nullptr, w));
       } else {
         ST(spmv_outer(ctx, GASA_MV_ASSIGN, vj, nullptr, t));
-        ST(apply_M(ctx, t, w, precision));
+        ST(apply_M_host(ctx, t, w, precision));
       }
       ++total;
       double *Hj = ctx->H + (size_t)j * ldh;
@@ -2294,7 +2391,7 @@ gasa_status gasa_vcycle(gasa_ctx *ctx, const double *r, double *z, int32_t preci
   if (precision < GASA_PREC_FP64 || precision > GASA_PREC_MIXED16)
     return fail(ctx, GASA_ERR_INVALID_ARG, "unknown precision");
   if (cudaSetDevice(ctx->device) != cudaSuccess) return fail(ctx, GASA_ERR_CUDA, "cudaSetDevice");
-  ST(apply_M(ctx, r, z, precision));
+  ST(apply_M_host(ctx, r, z, precision));
   return check_wait_flag(ctx);
 }
 
