@@ -366,10 +366,7 @@ __global__ void tentative_kernel(int bs, const int *__restrict__ child_ptr,
     const double *gc = G + (size_t)c * rows;
     for (int i = lane; i < rows; i += 32) a = fma(gc[i], gc[i], a);
     a = warp_sum(a);
-    if (lane == 0) {
-      sv[c] = sqrt(a);
-      order[c] = c;     // ranks of non-finite norms leave gaps
-    }
+    if (lane == 0) sv[c] = sqrt(a);
   }
   __syncthreads();
   for (int c = threadIdx.x; c < r; c += blockDim.x) {
@@ -482,354 +479,6 @@ __global__ void tentative_kernel(int bs, const int *__restrict__ child_ptr,
   }
 }
 
-// ----------------------------------------------------------------------------
-// The same singular vectors with the Jacobi sweeps on a preconditioned factor
-// (Drmac & Veselic, "New fast and accurate Jacobi SVD algorithm", SIAM J.
-// Matrix Anal. Appl. 29, 2008): G = Q R by Householder QR with column
-// pivoting, R = L Q2^T by a second one on R^T, then one-sided Jacobi on the
-// lower triangular L (k x k, k = min(rows, r)), whose columns are nearly
-// orthogonal already; the kept vectors are Q times L's.  The right factors
-// (pivoting, Q2, the rotations) are never needed.  The relaxed candidates'
-// singular values span 5 to 16 decades, and on G itself Jacobi took 13 to 23
-// sweeps with nearly every pair rotated; on L it takes 7 or 8, the last two
-// of which rotate next to nothing.
-//
-// Bound: FP64 arithmetic (an SM does two FP64 FMAs a clock).  Eight lanes own
-// a column pair, so a round of k/2 disjoint pairs is one pass of the CTA; the
-// squared norms come from an update and are recomputed once per sweep, the
-// rotation's tangent from FP32 (a relative error of 1e-7 in the angle only
-// costs a later sweep a smaller rotation), its cosine from FP64.  The three
-// levels of a P2 8^3 tet mesh (384, 48 and 6 aggregates of 80, 104 and 136 rows
-// by 80 candidates), GB300: 204.7 -> 22.9 ms (13.5, 4.4 and 5.0 ms).
-// ----------------------------------------------------------------------------
-constexpr int kTentQrMaxR = 256;
-
-// sum over a group of eight neighbouring lanes
-__device__ __forceinline__ double group8_sum(double v) {
-  v += __shfl_xor_sync(0xffffffffu, v, 4);
-  v += __shfl_xor_sync(0xffffffffu, v, 2);
-  v += __shfl_xor_sync(0xffffffffu, v, 1);
-  return v;
-}
-
-// Householder QR of the rows x cols matrix M (column-major, pitch ld) by the
-// whole CTA: nref reflectors, R above and on the diagonal.  Reflector i is
-// I - f[i] v v^T with v = (vd[i], M[i+1.., i]) from row i on.  cn holds the
-// squared norms of the remaining rows of every column (recomputed exactly as
-// each column is updated); with `pivot` the largest is swapped to the front.
-__device__ void house_qr(double *M, int ld, int rows, int cols, int nref, bool pivot, double *cn,
-                         double *vd, double *f, double *bc) {
-  const int lane8 = threadIdx.x & 7, grp = threadIdx.x >> 3, ngrp = blockDim.x >> 3;
-  const int jround = ((cols + ngrp - 1) / ngrp) * ngrp;
-  for (int j = grp; j < jround; j += ngrp) {
-    double s = 0.0;
-    if (j < cols)
-      for (int q = lane8; q < rows; q += 8) s = fma(M[(size_t)j * ld + q], M[(size_t)j * ld + q], s);
-    s = group8_sum(s);
-    if (j < cols && lane8 == 0) cn[j] = s;
-  }
-  __syncthreads();
-  __shared__ int piv_s;
-  for (int i = 0; i < nref; ++i) {
-    if (pivot) {
-      if (threadIdx.x < 32) {
-        double best = -1.0;
-        int bi = INT_MAX;
-        for (int j = i + (int)threadIdx.x; j < cols; j += 32)
-          if (cn[j] > best) { best = cn[j]; bi = j; }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-          const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-          if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-        }
-        if (threadIdx.x == 0) piv_s = bi < cols ? bi : i;
-      }
-      __syncthreads();
-      const int p = piv_s;
-      if (p != i) {
-        for (int q = threadIdx.x; q < rows; q += blockDim.x) {
-          const double t = M[(size_t)i * ld + q];
-          M[(size_t)i * ld + q] = M[(size_t)p * ld + q];
-          M[(size_t)p * ld + q] = t;
-        }
-        if (threadIdx.x == 0) {
-          const double t = cn[i];
-          cn[i] = cn[p];
-          cn[p] = t;
-        }
-        __syncthreads();
-      }
-    }
-    if (threadIdx.x == 0) {
-      const double alpha = M[(size_t)i * ld + i], nr = sqrt(cn[i]);
-      const double beta = alpha > 0.0 ? -nr : nr;
-      const double den = beta * (beta - alpha);
-      const bool on = den > 0.0;            // zero column (or one whose square underflows): no reflection
-      vd[i] = on ? alpha - beta : 0.0;
-      f[i] = on ? 1.0 / den : 0.0;
-      bc[0] = on ? beta : alpha;
-    }
-    __syncthreads();
-    const double vi = vd[i], fi = f[i];
-    const double *v = M + (size_t)i * ld;
-    const int jr = i + 1 + ((cols - i - 1 + ngrp - 1) / ngrp) * ngrp;
-    for (int j = i + 1 + grp; j < jr; j += ngrp) {
-      double *g = M + (size_t)j * ld;
-      const bool act = j < cols;
-      double w = 0.0;
-      if (act) {
-        for (int q = i + 1 + lane8; q < rows; q += 8) w = fma(v[q], g[q], w);
-        if (lane8 == 0) w = fma(vi, g[i], w);
-      }
-      w = group8_sum(w) * fi;
-      double s = 0.0;
-      if (act) {
-        for (int q = i + 1 + lane8; q < rows; q += 8) {
-          const double t = fma(-w, v[q], g[q]);
-          g[q] = t;
-          s = fma(t, t, s);
-        }
-        if (lane8 == 0) g[i] = fma(-w, vi, g[i]);
-      }
-      s = group8_sum(s);
-      if (act && lane8 == 0) cn[j] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) M[(size_t)i * ld + i] = bc[0];
-  }
-  __syncthreads();
-}
-
-__global__ void __launch_bounds__(512)
-tentative_qr_kernel(int bs, const int *__restrict__ child_ptr, const int *__restrict__ child_idx,
-                    const double *__restrict__ B, int64_t ldb, int r, int s_next, int max_rows,
-                    double *__restrict__ T, double *__restrict__ sigma, int *status,
-                    const int *__restrict__ unit_size, const int *__restrict__ keep) {
-  extern __shared__ double smem_t[];
-  __shared__ double sv[kTentQrMaxR], cn[kTentQrMaxR], vd[kTentQrMaxR], ff[kTentQrMaxR],
-      scr[kTentQrMaxR];
-  __shared__ int order[kTentQrMaxR];
-  __shared__ double bc[1];
-  __shared__ int rows_s, rotated;
-  const int J = blockIdx.x;
-  const int c0 = child_ptr[J], nch = child_ptr[J + 1] - c0;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  const int lane8 = threadIdx.x & 7, grp = threadIdx.x >> 3, ngrp = blockDim.x >> 3;
-  const int kmax = min(max_rows, r), ldx = r | 1;
-  double *G = smem_t;                              // rows x r
-  double *X = G + (size_t)max_rows * r;            // R^T, then L: pitch ldx
-  double *U = X + (size_t)ldx * kmax;              // rows x s_next
-  int *rowg = reinterpret_cast<int *>(U + (size_t)max_rows * s_next);
-  // the aggregate's real rows, in unit then dof order (padded levels: unit u
-  // holds unit_size[u] real dofs followed by zeros)
-  if (threadIdx.x == 0) {
-    int m = 0;
-    for (int ch = 0; ch < nch; ++ch) {
-      const int u = child_idx[c0 + ch], nu = unit_size ? unit_size[u] : bs;
-      for (int d = 0; d < nu; ++d) rowg[m++] = u * bs + d;
-    }
-    rows_s = m;
-  }
-  __syncthreads();
-  const int rows = rows_s;
-  const int k = min(rows, r);
-  const int sJ = keep ? keep[J] : s_next;
-  for (int e = threadIdx.x; e < rows * r; e += blockDim.x) {
-    const int c = e / rows, q = e - c * rows;
-    G[e] = B[(size_t)c * ldb + rowg[q]];
-  }
-  __syncthreads();
-  house_qr(G, rows, rows, r, k, true, cn, vd, ff, bc);
-  // X = R^T (r x k, lower trapezoidal)
-  for (int e = threadIdx.x; e < r * k; e += blockDim.x) {
-    const int i = e / r, j = e - i * r;
-    X[(size_t)i * ldx + j] = j >= i ? G[(size_t)j * rows + i] : 0.0;
-  }
-  __syncthreads();
-  house_qr(X, ldx, r, k, k, false, cn, sv, scr, bc);   // its reflectors are not needed
-  // L = R2^T in place: lower triangle from the upper one
-  for (int e = threadIdx.x; e < k * k; e += blockDim.x) {
-    const int c = e / k, q = e - c * k;
-    if (q > c) {
-      X[(size_t)c * ldx + q] = X[(size_t)q * ldx + c];
-      X[(size_t)q * ldx + c] = 0.0;
-    }
-  }
-  __syncthreads();
-  // one-sided Jacobi on L's columns, a group of eight lanes per pair
-  const int m = (k + 1) & ~1;
-  const double tol = 2.220446049250313e-16 * (double)rows;
-  const double tol2 = tol * tol;
-  const int half = m / 2, hround = ((half + ngrp - 1) / ngrp) * ngrp;
-  const int cround = ((k + ngrp - 1) / ngrp) * ngrp;
-  auto norms = [&]() {
-    for (int c = grp; c < cround; c += ngrp) {
-      double s = 0.0;
-      if (c < k)
-        for (int q = lane8; q < k; q += 8) s = fma(X[(size_t)c * ldx + q], X[(size_t)c * ldx + q], s);
-      s = group8_sum(s);
-      if (c < k && lane8 == 0) cn[c] = s;
-    }
-  };
-  for (int sweep = 0; sweep < 60; ++sweep) {
-    norms();
-    if (threadIdx.x == 0) rotated = 0;
-    __syncthreads();
-    for (int t = 0; t < m - 1; ++t) {
-      for (int h = grp; h < hround; h += ngrp) {
-        const int a = (h == 0) ? 0 : ((h - 1 + t) % (m - 1)) + 1;
-        const int b = ((m - 1 - h - 1 + t) % (m - 1)) + 1;
-        const int p = min(a, b), q = max(a, b);
-        const bool act = h < half && q < k;     // else idle group or dummy player
-        double *gp = X + (size_t)(act ? p : 0) * ldx, *gq = X + (size_t)(act ? q : 0) * ldx;
-        double ga = 0.0, al = 0.0, be = 0.0;
-        if (act) {
-          al = cn[p];               // every lane reads the norms before the group's sum, and
-          be = cn[q];               // lane 0 replaces them after it
-          for (int i = lane8; i < k; i += 8) ga = fma(gp[i], gq[i], ga);
-        }
-        ga = group8_sum(ga);
-        if (act) {
-          if (ga * ga > tol2 * (al * be)) {
-            const double zeta = (be - al) / (2.0 * ga);
-            double tt;
-            if (fabs(zeta) < 1e8) {
-              const float z = (float)zeta;
-              tt = (double)((z >= 0.f ? 1.f : -1.f) / (fabsf(z) + sqrtf(fmaf(z, z, 1.f))));
-            } else {
-              tt = 0.5 / zeta;
-            }
-            const double cs = rsqrt(fma(tt, tt, 1.0));
-            const double sn = cs * tt;
-            for (int i = lane8; i < k; i += 8) {
-              const double x = gp[i], y = gq[i];
-              gp[i] = cs * x - sn * y;
-              gq[i] = sn * x + cs * y;
-            }
-            if (lane8 == 0) {
-              cn[p] = fmax(fma(-tt, ga, al), 0.0);
-              cn[q] = fma(tt, ga, be);
-              rotated = 1;
-            }
-          }
-        }
-      }
-      __syncthreads();
-    }
-    if (!rotated) break;
-    __syncthreads();
-  }
-  norms();
-  __syncthreads();
-  for (int c = threadIdx.x; c < k; c += blockDim.x) {
-    sv[c] = sqrt(cn[c]);
-    order[c] = c;     // ranks of non-finite norms leave gaps
-  }
-  __syncthreads();
-  // descending order, ties by column index
-  for (int c = threadIdx.x; c < k; c += blockDim.x) {
-    int rank = 0;
-    const double s0 = sv[c];
-    for (int d = 0; d < k; ++d) {
-      const double s1 = sv[d];
-      if (s1 > s0 || (s1 == s0 && d < c)) ++rank;
-    }
-    order[rank] = c;
-  }
-  __syncthreads();
-  if (sigma)
-    for (int l = threadIdx.x; l < r; l += blockDim.x)
-      sigma[(size_t)J * r + l] = l < k ? sv[order[l]] : 0.0;
-  if (!T) return;
-  constexpr double kNullSigma = 1e-10;   // as in tentative_kernel
-  const double snull = kNullSigma * sv[order[0]];
-  // kept columns: U_l = Q (L_c / sigma_c), a warp per column
-  for (int l = wid; l < sJ && l < k; l += nwarps) {
-    const int c = order[l];
-    if (!(sv[c] > snull)) continue;
-    const double inv = 1.0 / sv[c];
-    double *u = U + (size_t)l * rows;
-    for (int q = lane; q < rows; q += 32) u[q] = q < k ? X[(size_t)c * ldx + q] * inv : 0.0;
-    __syncwarp();
-    for (int i = k - 1; i >= 0; --i) {
-      const double *v = G + (size_t)i * rows;
-      const double vi = vd[i];
-      double w = 0.0;
-      for (int q = i + 1 + lane; q < rows; q += 32) w = fma(v[q], u[q], w);
-      if (lane == 0) w = fma(vi, u[i], w);
-      w = warp_sum(w) * ff[i];
-      for (int q = i + 1 + lane; q < rows; q += 32) u[q] = fma(-w, v[q], u[q]);
-      if (lane == 0) u[i] = fma(-w, vi, u[i]);
-      __syncwarp();
-    }
-  }
-  __syncthreads();
-  // numerically null columns, in order: unit vectors e_t (t = l, l+1, ...
-  // cyclically) orthogonalised twice against the columns already fixed, the
-  // first with norm above 1/2 being kept
-  if (wid == 0) {
-    for (int l = 0; l < sJ && l < rows; ++l) {
-      if (l < k && sv[order[l]] > snull) continue;
-      double *u = U + (size_t)l * rows;
-      bool done = false;
-      for (int t = 0; t < rows && !done; ++t) {
-        const int e = (l + t) % rows;
-        for (int i = lane; i < rows; i += 32) u[i] = (i == e) ? 1.0 : 0.0;
-        __syncwarp();
-        for (int pass = 0; pass < 2; ++pass) {
-          for (int j = 0; j < l; ++j) {
-            const double *uj = U + (size_t)j * rows;
-            double d = 0.0;
-            for (int i = lane; i < rows; i += 32) d = fma(uj[i], u[i], d);
-            d = warp_sum(d);
-            for (int i = lane; i < rows; i += 32) u[i] = fma(-d, uj[i], u[i]);
-            __syncwarp();
-          }
-        }
-        double nn = 0.0;
-        for (int i = lane; i < rows; i += 32) nn = fma(u[i], u[i], nn);
-        nn = warp_sum(nn);
-        if (nn > 0.25) {
-          const double inv = 1.0 / sqrt(nn);
-          for (int i = lane; i < rows; i += 32) u[i] *= inv;
-          done = true;
-        }
-        __syncwarp();
-      }
-      if (!done && lane == 0) atomicExch(status, 1);
-    }
-  }
-  __syncthreads();
-  // sign so that the largest |entry| (lowest row on ties) is positive, then
-  // write; padding columns and padding rows of T are zero
-  for (int l = wid; l < s_next; l += nwarps) {
-    const bool ok = l < sJ && l < rows;
-    const double *u = U + (size_t)l * rows;
-    double best = -1.0;
-    int bi = INT_MAX;
-    for (int i = lane; ok && i < rows; i += 32) {
-      const double a = fabs(u[i]);
-      if (a > best) { best = a; bi = i; }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-    }
-    const double sgn = (ok && bi < rows && u[bi] < 0.0) ? -1.0 : 1.0;
-    for (int i = lane; i < rows; i += 32) T[(size_t)rowg[i] * s_next + l] = ok ? u[i] * sgn : 0.0;
-    if (unit_size)
-      for (int ch = 0; ch < nch; ++ch) {
-        const int un = child_idx[c0 + ch];
-        for (int d = unit_size[un] + lane; d < bs; d += 32)
-          T[((size_t)un * bs + d) * s_next + l] = 0.0;
-      }
-    if (l < sJ && !ok && lane == 0) atomicExch(status, 1);
-  }
-}
-
 // Padded level: the Galerkin product leaves the padding rows and columns of
 // A zero; put 1 on their diagonal so that the block inverses exist.  The
 // padding then stays exactly zero through every smoothing step.
@@ -853,34 +502,13 @@ cudaError_t launch_pad_identity(int n_units, int s_pad, const int *usize, const 
   return cudaGetLastError();
 }
 
-// The preconditioned kernel takes every aggregate whose block, its triangular
-// factor and the kept vectors fit in shared memory together; plain Jacobi
-// needs the block alone and keeps the largest ones.  Measured on both sides
-// down to r = 12 (2,048 aggregates of 12 x 12: 4.84 -> 0.78 ms) and r = 4.
 // shared memory holds the largest aggregate's rows x r block of B
 cudaError_t launch_tentative(int bs, int n_agg, int max_children, const int *child_ptr,
                                    const int *child_idx, const double *B, int64_t ldb, int r,
                                    int s_next, double *T, double *sigma, int *status,
                                    cudaStream_t s, const int *unit_size, const int *keep) {
   if (n_agg == 0) return cudaSuccess;
-  const size_t rows = (size_t)max_children * bs;
-  if (r <= kTentQrMaxR) {
-    const int k = (int)std::min<size_t>(rows, r);
-    const size_t sq = (rows * r + (size_t)(r | 1) * k + rows * s_next) * sizeof(double) +
-                      rows * sizeof(int);
-    if (sq <= 212 * 1024) {   // of 227 KB, beside 12 KB of static arrays
-      cudaError_t e = cudaFuncSetAttribute(tentative_qr_kernel,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sq);
-      if (e != cudaSuccess) return e;
-      int th = ((8 * ((k + 1) / 2) + 31) / 32) * 32;
-      th = th < 64 ? 64 : (th > 512 ? 512 : th);
-      launch_k(tentative_qr_kernel, n_agg, th, sq, s, bs, child_ptr, child_idx, B, ldb, r, s_next,
-               (int)rows, T, sigma, status, unit_size, keep);
-      note_launch();
-      return cudaGetLastError();
-    }
-  }
-  const size_t sm = rows * r * sizeof(double);
+  const size_t sm = (size_t)max_children * bs * r * sizeof(double);
   cudaError_t e = cudaFuncSetAttribute(tentative_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
