@@ -493,20 +493,25 @@ gasa_status dense_tail_build(gasa_ctx *ctx) {
     kt = k;
   }
   if (kt == N) return GASA_OK;
-  constexpr int K = 8;
   cudaStream_t s = ctx->stream;
   const int n = (int)ctx->L[kt].ndof;
   const int tpre = o.t_pre, tpost = o.t_post;
-  // scratch per level kt .. N: x, x2, b, r of K interleaved columns
-  size_t tot = 0;
-  for (int k = kt; k <= N; ++k) tot += 4 * (size_t)ctx->L[k].ndof * K;
+  // rows of M 128-byte aligned and 129 * 128 bytes apart for n = 2048 (a row
+  // pitch that is no power of two)
+  const int ld = ((n + 15) / 16) * 16 + 16;
+  // columns per pass: as many as keep the scratch (x, x2, b, r per level
+  // kt .. N) within the size of M, whose FP32 split follows when it is freed
+  size_t dofs = 0;
+  for (int k = kt; k <= N; ++k) dofs += (size_t)ctx->L[k].ndof;
+  const int C = std::min(n, std::max(64, (int)((size_t)n * ld / (4 * dofs)) / 32 * 32));
+  const size_t tot = 4 * dofs * C;
   double *scr = nullptr;
   ST(dalloc(ctx, &scr, tot));
   std::vector<double *> X(N + 1), X2(N + 1), B(N + 1), Rv(N + 1);
   {
     double *p = scr;
     for (int k = kt; k <= N; ++k) {
-      const size_t m = (size_t)ctx->L[k].ndof * K;
+      const size_t m = (size_t)ctx->L[k].ndof * C;
       X[k] = p;
       X2[k] = p + m;
       B[k] = p + 2 * m;
@@ -514,68 +519,62 @@ gasa_status dense_tail_build(gasa_ctx *ctx) {
       p += 4 * m;
     }
   }
-  // rows of M 128-byte aligned and 129 * 128 bytes apart for n = 2048 (a row
-  // pitch that is no power of two)
-  const int ld = ((n + 15) / 16) * 16 + 16;
   double *M = nullptr;
   gasa_status st = dalloc(ctx, &M, (size_t)n * ld);
-  if (st == GASA_OK) CU(cudaMemsetAsync(M, 0, (size_t)n * ld * sizeof(double), s));
   cudaError_t e = cudaSuccess;
   auto ok = [&](cudaError_t r) {
     if (e == cudaSuccess) e = r;
     return e == cudaSuccess;
   };
-  for (int c0 = 0; st == GASA_OK && e == cudaSuccess && c0 < n; c0 += K) {
+  if (st == GASA_OK) ok(cudaMemsetAsync(M, 0, (size_t)n * ld * sizeof(double), s));
+  for (int c0 = 0; st == GASA_OK && e == cudaSuccess && c0 < n; c0 += C) {
+    const int w = std::min(C, n - c0);
     std::vector<double *> xk(N + 1);
-    if (!ok(launch_bunit_columns(n, K, c0, B[kt], s))) break;
+    if (!ok(launch_mm_identity(n, c0, w, B[kt], s))) break;
+    auto mm = [&](int op, const DevBSR &m, const double *W, const double *x, const double *b,
+                  double *y) {
+      ok(launch_mm(op, m.nrows, m.br, m.bc, w, m.rp, m.col, m.val, W, x, b, y, s));
+    };
     for (int k = kt; k < N && e == cudaSuccess; ++k) {
       Level &l = ctx->L[k];
       double *x = X[k], *x2 = X2[k];
       if (tpre == 0) {
-        ok(cudaMemsetAsync(x, 0, (size_t)l.ndof * K * sizeof(double), s));
+        ok(cudaMemsetAsync(x, 0, (size_t)l.ndof * w * sizeof(double), s));
       } else {
-        ok(launch_bjacobi<double>(JAC_FIRST, l.n, l.s, l.A.rp, l.A.col, l.A.val, l.W, nullptr,
-                                  B[k], x, K, s, l.A.nnzb));
+        mm(MM_FIRST, l.A, l.W, nullptr, B[k], x);
         for (int t = 1; t < tpre; ++t) {
-          ok(launch_bjacobi<double>(JAC_SWEEP, l.n, l.s, l.A.rp, l.A.col, l.A.val, l.W, x, B[k],
-                                    x2, K, s, l.A.nnzb));
+          mm(MM_SWEEP, l.A, l.W, x, B[k], x2);
           std::swap(x, x2);
         }
       }
       xk[k] = x;
-      ok(launch_bmv<double>(GASA_MV_RESIDUAL, l.n, l.s, l.s, l.A.rp, l.A.col, l.A.val, x, B[k],
-                            Rv[k], K, s, l.A.nnzb));
-      ok(launch_bmv<double>(GASA_MV_ASSIGN, l.R.nrows, l.R.br, l.R.bc, l.R.rp, l.R.col, l.R.val,
-                            Rv[k], nullptr, B[k + 1], K, s, l.R.nnzb));
+      mm(MM_RESIDUAL, l.A, nullptr, x, B[k], Rv[k]);
+      mm(MM_ASSIGN, l.R, nullptr, Rv[k], nullptr, B[k + 1]);
     }
-    ok(launch_bdense<double>(ctx->nc, ctx->coarse_inv, B[N], X[N], K, s));
+    ok(launch_mm_dense(ctx->nc, w, ctx->coarse_inv, B[N], X[N], s));
     xk[N] = X[N];
     for (int k = N - 1; k >= kt && e == cudaSuccess; --k) {
       Level &l = ctx->L[k];
       double *x = xk[k];
       double *x2 = (x == X[k]) ? X2[k] : X[k];
-      ok(launch_bmv<double>(GASA_MV_ADD, l.P.nrows, l.P.br, l.P.bc, l.P.rp, l.P.col, l.P.val,
-                            xk[k + 1], nullptr, x, K, s, l.P.nnzb));
+      mm(MM_ADD, l.P, nullptr, xk[k + 1], nullptr, x);
       for (int t = 0; t < tpost; ++t) {
-        ok(launch_bjacobi<double>(JAC_SWEEP, l.n, l.s, l.A.rp, l.A.col, l.A.val, l.W, x, B[k], x2,
-                                  K, s, l.A.nnzb));
+        mm(MM_SWEEP, l.A, l.W, x, B[k], x2);
         std::swap(x, x2);
       }
       xk[k] = x;
     }
-    // row i of the K interleaved columns is M[i][c0 .. c0 + K)
-    const int w = std::min(K, n - c0);
-    ok(cudaMemcpy2DAsync(M + c0, (size_t)ld * sizeof(double), xk[kt], K * sizeof(double),
-                         w * sizeof(double), n, cudaMemcpyDeviceToDevice, s));
+    ok(cudaMemcpy2DAsync(M + c0, (size_t)ld * sizeof(double), xk[kt], (size_t)w * sizeof(double),
+                         (size_t)w * sizeof(double), n, cudaMemcpyDeviceToDevice, s));
   }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  dfree(ctx, scr);
+  ctx->device_bytes -= (int64_t)(tot * sizeof(double));
   // the FP32 cycle applies M from its exact two-term FP32 split
   float *Mh = nullptr, *Ml = nullptr;
   if (st == GASA_OK) st = dalloc(ctx, &Mh, (size_t)n * ld);
   if (st == GASA_OK) st = dalloc(ctx, &Ml, (size_t)n * ld);
   if (st == GASA_OK && e == cudaSuccess) e = launch_split((int64_t)n * ld, M, Mh, Ml, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  dfree(ctx, scr);
-  ctx->device_bytes -= (int64_t)(tot * sizeof(double));
   if (st != GASA_OK) return st;
   CU(e);
   ctx->dtail_Mh = Mh;

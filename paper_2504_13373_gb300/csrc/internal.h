@@ -271,6 +271,16 @@ cudaError_t launch_numeric_AB(int n, int br, int bm, int bc, const int *Arp, con
 cudaError_t launch_transpose(int n_rows, int n_cols, int br, int bc, const int *Prp,
                              const int *Pcol, const double *Pval, int *Rrp, int *Rcol,
                              double *Rval, int *scratch_pos, int *scratch_cnt, cudaStream_t s);
+// products and smoothing steps on ncol columns at once (FP64; X, B, Y row-major,
+// entry i of column c at i * ncol + c; br <= 192): Y = A X, B - A X, Y + A X,
+// X + W (B - A X), W B
+enum MmOp { MM_ASSIGN = 0, MM_RESIDUAL = 1, MM_ADD = 2, MM_SWEEP = 3, MM_FIRST = 4 };
+cudaError_t launch_mm(int op, int n_brows, int br, int bc, int ncol, const int *rp, const int *col,
+                      const double *val, const double *W, const double *X, const double *B,
+                      double *Y, cudaStream_t s);
+cudaError_t launch_mm_identity(int n, int c0, int ncol, double *X, cudaStream_t s);
+cudaError_t launch_mm_dense(int n, int ncol, const double *A, const double *X, double *Y,
+                            cudaStream_t s);
 cudaError_t launch_bsr_to_dense(int n, int bs, const int *rp, const int *col, const double *val,
                                 double *D, cudaStream_t s);
 cudaError_t launch_dense_inverse(int n, const double *A, double *Ainv, double *work,

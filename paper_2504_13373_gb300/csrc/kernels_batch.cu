@@ -739,15 +739,6 @@ __global__ void bcolcopy_kernel(int64_t n, int K, int c, const T *__restrict__ s
   if (i < n) dst[i * K + c] = src[i * K + c];
 }
 
-// B (n x K interleaved) = columns c0 .. c0 + K - 1 of the n x n identity
-// (columns past n are zero)
-__global__ void bunit_columns_kernel(int n, int K, int c0, double *__restrict__ B) {
-  const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  if (t >= (int64_t)n * K) return;
-  const int64_t i = t / K, c = t - i * K;
-  B[t] = (i == c0 + c) ? 1.0 : 0.0;
-}
-
 // X = A B for a dense row-major n x n FP64 A and K interleaved columns, FP64
 // arithmetic: a warp per row, lane l takes columns j = l, l + 32, ... of the
 // row in order (four rows of B in flight), then an xor-shuffle tree; a
@@ -1051,13 +1042,6 @@ cudaError_t launch_bscatter(int64_t n, int K, int c, const T *src, T *dst, cudaS
 template <typename T>
 cudaError_t launch_bgather(int64_t n, int K, int c, const T *src, T *dst, cudaStream_t s) {
   launch_k(bgather_kernel<T>, div_up(n, kThreads), kThreads, 0, s, n, K, c, src, dst);
-  note_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_bunit_columns(int n, int K, int c0, double *B, cudaStream_t s) {
-  if (n <= 0 || K <= 0) return cudaSuccess;
-  launch_k(bunit_columns_kernel, div_up((int64_t)n * K, kThreads), kThreads, 0, s, n, K, c0, B);
   note_launch();
   return cudaGetLastError();
 }

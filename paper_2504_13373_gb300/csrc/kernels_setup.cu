@@ -934,6 +934,143 @@ cudaError_t launch_transpose(int n_rows, int n_cols, int br, int bc, const int *
 }
 
 // ----------------------------------------------------------------------------
+// block-sparse products and smoothing steps on many columns at once (setup of
+// the dense bottom operator: the columns of the identity).  X, B and Y are
+// row-major with the columns contiguous (entry i of column c at i * ncol + c),
+// FP64 throughout.
+//
+// A CTA owns `units` block rows and 32 columns, a lane per column, so X is read
+// in 256-byte runs and a matrix value is one broadcast load for 32 FMAs; its
+// warps take the scalar rows in turn, and a smoothing step meets the block
+// row's residual in shared memory.  Sums run in block order, then column
+// order.  An SM does two FP64 FMAs a clock, so this is bound by that as soon as
+// there are columns enough; eight columns per launch were not enough (levels of
+// 48 units: 63 us a step for 9 us of FMAs).  Setting up the operator of a P2
+// 8^3 tet hierarchy (order 816) took 47 ms in eight-column passes and takes
+// 9.9 ms, 6.4 of them FMAs; order 2,048 with 4 x 4 blocks 138 -> 11.4 ms.
+// ----------------------------------------------------------------------------
+constexpr int kMmRows = 4;        // rows a warp carries at once, at most
+constexpr int kMmWarps = 8;
+
+// the product of CNT rows (kMmWarps apart) of block row u with column c; CNT is
+// a constant because a predicated-off FP64 instruction takes the pipe as long
+// as one that runs
+template <int CNT>
+__device__ __forceinline__ void mm_rows(int beg, int end, int br, int bc, int ncol,
+                                        const int *__restrict__ col, const double *__restrict__ a0,
+                                        const double *__restrict__ Xc, double *acc) {
+  for (int k = beg; k < end; ++k) {
+    const double *ab = a0 + (size_t)k * br * bc;
+    const double *x = Xc + (size_t)__ldg(col + k) * bc * ncol;
+#pragma unroll 4
+    for (int m = 0; m < bc; ++m) {
+      const double xv = __ldg(x + (size_t)m * ncol);
+#pragma unroll
+      for (int q = 0; q < CNT; ++q)
+        acc[q] = fma(__ldg(ab + (size_t)q * kMmWarps * bc + m), xv, acc[q]);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(32 * kMmWarps)
+mm_kernel(int op, int n_brows, int br, int bc, int units, int ncol, const int *__restrict__ rp,
+          const int *__restrict__ col, const double *__restrict__ val,
+          const double *__restrict__ W, const double *__restrict__ X,
+          const double *__restrict__ B, double *__restrict__ Y) {
+  extern __shared__ double res[];       // [units * br][32], smoothing steps only
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const bool on = (int)(blockIdx.y * 32 + lane) < ncol;
+  const int c = on ? blockIdx.y * 32 + lane : 0;    // lanes past the last column repeat column 0
+  const int u0 = blockIdx.x * units;
+  const int nrow = min(units, n_brows - u0) * br;
+  const bool smooth = op == MM_SWEEP || op == MM_FIRST;
+  for (int t = wid; t < nrow; ) {
+    // rows t, t + 8, ... inside one block row share its loads of X
+    const int lu = t / br, u = u0 + lu, r0 = t - lu * br;
+    const int cnt = min(kMmRows, (br - r0 - 1) / kMmWarps + 1);
+    double acc[kMmRows] = {};
+    if (op != MM_FIRST) {
+      const int beg = __ldg(rp + u), end = __ldg(rp + u + 1);
+      const double *a0 = val + (size_t)r0 * bc;
+      switch (cnt) {
+        case 1: mm_rows<1>(beg, end, br, bc, ncol, col, a0, X + c, acc); break;
+        case 2: mm_rows<2>(beg, end, br, bc, ncol, col, a0, X + c, acc); break;
+        case 3: mm_rows<3>(beg, end, br, bc, ncol, col, a0, X + c, acc); break;
+        default: mm_rows<4>(beg, end, br, bc, ncol, col, a0, X + c, acc); break;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kMmRows; ++q) {
+      if (q >= cnt) break;
+      const int tq = t + q * kMmWarps;
+      const size_t e = ((size_t)u0 * br + tq) * ncol + c;
+      if (smooth) res[tq * 32 + lane] = B[e] - acc[q];
+      else if (on) Y[e] = op == MM_RESIDUAL ? B[e] - acc[q] : op == MM_ADD ? Y[e] + acc[q] : acc[q];
+    }
+    t += cnt * kMmWarps;
+  }
+  if (!smooth) return;
+  __syncthreads();
+  for (int t = wid; t < nrow; t += kMmWarps) {
+    const int lu = t / br;
+    const double *w = W + ((size_t)u0 * br + t) * br;
+    const double *rl = res + (size_t)lu * br * 32 + lane;
+    double out = 0.0;
+#pragma unroll 4
+    for (int m = 0; m < br; ++m) out = fma(__ldg(w + m), rl[m * 32], out);
+    const size_t e = ((size_t)u0 * br + t) * ncol + c;
+    if (on) Y[e] = op == MM_SWEEP ? X[e] + out : out;
+  }
+}
+
+cudaError_t launch_mm(int op, int n_brows, int br, int bc, int ncol, const int *rp, const int *col,
+                      const double *val, const double *W, const double *X, const double *B,
+                      double *Y, cudaStream_t s) {
+  if (n_brows == 0 || ncol == 0) return cudaSuccess;
+  const int units = br >= kMmWarps ? 1 : div_up(kMmWarps, br);
+  const bool smooth = op == MM_SWEEP || op == MM_FIRST;
+  const size_t sm = smooth ? (size_t)units * br * 32 * sizeof(double) : 0;   // 48 KB at br = 192
+  launch_k(mm_kernel, dim3(div_up(n_brows, units), div_up(ncol, 32)), 32 * kMmWarps, sm, s, op,
+           n_brows, br, bc, units, ncol, rp, col, val, W, X, B, Y);
+  note_launch();
+  return cudaGetLastError();
+}
+
+// X = columns c0 .. c0 + ncol - 1 of the n x n identity, or Y = A X for a dense
+// row-major n x n A (a warp per row and 32 columns, in column order)
+__global__ void mm_identity_kernel(int n, int c0, int ncol, double *__restrict__ X) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (int64_t)n * ncol) return;
+  X[t] = t / ncol == c0 + t % ncol ? 1.0 : 0.0;
+}
+cudaError_t launch_mm_identity(int n, int c0, int ncol, double *X, cudaStream_t s) {
+  if (n == 0 || ncol == 0) return cudaSuccess;
+  launch_k(mm_identity_kernel, div_up((int64_t)n * ncol, 256), 256, 0, s, n, c0, ncol, X);
+  note_launch();
+  return cudaGetLastError();
+}
+
+__global__ void __launch_bounds__(256)
+mm_dense_kernel(int n, int ncol, const double *__restrict__ A, const double *__restrict__ X,
+                double *__restrict__ Y) {
+  const int lane = threadIdx.x & 31;
+  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), c = blockIdx.y * 32 + lane;
+  if (row >= n || c >= ncol) return;
+  double acc = 0.0;
+#pragma unroll 8
+  for (int j = 0; j < n; ++j)
+    acc = fma(__ldg(A + (size_t)row * n + j), __ldg(X + (size_t)j * ncol + c), acc);
+  Y[(size_t)row * ncol + c] = acc;
+}
+cudaError_t launch_mm_dense(int n, int ncol, const double *A, const double *X, double *Y,
+                            cudaStream_t s) {
+  if (n == 0 || ncol == 0) return cudaSuccess;
+  launch_k(mm_dense_kernel, dim3(div_up(n, 8), div_up(ncol, 32)), 256, 0, s, n, ncol, A, X, Y);
+  note_launch();
+  return cudaGetLastError();
+}
+
+// ----------------------------------------------------------------------------
 // coarsest level: BSR -> dense row-major, Gauss-Jordan inverse on [A | I]
 // ----------------------------------------------------------------------------
 __global__ void bsr_to_dense_kernel(int n, int bs, const int *__restrict__ rp,
