@@ -1560,7 +1560,7 @@ gasa_status spgemm(gasa_ctx *ctx, const DevBSR &A, const DevBSR &B, DevBSR &C,
   ST(dalloc(ctx, &C.val, (size_t)nnz * C.br * C.bc));
   CU(launch_pattern_AB(n, A.rp, A.col, B.rp, B.col, nullptr, C.rp, C.col, maxc, B.ncols, s));
   CU(launch_numeric_AB(n, A.br, A.bc, B.bc, A.rp, A.col, A.val, B.rp, B.col, B.val, C.rp, C.col,
-                       C.val, s));
+                       C.val, C.nnzb, s));
   CU(cudaStreamSynchronize(s));
   dfree(ctx, cand);
   dfree(ctx, mx);
@@ -1845,8 +1845,7 @@ gasa_status setup_impl(gasa_ctx *ctx, const gasa_bsr *Ain, const int32_t *adj_pt
         std::vector<const double *> tab(r);
         for (int c = 0; c < r; ++c) tab[c] = cur[c];
         CU(cudaMemcpyAsync(ptab, tab.data(), sizeof(double *) * r, cudaMemcpyHostToDevice, s));
-        CU(launch_colnorm_partials(nd, (const double *const *)ptab, r, ctx->part, s));
-        CU(launch_finalize(ctx->part, r, nrmbuf, s));
+        CU(launch_colnorms(nd, (const double *const *)ptab, r, ctx->part, nrmbuf, s));
         CU(cudaMemcpyAsync(nrm.data(), nrmbuf, sizeof(double) * r, cudaMemcpyDeviceToHost, s));
         CU(cudaStreamSynchronize(s));
         for (auto &v : nrm) v = std::sqrt(v);
@@ -1862,8 +1861,7 @@ gasa_status setup_impl(gasa_ctx *ctx, const gasa_bsr *Ain, const int32_t *adj_pt
         CU(cudaMemcpyAsync(ptab, tab.data(), sizeof(double *) * 2 * na, cudaMemcpyHostToDevice, s));
         CU(launch_relax_multi(l.n, l.s, l.A.rp, l.A.col, l.A.val, l.W, (const double *const *)ptab,
                               (double *const *)(ptab + na), na, s));
-        CU(launch_colnorm_partials(nd, (const double *const *)(ptab + na), na, ctx->part, s));
-        CU(launch_finalize(ctx->part, na, nrmbuf, s));
+        CU(launch_colnorms(nd, (const double *const *)(ptab + na), na, ctx->part, nrmbuf, s));
         CU(cudaMemcpyAsync(nn.data(), nrmbuf, sizeof(double) * na, cudaMemcpyDeviceToHost, s));
         CU(cudaStreamSynchronize(s));
         std::vector<int> still;
@@ -2694,8 +2692,7 @@ gasa_status gasa_relax_candidates(int32_t n_units, int32_t bs, const int32_t *ro
   if (e == cudaSuccess) {
     for (int c = 0; c < r; ++c) htab[c] = cur[c];
     e = cudaMemcpyAsync(tab, htab.data(), sizeof(double *) * r, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = launch_colnorm_partials(n, (const double *const *)tab, r, part, s);
-    if (e == cudaSuccess) e = launch_finalize(part, r, nr, s);
+    if (e == cudaSuccess) e = launch_colnorms(n, (const double *const *)tab, r, part, nr, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(nrm.data(), nr, sizeof(double) * r, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     for (auto &v : nrm) v = std::sqrt(v);
@@ -2710,8 +2707,7 @@ gasa_status gasa_relax_candidates(int32_t n_units, int32_t bs, const int32_t *ro
     if (e == cudaSuccess)
       e = launch_relax_multi(n_units, bs, row_ptr, col, val, W, (const double *const *)tab,
                              (double *const *)(tab + na), na, s);
-    if (e == cudaSuccess) e = launch_colnorm_partials(n, (const double *const *)(tab + na), na, part, s);
-    if (e == cudaSuccess) e = launch_finalize(part, na, nr, s);
+    if (e == cudaSuccess) e = launch_colnorms(n, (const double *const *)(tab + na), na, part, nr, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(nn.data(), nr, sizeof(double) * na, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) break;

@@ -164,9 +164,9 @@ cudaError_t launch_dense_mv_ds(int n, int ld, const float *Mh, const float *Ml, 
 // partials[kRedBlocks] of sum_i x_i y_i (y == nullptr: sum x_i^2)
 cudaError_t launch_dot_partials(int64_t n, const double *x, const double *y, double *partials,
                                 cudaStream_t s);
-// multi-column squared norms: partials[c * kRedBlocks + blk]
-cudaError_t launch_colnorm_partials(int64_t n, const double *const *cols, int nc,
-                                    double *partials, cudaStream_t s);
+// multi-column squared norms out[c]; partials: at least kRedBlocks * nc doubles of scratch
+cudaError_t launch_colnorms(int64_t n, const double *const *cols, int nc, double *partials,
+                            double *out, cudaStream_t s);
 // out[c] = sum of partials of column c (one block per column)
 cudaError_t launch_finalize(const double *partials, int nc, double *out, cudaStream_t s);
 // out[0] = sum of n partials
@@ -267,7 +267,7 @@ cudaError_t launch_numeric_P(int n, int sk, int sn, const int *Arp, const int *A
 cudaError_t launch_numeric_AB(int n, int br, int bm, int bc, const int *Arp, const int *Acol,
                               const double *Aval, const int *Brp, const int *Bcol,
                               const double *Bval, const int *Crp, const int *Ccol,
-                              double *Cval, cudaStream_t s);
+                              double *Cval, int64_t nnzb, cudaStream_t s);
 cudaError_t launch_transpose(int n_rows, int n_cols, int br, int bc, const int *Prp,
                              const int *Pcol, const double *Pval, int *Rrp, int *Rcol,
                              double *Rval, int *scratch_pos, int *scratch_cnt, cudaStream_t s);

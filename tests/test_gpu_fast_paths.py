@@ -79,4 +79,4 @@ def test_tentative_packed_sums(n_units, bs, size, r, s_next):
         eps = 1e-15 * max(rows.size, r)
         assert np.max(np.abs(sg[J, :s.size] - s)) <= eps * s[0]
         assert np.max(np.abs(Tg[rows] - Td)) <= 10 * eps / gap, J
-        assert np.max(np.abs(Tg[rows].T @ Tg[rows] - np.eye(s_next))) <= 1e-8
+        assert np.max(np.abs(Tg[rows].T @ Tg[rows] - np.eye(s_next))) <= 1e-12
