@@ -53,23 +53,27 @@ template <typename T>
 cudaError_t launch_bdense(int nc, const double *Ainv, const T *B, T *X, int K, cudaStream_t s,
                           int ld = 0);
 
+// X = M B from the exact two-term FP32 split of M (row pitch ld), double-single arithmetic
+cudaError_t launch_bdense_ds(int n, int ld, const float *Mh, const float *Ml, const float *B,
+                             float *X, int K, cudaStream_t s);
+
+// partial sums of x . y (y null: x . x) and, with Z, of x . z; the launchers
+// that add partials up take the n of the dot product
 cudaError_t launch_bdot(int64_t n, const double *X, const double *Y, double *part, int K,
-                        cudaStream_t s);
-cudaError_t launch_bfinalize(const double *part, double *out, int K, cudaStream_t s);
-cudaError_t launch_bnorm(const double *part, double *out, int K, cudaStream_t s);
+                        cudaStream_t s, const double *Z = nullptr, double *part2 = nullptr);
+cudaError_t launch_bfinalize(int64_t n, const double *part, double *out, int K, cudaStream_t s);
+cudaError_t launch_bnorm(int64_t n, const double *part, double *out, int K, cudaStream_t s);
 cudaError_t launch_bnormalize(int64_t n, const double *w, const double *nrm, double *v, int K,
                               cudaStream_t s);
 
-cudaError_t launch_bcg_beta(const double *part_rz, const double *part_rzo, double *sc,
-                            const int *st, int flex, int K, cudaStream_t s);
 cudaError_t launch_bcg_update_p(int64_t n, double *p, const double *z, double *zold,
-                                const double *sc, int K, cudaStream_t s);
-cudaError_t launch_bcg_alpha(const double *part_pq, double *sc, const int *st, int K,
-                             cudaStream_t s);
+                                const double *part_rz, const double *part_rzo, double *sc,
+                                const int *st, int flex, int K, cudaStream_t s);
 cudaError_t launch_bcg_update_xr(int64_t n, double *x, double *r, const double *p, const double *q,
-                                 const double *sc, double *part_rr, int K, cudaStream_t s);
-cudaError_t launch_bcg_check(const double *part_rr, double *sc, int *st, int *ctl, int flex,
-                             cudaGraphConditionalHandle h, int K, cudaStream_t s);
+                                 const double *part_pq, double *sc, const int *st, double *part_rr,
+                                 int K, cudaStream_t s);
+cudaError_t launch_bcg_check(int64_t n, const double *part_rr, double *sc, int *st, int *ctl,
+                             int flex, cudaGraphConditionalHandle h, int K, cudaStream_t s);
 
 // GMRES: the Arnoldi step j is read from device memory (*dj)
 cudaError_t launch_bgm_load(int64_t nk, const double *base, int64_t ld, const int *dj, int off,
@@ -78,11 +82,11 @@ cudaError_t launch_bgm_store(int64_t nk, const double *src, double *base, int64_
                              int off, cudaStream_t s);
 cudaError_t launch_bmulti_dot(int64_t n, const double *V, int64_t ldv, int max_k, const int *dj,
                               const double *w, double *part, int K, cudaStream_t s);
-cudaError_t launch_bmulti_finalize(const double *part, int m, const int *dj, double *h, double *H,
-                                   int accumulate, int K, cudaStream_t s);
+cudaError_t launch_bmulti_finalize(int64_t n, const double *part, int m, const int *dj, double *h,
+                                   double *H, int accumulate, int K, cudaStream_t s);
 cudaError_t launch_bgs_update(int64_t n, const double *V, int64_t ldv, const int *dj, const double *h,
                               double *w, int K, cudaStream_t s);
-cudaError_t launch_bgm_norm(const double *part, int m, const int *dj, double *H, int K,
+cudaError_t launch_bgm_norm(int64_t n, const double *part, int m, const int *dj, double *H, int K,
                             cudaStream_t s);
 cudaError_t launch_bgm_normalize(int64_t n, const double *w, const double *H, int m, const int *dj,
                                  double *V, int K, cudaStream_t s);
@@ -94,7 +98,7 @@ cudaError_t launch_bgm_backsolve(int m, const double *H, const double *g, double
                                  int K, cudaStream_t s);
 cudaError_t launch_bgm_combine(int64_t n, const double *Bv, int64_t ldb, const double *y,
                                const int *st, double *x, int K, cudaStream_t s);
-cudaError_t launch_bgm_check(const double *part_rr, double *sc, int *st, int K, cudaStream_t s);
+cudaError_t launch_bgm_check(int64_t n, const double *part_rr, double *sc, int *st, int K, cudaStream_t s);
 
 template <typename T>
 cudaError_t launch_bscatter(int64_t n, int K, int c, const T *src, T *dst, cudaStream_t s);

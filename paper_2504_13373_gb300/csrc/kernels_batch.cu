@@ -54,6 +54,144 @@ __device__ __forceinline__ void row_dot_k(int beg, int end, int r, int br, int b
 }
 
 // ---------------------------------------------------------------------------
+// Served meshes of a few thousand rows: eight slices per scalar row.  A thread
+// per row leaves most SMs empty and walks its 40 to 700 values one dependent
+// load after another; here the row's values are dealt to eight lanes (slice q
+// takes entries q, q + 8, ... of the row), each for two of the K columns, so a
+// row is 4 K lanes that read whole runs of A and X, and the slices' sums meet
+// in a shuffle tree (slices 4, 2, 1 apart).  The slicing depends on the matrix
+// alone, so a column's bits do not depend on K.  Launch-latency bound:
+// 5,120 to 9,216 dofs, K = 8, GB300: smoothing step 12.1 -> 9.9 us, product
+// 17.1 -> 9.1 us on average over a V-cycle's, FP64 outer product 37.1 ->
+// 11.5 us (three engines at once).
+// ---------------------------------------------------------------------------
+template <int K>
+struct Slices {
+  static constexpr int C = K < 2 ? 1 : 2;      // columns per lane
+  static constexpr int CG = K / C;             // lanes side by side on one entry
+  static constexpr int lanes = 8 * CG;         // lanes per scalar row
+};
+
+// Sum over `len` entries dealt to the slices: entry f of the row is a(f) and
+// x(f) points at its K columns.  Returns the sum of column column_of(sub).
+template <typename T, int K, typename FA, typename FX>
+__device__ __forceinline__ T sliced_sum(int sub, int len, FA a, FX x) {
+  using S = Slices<K>;
+  const int sl = sub / S::CG, cg = sub % S::CG;
+  T acc[S::C];
+#pragma unroll
+  for (int c = 0; c < S::C; ++c) acc[c] = T(0);
+#pragma unroll 4
+  for (int f = sl; f < len; f += 8) {
+    const T av = a(f);
+    const T *xp = x(f) + cg * S::C;
+#pragma unroll
+    for (int c = 0; c < S::C; ++c) acc[c] = fma(av, xp[c], acc[c]);
+  }
+  T v;
+  if constexpr (S::C == 2) {
+    const bool hi = sl & 4;                    // carries on with the second column
+    v = (hi ? acc[1] : acc[0]) + __shfl_xor_sync(0xffffffffu, hi ? acc[0] : acc[1], 4 * S::CG);
+  } else {
+    v = acc[0] + __shfl_xor_sync(0xffffffffu, acc[0], 4 * S::CG);
+  }
+  v += __shfl_xor_sync(0xffffffffu, v, 2 * S::CG);
+  v += __shfl_xor_sync(0xffffffffu, v, S::CG);
+  return v;
+}
+template <int K>
+__device__ __forceinline__ int column_of(int sub) {
+  using S = Slices<K>;
+  return (sub % S::CG) * S::C + (S::C == 2 && (sub / S::CG & 4) ? 1 : 0);
+}
+// one lane per column stores
+template <int K>
+__device__ __forceinline__ bool stores(int sub) {
+  using S = Slices<K>;
+  return S::C == 2 ? (sub / S::CG & 3) == 0 : sub == 0;
+}
+
+// sliced sum of scalar row r of block row [beg, end)
+template <typename T, int K>
+__device__ __forceinline__ T sliced_row(int sub, int beg, int end, int r, int br, int bc,
+                                        const int *__restrict__ col, const T *__restrict__ val,
+                                        const T *__restrict__ X) {
+  const T *a0 = val + ((size_t)beg * br + r) * bc;
+  const size_t bstep = (size_t)(br - 1) * bc;     // skip of one block beyond its row r
+  return sliced_sum<T, K>(
+      sub, (end - beg) * bc,
+      [&](int f) { return __ldg(a0 + f + (f / bc) * bstep); },
+      [&](int f) {
+        const int k = f / bc;
+        return X + ((size_t)__ldg(col + beg + k) * bc + (f - k * bc)) * K;
+      });
+}
+
+template <typename T, int K>
+__global__ void __launch_bounds__(kThreads)
+bmv_sliced_kernel(int mode, int64_t n_rows, int br, int bc, const int *__restrict__ rp,
+                  const int *__restrict__ col, const T *__restrict__ val, const T *__restrict__ X,
+                  const T *__restrict__ B, T *__restrict__ Y) {
+  constexpr int L = Slices<K>::lanes;
+  const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  const int sub = (int)(t % L);
+  const bool on = t / L < n_rows;
+  const int64_t row = on ? t / L : n_rows - 1;
+  const int i = (int)(row / br);
+  const int r = (int)(row - (int64_t)i * br);
+  const T v = sliced_row<T, K>(sub, __ldg(rp + i), __ldg(rp + i + 1), r, br, bc, col, val, X);
+  if (!on || !stores<K>(sub)) return;
+  const size_t e = (size_t)row * K + column_of<K>(sub);
+  Y[e] = mode == GASA_MV_RESIDUAL ? B[e] - v : mode == GASA_MV_ADD ? Y[e] + v : v;
+}
+
+// block-Jacobi step, `units` whole block rows per CTA (blockDim = units * bs rows' lanes,
+// rounded up to warps)
+template <typename T, int K>
+__global__ void __launch_bounds__(1024)
+bjacobi_sliced_kernel(int mode, int n, int bs, int units, const int *__restrict__ rp,
+                      const int *__restrict__ col, const T *__restrict__ A,
+                      const T *__restrict__ W, const T *__restrict__ X, const T *__restrict__ B,
+                      T *__restrict__ Xo) {
+  constexpr int L = Slices<K>::lanes;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T *res = reinterpret_cast<T *>(smem_raw);          // [units * bs][K]
+  const int sub = threadIdx.x % L;
+  const int u0 = blockIdx.x * units;
+  const int nrow = min(units, n - u0) * bs;
+  const int step = blockDim.x / L;
+  const int rounds = (nrow + step - 1) / step;
+  for (int it = 0; it < rounds; ++it) {
+    const int t = threadIdx.x / L + it * step;
+    const bool on = t < nrow;
+    const int tr = on ? t : nrow - 1;
+    const int i = u0 + tr / bs, r = tr % bs;
+    T v = T(0);
+    if (mode == JAC_SWEEP)
+      v = sliced_row<T, K>(sub, __ldg(rp + i), __ldg(rp + i + 1), r, bs, bs, col, A, X);
+    if (on && stores<K>(sub)) {
+      const int c = column_of<K>(sub);
+      const T b = B[((size_t)u0 * bs + t) * K + c];
+      res[t * K + c] = mode == JAC_SWEEP ? b - v : b;
+    }
+  }
+  __syncthreads();
+  for (int it = 0; it < rounds; ++it) {
+    const int t = threadIdx.x / L + it * step;
+    const bool on = t < nrow;
+    const int tr = on ? t : nrow - 1;
+    const T *w = W + ((size_t)u0 * bs + tr) * bs;
+    const T *rl = res + (size_t)(tr / bs) * bs * K;
+    const T v = sliced_sum<T, K>(sub, bs, [&](int f) { return __ldg(w + f); },
+                                 [&](int f) { return rl + f * K; });
+    if (on && stores<K>(sub)) {
+      const size_t g = ((size_t)u0 * bs + t) * K + column_of<K>(sub);
+      Xo[g] = mode == JAC_SWEEP ? X[g] + v : v;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
 // block SpMV over K columns: Y = A X, Y += A X or Y = B - A X.  Short rows:
 // one thread per scalar row computes all K columns (each matrix value is
 // read once per batch); long rows (coarse levels): one warp per scalar row.
@@ -325,64 +463,112 @@ bdense_kernel(int nc, int ld, const double *__restrict__ Ainv, const T *__restri
 }
 
 // ---------------------------------------------------------------------------
-// per-column reductions on a fixed grid of kRedBlocks CTAs.  Thread t of CTA
-// blk takes rows blk * 256 + t, + kRedBlocks * 256, ... for all K columns,
-// then a fixed tree over the 256 threads: the partial sums of a column do not
-// depend on K, on the slot or on the other columns.
+// per-column reductions on a grid of nb = bred_blocks(n) CTAs (kRedBlocks at
+// most).  Thread t of CTA blk takes rows blk * 256 + t, + nb * 256, ... for all
+// K columns, then a fixed tree: a shuffle tree over the warp, the warps in
+// order.  The partial sums of a column do not depend on K, on the slot or on
+// the other columns.  The warp's tree is packed: at each distance half of the
+// lanes carry on with half of the columns, so K columns cost K + 1 FP64
+// additions a warp and not 5 K (an FP64 instruction takes an SM quarter 64
+// clocks whatever its active lanes).
 // ---------------------------------------------------------------------------
-template <int K>
-__device__ __forceinline__ void column_tree(const double (&acc)[K], double *part) {
-  __shared__ double sh[K][kThreads];
-#pragma unroll
-  for (int c = 0; c < K; ++c) sh[c][threadIdx.x] = acc[c];
-  __syncthreads();
-  for (int s = kThreads / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) {
-#pragma unroll
-      for (int c = 0; c < K; ++c) sh[c][threadIdx.x] += sh[c][threadIdx.x + s];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x < K) part[(size_t)threadIdx.x * kRedBlocks + blockIdx.x] = sh[threadIdx.x][0];
+int bred_blocks(int64_t n) {
+  return (int)std::min<int64_t>(kRedBlocks, std::max<int64_t>(1, (n + kThreads - 1) / kThreads));
 }
 
-// part[c * kRedBlocks + blk]: partial sums of x_c . y_c (y null: x_c . x_c)
+// sums of K <= 8 quantities over the warp; the sum of column c ends in the
+// lanes whose upper log2(K) bits are c
 template <int K>
+__device__ __forceinline__ double warp_columns(const double (&acc)[K], int lane) {
+  double v[K];
+#pragma unroll
+  for (int c = 0; c < K; ++c) v[c] = acc[c];
+  int width = K;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    if (width > 1) {
+      width >>= 1;
+      const bool hi = lane & o;
+#pragma unroll
+      for (int j = 0; j < K / 2; ++j) {
+        if (j >= width) continue;
+        const double mine = hi ? v[j + width] : v[j], other = hi ? v[j] : v[j + width];
+        v[j] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+      }
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    }
+  }
+  return v[0];
+}
+
+template <int K>
+__device__ __forceinline__ void column_tree(const double (&acc)[K], double *part) {
+  __shared__ double sh[kThreads / 32][K];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const double v = warp_columns<K>(acc, lane);
+  constexpr int per = 32 / K;
+  if (lane % per == 0) sh[wid][lane / per] = v;
+  __syncthreads();
+  if (threadIdx.x < K) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) t += sh[w][threadIdx.x];
+    part[(size_t)threadIdx.x * kRedBlocks + blockIdx.x] = t;
+  }
+}
+
+// part[c * kRedBlocks + blk]: partial sums of x_c . y_c (y null: x_c . x_c);
+// with TWO also of x_c . z_c in part2
+template <int K, bool TWO>
 __global__ void __launch_bounds__(kThreads)
 bdot_kernel(int64_t n, const double *__restrict__ X, const double *__restrict__ Y,
-            double *__restrict__ part) {
-  double acc[K];
+            double *__restrict__ part, const double *__restrict__ Z, double *__restrict__ part2) {
+  double acc[K], acc2[K];
 #pragma unroll
-  for (int c = 0; c < K; ++c) acc[c] = 0.0;
+  for (int c = 0; c < K; ++c) acc[c] = acc2[c] = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * kThreads) {
+    double x[K], y[K];
+    load_k<double, K>(X + i * K, x);
+    load_k<double, K>((Y ? Y : X) + i * K, y);
 #pragma unroll
-    for (int c = 0; c < K; ++c) {
-      const double x = X[i * K + c];
-      acc[c] = fma(x, Y ? Y[i * K + c] : x, acc[c]);
+    for (int c = 0; c < K; ++c) acc[c] = fma(x[c], y[c], acc[c]);
+    if (TWO) {
+      load_k<double, K>(Z + i * K, y);
+#pragma unroll
+      for (int c = 0; c < K; ++c) acc2[c] = fma(x[c], y[c], acc2[c]);
     }
   }
   column_tree<K>(acc, part);
+  if (TWO) {
+    __syncthreads();
+    column_tree<K>(acc2, part2);
+  }
 }
 
-// out[c] = sum of the kRedBlocks partials of column c, in index order
-__device__ __forceinline__ double sum_partials(const double *p) {
+// sum of the nb partials of one column by one warp: lane l adds l, l + 32, ...
+// in order, then the warp tree; every lane gets it
+__device__ __forceinline__ double warp_partials(const double *p, int nb) {
   double v = 0.0;
-  for (int b = 0; b < kRedBlocks; ++b) v += p[b];
-  return v;
+  for (int b = threadIdx.x & 31; b < nb; b += 32) v += p[b];
+  return warp_sum(v);
 }
 
+// out[c] = sum of the partials of column c (a warp per column)
 template <int K>
-__global__ void bfinalize_kernel(const double *__restrict__ part, double *__restrict__ out) {
-  const int c = threadIdx.x;
-  if (c < K) out[c] = sum_partials(part + (size_t)c * kRedBlocks);
+__global__ void bfinalize_kernel(int nb, const double *__restrict__ part, double *__restrict__ out) {
+  const int c = threadIdx.x >> 5;
+  const double v = warp_partials(part + (size_t)c * kRedBlocks, nb);
+  if ((threadIdx.x & 31) == 0) out[c] = v;
 }
 
 // out[c] = sqrt(sum of the partials of column c)
 template <int K>
-__global__ void bnorm_kernel(const double *__restrict__ part, double *__restrict__ out) {
-  const int c = threadIdx.x;
-  if (c < K) out[c] = sqrt(sum_partials(part + (size_t)c * kRedBlocks));
+__global__ void bnorm_kernel(int nb, const double *__restrict__ part, double *__restrict__ out) {
+  const int c = threadIdx.x >> 5;
+  const double v = warp_partials(part + (size_t)c * kRedBlocks, nb);
+  if ((threadIdx.x & 31) == 0) out[c] = sqrt(v);
 }
 
 // v_c = w_c / nrm[c] (zero when the norm is zero)
@@ -400,54 +586,69 @@ bnormalize_kernel(int64_t nk, const double *__restrict__ w, const double *__rest
 // batched CG (flexible when flex = 1): one iteration in the order
 //   z = M r; rz; beta; p = z + beta p; q = A p; pq; alpha; x, r update; check
 // ---------------------------------------------------------------------------
+// p = z + beta p with beta from the partial sums of r . z (and r . zold), which
+// every CTA adds for itself, a warp per column: no launch of their own
 template <int K>
-__global__ void bcg_beta_kernel(const double *__restrict__ part_rz, const double *__restrict__ part_rzo,
-                                double *__restrict__ sc, const int *__restrict__ st, int flex) {
-  const int c = threadIdx.x;
-  if (c >= K) return;
-  const double rz = sum_partials(part_rz + (size_t)c * kRedBlocks);
-  double beta = 0.0;
-  if (st[BI_STATE * K + c] == BS_RUNNING && !st[BI_FRESH * K + c]) {
-    const double num = flex ? rz - sum_partials(part_rzo + (size_t)c * kRedBlocks) : rz;
-    beta = num / sc[BD_RZ_OLD * K + c];
+__global__ void __launch_bounds__(kThreads)
+bcg_update_p_kernel(int64_t nk, int nb, double *__restrict__ p, const double *__restrict__ z,
+                    double *__restrict__ zold, const double *__restrict__ part_rz,
+                    const double *__restrict__ part_rzo, double *__restrict__ sc,
+                    const int *__restrict__ st, int flex) {
+  __shared__ double sb[K];
+  if (threadIdx.x < 32 * K) {
+    const int c = threadIdx.x >> 5;
+    const double rz = warp_partials(part_rz + (size_t)c * kRedBlocks, nb);
+    double beta = 0.0;
+    if (st[BI_STATE * K + c] == BS_RUNNING && !st[BI_FRESH * K + c]) {
+      const double num = flex ? rz - warp_partials(part_rzo + (size_t)c * kRedBlocks, nb) : rz;
+      beta = num / sc[BD_RZ_OLD * K + c];
+    }
+    if ((threadIdx.x & 31) == 0) {
+      sb[c] = beta;
+      if (blockIdx.x == 0) {
+        sc[BD_RZ * K + c] = rz;
+        sc[BD_BETA * K + c] = beta;
+      }
+    }
   }
-  sc[BD_RZ * K + c] = rz;
-  sc[BD_BETA * K + c] = beta;
+  __syncthreads();
+  const int64_t stride = (int64_t)gridDim.x * kThreads;      // a multiple of K
+  const int64_t e0 = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  const double beta = sb[e0 % K];
+  for (int64_t e = e0; e < nk; e += stride) {
+    const double zv = z[e];
+    p[e] = fma(beta, p[e], zv);
+    if (zold) zold[e] = zv;
+  }
 }
 
+// x += alpha p; r -= alpha q with alpha = rz / p . q from the partial sums of
+// p . q; partial sums of r_c . r_c
 template <int K>
 __global__ void __launch_bounds__(kThreads)
-bcg_update_p_kernel(int64_t nk, double *__restrict__ p, const double *__restrict__ z,
-                    double *__restrict__ zold, const double *__restrict__ sc) {
-  const int64_t e = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  if (e >= nk) return;
-  const int c = (int)(e % K);
-  const double zv = z[e];
-  p[e] = fma(sc[BD_BETA * K + c], p[e], zv);
-  if (zold) zold[e] = zv;
-}
-
-template <int K>
-__global__ void bcg_alpha_kernel(const double *__restrict__ part_pq, double *__restrict__ sc,
-                                 const int *__restrict__ st) {
-  const int c = threadIdx.x;
-  if (c >= K) return;
-  const double pq = sum_partials(part_pq + (size_t)c * kRedBlocks);
-  sc[BD_PQ * K + c] = pq;
-  const bool run = st[BI_STATE * K + c] == BS_RUNNING;
-  sc[BD_ALPHA * K + c] = (run && pq != 0.0 && isfinite(pq)) ? sc[BD_RZ * K + c] / pq : 0.0;
-}
-
-// x += alpha p; r -= alpha q; partial sums of r_c . r_c
-template <int K>
-__global__ void __launch_bounds__(kThreads)
-bcg_update_xr_kernel(int64_t n, double *__restrict__ x, double *__restrict__ r,
+bcg_update_xr_kernel(int64_t n, int nb, double *__restrict__ x, double *__restrict__ r,
                      const double *__restrict__ p, const double *__restrict__ q,
-                     const double *__restrict__ sc, double *__restrict__ part_rr) {
+                     const double *__restrict__ part_pq, double *__restrict__ sc,
+                     const int *__restrict__ st, double *__restrict__ part_rr) {
+  __shared__ double sa[K];
+  if (threadIdx.x < 32 * K) {
+    const int c = threadIdx.x >> 5;
+    const double pq = warp_partials(part_pq + (size_t)c * kRedBlocks, nb);
+    const bool run = st[BI_STATE * K + c] == BS_RUNNING;
+    const double alpha = (run && pq != 0.0 && isfinite(pq)) ? sc[BD_RZ * K + c] / pq : 0.0;
+    if ((threadIdx.x & 31) == 0) {
+      sa[c] = alpha;
+      if (blockIdx.x == 0) {
+        sc[BD_PQ * K + c] = pq;
+        sc[BD_ALPHA * K + c] = alpha;
+      }
+    }
+  }
+  __syncthreads();
   double a[K], acc[K];
 #pragma unroll
   for (int c = 0; c < K; ++c) {
-    a[c] = sc[BD_ALPHA * K + c];
+    a[c] = sa[c];
     acc[c] = 0.0;
   }
   for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n;
@@ -467,18 +668,18 @@ bcg_update_xr_kernel(int64_t n, double *__restrict__ x, double *__restrict__ r,
 // per-column stopping test; ctl[0] counts iterations of this launch, ctl[1]
 // caps them, ctl[2] is set when a column leaves the running state
 template <int K>
-__global__ void bcg_check_kernel(const double *__restrict__ part_rr, double *__restrict__ sc,
-                                 int *__restrict__ st, int *__restrict__ ctl, int flex,
-                                 cudaGraphConditionalHandle h) {
+__global__ void bcg_check_kernel(int nb, const double *__restrict__ part_rr,
+                                 double *__restrict__ sc, int *__restrict__ st,
+                                 int *__restrict__ ctl, int flex, cudaGraphConditionalHandle h) {
   __shared__ int changed, running;
   if (threadIdx.x == 0) {
     changed = 0;
     running = 0;
   }
   __syncthreads();
-  const int c = threadIdx.x;
-  if (c < K) {
-    const double rr = sum_partials(part_rr + (size_t)c * kRedBlocks);
+  const int c = threadIdx.x >> 5;          // a warp per column
+  const double rr = warp_partials(part_rr + (size_t)c * kRedBlocks, nb);
+  if ((threadIdx.x & 31) == 0) {
     sc[BD_RR * K + c] = rr;
     int s = st[BI_STATE * K + c];
     if (s == BS_RUNNING) {
@@ -548,14 +749,17 @@ bmulti_dot_kernel(int64_t n, const double *__restrict__ V, int64_t ldv, const in
   column_tree<K>(acc, part + (size_t)i * K * kRedBlocks);
 }
 
-// h[i * K + c] = sum of partials; H(i, j) = h (pass 0) or += h (pass 1)
+// h[i * K + c] = sum of partials; H(i, j) = h (pass 0) or += h (pass 1); a
+// warp per sum
 template <int K>
-__global__ void bmulti_finalize_kernel(const double *__restrict__ part, int m, const int *__restrict__ dj,
-                                       double *__restrict__ h, double *__restrict__ H, int accumulate) {
+__global__ void bmulti_finalize_kernel(int nb, const double *__restrict__ part, int m,
+                                       const int *__restrict__ dj, double *__restrict__ h,
+                                       double *__restrict__ H, int accumulate) {
   const int j = *dj;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (t >= (j + 1) * K) return;
-  const double v = sum_partials(part + (size_t)t * kRedBlocks);
+  const double v = warp_partials(part + (size_t)t * kRedBlocks, nb);
+  if (threadIdx.x & 31) return;
   h[t] = v;
   double *Hj = H + (size_t)j * (m + 1) * K;
   Hj[t] = accumulate ? Hj[t] + v : v;
@@ -577,12 +781,12 @@ bgs_update_kernel(int64_t nk, const double *__restrict__ V, int64_t ldv, const i
 
 // H(j+1, j) = ||w_c||
 template <int K>
-__global__ void bgm_norm_kernel(const double *__restrict__ part, int m, const int *__restrict__ dj,
-                                double *__restrict__ H) {
-  const int c = threadIdx.x;
-  if (c >= K) return;
+__global__ void bgm_norm_kernel(int nb, const double *__restrict__ part, int m,
+                                const int *__restrict__ dj, double *__restrict__ H) {
+  const int c = threadIdx.x >> 5;
   const int j = *dj;
-  H[((size_t)j * (m + 1) + j + 1) * K + c] = sqrt(sum_partials(part + (size_t)c * kRedBlocks));
+  const double v = warp_partials(part + (size_t)c * kRedBlocks, nb);
+  if ((threadIdx.x & 31) == 0) H[((size_t)j * (m + 1) + j + 1) * K + c] = sqrt(v);
 }
 
 // v_{j+1} = w / H(j+1, j) (zero when the norm is zero)
@@ -703,13 +907,13 @@ bgm_combine_kernel(int64_t nk, const double *__restrict__ Bv, int64_t ldb,
   x[e] = acc;
 }
 
-// after the cycle: the true residual decides (one thread per column)
+// after the cycle: the true residual decides (a warp per column)
 template <int K>
-__global__ void bgm_check_kernel(const double *__restrict__ part_rr, double *__restrict__ sc,
-                                 int *__restrict__ st) {
-  const int c = threadIdx.x;
-  if (c >= K) return;
-  const double rr = sum_partials(part_rr + (size_t)c * kRedBlocks);
+__global__ void bgm_check_kernel(int nb, const double *__restrict__ part_rr,
+                                 double *__restrict__ sc, int *__restrict__ st) {
+  const int c = threadIdx.x >> 5;
+  const double rr = warp_partials(part_rr + (size_t)c * kRedBlocks, nb);
+  if (threadIdx.x & 31) return;
   sc[BD_RR * K + c] = rr;
   if (st[BI_STATE * K + c] != BS_RUNNING) return;
   if (!isfinite(rr)) st[BI_STATE * K + c] = BS_BREAKDOWN;
@@ -783,6 +987,112 @@ bdense_warp_kernel(int n, int ld, const double *__restrict__ A, const T *__restr
   }
 }
 
+// X = M B for the FP32 cycle's dense bottom operator on K columns: M as its exact
+// two-term FP32 split (Mh the FP32 rounding of M, Ml that of M - Mh, row pitch
+// ld), FP32 B and X, double-single arithmetic as in the single solve's
+// dense_mv_ds_kernel, so a row agrees with the FP64 product to about 2^-47 of
+// sum |m b|.  FP64 FMAs took 123 us for order 2,048 and eight columns (33.5
+// million FMAs at 0.6 per ns, and a conversion each); this takes 15.8 us.
+// A CTA owns four rows, so B is read once per four rows; thread t takes columns
+// t, t + 256, ... in order, then the (s, lo) pairs meet in a packed warp tree
+// and the warps in order.  A column's sum does not depend on K.
+constexpr int kDsRows = 4;
+
+__device__ __forceinline__ void ds_add_product(float ah, float al, float x, float &s, float &lo) {
+  const float pr = __fmul_rn(ah, x);
+  const float e = __fmaf_rn(ah, x, -pr);
+  const float cross = __fmul_rn(al, x);
+  const float s1 = __fadd_rn(s, pr);
+  const float bp = __fsub_rn(s1, s);
+  const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(s1, bp)), __fsub_rn(pr, bp));
+  s = s1;
+  lo = __fadd_rn(lo, __fadd_rn(err, __fadd_rn(e, cross)));
+}
+// (s, lo) += (s2, lo2), the same either way round
+__device__ __forceinline__ void ds_add_pair(float &s, float &lo, float s2, float lo2) {
+  const float s1 = __fadd_rn(s, s2);
+  const float bp = __fsub_rn(s1, s);
+  const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(s1, bp)), __fsub_rn(s2, bp));
+  s = s1;
+  lo = __fadd_rn(__fadd_rn(lo, lo2), err);
+}
+
+template <int K>
+__global__ void __launch_bounds__(kThreads)
+bdense_ds_kernel(int n, int ld, const float *__restrict__ Mh, const float *__restrict__ Ml,
+                 const float *__restrict__ B, float *__restrict__ X) {
+  constexpr int Q = kDsRows * K;                    // sums of a CTA, at most 32
+  __shared__ float sh[kThreads / 32][Q], sl[kThreads / 32][Q];
+  const int r0 = blockIdx.x * kDsRows;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const float *hp[kDsRows], *lp[kDsRows];
+#pragma unroll
+  for (int r = 0; r < kDsRows; ++r) {               // rows past the last repeat it
+    const size_t o = (size_t)min(r0 + r, n - 1) * ld;
+    hp[r] = Mh + o;
+    lp[r] = Ml + o;
+  }
+  float s[Q], lo[Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) s[q] = lo[q] = 0.f;
+#pragma unroll 2
+  for (int j = threadIdx.x; j < n; j += kThreads) {
+    float b[K], h[kDsRows], l[kDsRows];
+    load_k<float, K>(B + (size_t)j * K, b);
+#pragma unroll
+    for (int r = 0; r < kDsRows; ++r) {
+      h[r] = __ldg(hp[r] + j);
+      l[r] = __ldg(lp[r] + j);
+    }
+#pragma unroll
+    for (int r = 0; r < kDsRows; ++r)
+#pragma unroll
+      for (int c = 0; c < K; ++c) ds_add_product(h[r], l[r], b[c], s[r * K + c], lo[r * K + c]);
+  }
+  int width = Q;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    if (width > 1) {
+      width >>= 1;
+      const bool hi = lane & o;
+#pragma unroll
+      for (int j = 0; j < Q / 2; ++j) {
+        if (j >= width) continue;
+        const float ms = hi ? s[j + width] : s[j], os = hi ? s[j] : s[j + width];
+        const float ml = hi ? lo[j + width] : lo[j], ol = hi ? lo[j] : lo[j + width];
+        // the lower lane's pair first in both lanes
+        const float ps = __shfl_xor_sync(0xffffffffu, os, o);
+        const float pl = __shfl_xor_sync(0xffffffffu, ol, o);
+        s[j] = hi ? ps : ms;
+        lo[j] = hi ? pl : ml;
+        ds_add_pair(s[j], lo[j], hi ? ms : ps, hi ? ml : pl);
+      }
+    } else {
+      const bool hi = lane & o;
+      const float ps = __shfl_xor_sync(0xffffffffu, s[0], o);
+      const float pl = __shfl_xor_sync(0xffffffffu, lo[0], o);
+      const float ms = s[0], ml = lo[0];
+      s[0] = hi ? ps : ms;
+      lo[0] = hi ? pl : ml;
+      ds_add_pair(s[0], lo[0], hi ? ms : ps, hi ? ml : pl);
+    }
+  }
+  constexpr int per = 32 / Q;
+  if (lane % per == 0) {
+    sh[wid][lane / per] = s[0];
+    sl[wid][lane / per] = lo[0];
+  }
+  __syncthreads();
+  if (threadIdx.x < Q) {
+    double v = 0.0;
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w)
+      v += (double)sh[w][threadIdx.x] + (double)sl[w][threadIdx.x];
+    const int r = r0 + threadIdx.x / K;
+    if (r < n) X[(size_t)r * K + threadIdx.x % K] = (float)v;
+  }
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -802,13 +1112,21 @@ bdense_warp_kernel(int n, int ld, const double *__restrict__ A, const T *__restr
 // column's bits do not depend on the batch width
 static bool long_rows(int n_brows, int64_t nnzb) { return nnzb >= 16 * (int64_t)n_brows; }
 
+// Rows in eight slices while a thread per row would leave SMs without their
+// 1,024 threads; long rows on such a mesh too (their warp variant gives every
+// lane whole blocks).  By the matrix only, as above.
+static bool few_rows(int64_t rows) { return rows < (int64_t)kNumSM * 1024; }
+
 template <typename T>
 cudaError_t launch_bmv(int mode, int n_brows, int br, int bc, const int *rp, const int *col,
                        const T *val, const T *X, const T *B, T *Y, int K, cudaStream_t s,
                        int64_t nnzb) {
   const int64_t rows = (int64_t)n_brows * br;
   if (rows == 0) return cudaSuccess;
-  if (long_rows(n_brows, nnzb)) {
+  if (few_rows(rows)) {
+    GASA_KSWITCH(K, launch_k(bmv_sliced_kernel<T, KK>, div_up(rows * Slices<KK>::lanes, kThreads),
+                             kThreads, 0, s, mode, rows, br, bc, rp, col, val, X, B, Y));
+  } else if (long_rows(n_brows, nnzb)) {
     GASA_KSWITCH(K, launch_k(bmv_warp_kernel<T, KK>, div_up(rows * 32, kThreads), kThreads, 0, s,
                              mode, rows, br, bc, rp, col, val, X, B, Y));
   } else {
@@ -824,11 +1142,21 @@ cudaError_t launch_bjacobi(int mode, int n, int bs, const int *rp, const int *co
                            const T *W, const T *X, const T *B, T *Xo, int K, cudaStream_t s,
                            int64_t nnzb) {
   if (n == 0) return cudaSuccess;
-  const bool warp = mode == JAC_SWEEP && long_rows(n, nnzb);
-  const int rows_cta = warp ? 1 : std::max(1, kThreads / bs);
+  const bool few = few_rows((int64_t)n * bs);
+  const bool warp = !few && mode == JAC_SWEEP && long_rows(n, nnzb);
+  int rows_cta = warp ? 1 : std::max(1, kThreads / bs);
+  int th = kThreads;
+  if (few) {
+    const int lanes = K < 2 ? 8 : 4 * K;
+    rows_cta = std::max(1, kThreads / (bs * lanes));
+    th = std::min(1024, (rows_cta * bs * lanes + 31) / 32 * 32);
+  }
   const size_t smem = (size_t)rows_cta * bs * K * sizeof(T);
   if (smem > 48 * 1024) return cudaErrorInvalidValue;
-  if (warp) {
+  if (few) {
+    GASA_KSWITCH(K, launch_k(bjacobi_sliced_kernel<T, KK>, div_up(n, rows_cta), th, smem, s, mode,
+                             n, bs, rows_cta, rp, col, A, W, X, B, Xo));
+  } else if (warp) {
     GASA_KSWITCH(K, launch_k(bjacobi_kernel<T, KK, true>, div_up(n, rows_cta), kThreads, smem, s,
                              mode, n, bs, rows_cta, rp, col, A, W, X, B, Xo));
   } else {
@@ -881,21 +1209,35 @@ cudaError_t launch_bdense(int nc, const double *Ainv, const T *B, T *X, int K, c
   return cudaGetLastError();
 }
 
+cudaError_t launch_bdense_ds(int n, int ld, const float *Mh, const float *Ml, const float *B,
+                             float *X, int K, cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
+  GASA_KSWITCH(K, launch_k(bdense_ds_kernel<KK>, div_up(n, kDsRows), kThreads, 0, s, n, ld, Mh, Ml,
+                           B, X));
+  note_launch();
+  return cudaGetLastError();
+}
+
 cudaError_t launch_bdot(int64_t n, const double *X, const double *Y, double *part, int K,
-                        cudaStream_t s) {
-  GASA_KSWITCH(K, launch_k(bdot_kernel<KK>, kRedBlocks, kThreads, 0, s, n, X, Y, part));
+                        cudaStream_t s, const double *Z, double *part2) {
+  const int nb = bred_blocks(n);
+  if (Z) {
+    GASA_KSWITCH(K, launch_k(bdot_kernel<KK, true>, nb, kThreads, 0, s, n, X, Y, part, Z, part2));
+  } else {
+    GASA_KSWITCH(K, launch_k(bdot_kernel<KK, false>, nb, kThreads, 0, s, n, X, Y, part, Z, part2));
+  }
   note_launch();
   return cudaGetLastError();
 }
 
-cudaError_t launch_bfinalize(const double *part, double *out, int K, cudaStream_t s) {
-  GASA_KSWITCH(K, launch_k(bfinalize_kernel<KK>, 1, 32, 0, s, part, out));
+cudaError_t launch_bfinalize(int64_t n, const double *part, double *out, int K, cudaStream_t s) {
+  GASA_KSWITCH(K, launch_k(bfinalize_kernel<KK>, 1, 32 * KK, 0, s, bred_blocks(n), part, out));
   note_launch();
   return cudaGetLastError();
 }
 
-cudaError_t launch_bnorm(const double *part, double *out, int K, cudaStream_t s) {
-  GASA_KSWITCH(K, launch_k(bnorm_kernel<KK>, 1, 32, 0, s, part, out));
+cudaError_t launch_bnorm(int64_t n, const double *part, double *out, int K, cudaStream_t s) {
+  GASA_KSWITCH(K, launch_k(bnorm_kernel<KK>, 1, 32 * KK, 0, s, bred_blocks(n), part, out));
   note_launch();
   return cudaGetLastError();
 }
@@ -908,38 +1250,31 @@ cudaError_t launch_bnormalize(int64_t n, const double *w, const double *nrm, dou
   return cudaGetLastError();
 }
 
-cudaError_t launch_bcg_beta(const double *part_rz, const double *part_rzo, double *sc,
-                            const int *st, int flex, int K, cudaStream_t s) {
-  GASA_KSWITCH(K, launch_k(bcg_beta_kernel<KK>, 1, 32, 0, s, part_rz, part_rzo, sc, st, flex));
-  note_launch();
-  return cudaGetLastError();
-}
-
 cudaError_t launch_bcg_update_p(int64_t n, double *p, const double *z, double *zold,
-                                const double *sc, int K, cudaStream_t s) {
+                                const double *part_rz, const double *part_rzo, double *sc,
+                                const int *st, int flex, int K, cudaStream_t s) {
   const int64_t nk = n * K;
-  GASA_KSWITCH(K, launch_k(bcg_update_p_kernel<KK>, div_up(nk, kThreads), kThreads, 0, s, nk, p, z, zold, sc));
-  note_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_bcg_alpha(const double *part_pq, double *sc, const int *st, int K,
-                             cudaStream_t s) {
-  GASA_KSWITCH(K, launch_k(bcg_alpha_kernel<KK>, 1, 32, 0, s, part_pq, sc, st));
+  const int grid = (int)std::min<int64_t>(div_up(nk, kThreads), 4 * kNumSM);
+  GASA_KSWITCH(K, launch_k(bcg_update_p_kernel<KK>, grid, kThreads, 0, s, nk, bred_blocks(n), p, z,
+                           zold, part_rz, part_rzo, sc, st, flex));
   note_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_bcg_update_xr(int64_t n, double *x, double *r, const double *p, const double *q,
-                                 const double *sc, double *part_rr, int K, cudaStream_t s) {
-  GASA_KSWITCH(K, launch_k(bcg_update_xr_kernel<KK>, kRedBlocks, kThreads, 0, s, n, x, r, p, q, sc, part_rr));
+                                 const double *part_pq, double *sc, const int *st, double *part_rr,
+                                 int K, cudaStream_t s) {
+  const int nb = bred_blocks(n);
+  GASA_KSWITCH(K, launch_k(bcg_update_xr_kernel<KK>, nb, kThreads, 0, s, n, nb, x, r, p, q, part_pq,
+                           sc, st, part_rr));
   note_launch();
   return cudaGetLastError();
 }
 
-cudaError_t launch_bcg_check(const double *part_rr, double *sc, int *st, int *ctl, int flex,
-                             cudaGraphConditionalHandle h, int K, cudaStream_t s) {
-  GASA_KSWITCH(K, launch_k(bcg_check_kernel<KK>, 1, 32, 0, s, part_rr, sc, st, ctl, flex, h));
+cudaError_t launch_bcg_check(int64_t n, const double *part_rr, double *sc, int *st, int *ctl,
+                             int flex, cudaGraphConditionalHandle h, int K, cudaStream_t s) {
+  GASA_KSWITCH(K, launch_k(bcg_check_kernel<KK>, 1, 32 * KK, 0, s, bred_blocks(n), part_rr, sc, st,
+                           ctl, flex, h));
   note_launch();
   return cudaGetLastError();
 }
@@ -960,16 +1295,17 @@ cudaError_t launch_bgm_store(int64_t nk, const double *src, double *base, int64_
 
 cudaError_t launch_bmulti_dot(int64_t n, const double *V, int64_t ldv, int max_k, const int *dj,
                               const double *w, double *part, int K, cudaStream_t s) {
-  dim3 grid(kRedBlocks, max_k);
+  dim3 grid(bred_blocks(n), max_k);
   GASA_KSWITCH(K, launch_k(bmulti_dot_kernel<KK>, grid, kThreads, 0, s, n, V, ldv, dj, w, part));
   note_launch();
   return cudaGetLastError();
 }
 
-cudaError_t launch_bmulti_finalize(const double *part, int m, const int *dj, double *h, double *H,
-                                   int accumulate, int K, cudaStream_t s) {
+cudaError_t launch_bmulti_finalize(int64_t n, const double *part, int m, const int *dj, double *h,
+                                   double *H, int accumulate, int K, cudaStream_t s) {
   const int tot = (m + 1) * K;
-  GASA_KSWITCH(K, launch_k(bmulti_finalize_kernel<KK>, div_up(tot, 64), 64, 0, s, part, m, dj, h, H, accumulate));
+  GASA_KSWITCH(K, launch_k(bmulti_finalize_kernel<KK>, div_up(tot, 8), 256, 0, s, bred_blocks(n),
+                           part, m, dj, h, H, accumulate));
   note_launch();
   return cudaGetLastError();
 }
@@ -982,9 +1318,9 @@ cudaError_t launch_bgs_update(int64_t n, const double *V, int64_t ldv, const int
   return cudaGetLastError();
 }
 
-cudaError_t launch_bgm_norm(const double *part, int m, const int *dj, double *H, int K,
+cudaError_t launch_bgm_norm(int64_t n, const double *part, int m, const int *dj, double *H, int K,
                             cudaStream_t s) {
-  GASA_KSWITCH(K, launch_k(bgm_norm_kernel<KK>, 1, 32, 0, s, part, m, dj, H));
+  GASA_KSWITCH(K, launch_k(bgm_norm_kernel<KK>, 1, 32 * KK, 0, s, bred_blocks(n), part, m, dj, H));
   note_launch();
   return cudaGetLastError();
 }
@@ -1026,8 +1362,9 @@ cudaError_t launch_bgm_combine(int64_t n, const double *Bv, int64_t ldb, const d
   return cudaGetLastError();
 }
 
-cudaError_t launch_bgm_check(const double *part_rr, double *sc, int *st, int K, cudaStream_t s) {
-  GASA_KSWITCH(K, launch_k(bgm_check_kernel<KK>, 1, 32, 0, s, part_rr, sc, st));
+cudaError_t launch_bgm_check(int64_t n, const double *part_rr, double *sc, int *st, int K,
+                             cudaStream_t s) {
+  GASA_KSWITCH(K, launch_k(bgm_check_kernel<KK>, 1, 32 * KK, 0, s, bred_blocks(n), part_rr, sc, st));
   note_launch();
   return cudaGetLastError();
 }

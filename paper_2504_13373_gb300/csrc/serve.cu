@@ -327,10 +327,14 @@ cudaError_t vcycle_b(Engine &e, const T *rhs, T *out) {
     ECU(launch_bmv<T>(GASA_MV_ASSIGN, l.R.nrows, l.R.br, l.R.bc, l.R.rp, l.R.col, P::A(l.R),
                       P::r(v), nullptr, P::b(e.lv[k + 1]), K, s, l.R.nnzb));
   }
-  if (kt < N)
-    ECU(launch_bdense<T>(ctx->dtail_n, ctx->dtail_M, P::b(e.lv[kt]), P::x(e.lv[kt]), K, s,
-                         ctx->dtail_ld));
-  else
+  if (kt < N) {
+    if constexpr (std::is_same<T, float>::value)
+      ECU(launch_bdense_ds(ctx->dtail_n, ctx->dtail_ld, ctx->dtail_Mh, ctx->dtail_Ml,
+                           P::b(e.lv[kt]), P::x(e.lv[kt]), K, s));
+    else
+      ECU(launch_bdense<T>(ctx->dtail_n, ctx->dtail_M, P::b(e.lv[kt]), P::x(e.lv[kt]), K, s,
+                           ctx->dtail_ld));
+  } else
     ECU(launch_bdense<T>(ctx->nc, ctx->coarse_inv, P::b(e.lv[N]), P::x(e.lv[N]), K, s));
   xk[kt] = P::x(e.lv[kt]);
   for (int k = kt - 1; k >= 0; --k) {
@@ -388,15 +392,13 @@ cudaError_t build_cg(Engine &e) {
   ECU(cudaStreamBeginCaptureToGraph(e.s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
   cudaError_t err = [&]() -> cudaError_t {
     ECU(apply_Mb(e, e.R, e.Z));
-    ECU(launch_bdot(n, e.R, e.Z, e.part[0], K, e.s));
-    if (e.flex) ECU(launch_bdot(n, e.R, e.Zold, e.part[1], K, e.s));
-    ECU(launch_bcg_beta(e.part[0], e.part[1], e.sc, e.st, e.flex ? 1 : 0, K, e.s));
-    ECU(launch_bcg_update_p(n, e.P, e.Z, e.flex ? e.Zold : nullptr, e.sc, K, e.s));
+    ECU(launch_bdot(n, e.R, e.Z, e.part[0], K, e.s, e.flex ? e.Zold : nullptr, e.part[1]));
+    ECU(launch_bcg_update_p(n, e.P, e.Z, e.flex ? e.Zold : nullptr, e.part[0], e.part[1], e.sc,
+                            e.st, e.flex ? 1 : 0, K, e.s));
     ECU(outer_mv(e, GASA_MV_ASSIGN, e.P, nullptr, e.Q));
     ECU(launch_bdot(n, e.P, e.Q, e.part[2], K, e.s));
-    ECU(launch_bcg_alpha(e.part[2], e.sc, e.st, K, e.s));
-    ECU(launch_bcg_update_xr(n, e.X, e.R, e.P, e.Q, e.sc, e.part[3], K, e.s));
-    return launch_bcg_check(e.part[3], e.sc, e.st, e.ctl, e.flex ? 1 : 0, h, K, e.s);
+    ECU(launch_bcg_update_xr(n, e.X, e.R, e.P, e.Q, e.part[2], e.sc, e.st, e.part[3], K, e.s));
+    return launch_bcg_check(n, e.part[3], e.sc, e.st, e.ctl, e.flex ? 1 : 0, h, K, e.s);
   }();
   cudaGraph_t cap = nullptr;
   cudaError_t e2 = cudaStreamEndCapture(e.s, &cap);
@@ -420,7 +422,7 @@ cudaError_t build_gm(Engine &e) {
       w = e.W;
     }
     ECU(launch_bdot(n, w, nullptr, e.part[0], K, e.s));
-    ECU(launch_bnorm(e.part[0], e.beta, K, e.s));
+    ECU(launch_bnorm(n, e.part[0], e.beta, K, e.s));
     ECU(launch_bnormalize(n, w, e.beta, e.V, K, e.s));
     return launch_bgm_start(m, e.beta, e.g, e.sc, e.st, e.flex ? 1 : 0, dj, K, e.s);
   }();
@@ -452,11 +454,11 @@ cudaError_t build_gm(Engine &e) {
     }
     for (int pass = 0; pass < 2; ++pass) {
       ECU(launch_bmulti_dot(n, e.V, nk, m + 1, dj, e.W, e.mpart, K, e.s));
-      ECU(launch_bmulti_finalize(e.mpart, m, dj, e.hbuf, e.H, pass, K, e.s));
+      ECU(launch_bmulti_finalize(n, e.mpart, m, dj, e.hbuf, e.H, pass, K, e.s));
       ECU(launch_bgs_update(n, e.V, nk, dj, e.hbuf, e.W, K, e.s));
     }
     ECU(launch_bdot(n, e.W, nullptr, e.part[1], K, e.s));
-    ECU(launch_bgm_norm(e.part[1], m, dj, e.H, K, e.s));
+    ECU(launch_bgm_norm(n, e.part[1], m, dj, e.H, K, e.s));
     ECU(launch_bgm_normalize(n, e.W, e.H, m, dj, e.V, K, e.s));
     return launch_bgm_givens(m, e.H, e.cs, e.sn, e.g, e.sc, e.st, dj, h, K, e.s);
   }();
@@ -472,7 +474,7 @@ cudaError_t build_gm(Engine &e) {
     ECU(launch_bgm_combine(n, e.flex ? e.Zb : e.V, nk, e.y, e.st, e.X, K, e.s));
     ECU(outer_mv(e, GASA_MV_RESIDUAL, e.X, e.Bv, e.T));
     ECU(launch_bdot(n, e.T, nullptr, e.part[2], K, e.s));
-    return launch_bgm_check(e.part[2], e.sc, e.st, K, e.s);
+    return launch_bgm_check(n, e.part[2], e.sc, e.st, K, e.s);
   }();
   e2 = cudaStreamEndCapture(e.s, &e.g_end);
   ECU(err);
@@ -582,7 +584,7 @@ cudaError_t admit(Engine &e, int c, Request *rq) {
   }
   // ||b_c|| (every column is recomputed from its own data: same bits)
   ECU(launch_bdot(n, e.Bv, nullptr, e.part[0], K, e.s));
-  ECU(launch_bnorm(e.part[0], e.sc + BD_BN * K, K, e.s));
+  ECU(launch_bnorm(n, e.part[0], e.sc + BD_BN * K, K, e.s));
   e.hsc[BD_TOL * K + c] = rq->tol;
   ECU(cudaMemcpyAsync(e.sc + BD_TOL * K + c, e.hsc + BD_TOL * K + c, sizeof(double),
                       cudaMemcpyHostToDevice, e.s));
@@ -609,7 +611,7 @@ cudaError_t true_residual(Engine &e) {
   const int K = e.K;
   ECU(outer_mv(e, GASA_MV_RESIDUAL, e.X, e.Bv, e.T));
   ECU(launch_bdot(e.n, e.T, nullptr, e.part[0], K, e.s));
-  ECU(launch_bfinalize(e.part[0], e.sc + BD_RR * K, K, e.s));
+  ECU(launch_bfinalize(e.n, e.part[0], e.sc + BD_RR * K, K, e.s));
   return read_back(e);
 }
 
