@@ -4,24 +4,32 @@
 // The Galerkin operators below level 0 of the 3-D and convection-diffusion
 // workloads have blocks of 12 to 36 rows and tens to hundreds of blocks per
 // block row, and at these sizes they hold more bytes than the level-0
-// operator.  A lane per whole block (kernels_blk.cu) would need s*s
-// registers; a thread per scalar row reads its row's blocks one after
-// another with little memory-level parallelism.  Here a team of NW warps
-// owns a block row; the lanes of a warp form G = 32 / br groups of br lanes
-// (one group, two rows per lane, when br > 32) and group g of warp w takes
-// the blocks beg + w*G + g, beg + (w + NW)*G + g, ...; lane r of a group
-// reads row r of its block (the group's lanes together read the block's
-// contiguous br*bc values) with 16- or 8-byte loads where bc and the
-// pointers allow, and the block's bc entries of x.  Each lane keeps one
-// partial sum per row it owns (even and odd columns apart, in column order,
-// whatever the load width); the team's partial sums meet in shared memory
-// and are added in a fixed order (warp, then group), so every row is summed
-// in an order that depends only on the matrix and NW.
+// operator; at full rate they are bound by HBM, or by L2 where a level fits it.
+//
+// A lane owns a fixed run of VW columns of a block (VW = 4, 2 or 1 by what
+// divides bc) in RPL of its rows: LC = bc / VW lanes read one row of the block
+// side by side, G = 32 / LC rows at once, so every load instruction reads one
+// contiguous run of the block whatever its width, the entries of x are loaded
+// once per block, and the lane keeps one partial sum per row over all blocks.
+// (A lane per row, as this file had it before, read a 13-wide block with 4-byte
+// loads 52 bytes apart, eleven 128-byte lines each.)  A team of ES x BS warps
+// owns a block row: ES of them share out the rows of a block (at most
+// kTeamRows each), BS the blocks (block beg + b, beg + b + BS, ...).  The
+// partial sums meet in shared memory and four lanes add up a row in a fixed
+// order, so every row is summed in an order that depends only on the matrix
+// and the team.
 //
 // Operations: y = A x, y = b - A x, y += A x for any br x bc blocks (at most
-// 40 x 40), the block-Jacobi step x_out = x + W (b - A x) of Alg. 1
-// (W = w D^{-1}, square blocks), and the fused residual and restriction
-// y = R b - (R A) x of Alg. 2 with the next level's first step W y.
+// 40 x 40, bc <= 32 where it is odd), the block-Jacobi step
+// x_out = x + W (b - A x) of Alg. 1 (W = w D^{-1}, square blocks), and the fused
+// residual and restriction y = R b - (R A) x of Alg. 2 with the next level's
+// first step W y.
+//
+// GB300, FP32: level 1 of a P2 16^3 tet hierarchy (3,072 rows of about 25 blocks
+// of 13 x 13, 53 MB): product 16.0 -> 14.8 us, smoothing step 20.4 -> 17.0 us;
+// level 2 (384 rows of about 275 blocks of 17 x 17, 122 MB): step 35.6 ->
+// 24.4 us; fused restriction of level 1 92.4 -> 60.3 us.  GMRES on Q2 96^2:
+// 5.97 -> 4.75 ms.
 #include "common.cuh"
 #include "internal.h"
 
@@ -29,189 +37,226 @@ namespace gasa {
 
 namespace {
 
-constexpr int kWideThreads = 256;
-constexpr int kWideWarps = kWideThreads / 32;
 constexpr int kWideMaxRows = 40;    // rows and columns of a block at most
+constexpr int kTeamRows = 8;        // rows per lane at most
+constexpr int kTeamWarps = 16;      // warps per team at most
 
 enum { WIDE_ASSIGN = 0, WIDE_RESID = 1, WIDE_ADD = 2, WIDE_SWEEP = 3, WIDE_RFUSED = 4 };
 
-// one lane's rows (r0 and, with two, r0 + 32) over the blocks kbeg, kbeg +
-// step, ... < end of one block row: adds sign * (row . x_col) to a0, a1
-template <int VW>
-__device__ __forceinline__ void lane_rows(int kbeg, int end, int step, int br, int bc, int r0,
-                                          bool two, const int *__restrict__ col,
-                                          const float *__restrict__ val,
-                                          const float *__restrict__ x, float sign, float &a0,
-                                          float &a1) {
-  for (int k = kbeg; k < end; k += step) {
-    const int j = __ldg(col + k);
-    const float *ar0 = val + ((size_t)k * br + r0) * bc;
-    const float *ar1 = ar0 + (size_t)32 * bc;
-    const float *xj = x + (size_t)j * bc;
-    float s0 = 0.f, s1 = 0.f, t0 = 0.f, t1 = 0.f;
-    if constexpr (VW == 4) {
-      for (int c = 0; c < bc; c += 4) {
-        const float4 xv = __ldg(reinterpret_cast<const float4 *>(xj + c));
-        const float4 av = __ldg(reinterpret_cast<const float4 *>(ar0 + c));
-        s0 = fmaf(av.x, xv.x, s0);
-        s1 = fmaf(av.y, xv.y, s1);
-        s0 = fmaf(av.z, xv.z, s0);
-        s1 = fmaf(av.w, xv.w, s1);
-        if (two) {
-          const float4 bv = __ldg(reinterpret_cast<const float4 *>(ar1 + c));
-          t0 = fmaf(bv.x, xv.x, t0);
-          t1 = fmaf(bv.y, xv.y, t1);
-          t0 = fmaf(bv.z, xv.z, t0);
-          t1 = fmaf(bv.w, xv.w, t1);
-        }
-      }
-    } else if constexpr (VW == 2) {
-      for (int c = 0; c < bc; c += 2) {
-        const float2 xv = __ldg(reinterpret_cast<const float2 *>(xj + c));
-        const float2 av = __ldg(reinterpret_cast<const float2 *>(ar0 + c));
-        s0 = fmaf(av.x, xv.x, s0);
-        s1 = fmaf(av.y, xv.y, s1);
-        if (two) {
-          const float2 bv = __ldg(reinterpret_cast<const float2 *>(ar1 + c));
-          t0 = fmaf(bv.x, xv.x, t0);
-          t1 = fmaf(bv.y, xv.y, t1);
-        }
-      }
-    } else {
-      int c = 0;
-      for (; c + 1 < bc; c += 2) {
-        const float x0 = __ldg(xj + c), x1 = __ldg(xj + c + 1);
-        s0 = fmaf(__ldg(ar0 + c), x0, s0);
-        s1 = fmaf(__ldg(ar0 + c + 1), x1, s1);
-        if (two) {
-          t0 = fmaf(__ldg(ar1 + c), x0, t0);
-          t1 = fmaf(__ldg(ar1 + c + 1), x1, t1);
-        }
-      }
-      if (c < bc) {
-        const float xc = __ldg(xj + c);
-        s0 = fmaf(__ldg(ar0 + c), xc, s0);
-        if (two) t0 = fmaf(__ldg(ar1 + c), xc, t0);
+// adds sign * (rows r0, r0 + rstep, ... of the blocks k0, k0 + BS, ... < end,
+// columns c .. c + VW) . x to acc; two blocks in flight, and the column indices
+// of the next two
+template <int VW, int RPL>
+__device__ __forceinline__ void team_blocks(int k0, int end, int step, int br, int bc, int r0,
+                                            int rstep, int c, const int *__restrict__ col,
+                                            const float *__restrict__ val,
+                                            const float *__restrict__ x, float sign,
+                                            float (&acc)[RPL]) {
+  const float *vp = val + (size_t)r0 * bc + c;
+  const size_t bb = (size_t)br * bc;
+  const float *xc = x + c;
+  bool row[RPL];
+#pragma unroll
+  for (int m = 0; m < RPL; ++m) row[m] = r0 + m * rstep < br;
+  int k = k0;
+  int j0 = k < end ? __ldg(col + k) : 0, j1 = k + step < end ? __ldg(col + k + step) : 0;
+  for (; k + step < end; k += 2 * step) {
+    float a0[RPL][VW], a1[RPL][VW], x0[VW], x1[VW];
+    const float *p0 = vp + (size_t)k * bb, *p1 = vp + (size_t)(k + step) * bb;
+#pragma unroll
+    for (int m = 0; m < RPL; ++m) {
+      if (row[m]) load_vec<float, VW>(p0 + (size_t)m * rstep * bc, a0[m]);
+      if (row[m]) load_vec<float, VW>(p1 + (size_t)m * rstep * bc, a1[m]);
+    }
+    load_vec<float, VW>(xc + (size_t)j0 * bc, x0);
+    load_vec<float, VW>(xc + (size_t)j1 * bc, x1);
+    j0 = k + 2 * step < end ? __ldg(col + k + 2 * step) : 0;
+    j1 = k + 3 * step < end ? __ldg(col + k + 3 * step) : 0;
+#pragma unroll
+    for (int m = 0; m < RPL; ++m) {
+      if (!row[m]) continue;
+#pragma unroll
+      for (int v = 0; v < VW; ++v) {
+        acc[m] = fmaf(sign * a0[m][v], x0[v], acc[m]);
+        acc[m] = fmaf(sign * a1[m][v], x1[v], acc[m]);
       }
     }
-    a0 += sign * (s0 + s1);
-    a1 += sign * (t0 + t1);
+  }
+  if (k < end) {
+    float a0[RPL][VW], x0[VW];
+    const float *p0 = vp + (size_t)k * bb;
+#pragma unroll
+    for (int m = 0; m < RPL; ++m)
+      if (row[m]) load_vec<float, VW>(p0 + (size_t)m * rstep * bc, a0[m]);
+    load_vec<float, VW>(xc + (size_t)j0 * bc, x0);
+#pragma unroll
+    for (int m = 0; m < RPL; ++m) {
+      if (!row[m]) continue;
+#pragma unroll
+      for (int v = 0; v < VW; ++v) acc[m] = fmaf(sign * a0[m][v], x0[v], acc[m]);
+    }
   }
 }
 
-// OP WIDE_ASSIGN / RESID / ADD / SWEEP on (rp, col, val); WIDE_RFUSED: the
+// op WIDE_ASSIGN / RESID / ADD / SWEEP on (rp, col, val); WIDE_RFUSED: the
 // fused residual and restriction y = R b - (R A) x with R = (rp, col, val),
 // R A = (rp2, col2, val2), and, with Wm (the next level's w D^{-1}), its first
-// smoothing step x2o = Wm y
-template <int OP, int VW>
-__global__ void __launch_bounds__(kWideThreads)
-bsr_wide_kernel(int n_brows, int br, int bc, int nw, const int *__restrict__ rp,
+// smoothing step x2o = Wm y.  blockDim = 32 * ES * BS * teams; dynamic shared
+// memory: 32 * RPL floats per warp and 40 per team.
+template <int VW, int RPL>
+__global__ void __launch_bounds__(32 * kTeamWarps)
+bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, const int *__restrict__ rp,
                 const int *__restrict__ col, const float *__restrict__ val,
                 const float *__restrict__ Wm, const float *__restrict__ x,
                 const float *__restrict__ b, float *__restrict__ y, const int *__restrict__ rp2,
                 const int *__restrict__ col2, const float *__restrict__ val2,
                 float *__restrict__ x2o) {
-  // red[warp][slot]: each lane's partial row sums (slot = lane, lane + 32)
-  __shared__ float red[kWideWarps][kWideMaxRows];
-  __shared__ float res[kWideWarps][kWideMaxRows];
+  extern __shared__ float sm[];
+  const int nw = ES * BS, warps = blockDim.x >> 5, teams = warps / nw;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int teams = kWideWarps / nw;
   const int team = warp / nw, wt = warp - team * nw;
+  const int es = wt % ES, bs = wt / ES;
+  const int LC = bc / VW, G = 32 / LC;
+  const int g = lane / LC, cl = lane - g * LC;
   const int u = blockIdx.x * teams + team;
-  const int G = br <= 32 ? 32 / br : 1;          // block groups per warp
-  const int g = br <= 32 ? lane / br : 0;
-  const int r0 = br <= 32 ? lane - g * br : lane;
-  const bool lane_on = g < G && r0 < br;
-  const bool two = br > 32 && lane + 32 < br;   // second row of this lane
-  float a0 = 0.f, a1 = 0.f;
-  if (u < n_brows && lane_on) {
-    const int step = nw * G, off = wt * G + g;
-    if (OP == WIDE_RFUSED) {
-      lane_rows<VW>(__ldg(rp + u) + off, __ldg(rp + u + 1), step, br, bc, r0, two, col, val, b,
-                    1.f, a0, a1);
-      lane_rows<VW>(__ldg(rp2 + u) + off, __ldg(rp2 + u + 1), step, br, bc, r0, two, col2, val2, x,
-                    -1.f, a0, a1);
-    } else {
-      lane_rows<VW>(__ldg(rp + u) + off, __ldg(rp + u + 1), step, br, bc, r0, two, col, val, x,
-                    1.f, a0, a1);
+  const bool on = u < n_brows;
+  float *part = sm + (size_t)team * nw * 32 * RPL;            // [nw][RPL][32]
+  float *res = sm + (size_t)warps * 32 * RPL + team * kWideMaxRows;
+  const bool smooth = op == WIDE_SWEEP || (op == WIDE_RFUSED && Wm);
+  if (smooth && on) {
+    // the block of Wm is needed last: bring it into L2 meanwhile
+    const int lines = (br * br * 4 + 127) / 128 + 1;
+    for (int q = wt * 32 + lane; q < lines; q += nw * 32) {
+      const int o = min(q * 32, br * br - 1);
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(Wm + (size_t)u * br * br + o));
     }
   }
-  // partial sums to shared memory: slot = g * br + r0 (br <= 32), else r0, r0 + 32
-  if (lane_on) red[warp][br <= 32 ? g * br + r0 : r0] = a0;
-  if (two) red[warp][lane + 32] = a1;
+  float acc[RPL];
+#pragma unroll
+  for (int m = 0; m < RPL; ++m) acc[m] = 0.f;
+  if (on && g < G) {
+    const int r0 = es * G + g, rs = ES * G;
+    const int beg = __ldg(rp + u), end = __ldg(rp + u + 1);
+    if (op == WIDE_RFUSED) {
+      const int beg2 = __ldg(rp2 + u), end2 = __ldg(rp2 + u + 1);
+      team_blocks<VW, RPL>(beg + bs, end, BS, br, bc, r0, rs, cl * VW, col, val, b, 1.f, acc);
+      team_blocks<VW, RPL>(beg2 + bs, end2, BS, br, bc, r0, rs, cl * VW, col2, val2, x, -1.f, acc);
+    } else {
+      team_blocks<VW, RPL>(beg + bs, end, BS, br, bc, r0, rs, cl * VW, col, val, x, 1.f, acc);
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < RPL; ++m) part[(wt * RPL + m) * 32 + lane] = acc[m];
   __syncthreads();
-  if (u >= n_brows || wt != 0) return;
-  // the team's first warp adds the partial sums of row r: warps in order, then groups
-  const int w0 = team * nw;
-  for (int r = lane; r < br; r += 32) {
+  // four lanes per row add the row's BS * LC partial sums: blocks' warps in
+  // order, columns sub, sub + 4, ... in order, then the four
+  const int sub = lane & 3;
+  const int rounds = (br * 4 + nw * 32 - 1) / (nw * 32);
+  for (int it = 0; it < rounds; ++it) {
+    const int r = (it * nw * 32 + wt * 32 + lane) >> 2;
     float v = 0.f;
-    for (int w = 0; w < nw; ++w) {
-      if (br <= 32) {
-        for (int q = 0; q < G; ++q) v += red[w0 + w][q * br + r];
+    if (r < br) {
+      const int m = r / (ES * G), q = r - m * ES * G;
+      const float *p = part + ((size_t)(q / G) * RPL + m) * 32 + (q % G) * LC;
+      for (int s = 0; s < BS; ++s)
+        for (int c = sub; c < LC; c += 4) v += p[(size_t)s * ES * RPL * 32 + c];
+    }
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    if (on && r < br && sub == 0) {
+      const size_t t = (size_t)u * br + r;
+      if (op == WIDE_ASSIGN) y[t] = v;
+      else if (op == WIDE_RESID) y[t] = b[t] - v;
+      else if (op == WIDE_ADD) y[t] = y[t] + v;
+      else if (op == WIDE_RFUSED) {
+        y[t] = v;
+        res[r] = v;
       } else {
-        v += red[w0 + w][r];
+        res[r] = b[t] - v;
       }
     }
-    const size_t t = (size_t)u * br + r;
-    if (OP == WIDE_ASSIGN) y[t] = v;
-    else if (OP == WIDE_RESID) y[t] = b[t] - v;
-    else if (OP == WIDE_ADD) y[t] = y[t] + v;
-    else if (OP == WIDE_RFUSED) {
-      y[t] = v;
-      res[w0][r] = v;
-    } else {
-      res[w0][r] = b[t] - v;
+  }
+  if (!smooth) return;
+  __syncthreads();
+  // SWEEP: x_out = x + W (b - A x); RFUSED: x2o = Wm y, four lanes per row
+  for (int it = 0; it < rounds; ++it) {
+    const int r = (it * nw * 32 + wt * 32 + lane) >> 2;
+    float v = 0.f;
+    if (on && r < br) {
+      const float *w = Wm + ((size_t)u * br + r) * br;
+      for (int c = sub; c < br; c += 4) v = fmaf(__ldg(w + c), res[c], v);
+    }
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    if (on && r < br && sub == 0) {
+      const size_t t = (size_t)u * br + r;
+      if (op == WIDE_SWEEP) y[t] = x[t] + v;
+      else x2o[t] = v;
     }
   }
-  if (OP == WIDE_RFUSED && !Wm) return;
-  if (OP != WIDE_SWEEP && OP != WIDE_RFUSED) return;
-  __syncwarp();
-  // SWEEP: x_out = x + W (b - A x); RFUSED: x2o = Wm y (W row r against res)
-  for (int r = lane; r < br; r += 32) {
-    const float *w = Wm + ((size_t)u * br + r) * br;
-    float o0 = 0.f, o1 = 0.f;
-    int c = 0;
-    for (; c + 1 < br; c += 2) {
-      o0 = fmaf(__ldg(w + c), res[w0][c], o0);
-      o1 = fmaf(__ldg(w + c + 1), res[w0][c + 1], o1);
-    }
-    if (c < br) o0 = fmaf(__ldg(w + c), res[w0][c], o0);
-    const size_t t = (size_t)u * br + r;
-    if (OP == WIDE_SWEEP) y[t] = x[t] + (o0 + o1);
-    else x2o[t] = o0 + o1;
-  }
-}
-
-// warps per block row: about four blocks per group, at most a CTA
-int wide_team(int br, double avg) {
-  const int G = br <= 32 ? 32 / br : 1;
-  int nw = 1;
-  while (nw < kWideWarps && nw * G * 4 < avg) nw *= 2;
-  return nw;
 }
 
 bool al(const void *p, size_t a) { return p == nullptr || ((uintptr_t)p % a) == 0; }
 
-// widest row load the block width and every row pointer allow
+// widest run the block width and every pointer allow
 int wide_vec(int bc, const void *v1, const void *x1, const void *v2, const void *x2) {
   if (bc % 4 == 0 && al(v1, 16) && al(x1, 16) && al(v2, 16) && al(x2, 16)) return 4;
   if (bc % 2 == 0 && al(v1, 8) && al(x1, 8) && al(v2, 8) && al(x2, 8)) return 2;
   return 1;
 }
 
-template <int OP>
-void wide_go(int vw, int grid, cudaStream_t s, int n_brows, int br, int bc, int nw, const int *rp,
-             const int *col, const float *val, const float *W, const float *x, const float *b,
-             float *y, const int *rp2, const int *col2, const float *val2, float *x2o) {
+template <int VW>
+cudaError_t team_go(int op, int n_brows, int br, int bc, double avg, const int *rp, const int *col,
+                    const float *val, const float *W, const float *x, const float *b, float *y,
+                    const int *rp2, const int *col2, const float *val2, float *x2o,
+                    cudaStream_t s) {
+  const int LC = bc / VW, G = 32 / LC;
+  const int rows = div_up(br, G);                  // row steps of one warp over a block
+  const int ES = div_up(rows, kTeamRows);
+  const int RPL = div_up(rows, ES);
+  // blocks shared out over warps while each keeps four or more and the GPU has
+  // fewer than 40 warps an SM; twice as many warps (or half as many blocks each)
+  // cost more in the teams' sums than they hide: 14.8 -> 16.7 us (25.0 us) for
+  // the 13 x 13 product above
+  int BS = 1;
+  while (ES * BS * 2 <= kTeamWarps && avg >= 8.0 * BS &&
+         (long long)n_brows * ES * BS < 40LL * kNumSM)
+    BS *= 2;
+  const int nw = ES * BS, teams = nw >= 8 ? 1 : 8 / nw, warps = nw * teams;
+  const size_t smem = ((size_t)warps * 32 * RPL + teams * kWideMaxRows) * sizeof(float);
+  const int grid = div_up(n_brows, teams);
+  auto go = [&](auto kern) {
+    launch_k(kern, grid, 32 * warps, smem, s, op, n_brows, br, bc, ES, BS, rp, col, val, W, x, b, y,
+             rp2, col2, val2, x2o);
+  };
+  switch (RPL) {
+    case 1: go(bsr_team_kernel<VW, 1>); break;
+    case 2: go(bsr_team_kernel<VW, 2>); break;
+    case 3: go(bsr_team_kernel<VW, 3>); break;
+    case 4: go(bsr_team_kernel<VW, 4>); break;
+    case 5: go(bsr_team_kernel<VW, 5>); break;
+    case 6: go(bsr_team_kernel<VW, 6>); break;
+    case 7: go(bsr_team_kernel<VW, 7>); break;
+    default: go(bsr_team_kernel<VW, 8>); break;
+  }
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t team_launch(int op, int n_brows, int br, int bc, int64_t nnzb, const int *rp,
+                        const int *col, const float *val, const float *W, const float *x,
+                        const float *b, float *y, const int *rp2, const int *col2,
+                        const float *val2, float *x2o, cudaStream_t s) {
+  const double avg = (double)nnzb / (double)n_brows;
+  // RFUSED multiplies val with b and val2 with x
+  const int vw = op == WIDE_RFUSED ? wide_vec(bc, val, b, val2, x)
+                                   : wide_vec(bc, val, x, nullptr, nullptr);
+  if (bc / vw > 32) return cudaErrorNotSupported;
   if (vw == 4)
-    launch_k(bsr_wide_kernel<OP, 4>, grid, kWideThreads, 0, s, n_brows, br, bc, nw, rp, col, val, W,
-             x, b, y, rp2, col2, val2, x2o);
-  else if (vw == 2)
-    launch_k(bsr_wide_kernel<OP, 2>, grid, kWideThreads, 0, s, n_brows, br, bc, nw, rp, col, val, W,
-             x, b, y, rp2, col2, val2, x2o);
-  else
-    launch_k(bsr_wide_kernel<OP, 1>, grid, kWideThreads, 0, s, n_brows, br, bc, nw, rp, col, val, W,
-             x, b, y, rp2, col2, val2, x2o);
+    return team_go<4>(op, n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2, val2, x2o, s);
+  if (vw == 2)
+    return team_go<2>(op, n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2, val2, x2o, s);
+  return team_go<1>(op, n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2, val2, x2o, s);
 }
 
 }  // namespace
@@ -227,29 +272,8 @@ cudaError_t launch_wide(int op, int n_brows, int br, int bc, int64_t nnzb, const
   if (n_brows == 0) return cudaSuccess;
   if (br > kWideMaxRows || bc > kWideMaxRows || (op == WIDE_SWEEP && br != bc))
     return cudaErrorNotSupported;
-  const int nw = wide_team(br, (double)nnzb / (double)n_brows);
-  const int grid = div_up(n_brows, kWideWarps / nw);
-  const int vw = wide_vec(bc, val, x, nullptr, nullptr);
-  switch (op) {
-    case WIDE_ASSIGN:
-      wide_go<WIDE_ASSIGN>(vw, grid, s, n_brows, br, bc, nw, rp, col, val, W, x, b, y, nullptr,
-                           nullptr, nullptr, nullptr);
-      break;
-    case WIDE_RESID:
-      wide_go<WIDE_RESID>(vw, grid, s, n_brows, br, bc, nw, rp, col, val, W, x, b, y, nullptr,
-                          nullptr, nullptr, nullptr);
-      break;
-    case WIDE_ADD:
-      wide_go<WIDE_ADD>(vw, grid, s, n_brows, br, bc, nw, rp, col, val, W, x, b, y, nullptr,
-                        nullptr, nullptr, nullptr);
-      break;
-    default:
-      wide_go<WIDE_SWEEP>(vw, grid, s, n_brows, br, bc, nw, rp, col, val, W, x, b, y, nullptr,
-                          nullptr, nullptr, nullptr);
-      break;
-  }
-  note_launch();
-  return cudaGetLastError();
+  return team_launch(op, n_brows, br, bc, nnzb, rp, col, val, W, x, b, y, nullptr, nullptr, nullptr,
+                     nullptr, s);
 }
 
 cudaError_t launch_wide_restrict(int n_brows, int br, int bc, int64_t nnzb, const int *rrp,
@@ -259,13 +283,8 @@ cudaError_t launch_wide_restrict(int n_brows, int br, int bc, int64_t nnzb, cons
                                  cudaStream_t s) {
   if (n_brows == 0) return cudaSuccess;
   if (br > kWideMaxRows || bc > kWideMaxRows) return cudaErrorNotSupported;
-  const int nw = wide_team(br, (double)nnzb / (double)n_brows);
-  const int grid = div_up(n_brows, kWideWarps / nw);
-  const int vw = wide_vec(bc, rval, b, aval, x);
-  wide_go<WIDE_RFUSED>(vw, grid, s, n_brows, br, bc, nw, rrp, rcol, rval, Wn, x, b, y, arp, acol,
-                       aval, xn);
-  note_launch();
-  return cudaGetLastError();
+  return team_launch(WIDE_RFUSED, n_brows, br, bc, nnzb, rrp, rcol, rval, Wn, x, b, y, arp, acol,
+                     aval, xn, s);
 }
 
 }  // namespace gasa

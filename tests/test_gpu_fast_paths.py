@@ -80,3 +80,53 @@ def test_tentative_packed_sums(n_units, bs, size, r, s_next):
         assert np.max(np.abs(sg[J, :s.size] - s)) <= eps * s[0]
         assert np.max(np.abs(Tg[rows] - Td)) <= 10 * eps / gap, J
         assert np.max(np.abs(Tg[rows].T @ Tg[rows] - np.eye(s_next))) <= 1e-12
+
+
+def _random_bsr(rng, n, ncols, br, bc, lo, hi):
+    """(row_ptr, col, val) with lo..hi blocks per row (one row empty when lo is 0)."""
+    counts = rng.integers(lo, hi + 1, n)
+    rp = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+    col = np.concatenate([np.sort(rng.choice(ncols, c, replace=False)) for c in counts] or
+                         [np.zeros(0)]).astype(np.int32)
+    return rp, col, rng.standard_normal((int(rp[-1]), br, bc))
+
+
+def _bsr_apply(rp, col, val, x):
+    n, br, bc = rp.size - 1, val.shape[1], val.shape[2]
+    y = np.zeros((n, br))
+    prod = np.einsum("kij,kj->ki", val, x.reshape(-1, bc)[col])
+    np.add.at(y, np.repeat(np.arange(n), np.diff(rp)), prod)
+    return y.ravel()
+
+
+@pytest.mark.parametrize("br,bc", [(9, 9), (13, 13), (17, 17), (12, 12), (22, 22), (31, 31),
+                                   (36, 36), (40, 40), (38, 38), (33, 33), (39, 13), (4, 30),
+                                   (13, 10), (1, 40), (40, 9)])
+@pytest.mark.parametrize("n,lo,hi", [(1, 9, 9), (45, 0, 30), (700, 8, 14)])
+def test_wide_team_products(br, bc, n, lo, hi):
+    """FP32 products and smoothing steps with wide blocks at every load width, team shape and
+    a ragged last team: n terms of a row to n 2^-23 of sum |a x|."""
+    gasa = _gasa()
+    rng = np.random.default_rng(br * 100 + bc + n)
+    ncols = max(n, hi)
+    rp, col, val = _random_bsr(rng, n, ncols, br, bc, lo, hi)
+    val = val.astype(np.float32)
+    x, b = rng.standard_normal(ncols * bc).astype(np.float32), rng.standard_normal(n * br).astype(np.float32)
+    ax = _bsr_apply(rp, col, val.astype(np.float64), x.astype(np.float64))
+    mag = _bsr_apply(rp, col, np.abs(val).astype(np.float64), np.abs(x).astype(np.float64))
+    tol = (hi * bc + 4) * 2.0 ** -23 * (mag + np.abs(b)) + 1e-30
+    d = [to_dev(a) for a in (rp, col, val.ravel(), x, b)]
+    for mode, ref in ((0, ax), (1, b - ax), (2, b + ax)):
+        y = d[4].clone()
+        gasa.gasa_bsr_mv_f32(mode, n, br, bc, *d[:4], d[4], y)
+        assert np.all(np.abs(y.cpu().numpy() - ref) <= tol)
+    if br != bc or ncols != n:
+        return
+    W = (rng.standard_normal((n, br, br)) / br).astype(np.float32)
+    out = to_dev(np.zeros(n * br, np.float32))
+    gasa.gasa_jacobi_sweep_f32(n, br, *d[:3], to_dev(W.ravel()), d[3], d[4], out)
+    r = (b - ax).reshape(n, br)
+    ref = x + np.einsum("nij,nj->ni", W.astype(np.float64), r).ravel()
+    wtol = np.einsum("nij,nj->ni", np.abs(W).astype(np.float64),
+                     (tol + np.abs(r).ravel() * br * 2.0 ** -23).reshape(n, br)).ravel()
+    assert np.all(np.abs(out.cpu().numpy() - ref) <= wtol + 2.0 ** -23 * (np.abs(x) + np.abs(ref)))
