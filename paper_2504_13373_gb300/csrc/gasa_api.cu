@@ -2574,7 +2574,7 @@ gasa_status gasa_bsr_mv(int32_t mode, int32_t n_brows, int32_t br, int32_t bc,
     return GASA_ERR_INVALID_ARG;
   return op_status(launch_bsr_mv<double>(mode, n_brows, br, bc, row_ptr, col, val, x, b, y,
                                          (cudaStream_t)stream,
-                                         op_nnzb(row_ptr, n_brows, (cudaStream_t)stream)));
+                                         kNnzbUnknown));
 }
 
 gasa_status gasa_bsr_mv_f32(int32_t mode, int32_t n_brows, int32_t br, int32_t bc,
@@ -2586,7 +2586,7 @@ gasa_status gasa_bsr_mv_f32(int32_t mode, int32_t n_brows, int32_t br, int32_t b
     return GASA_ERR_INVALID_ARG;
   return op_status(launch_bsr_mv<float>(mode, n_brows, br, bc, row_ptr, col, val, x, b, y,
                                         (cudaStream_t)stream,
-                                        op_nnzb(row_ptr, n_brows, (cudaStream_t)stream)));
+                                        kNnzbUnknown));
 }
 
 gasa_status gasa_bsr_mv_ds(int32_t n_brows, int32_t br, int32_t bc, const int32_t *row_ptr,
@@ -2609,7 +2609,7 @@ gasa_status gasa_jacobi_sweep(int32_t n_units, int32_t bs, const int32_t *row_pt
     return GASA_ERR_INVALID_ARG;
   return op_status(launch_jacobi<double>(first ? JAC_FIRST : JAC_SWEEP, n_units, bs, row_ptr, col,
                                          val, W, x, b, x_out, (cudaStream_t)stream,
-                                         first ? -1 : op_nnzb(row_ptr, n_units, (cudaStream_t)stream)));
+                                         first ? -1 : kNnzbUnknown));
 }
 
 gasa_status gasa_jacobi_sweep_f32(int32_t n_units, int32_t bs, const int32_t *row_ptr,
@@ -2622,7 +2622,7 @@ gasa_status gasa_jacobi_sweep_f32(int32_t n_units, int32_t bs, const int32_t *ro
     return GASA_ERR_INVALID_ARG;
   return op_status(launch_jacobi<float>(first ? JAC_FIRST : JAC_SWEEP, n_units, bs, row_ptr, col,
                                         val, W, x, b, x_out, (cudaStream_t)stream,
-                                        first ? -1 : op_nnzb(row_ptr, n_units, (cudaStream_t)stream)));
+                                        first ? -1 : kNnzbUnknown));
 }
 
 gasa_status gasa_block_inverse(int32_t n_units, int32_t bs, const int32_t *row_ptr,

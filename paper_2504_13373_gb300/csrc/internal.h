@@ -55,6 +55,13 @@ long long launch_count();
 
 enum JacobiMode { JAC_SWEEP = 0, JAC_FIRST = 1, JAC_APPLY = 2, JAC_RELAX = 3 };
 
+// nnzb argument of the launchers below when the host does not know it (reading
+// it from the device would wait for the stream)
+constexpr int64_t kNnzbUnknown = -2;
+// rows of at least this many wide FP32 blocks take the team kernel when the
+// host does not know the matrix's average
+constexpr int kLongRow = 8;
+
 // ---- kernels_wide.cu: FP32 blocks wider than 8, a team of warps per block row
 // true for blocks with more than 8 rows or columns (at most 40 of either) and
 // at least 8 blocks per block row on average
@@ -67,14 +74,18 @@ cudaError_t launch_wide_restrict(int n_brows, int br, int bc, int64_t nnzb, cons
                                  const int *acol, const float *aval, const float *b,
                                  const float *x, float *y, const float *Wn, float *xn,
                                  cudaStream_t s);
-// op: 0 y = A x, 1 y = b - A x, 2 y += A x, 3 y = x + W (b - A x) (square)
+// op: 0 y = A x, 1 y = b - A x, 2 y += A x, 3 y = x + W (b - A x) (square);
+// min_len > 0: only the block rows of at least min_len blocks
 cudaError_t launch_wide(int op, int n_brows, int br, int bc, int64_t nnzb, const int *rp,
                         const int *col, const float *val, const float *W, const float *x,
-                        const float *b, float *y, cudaStream_t s);
+                        const float *b, float *y, cudaStream_t s, int min_len = 0);
+// whether launch_wide takes these blocks, whatever the row lengths
+bool wide_shape(int br, int bc, const float *val, const float *x);
 
 // ---- kernels_blk.cu: small square blocks, one lane per block ---------------
-// true when square s x s blocks (2 <= s <= 8) average at least 6 per block row;
-// launch_blk then takes FP32 operands (FP64 returns cudaErrorNotSupported)
+// true when square s x s blocks (2 <= s <= 8) average at least 6 per block row
+// (or nnzb is kNnzbUnknown); launch_blk then takes FP32 operands (FP64 returns
+// cudaErrorNotSupported)
 bool blk_applies(int bs, int n_brows, int64_t nnzb);
 // fused residual + restriction y = R b - (R A) x (FP32, s x s blocks, s <= 8)
 // with the next level's first step xn = Wn y when Wn is given; nnzb: blocks
@@ -99,8 +110,9 @@ cudaError_t launch_blk(int op, int n_brows, int bs, int64_t nnzb, const int *rp,
                        const T *val, const T *W, const T *x, const T *b, T *y, cudaStream_t s);
 
 // ---- kernels_mv.cu ---------------------------------------------------------
-// nnzb >= 0 lets the launcher pick a warp per block row when rows are long
-// (>= 12 blocks on average); nnzb < 0 always uses one thread per scalar row.
+// nnzb >= 0 lets the launcher pick by the average row length; kNnzbUnknown
+// picks by sizes alone or row by row on the device; -1 always uses one thread
+// per scalar row.
 template <typename T>
 cudaError_t launch_bsr_mv(int mode, int n_brows, int br, int bc, const int *rp, const int *col,
                           const T *val, const T *x, const T *b, T *y, cudaStream_t s,

@@ -236,7 +236,17 @@ blk_restrict_kernel(int n_brows, const int *__restrict__ rrp, const int *__restr
 // Lanes per block row: about 2.5 blocks per lane (two in flight, a short
 // tail), a power of two in [4, 64] and at least s, so that lanes 0..s-1 of
 // the team can write the s rows.
+// Without the average, by the number of rows: as many lanes as give the GPU
+// 1,024 per SM, at most 32 (coarse levels have fewer and longer rows; the
+// benchmark's 32,768, 8,192 and 2,048 rows of 13, 31 and 75 blocks get the 8, 32
+// and 32 lanes that the averages would give them to within one step).
 int blk_team(int bs, int n_brows, int64_t nnzb) {
+  if (nnzb < 0) {
+    int tl = 4;
+    while (tl < 32 && (long long)tl * n_brows < 1024LL * kNumSM) tl *= 2;
+    while (tl < bs) tl *= 2;
+    return tl;
+  }
   const double avg = (double)nnzb / (double)(n_brows > 0 ? n_brows : 1);
   int tl = 4;
   while (tl < 64 && tl * 2.5 < avg) tl *= 2;
@@ -307,7 +317,8 @@ bool aligned_to(const void *p, size_t a) { return ((uintptr_t)p % a) == 0; }
 }  // namespace
 
 bool blk_applies(int bs, int n_brows, int64_t nnzb) {
-  return bs >= 2 && bs <= 8 && n_brows > 0 && nnzb >= 6LL * n_brows;
+  return bs >= 2 && bs <= 8 && n_brows > 0 &&
+         (nnzb >= 6LL * n_brows || nnzb == kNnzbUnknown);
 }
 
 // rectangular blocks from the finest level: br coarse rows (4 or 8) by bc

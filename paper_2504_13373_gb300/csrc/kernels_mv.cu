@@ -9,6 +9,7 @@
 // cover whole 32-byte sectors and every matrix byte crosses HBM once per
 // pass.  The block-Jacobi step additionally exchanges the block row's
 // residual through shared memory and applies the precomputed w D^{-1}.
+#include <climits>
 #include <type_traits>
 
 #include "common.cuh"
@@ -23,13 +24,14 @@ template <typename T, int BC, int MODE>
 __global__ void __launch_bounds__(256)
 bsr_mv_kernel(int n_brows, int br, const int *__restrict__ rp, const int *__restrict__ col,
               const T *__restrict__ val, const T *__restrict__ x, const T *__restrict__ b,
-              T *__restrict__ y) {
+              T *__restrict__ y, int lim) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long long)n_brows * br) return;
   const int i = (int)(t / br);
   const int r = (int)(t - (long long)i * br);
   constexpr int W = RowVec<T, BC>::value;
   const int beg = __ldg(rp + i), end = __ldg(rp + i + 1);
+  if (end - beg >= lim) return;      // a long row: the team kernel's
   T acc = T(0);
   for (int k = beg; k < end; ++k) {
     const int j = __ldg(col + k);
@@ -280,19 +282,30 @@ static inline bool cta_rows(int n_brows, int br) { return n_brows <= 4096 && br 
 
 // A warp per block row pays when the thread-per-row grid would fill less
 // than about half of the GPU, or when rows are very long.
+// Without the average, by the first of these alone.
+static inline bool few_scalar_rows(int n_brows, int br) { return (long long)n_brows * br < 65536; }
 static inline bool warp_rows(int n_brows, int br, int64_t nnzb) {
-  if (nnzb < 0 || br > 64) return false;
+  if (br > 64) return false;
+  if (nnzb == kNnzbUnknown) return few_scalar_rows(n_brows, br);
+  if (nnzb < 0) return false;
   const long long threads = (long long)n_brows * br;
   return (threads < 65536 && nnzb >= 4LL * n_brows) || nnzb >= 64LL * n_brows;
+}
+
+// small blocks in rows of unknown length: a warp per block row, not a CTA (a
+// CTA for four 3 x 3 blocks adds up 85 groups: 2,048 rows 15 us)
+static inline bool maybe_short(int br, int bc, int64_t nnzb) {
+  return nnzb == kNnzbUnknown && br * bc < 32;
 }
 
 static inline bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 template <typename T, int MODE>
 static cudaError_t mv_warp_dispatch(int n_brows, int br, int bc, const int *rp, const int *col,
-                                    const T *val, const T *x, const T *b, T *y, cudaStream_t s) {
+                                    const T *val, const T *x, const T *b, T *y, cudaStream_t s,
+                                    int64_t nnzb) {
   const int grid = div_up((long long)n_brows * 32, 256);
-  if (cta_rows(n_brows, br)) {
+  if (cta_rows(n_brows, br) && !maybe_short(br, bc, nnzb)) {
     launch_k(bsr_mv_cta_kernel<T, MODE>, n_brows, 256, (256 + br) * sizeof(T), s, n_brows, br, bc, rp, col, val, x, b, y);
     note_launch();
     return cudaGetLastError();
@@ -309,15 +322,17 @@ static cudaError_t mv_warp_dispatch(int n_brows, int br, int bc, const int *rp, 
 
 template <typename T, int MODE>
 static cudaError_t mv_dispatch(int n_brows, int br, int bc, const int *rp, const int *col,
-                               const T *val, const T *x, const T *b, T *y, cudaStream_t s) {
+                               const T *val, const T *x, const T *b, T *y, cudaStream_t s,
+                               int lim = INT_MAX) {
   const long long rows = (long long)n_brows * br;
   if (rows == 0) return cudaSuccess;
   const int th = 256;
   const int grid = div_up(rows, th);
   const bool al = aligned16(val) && aligned16(x);
+  if (lim != INT_MAX && (!al || bc > 16)) return cudaErrorNotSupported;
 #define GASA_MV_CASE(BC)                                                                   \
   case BC:                                                                                 \
-    launch_k(bsr_mv_kernel<T, BC, MODE>, grid, th, 0, s, n_brows, br, rp, col, val, x, b, y); note_launch();    \
+    launch_k(bsr_mv_kernel<T, BC, MODE>, grid, th, 0, s, n_brows, br, rp, col, val, x, b, y, lim); note_launch();    \
     return cudaGetLastError();
   if (al) {
     switch (bc) {
@@ -331,6 +346,12 @@ static cudaError_t mv_dispatch(int n_brows, int br, int bc, const int *rp, const
 #undef GASA_MV_CASE
   launch_k(bsr_mv_generic<T, MODE>, grid, th, 0, s, n_brows, br, bc, rp, col, val, x, b, y); note_launch();
   return cudaGetLastError();
+}
+
+// rows of unknown length, small blocks: from 16,384 scalar rows on a thread each
+// (8,192 rows of four 3 x 3 blocks: sweep 22.6 us with a warp per block row)
+static inline bool short_enough(int n_brows, int br, int bc, int64_t nnzb) {
+  return maybe_short(br, bc, nnzb) && (long long)n_brows * br >= 16384;
 }
 
 template <typename T>
@@ -348,14 +369,37 @@ cudaError_t launch_bsr_mv(int mode, int n_brows, int br, int bc, const int *rp, 
       if (e != cudaErrorNotSupported) return e;
     }
   }
-  if (n_brows > 0 && warp_rows(n_brows, br, nnzb)) {
+  if constexpr (std::is_same<T, float>::value) {
+    if (nnzb == kNnzbUnknown && wide_shape(br, bc, val, x)) {
+      // few scalar rows: a team per block row whatever its length.  Many: each
+      // row's own length decides on the device, short rows a thread per scalar
+      // row, long ones the team kernel's second launch, which looks through the
+      // row pointers for them (2 us for 131,072 rows; the read-back it replaces
+      // cost the call 10 to 20 us and drained the stream)
+      if (few_scalar_rows(n_brows, br))
+        return launch_wide(mode, n_brows, br, bc, nnzb, rp, col, val, nullptr, x, b, y, s);
+      const cudaError_t e =
+          mode == GASA_MV_ASSIGN
+              ? mv_dispatch<T, GASA_MV_ASSIGN>(n_brows, br, bc, rp, col, val, x, b, y, s, kLongRow)
+          : mode == GASA_MV_RESIDUAL
+              ? mv_dispatch<T, GASA_MV_RESIDUAL>(n_brows, br, bc, rp, col, val, x, b, y, s, kLongRow)
+              : mv_dispatch<T, GASA_MV_ADD>(n_brows, br, bc, rp, col, val, x, b, y, s, kLongRow);
+      if (e != cudaErrorNotSupported)
+        return e != cudaSuccess ? e
+                                : launch_wide(mode, n_brows, br, bc, nnzb, rp, col, val, nullptr, x,
+                                              b, y, s, kLongRow);
+      // no thread-per-row kernel for these blocks: teams for all rows
+      return launch_wide(mode, n_brows, br, bc, nnzb, rp, col, val, nullptr, x, b, y, s);
+    }
+  }
+  if (n_brows > 0 && warp_rows(n_brows, br, nnzb) && !short_enough(n_brows, br, bc, nnzb)) {
     switch (mode) {
       case GASA_MV_ASSIGN:
-        return mv_warp_dispatch<T, GASA_MV_ASSIGN>(n_brows, br, bc, rp, col, val, x, b, y, s);
+        return mv_warp_dispatch<T, GASA_MV_ASSIGN>(n_brows, br, bc, rp, col, val, x, b, y, s, nnzb);
       case GASA_MV_RESIDUAL:
-        return mv_warp_dispatch<T, GASA_MV_RESIDUAL>(n_brows, br, bc, rp, col, val, x, b, y, s);
+        return mv_warp_dispatch<T, GASA_MV_RESIDUAL>(n_brows, br, bc, rp, col, val, x, b, y, s, nnzb);
       default:
-        return mv_warp_dispatch<T, GASA_MV_ADD>(n_brows, br, bc, rp, col, val, x, b, y, s);
+        return mv_warp_dispatch<T, GASA_MV_ADD>(n_brows, br, bc, rp, col, val, x, b, y, s, nnzb);
     }
   }
   switch (mode) {
@@ -623,21 +667,26 @@ template <typename T, int BS, int MODE>
 __global__ void __launch_bounds__(256)
 jacobi_kernel(int n_units, const int *__restrict__ rp, const int *__restrict__ col,
               const T *__restrict__ val, const T *__restrict__ Wm, const T *__restrict__ x,
-              const T *__restrict__ b, T *__restrict__ xo) {
+              const T *__restrict__ b, T *__restrict__ xo, int lim) {
   __shared__ T res[256];
   constexpr int RPB = 256 / BS;
   constexpr int W = RowVec<T, BS>::value;
   const int li = threadIdx.x / BS;
   const int r = threadIdx.x - li * BS;
   const int i = blockIdx.x * RPB + li;
-  const bool active = (li < RPB) && (i < n_units);
+  bool active = (li < RPB) && (i < n_units);
   const size_t row = (size_t)i * BS + r;
   T v = T(0);
   if (active) {
     if (MODE == JAC_FIRST) {
       v = b[row];
     } else {
-      const int beg = __ldg(rp + i), end = __ldg(rp + i + 1);
+      const int beg = __ldg(rp + i);
+      int end = __ldg(rp + i + 1);
+      if (end - beg >= lim) {        // a long row: the team kernel's
+        active = false;
+        end = beg;
+      }
       T acc = T(0);
       for (int k = beg; k < end; ++k) {
         const int j = __ldg(col + k);
@@ -859,9 +908,9 @@ jacobi_group_kernel(int n_units, int bs, const int *__restrict__ rp, const int *
 template <typename T, int MODE>
 static cudaError_t jac_warp_dispatch(int n_units, int bs, const int *rp, const int *col,
                                      const T *val, const T *W, const T *x, const T *b, T *xo,
-                                     cudaStream_t s) {
+                                     cudaStream_t s, int64_t nnzb) {
   const int grid = div_up((long long)n_units * 32, 256);
-  if (cta_rows(n_units, bs)) {
+  if (cta_rows(n_units, bs) && !maybe_short(bs, bs, nnzb)) {
     launch_k(jacobi_cta_kernel<T, MODE>, n_units, 256, (256 + bs) * sizeof(T), s, n_units, bs, rp, col, val, W, x, b, xo);
     note_launch();
     return cudaGetLastError();
@@ -879,14 +928,15 @@ static cudaError_t jac_warp_dispatch(int n_units, int bs, const int *rp, const i
 template <typename T, int MODE>
 static cudaError_t jac_dispatch(int n_units, int bs, const int *rp, const int *col,
                                 const T *val, const T *W, const T *x, const T *b, T *xo,
-                                cudaStream_t s) {
+                                cudaStream_t s, int lim = INT_MAX) {
   if (n_units == 0) return cudaSuccess;
   const bool al = aligned16(val) && aligned16(W) && (MODE == JAC_FIRST || aligned16(x));
+  if (lim != INT_MAX && (!al || bs > 16)) return cudaErrorNotSupported;
 #define GASA_JAC_CASE(BS)                                                                   \
   case BS: {                                                                                \
     constexpr int rpb = 256 / BS;                                                           \
     launch_k(jacobi_kernel<T, BS, MODE>, div_up(n_units, rpb), 256, 0, s, n_units, rp, col, val,  \
-                                                                    W, x, b, xo); note_launch();           \
+                                                                    W, x, b, xo, lim); note_launch();      \
     return cudaGetLastError();                                                              \
   }
   if (al && bs <= 16) {
@@ -923,11 +973,26 @@ cudaError_t launch_jacobi(int mode, int n_units, int bs, const int *rp, const in
       if (e != cudaErrorNotSupported) return e;
     }
   }
-  if (n_units > 0 && mode != JAC_FIRST && warp_rows(n_units, bs, nnzb)) {
+  if constexpr (std::is_same<T, float>::value) {
+    // as in launch_bsr_mv
+    if (mode == JAC_SWEEP && nnzb == kNnzbUnknown && wide_shape(bs, bs, val, x)) {
+      if (few_scalar_rows(n_units, bs))
+        return launch_wide(3, n_units, bs, bs, nnzb, rp, col, val, W, x, b, xo, s);
+      const cudaError_t e = jac_dispatch<T, JAC_SWEEP>(n_units, bs, rp, col, val, W, x, b, xo, s,
+                                                       kLongRow);
+      if (e == cudaErrorNotSupported)
+        return launch_wide(3, n_units, bs, bs, nnzb, rp, col, val, W, x, b, xo, s);
+      return e != cudaSuccess ? e
+                              : launch_wide(3, n_units, bs, bs, nnzb, rp, col, val, W, x, b, xo, s,
+                                            kLongRow);
+    }
+  }
+  if (n_units > 0 && mode != JAC_FIRST && warp_rows(n_units, bs, nnzb) &&
+      !short_enough(n_units, bs, bs, nnzb)) {
     switch (mode) {
-      case JAC_SWEEP: return jac_warp_dispatch<T, JAC_SWEEP>(n_units, bs, rp, col, val, W, x, b, xo, s);
-      case JAC_APPLY: return jac_warp_dispatch<T, JAC_APPLY>(n_units, bs, rp, col, val, W, x, b, xo, s);
-      default: return jac_warp_dispatch<T, JAC_RELAX>(n_units, bs, rp, col, val, W, x, b, xo, s);
+      case JAC_SWEEP: return jac_warp_dispatch<T, JAC_SWEEP>(n_units, bs, rp, col, val, W, x, b, xo, s, nnzb);
+      case JAC_APPLY: return jac_warp_dispatch<T, JAC_APPLY>(n_units, bs, rp, col, val, W, x, b, xo, s, nnzb);
+      default: return jac_warp_dispatch<T, JAC_RELAX>(n_units, bs, rp, col, val, W, x, b, xo, s, nnzb);
     }
   }
   switch (mode) {

@@ -30,6 +30,8 @@
 // level 2 (384 rows of about 275 blocks of 17 x 17, 122 MB): step 35.6 ->
 // 24.4 us; fused restriction of level 1 92.4 -> 60.3 us.  GMRES on Q2 96^2:
 // 5.97 -> 4.75 ms.
+#include <algorithm>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -103,14 +105,17 @@ __device__ __forceinline__ void team_blocks(int k0, int end, int step, int br, i
 // R A = (rp2, col2, val2), and, with Wm (the next level's w D^{-1}), its first
 // smoothing step x2o = Wm y.  blockDim = 32 * ES * BS * teams; dynamic shared
 // memory: 32 * RPL floats per warp and 40 per team.
-template <int VW, int RPL>
-__global__ void __launch_bounds__(32 * kTeamWarps)
+// LONG: only the block rows of at least min_len blocks, the others being
+// left to the thread-per-row kernels.  A CTA then looks through 32 rows at a
+// time and its teams take the long ones among them.
+template <int VW, int RPL, bool LONG>
+__global__ void __launch_bounds__(32 * kTeamWarps, LONG ? 2 : 1)
 bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, const int *__restrict__ rp,
                 const int *__restrict__ col, const float *__restrict__ val,
                 const float *__restrict__ Wm, const float *__restrict__ x,
                 const float *__restrict__ b, float *__restrict__ y, const int *__restrict__ rp2,
                 const int *__restrict__ col2, const float *__restrict__ val2,
-                float *__restrict__ x2o) {
+                float *__restrict__ x2o, int min_len) {
   extern __shared__ float sm[];
   const int nw = ES * BS, warps = blockDim.x >> 5, teams = warps / nw;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -118,80 +123,104 @@ bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, const int *
   const int es = wt % ES, bs = wt / ES;
   const int LC = bc / VW, G = 32 / LC;
   const int g = lane / LC, cl = lane - g * LC;
-  const int u = blockIdx.x * teams + team;
-  const bool on = u < n_brows;
   float *part = sm + (size_t)team * nw * 32 * RPL;            // [nw][RPL][32]
   float *res = sm + (size_t)warps * 32 * RPL + team * kWideMaxRows;
   const bool smooth = op == WIDE_SWEEP || (op == WIDE_RFUSED && Wm);
-  if (smooth && on) {
-    // the block of Wm is needed last: bring it into L2 meanwhile
-    const int lines = (br * br * 4 + 127) / 128 + 1;
-    for (int q = wt * 32 + lane; q < lines; q += nw * 32) {
-      const int o = min(q * 32, br * br - 1);
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(Wm + (size_t)u * br * br + o));
-    }
-  }
-  float acc[RPL];
-#pragma unroll
-  for (int m = 0; m < RPL; ++m) acc[m] = 0.f;
-  if (on && g < G) {
-    const int r0 = es * G + g, rs = ES * G;
-    const int beg = __ldg(rp + u), end = __ldg(rp + u + 1);
-    if (op == WIDE_RFUSED) {
-      const int beg2 = __ldg(rp2 + u), end2 = __ldg(rp2 + u + 1);
-      team_blocks<VW, RPL>(beg + bs, end, BS, br, bc, r0, rs, cl * VW, col, val, b, 1.f, acc);
-      team_blocks<VW, RPL>(beg2 + bs, end2, BS, br, bc, r0, rs, cl * VW, col2, val2, x, -1.f, acc);
-    } else {
-      team_blocks<VW, RPL>(beg + bs, end, BS, br, bc, r0, rs, cl * VW, col, val, x, 1.f, acc);
-    }
-  }
-#pragma unroll
-  for (int m = 0; m < RPL; ++m) part[(wt * RPL + m) * 32 + lane] = acc[m];
-  __syncthreads();
-  // four lanes per row add the row's BS * LC partial sums: blocks' warps in
-  // order, columns sub, sub + 4, ... in order, then the four
-  const int sub = lane & 3;
-  const int rounds = (br * 4 + nw * 32 - 1) / (nw * 32);
-  for (int it = 0; it < rounds; ++it) {
-    const int r = (it * nw * 32 + wt * 32 + lane) >> 2;
-    float v = 0.f;
-    if (r < br) {
-      const int m = r / (ES * G), q = r - m * ES * G;
-      const float *p = part + ((size_t)(q / G) * RPL + m) * 32 + (q % G) * LC;
-      for (int s = 0; s < BS; ++s)
-        for (int c = sub; c < LC; c += 4) v += p[(size_t)s * ES * RPL * 32 + c];
-    }
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    v += __shfl_xor_sync(0xffffffffu, v, 2);
-    if (on && r < br && sub == 0) {
-      const size_t t = (size_t)u * br + r;
-      if (op == WIDE_ASSIGN) y[t] = v;
-      else if (op == WIDE_RESID) y[t] = b[t] - v;
-      else if (op == WIDE_ADD) y[t] = y[t] + v;
-      else if (op == WIDE_RFUSED) {
-        y[t] = v;
-        res[r] = v;
-      } else {
-        res[r] = b[t] - v;
+  auto block_row = [&](int u, bool on) {
+    if (smooth && on) {
+      // the block of Wm is needed last: bring it into L2 meanwhile
+      const int lines = (br * br * 4 + 127) / 128 + 1;
+      for (int q = wt * 32 + lane; q < lines; q += nw * 32) {
+        const int o = min(q * 32, br * br - 1);
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(Wm + (size_t)u * br * br + o));
       }
     }
-  }
-  if (!smooth) return;
-  __syncthreads();
-  // SWEEP: x_out = x + W (b - A x); RFUSED: x2o = Wm y, four lanes per row
-  for (int it = 0; it < rounds; ++it) {
-    const int r = (it * nw * 32 + wt * 32 + lane) >> 2;
-    float v = 0.f;
-    if (on && r < br) {
-      const float *w = Wm + ((size_t)u * br + r) * br;
-      for (int c = sub; c < br; c += 4) v = fmaf(__ldg(w + c), res[c], v);
+    float acc[RPL];
+  #pragma unroll
+    for (int m = 0; m < RPL; ++m) acc[m] = 0.f;
+    if (on && g < G) {
+      const int r0 = es * G + g, rs = ES * G;
+      const int beg = __ldg(rp + u), end = __ldg(rp + u + 1);
+      if (op == WIDE_RFUSED) {
+        const int beg2 = __ldg(rp2 + u), end2 = __ldg(rp2 + u + 1);
+        team_blocks<VW, RPL>(beg + bs, end, BS, br, bc, r0, rs, cl * VW, col, val, b, 1.f, acc);
+        team_blocks<VW, RPL>(beg2 + bs, end2, BS, br, bc, r0, rs, cl * VW, col2, val2, x, -1.f, acc);
+      } else {
+        team_blocks<VW, RPL>(beg + bs, end, BS, br, bc, r0, rs, cl * VW, col, val, x, 1.f, acc);
+      }
     }
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    v += __shfl_xor_sync(0xffffffffu, v, 2);
-    if (on && r < br && sub == 0) {
-      const size_t t = (size_t)u * br + r;
-      if (op == WIDE_SWEEP) y[t] = x[t] + v;
-      else x2o[t] = v;
+  #pragma unroll
+    for (int m = 0; m < RPL; ++m) part[(wt * RPL + m) * 32 + lane] = acc[m];
+    __syncthreads();
+    // four lanes per row add the row's BS * LC partial sums: blocks' warps in
+    // order, columns sub, sub + 4, ... in order, then the four
+    const int sub = lane & 3;
+    const int rounds = (br * 4 + nw * 32 - 1) / (nw * 32);
+    for (int it = 0; it < rounds; ++it) {
+      const int r = (it * nw * 32 + wt * 32 + lane) >> 2;
+      float v = 0.f;
+      if (r < br) {
+        const int m = r / (ES * G), q = r - m * ES * G;
+        const float *p = part + ((size_t)(q / G) * RPL + m) * 32 + (q % G) * LC;
+        for (int s = 0; s < BS; ++s)
+          for (int c = sub; c < LC; c += 4) v += p[(size_t)s * ES * RPL * 32 + c];
+      }
+      v += __shfl_xor_sync(0xffffffffu, v, 1);
+      v += __shfl_xor_sync(0xffffffffu, v, 2);
+      if (on && r < br && sub == 0) {
+        const size_t t = (size_t)u * br + r;
+        if (op == WIDE_ASSIGN) y[t] = v;
+        else if (op == WIDE_RESID) y[t] = b[t] - v;
+        else if (op == WIDE_ADD) y[t] = y[t] + v;
+        else if (op == WIDE_RFUSED) {
+          y[t] = v;
+          res[r] = v;
+        } else {
+          res[r] = b[t] - v;
+        }
+      }
+    }
+    if (!smooth) return;
+    __syncthreads();
+    // SWEEP: x_out = x + W (b - A x); RFUSED: x2o = Wm y, four lanes per row
+    for (int it = 0; it < rounds; ++it) {
+      const int r = (it * nw * 32 + wt * 32 + lane) >> 2;
+      float v = 0.f;
+      if (on && r < br) {
+        const float *w = Wm + ((size_t)u * br + r) * br;
+        for (int c = sub; c < br; c += 4) v = fmaf(__ldg(w + c), res[c], v);
+      }
+      v += __shfl_xor_sync(0xffffffffu, v, 1);
+      v += __shfl_xor_sync(0xffffffffu, v, 2);
+      if (on && r < br && sub == 0) {
+        const size_t t = (size_t)u * br + r;
+        if (op == WIDE_SWEEP) y[t] = x[t] + v;
+        else x2o[t] = v;
+      }
+    }
+  };
+  if constexpr (!LONG) {
+    const int u = blockIdx.x * teams + team;
+    block_row(u, u < n_brows);
+  } else {
+    __shared__ unsigned longs;
+    for (int base = blockIdx.x * 32; base < n_brows; base += gridDim.x * 32) {
+      if (warp == 0) {
+        const int i = base + lane;
+        const unsigned m =
+            __ballot_sync(0xffffffffu, i < n_brows && __ldg(rp + i + 1) - __ldg(rp + i) >= min_len);
+        if (lane == 0) longs = m;
+      }
+      __syncthreads();
+      unsigned m = longs;
+      while (m) {                       // uniform over the CTA: `teams` long rows per turn
+        unsigned t = m;
+        for (int q = 0; q < team && t; ++q) t &= t - 1u;
+        block_row(base + (t ? __ffs(t) - 1 : 0), t != 0);
+        for (int q = 0; q < teams && m; ++q) m &= m - 1u;
+        __syncthreads();
+      }
+      __syncthreads();
     }
   }
 }
@@ -209,7 +238,7 @@ template <int VW>
 cudaError_t team_go(int op, int n_brows, int br, int bc, double avg, const int *rp, const int *col,
                     const float *val, const float *W, const float *x, const float *b, float *y,
                     const int *rp2, const int *col2, const float *val2, float *x2o,
-                    cudaStream_t s) {
+                    int min_len, cudaStream_t s) {
   const int LC = bc / VW, G = 32 / LC;
   const int rows = div_up(br, G);                  // row steps of one warp over a block
   const int ES = div_up(rows, kTeamRows);
@@ -222,23 +251,24 @@ cudaError_t team_go(int op, int n_brows, int br, int bc, double avg, const int *
   while (ES * BS * 2 <= kTeamWarps && avg >= 8.0 * BS &&
          (long long)n_brows * ES * BS < 40LL * kNumSM)
     BS *= 2;
+  if (min_len == 0 && avg > 1e8) BS = std::min(BS, 4);   // rows of unknown length
   const int nw = ES * BS, teams = nw >= 8 ? 1 : 8 / nw, warps = nw * teams;
   const size_t smem = ((size_t)warps * 32 * RPL + teams * kWideMaxRows) * sizeof(float);
-  const int grid = div_up(n_brows, teams);
+  const int grid = min_len > 0 ? std::min(div_up(n_brows, 32), 8 * kNumSM) : div_up(n_brows, teams);
   auto go = [&](auto kern) {
     launch_k(kern, grid, 32 * warps, smem, s, op, n_brows, br, bc, ES, BS, rp, col, val, W, x, b, y,
-             rp2, col2, val2, x2o);
+             rp2, col2, val2, x2o, min_len);
   };
+#define GASA_TEAM(N)                              \
+  case N:                                         \
+    if (min_len > 0) go(bsr_team_kernel<VW, N, true>); \
+    else go(bsr_team_kernel<VW, N, false>);       \
+    break;
   switch (RPL) {
-    case 1: go(bsr_team_kernel<VW, 1>); break;
-    case 2: go(bsr_team_kernel<VW, 2>); break;
-    case 3: go(bsr_team_kernel<VW, 3>); break;
-    case 4: go(bsr_team_kernel<VW, 4>); break;
-    case 5: go(bsr_team_kernel<VW, 5>); break;
-    case 6: go(bsr_team_kernel<VW, 6>); break;
-    case 7: go(bsr_team_kernel<VW, 7>); break;
-    default: go(bsr_team_kernel<VW, 8>); break;
+    GASA_TEAM(1) GASA_TEAM(2) GASA_TEAM(3) GASA_TEAM(4) GASA_TEAM(5) GASA_TEAM(6) GASA_TEAM(7)
+    GASA_TEAM(8)
   }
+#undef GASA_TEAM
   note_launch();
   return cudaGetLastError();
 }
@@ -246,34 +276,40 @@ cudaError_t team_go(int op, int n_brows, int br, int bc, double avg, const int *
 cudaError_t team_launch(int op, int n_brows, int br, int bc, int64_t nnzb, const int *rp,
                         const int *col, const float *val, const float *W, const float *x,
                         const float *b, float *y, const int *rp2, const int *col2,
-                        const float *val2, float *x2o, cudaStream_t s) {
-  const double avg = (double)nnzb / (double)n_brows;
+                        const float *val2, float *x2o, int min_len, cudaStream_t s) {
+  // unknown: long enough for the number of rows alone to decide (team_go caps it)
+  const double avg = nnzb >= 0 ? (double)nnzb / (double)n_brows : 1e9;
   // RFUSED multiplies val with b and val2 with x
   const int vw = op == WIDE_RFUSED ? wide_vec(bc, val, b, val2, x)
                                    : wide_vec(bc, val, x, nullptr, nullptr);
   if (bc / vw > 32) return cudaErrorNotSupported;
   if (vw == 4)
-    return team_go<4>(op, n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2, val2, x2o, s);
+    return team_go<4>(op, n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2, val2, x2o, min_len, s);
   if (vw == 2)
-    return team_go<2>(op, n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2, val2, x2o, s);
-  return team_go<1>(op, n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2, val2, x2o, s);
+    return team_go<2>(op, n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2, val2, x2o, min_len, s);
+  return team_go<1>(op, n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2, val2, x2o, min_len, s);
 }
 
 }  // namespace
 
 bool wide_applies(int br, int bc, int n_brows, int64_t nnzb) {
   return (br > 8 || bc > 8) && br <= kWideMaxRows && bc <= kWideMaxRows && n_brows > 0 &&
-         nnzb >= 8LL * n_brows;
+         nnzb >= (long long)kLongRow * n_brows;
+}
+
+bool wide_shape(int br, int bc, const float *val, const float *x) {
+  return (br > 8 || bc > 8) && br <= kWideMaxRows && bc <= kWideMaxRows &&
+         bc / wide_vec(bc, val, x, nullptr, nullptr) <= 32;
 }
 
 cudaError_t launch_wide(int op, int n_brows, int br, int bc, int64_t nnzb, const int *rp,
                         const int *col, const float *val, const float *W, const float *x,
-                        const float *b, float *y, cudaStream_t s) {
+                        const float *b, float *y, cudaStream_t s, int min_len) {
   if (n_brows == 0) return cudaSuccess;
   if (br > kWideMaxRows || bc > kWideMaxRows || (op == WIDE_SWEEP && br != bc))
     return cudaErrorNotSupported;
   return team_launch(op, n_brows, br, bc, nnzb, rp, col, val, W, x, b, y, nullptr, nullptr, nullptr,
-                     nullptr, s);
+                     nullptr, min_len, s);
 }
 
 cudaError_t launch_wide_restrict(int n_brows, int br, int bc, int64_t nnzb, const int *rrp,
@@ -284,7 +320,7 @@ cudaError_t launch_wide_restrict(int n_brows, int br, int bc, int64_t nnzb, cons
   if (n_brows == 0) return cudaSuccess;
   if (br > kWideMaxRows || bc > kWideMaxRows) return cudaErrorNotSupported;
   return team_launch(WIDE_RFUSED, n_brows, br, bc, nnzb, rrp, rcol, rval, Wn, x, b, y, arp, acol,
-                     aval, xn, s);
+                     aval, xn, 0, s);
 }
 
 }  // namespace gasa

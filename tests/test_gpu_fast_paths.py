@@ -130,3 +130,50 @@ def test_wide_team_products(br, bc, n, lo, hi):
     wtol = np.einsum("nij,nj->ni", np.abs(W).astype(np.float64),
                      (tol + np.abs(r).ravel() * br * 2.0 ** -23).reshape(n, br)).ravel()
     assert np.all(np.abs(out.cpu().numpy() - ref) <= wtol + 2.0 ** -23 * (np.abs(x) + np.abs(ref)))
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "fp64"])
+@pytest.mark.parametrize("br,bc,n,lo,hi", [
+    (10, 10, 7000, 0, 16),      # many scalar rows, short and long ones mixed: each takes its kernel
+    (13, 13, 5100, 7, 8),       # lengths on both sides of the line
+    (20, 20, 3300, 2, 12),      # no thread-per-row kernel at this width
+    (10, 10, 900, 0, 12),       # few scalar rows
+    (3, 3, 2048, 2, 5), (4, 4, 40000, 1, 9), (8, 8, 300, 20, 40), (1, 1, 5, 1, 3),
+    (4, 10, 20000, 1, 12), (10, 4, 8000, 1, 4), (45, 45, 30, 1, 9),
+])
+def test_products_without_a_known_row_length(dtype, br, bc, n, lo, hi):
+    """Single operations choose by sizes and by each row's own length: against the product
+    in 64 bits, aligned and not, n terms of a row to n eps of sum |a x|."""
+    import torch
+    gasa = _gasa()
+    rng = np.random.default_rng(br * 1000 + n)
+    t, eps = (np.float32, 2.0 ** -23) if dtype == "fp32" else (np.float64, 2.0 ** -52)
+    ncols = max(n, hi) if br == bc else 4000
+    rp, col, val = _random_bsr(rng, n, ncols, br, bc, lo, hi)
+    val = val.astype(t)
+    x, b = rng.standard_normal(ncols * bc).astype(t), rng.standard_normal(n * br).astype(t)
+    ax = _bsr_apply(rp, col, val.astype(np.float64), x.astype(np.float64))
+    mag = _bsr_apply(rp, col, np.abs(val).astype(np.float64), np.abs(x).astype(np.float64))
+    tol = (hi * bc + 4) * eps * (mag + np.abs(b)) + 1e-30
+    f = gasa.gasa_bsr_mv_f32 if dtype == "fp32" else gasa.gasa_bsr_mv
+    sweep = gasa.gasa_jacobi_sweep_f32 if dtype == "fp32" else gasa.gasa_jacobi_sweep
+    drp, dcol, db = to_dev(rp), to_dev(col), to_dev(b)
+    for shift in (0, 1):        # 1: values and x one element off their allocation's alignment
+        dval = torch.empty(val.size + 1, dtype=torch.from_numpy(val).dtype, device="cuda")[shift:shift + val.size]
+        dx = torch.empty(x.size + 1, dtype=dval.dtype, device="cuda")[shift:shift + x.size]
+        dval.copy_(to_dev(val.ravel()))
+        dx.copy_(to_dev(x))
+        for mode, ref in ((0, ax), (1, b - ax), (2, b + ax)):
+            y = db.clone()
+            f(mode, n, br, bc, drp, dcol, dval, dx, db, y)
+            assert np.all(np.abs(y.cpu().numpy() - ref) <= tol), (mode, shift)
+        if br == bc and ncols == n:
+            W = (rng.standard_normal((n, br, br)) / br).astype(t)
+            out = torch.zeros_like(db)
+            sweep(n, br, drp, dcol, dval, to_dev(W.ravel()), dx, db, out)
+            r = (b - ax).reshape(n, br)
+            ref = x + np.einsum("nij,nj->ni", W.astype(np.float64), r).ravel()
+            wtol = np.einsum("nij,nj->ni", np.abs(W).astype(np.float64),
+                             (tol + np.abs(r).ravel() * br * eps).reshape(n, br)).ravel()
+            assert np.all(np.abs(out.cpu().numpy() - ref) <= wtol + eps * (np.abs(x) + np.abs(ref))), shift
+
