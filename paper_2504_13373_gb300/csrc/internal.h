@@ -82,6 +82,12 @@ cudaError_t launch_wide(int op, int n_brows, int br, int bc, int64_t nnzb, const
 // whether launch_wide takes these blocks, whatever the row lengths
 bool wide_shape(int br, int bc, const float *val, const float *x);
 
+// ---- kernels_team64.cu: FP64, a team of warps per block row ------------------
+// op as launch_wide, blocks up to 64 x 64; cudaErrorNotSupported for others
+cudaError_t launch_team64(int op, int n_brows, int br, int bc, int64_t nnzb, const int *rp,
+                          const int *col, const double *val, const double *W, const double *x,
+                          const double *b, double *y, cudaStream_t s);
+
 // ---- kernels_blk.cu: small square blocks, one lane per block ---------------
 // true when square s x s blocks (2 <= s <= 8) average at least 6 per block row
 // (or nnzb is kNnzbUnknown); launch_blk then takes FP32 operands (FP64 returns

@@ -298,6 +298,15 @@ static inline bool maybe_short(int br, int bc, int64_t nnzb) {
   return nnzb == kNnzbUnknown && br * bc < 32;
 }
 
+// FP64: the team kernel of kernels_team64.cu instead of these, for blocks that
+// fill a warp's lanes at least (smaller ones leave them idle, which FP64
+// instructions do not forgive) or rows long enough to be worth it anyway;
+// without the average, blocks of 32 values on
+static inline bool team64_rows(int n_brows, int br, int bc, int64_t nnzb) {
+  if (!warp_rows(n_brows, br, nnzb)) return false;
+  return br * bc >= 32 || nnzb >= 16LL * n_brows;
+}
+
 static inline bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 template <typename T, int MODE>
@@ -390,6 +399,12 @@ cudaError_t launch_bsr_mv(int mode, int n_brows, int br, int bc, const int *rp, 
                                               b, y, s, kLongRow);
       // no thread-per-row kernel for these blocks: teams for all rows
       return launch_wide(mode, n_brows, br, bc, nnzb, rp, col, val, nullptr, x, b, y, s);
+    }
+  }
+  if constexpr (std::is_same<T, double>::value) {
+    if (n_brows > 0 && team64_rows(n_brows, br, bc, nnzb)) {
+      const cudaError_t e = launch_team64(mode, n_brows, br, bc, nnzb, rp, col, val, nullptr, x, b, y, s);
+      if (e != cudaErrorNotSupported) return e;
     }
   }
   if (n_brows > 0 && warp_rows(n_brows, br, nnzb) && !short_enough(n_brows, br, bc, nnzb)) {
@@ -985,6 +1000,14 @@ cudaError_t launch_jacobi(int mode, int n_units, int bs, const int *rp, const in
       return e != cudaSuccess ? e
                               : launch_wide(3, n_units, bs, bs, nnzb, rp, col, val, W, x, b, xo, s,
                                             kLongRow);
+    }
+  }
+  if constexpr (std::is_same<T, double>::value) {
+    // smoothing steps only: JAC_APPLY is the power iteration of Alg. 4, whose
+    // rounding the candidates downstream of it amplify
+    if (mode == JAC_SWEEP && n_units > 0 && team64_rows(n_units, bs, bs, nnzb)) {
+      const cudaError_t e = launch_team64(3, n_units, bs, bs, nnzb, rp, col, val, W, x, b, xo, s);
+      if (e != cudaErrorNotSupported) return e;
     }
   }
   if (n_units > 0 && mode != JAC_FIRST && warp_rows(n_units, bs, nnzb) &&

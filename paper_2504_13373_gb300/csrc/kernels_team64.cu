@@ -1,0 +1,164 @@
+// FP64 block-sparse products and smoothing steps on levels with few scalar
+// rows, where a thread per scalar row would leave the GPU short of warps.
+//
+// An SM does two FP64 FMAs a clock, a warp's instruction taking an SM quarter
+// 64 clocks whether one lane is active or all, so these products are bound by
+// the number of FP64 instructions.  The lanes of a warp therefore take a
+// block's br * bc values side by side (lane l the values l, l + 32, ..., EPL of
+// them), the same positions of every block, and keep one partial sum per
+// position: every lane works on every block, the matrix is read in runs of 256
+// bytes, and nothing is added up before the row's end.  A team of ES x BS warps
+// owns a block row: ES share out a block's positions (at most 32 * 8 each), BS
+// the blocks.  At the end the sums of a row's positions meet in shared memory;
+// four lanes add up a row in a fixed order, which depends only on the matrix
+// and the team.  (A CTA per block row with a thread per row of a block, as
+// before, spent half of its FP64 instructions on adding up 256 / br groups one
+// after another.)
+//
+// Operations: y = A x, y = b - A x, y += A x for br x bc blocks up to 64 x 64,
+// and the block-Jacobi step x_out = x + W (b - A x) (square blocks).
+//
+// GB300, Q2 128^2 V-cycle, FP64, levels of 4,096, 1,024 and 256 units (12 x 12,
+// 16 x 16 and 21 x 21 blocks): these products took 1,084 us of the V-cycle and
+// take 940 (smoothing steps 47.3 us on average before; now 34.5, 36.3 and 49.2).
+#include "common.cuh"
+#include "internal.h"
+
+namespace gasa {
+
+namespace {
+
+constexpr int kT64Values = 8;       // values of a block per lane at most
+constexpr int kT64Warps = 16;       // warps per team at most
+
+template <int EPL>
+__global__ void __launch_bounds__(32 * kT64Warps)
+team64_kernel(int op, int n_brows, int br, int bc, int ES, int BS, const int *__restrict__ rp,
+              const int *__restrict__ col, const double *__restrict__ val,
+              const double *__restrict__ Wm, const double *__restrict__ x,
+              const double *__restrict__ b, double *__restrict__ y) {
+  extern __shared__ double sm64[];
+  const int nw = ES * BS, warps = blockDim.x >> 5, teams = warps / nw;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int team = warp / nw, wt = warp - team * nw;
+  const int es = wt % ES, bs = wt / ES;
+  const int u = blockIdx.x * teams + team;
+  const bool on = u < n_brows;
+  const int E = br * bc, pitch = ES * EPL * 32;
+  double *part = sm64 + (size_t)team * BS * pitch;              // [BS][positions]
+  double *res = sm64 + (size_t)teams * BS * pitch + (size_t)team * br;
+  double acc[EPL];
+  int e[EPL], q[EPL];
+#pragma unroll
+  for (int m = 0; m < EPL; ++m) {
+    // positions past the block's end repeat its last value; their sums are not used
+    e[m] = min((es * EPL + m) * 32 + lane, E - 1);
+    q[m] = e[m] % bc;
+    acc[m] = 0.0;
+  }
+  if (on) {
+    const int beg = __ldg(rp + u), end = __ldg(rp + u + 1);
+    int k = beg + bs;
+    int j0 = k < end ? __ldg(col + k) : 0, j1 = k + BS < end ? __ldg(col + k + BS) : 0;
+    for (; k + BS < end; k += 2 * BS) {
+      const double *a0 = val + (size_t)k * E, *a1 = val + (size_t)(k + BS) * E;
+      const double *x0 = x + (size_t)j0 * bc, *x1 = x + (size_t)j1 * bc;
+      double av0[EPL], av1[EPL], xv0[EPL], xv1[EPL];
+#pragma unroll
+      for (int m = 0; m < EPL; ++m) {
+        av0[m] = __ldg(a0 + e[m]);
+        av1[m] = __ldg(a1 + e[m]);
+      }
+#pragma unroll
+      for (int m = 0; m < EPL; ++m) {
+        xv0[m] = __ldg(x0 + q[m]);
+        xv1[m] = __ldg(x1 + q[m]);
+      }
+      j0 = k + 2 * BS < end ? __ldg(col + k + 2 * BS) : 0;
+      j1 = k + 3 * BS < end ? __ldg(col + k + 3 * BS) : 0;
+#pragma unroll
+      for (int m = 0; m < EPL; ++m) acc[m] = fma(av1[m], xv1[m], fma(av0[m], xv0[m], acc[m]));
+    }
+    if (k < end) {
+      const double *a0 = val + (size_t)k * E, *x0 = x + (size_t)j0 * bc;
+#pragma unroll
+      for (int m = 0; m < EPL; ++m) acc[m] = fma(__ldg(a0 + e[m]), __ldg(x0 + q[m]), acc[m]);
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < EPL; ++m) part[(size_t)bs * pitch + (es * EPL + m) * 32 + lane] = acc[m];
+  __syncthreads();
+  // four lanes per row: the warps' sums in order, columns sub, sub + 4, ... in
+  // order, then the four; warps without a row skip it
+  const int sub = lane & 3;
+  for (int t0 = wt * 32; t0 < br * 4; t0 += nw * 32) {
+    const int r = (t0 + lane) >> 2;
+    double v = 0.0;
+    if (r < br)
+      for (int s = 0; s < BS; ++s)
+        for (int c = sub; c < bc; c += 4) v += part[(size_t)s * pitch + r * bc + c];
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    if (on && r < br && sub == 0) {
+      const size_t t = (size_t)u * br + r;
+      if (op == 0) y[t] = v;
+      else if (op == 1) y[t] = b[t] - v;
+      else if (op == 2) y[t] = y[t] + v;
+      else res[r] = b[t] - v;
+    }
+  }
+  if (op != 3) return;
+  __syncthreads();
+  for (int t0 = wt * 32; t0 < br * 4; t0 += nw * 32) {
+    const int r = (t0 + lane) >> 2;
+    double v = 0.0;
+    if (on && r < br) {
+      const double *w = Wm + ((size_t)u * br + r) * br;
+      for (int c = sub; c < br; c += 4) v = fma(__ldg(w + c), res[c], v);
+    }
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    if (on && r < br && sub == 0) {
+      const size_t t = (size_t)u * br + r;
+      y[t] = x[t] + v;
+    }
+  }
+}
+
+}  // namespace
+
+cudaError_t launch_team64(int op, int n_brows, int br, int bc, int64_t nnzb, const int *rp,
+                          const int *col, const double *val, const double *W, const double *x,
+                          const double *b, double *y, cudaStream_t s) {
+  if (n_brows == 0) return cudaSuccess;
+  if (br > 64 || bc > 64 || (op == 3 && br != bc)) return cudaErrorNotSupported;
+  const int per = div_up(br * bc, 32);
+  const int ES = div_up(per, kT64Values), EPL = div_up(per, ES);
+  // blocks shared out over warps while each keeps eight or more (its sums cost
+  // about as much as one) and the GPU has fewer than 16 warps an SM
+  const double avg = nnzb >= 0 ? (double)nnzb / (double)n_brows : 1e9;
+  int BS = 1;
+  while (ES * BS * 2 <= kT64Warps && avg >= 16.0 * BS && (long long)n_brows * ES * BS < 16LL * kNumSM)
+    BS *= 2;
+  if (nnzb < 0 && BS > 4) BS = 4;
+  const int nw = ES * BS, teams = nw >= 4 ? 1 : 4 / nw, warps = nw * teams;
+  const size_t smem = ((size_t)warps * 32 * EPL + (size_t)teams * br) * sizeof(double);
+  auto go = [&](auto kern) {
+    launch_k(kern, div_up(n_brows, teams), 32 * warps, smem, s, op, n_brows, br, bc, ES, BS, rp, col,
+             val, W, x, b, y);
+  };
+  switch (EPL) {
+    case 1: go(team64_kernel<1>); break;
+    case 2: go(team64_kernel<2>); break;
+    case 3: go(team64_kernel<3>); break;
+    case 4: go(team64_kernel<4>); break;
+    case 5: go(team64_kernel<5>); break;
+    case 6: go(team64_kernel<6>); break;
+    case 7: go(team64_kernel<7>); break;
+    default: go(team64_kernel<8>); break;
+  }
+  note_launch();
+  return cudaGetLastError();
+}
+
+}  // namespace gasa

@@ -177,3 +177,31 @@ def test_products_without_a_known_row_length(dtype, br, bc, n, lo, hi):
                              (tol + np.abs(r).ravel() * br * eps).reshape(n, br)).ravel()
             assert np.all(np.abs(out.cpu().numpy() - ref) <= wtol + eps * (np.abs(x) + np.abs(ref))), shift
 
+
+@pytest.mark.parametrize("br,bc", [(12, 12), (16, 16), (21, 21), (13, 13), (64, 64), (4, 9),
+                                   (36, 9), (1, 33), (40, 2), (6, 6)])
+@pytest.mark.parametrize("n,lo,hi", [(1, 1, 1), (37, 0, 70), (300, 16, 40)])
+def test_fp64_team_products(br, bc, n, lo, hi):
+    """FP64 products on few rows, every split of a block's values over lanes and warps: n
+    terms of a row to n 2^-52 of sum |a x|."""
+    gasa = _gasa()
+    rng = np.random.default_rng(br * 100 + bc + n)
+    ncols = max(n, hi)
+    rp, col, val = _random_bsr(rng, n, ncols, br, bc, lo, hi)
+    x, b = rng.standard_normal(ncols * bc), rng.standard_normal(n * br)
+    ax, mag = _bsr_apply(rp, col, val, x), _bsr_apply(rp, col, np.abs(val), np.abs(x))
+    tol = (hi * bc + 4) * 2.0 ** -52 * (mag + np.abs(b)) + 1e-300
+    d = [to_dev(a) for a in (rp, col, val.ravel(), x, b)]
+    for mode, ref in ((0, ax), (1, b - ax), (2, b + ax)):
+        y = d[4].clone()
+        gasa.gasa_bsr_mv(mode, n, br, bc, *d[:4], d[4], y)
+        assert np.all(np.abs(y.cpu().numpy() - ref) <= tol)
+    if br == bc and ncols == n:
+        W = rng.standard_normal((n, br, br)) / br
+        out = to_dev(np.zeros(n * br))
+        gasa.gasa_jacobi_sweep(n, br, *d[:3], to_dev(W.ravel()), d[3], d[4], out)
+        r = (b - ax).reshape(n, br)
+        ref = x + np.einsum("nij,nj->ni", W, r).ravel()
+        wtol = np.einsum("nij,nj->ni", np.abs(W),
+                         (tol + np.abs(r).ravel() * br * 2.0 ** -52).reshape(n, br)).ravel()
+        assert np.all(np.abs(out.cpu().numpy() - ref) <= wtol + 2.0 ** -52 * (np.abs(x) + np.abs(ref)))
