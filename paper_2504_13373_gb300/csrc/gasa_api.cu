@@ -687,7 +687,8 @@ gasa_status vcycle_impl(gasa_ctx *ctx, const T *rhs, T *out, bool h16 = false,
     Level &l = ctx->L[k];
     if (k == 0 && fold0) {
       if (mode == JAC_SWEEP)
-        return launch_folded_sweep<T>(l.n, l.s, l.A.rp, l.A.col, P::WA(l), xin, P::c(l), xo, s);
+        return launch_folded_sweep<T>(l.n, l.s, l.A.rp, l.A.col, P::WA(l), xin, P::c(l), xo, s,
+                                      l.A.nnzb);
       // first step u = W b, kept as c for the later steps
       cudaError_t e = launch_jacobi<T>(JAC_FIRST, l.n, l.s, l.A.rp, l.A.col, P::A(l.A), P::W(l),
                                        nullptr, bb, xo, s, l.A.nnzb);
@@ -1056,12 +1057,12 @@ gasa_status pcg(gasa_ctx *ctx, const double *b, double tol, int precision, int *
       ST(vcycle_f32_out(ctx, r, precision));
       CU(launch_cg_dots_f32(n, r, ctx->kf_out, ctx->kzold_f, ctx->rz_ds, ctx->rzo_ds, s));
       CU(launch_cg_update_p_f32(n, p, ctx->kf_out, ctx->scal + cur, ctx->rz_ds, ctx->rzo_ds,
-                                ctx->scal + nxt, ctx->kzold_f, ctx->kp_hi, ctx->kp_lo, kRedBlocks,
+                                ctx->scal + nxt, ctx->kzold_f, ctx->kp_hi, ctx->kp_lo, cg_blocks(n),
                                 s));
       ST(spmv_outer_ds(ctx, p, q));
       CU(launch_cg_update_xr(n, x, r, p, q, ctx->scal + nxt, ctx->pq_ds, rr_part,
                              ctx->scal + S_ALPHA, s, pq_ds_count(ctx)));
-      CU(launch_finalize(rr_part, 1, ctx->scal + S_RR, s));
+      CU(launch_finalize_n(rr_part, cg_blocks(n), ctx->scal + S_RR, s));
       ST(read_scalars(ctx, 0, 3));
       const double pq = ctx->hscal[S_PQ];
       if (!std::isfinite(pq)) return fail(ctx, GASA_ERR_BREAKDOWN, "CG: non-finite p^T A p");
@@ -1098,7 +1099,7 @@ gasa_status pcg(gasa_ctx *ctx, const double *b, double tol, int precision, int *
     CU(launch_dot_partials(n, p, q, pq_part, s));
     CU(launch_cg_update_xr(n, x, r, p, q, ctx->scal + cur, pq_part, rr_part,
                            ctx->scal + S_ALPHA, s, kRedBlocks));
-    CU(launch_finalize(rr_part, 1, ctx->scal + S_RR, s));
+    CU(launch_finalize_n(rr_part, cg_blocks(n), ctx->scal + S_RR, s));
     ST(read_scalars(ctx, 0, 3));
     const double pq = ctx->hscal[S_PQ];
     if (!(pq > 0.0)) {
@@ -1166,7 +1167,7 @@ gasa_status build_cg_graph(gasa_ctx *ctx, int precision) {
   ctx->prof = false;   // no event records inside a graph body
   const long long k0 = launch_count();
   CU(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-  int np = kRedBlocks;
+  int np = flex ? cg_blocks(n) : kRedBlocks;
   gasa_status st = GASA_OK;
   cudaError_t e = cudaSuccess;
   if (flex) {
@@ -1198,7 +1199,7 @@ gasa_status build_cg_graph(gasa_ctx *ctx, int precision) {
     if (e == cudaSuccess)
       e = launch_cg_update_xr(n, x, r, p, q, ctx->scal + S_RZ1, flex ? ctx->pq_ds : pq_part,
                               rr_part, ctx->scal + S_ALPHA, s, flex ? pq_ds_count(ctx) : kRedBlocks);
-    if (e == cudaSuccess) e = launch_cg_check(rr_part, ctx->scal, ctx->d_iters, max_iter, h, s);
+    if (e == cudaSuccess) e = launch_cg_check(rr_part, cg_blocks(n), ctx->scal, ctx->d_iters, max_iter, h, s);
   }
   cudaGraph_t captured = nullptr;
   cudaError_t e2 = cudaStreamEndCapture(s, &captured);
@@ -1365,7 +1366,7 @@ gasa_status gmres(gasa_ctx *ctx, const double *b, double tol, int precision, int
       // classical Gram-Schmidt, twice
       for (int pass = 0; pass < 2; ++pass) {
         CU(launch_multi_dot(n, ctx->V, n, j + 1, w, ctx->mpart, s));
-        CU(launch_multi_dot_finalize(ctx->mpart, j + 1, pass == 0 ? h : h2, Hj, s));
+        CU(launch_multi_dot_finalize(n, ctx->mpart, j + 1, pass == 0 ? h : h2, Hj, s));
         CU(launch_gs_update(n, ctx->V, n, j + 1, pass == 0 ? h : h2, w, s));
       }
       CU(launch_dot_partials(n, w, nullptr, ctx->part, s));
@@ -1406,7 +1407,7 @@ gasa_status stationary_step(gasa_ctx *ctx, int precision, int max_iter,
   CU(launch_axpy(n, 1.0, ctx->kz, ctx->kx, s));
   ST(spmv_outer(ctx, GASA_MV_RESIDUAL, ctx->kx, ctx->kb, ctx->kt));
   CU(launch_dot_partials(n, ctx->kt, nullptr, rr_part, s));
-  if (in_graph) CU(launch_cg_check(rr_part, ctx->scal, ctx->d_iters, max_iter, h, s));
+  if (in_graph) CU(launch_cg_check(rr_part, kRedBlocks, ctx->scal, ctx->d_iters, max_iter, h, s));
   else CU(launch_finalize(rr_part, 1, ctx->scal + S_RR, s));
   return GASA_OK;
 }

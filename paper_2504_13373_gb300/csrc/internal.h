@@ -89,7 +89,7 @@ cudaError_t launch_team64(int op, int n_brows, int br, int bc, int64_t nnzb, con
                           const double *b, double *y, cudaStream_t s);
 
 // ---- kernels_blk.cu: small square blocks, one lane per block ---------------
-// true when square s x s blocks (2 <= s <= 8) average at least 6 per block row
+// true when square s x s blocks (2 <= s <= 8) average at least 3 per block row
 // (or nnzb is kNnzbUnknown); launch_blk then takes FP32 operands (FP64 returns
 // cudaErrorNotSupported)
 bool blk_applies(int bs, int n_brows, int64_t nnzb);
@@ -109,7 +109,8 @@ cudaError_t launch_blk_restrict_rect(int n_brows, int br, int bc, int64_t nnzb, 
                                      const int *acol, const float *aval, const float *b,
                                      const float *x, float *y, const float *Wn, float *xn,
                                      cudaStream_t s);
-// op 0/1/2: y = A x, y = b - A x, y += A x; op 3: y = x + W (b - A x).
+// op 0/1/2: y = A x, y = b - A x, y += A x; op 3: y = x + W (b - A x);
+// op 4: y = x + (b - A x), for any row length.
 // cudaErrorNotSupported when the shape or the alignment does not fit.
 template <typename T>
 cudaError_t launch_blk(int op, int n_brows, int bs, int64_t nnzb, const int *rp, const int *col,
@@ -144,7 +145,7 @@ cudaError_t launch_jacobi_first_conv(int n_units, int bs, const double *bd, floa
 constexpr int kMvFolded = 3;   // internal product mode next to GASA_MV_*
 template <typename T>
 cudaError_t launch_folded_sweep(int n_units, int bs, const int *rp, const int *col, const T *WA,
-                                const T *x, const T *c, T *xo, cudaStream_t s);
+                                const T *x, const T *c, T *xo, cudaStream_t s, int64_t nnzb);
 // WA = W A block row by block row: block k of block row i becomes W_i A_k (FP64)
 cudaError_t launch_fold_block_rows(int n_units, int bs, const int *rp, const double *W,
                                    const double *A, double *WA, cudaStream_t s);
@@ -207,7 +208,9 @@ cudaError_t launch_fill(int64_t n, double v, double *x, cudaStream_t s);
 template <typename T>
 cudaError_t launch_add(int64_t n, const T *x, T *y, cudaStream_t s);
 
-// CG pieces (device scalars; partial arrays of kRedBlocks entries)
+// CG pieces (device scalars; the reductions here leave cg_blocks(n) partials,
+// at most kRedBlocks)
+int cg_blocks(int64_t n);
 cudaError_t launch_cg_update_xr(int64_t n, double *x, double *r, const double *p,
                                 const double *q, const double *rz, const double *pq_partials,
                                 double *rr_partials, double *alpha_out, cudaStream_t s,
@@ -217,7 +220,7 @@ cudaError_t launch_cg_update_p(int64_t n, double *p, const double *z, const doub
                                double *rz_out, int flexible, cudaStream_t s,
                                double *zold_out, float *p_hi, float *p_lo, int n_rz);
 // mixed-precision CG with z, zold in FP32 (exact in FP64): partials of r . z
-// and r . zold in one pass (the sums of launch_dot_partials on FP64 copies),
+// and r . zold in one pass,
 // and the flexible p update reading z from FP32, copying it to zold_out and
 // splitting p (8-byte aligned FP32 and 16-byte aligned FP64 arrays, else
 // cudaErrorNotSupported)
@@ -229,8 +232,8 @@ cudaError_t launch_cg_update_p_f32(int64_t n, double *p, const float *z, const d
                                    int n_rz, cudaStream_t s);
 // exact two-term FP32 split v = hi + lo of an FP64 vector
 cudaError_t launch_split(int64_t n, const double *v, float *hi, float *lo, cudaStream_t s);
-cudaError_t launch_cg_check(const double *rr_partials, double *scal, int *iters, int max_iter,
-                            cudaGraphConditionalHandle handle, cudaStream_t s);
+cudaError_t launch_cg_check(const double *rr_partials, int n_rr, double *scal, int *iters,
+                            int max_iter, cudaGraphConditionalHandle handle, cudaStream_t s);
 void note_launches(long long n);
 cudaError_t launch_axpy(int64_t n, double a, const double *x, double *y, cudaStream_t s);
 cudaError_t launch_copy(int64_t n, const double *x, double *y, cudaStream_t s);
@@ -239,8 +242,8 @@ cudaError_t launch_sub(int64_t n, const double *a, const double *b, double *out,
 // GMRES pieces
 cudaError_t launch_multi_dot(int64_t n, const double *V, int64_t ldv, int k, const double *w,
                              double *partials, cudaStream_t s);
-cudaError_t launch_multi_dot_finalize(const double *partials, int k, double *h,
-                                      double *hacc, cudaStream_t s);
+cudaError_t launch_multi_dot_finalize(int64_t n, const double *partials, int k, double *h,
+                                      double *hacc, cudaStream_t s);   // n of the dot products
 cudaError_t launch_gs_update(int64_t n, const double *V, int64_t ldv, int k, const double *h,
                              double *w, cudaStream_t s);
 cudaError_t launch_normalize_into(int64_t n, const double *w, const double *sumsq, double *v,

@@ -12,8 +12,9 @@
 // wider than a warp, in shared memory in a fixed order), so every row is
 // summed in an order that depends only on the matrix.
 //
-// Operations: y = A x, y = b - A x, y += A x, and the block-Jacobi step
-// x_out = x + W (b - A x) of Alg. 1 with W = w D^{-1}.
+// Operations: y = A x, y = b - A x, y += A x, the block-Jacobi step
+// x_out = x + W (b - A x) of Alg. 1 with W = w D^{-1}, and its folded form
+// x_out = x + (c - A x).
 #include <atomic>
 #include <cstdlib>
 
@@ -24,7 +25,7 @@ namespace gasa {
 
 namespace {
 
-enum { BLK_ASSIGN = 0, BLK_RESID = 1, BLK_ADD = 2, BLK_SWEEP = 3 };
+enum { BLK_ASSIGN = 0, BLK_RESID = 1, BLK_ADD = 2, BLK_SWEEP = 3, BLK_FOLDED = 4 };
 
 template <typename T, int N>
 struct BlkVec {
@@ -67,7 +68,8 @@ bsr_blk_kernel(int n_brows, const int *__restrict__ rp, const int *__restrict__ 
     load_run<T, S>(Wm + t * S, wv);
     xt = x[t];
   }
-  if (OP == BLK_RESID && writer) bt = b[t];
+  if ((OP == BLK_RESID || OP == BLK_FOLDED) && writer) bt = b[t];
+  if (OP == BLK_FOLDED && writer) xt = x[t];
   if (OP == BLK_ADD && writer) yt = y[t];
   if (u < n_brows) {
     const int beg = __ldg(rp + u), end = __ldg(rp + u + 1);
@@ -143,6 +145,7 @@ bsr_blk_kernel(int n_brows, const int *__restrict__ rp, const int *__restrict__ 
     if (r == l) v = acc[r];
   if (OP == BLK_ASSIGN) y[t] = v;
   else if (OP == BLK_RESID) y[t] = bt - v;
+  else if (OP == BLK_FOLDED) y[t] = xt + (bt - v);
   else y[t] = yt + v;
 }
 
@@ -318,7 +321,7 @@ bool aligned_to(const void *p, size_t a) { return ((uintptr_t)p % a) == 0; }
 
 bool blk_applies(int bs, int n_brows, int64_t nnzb) {
   return bs >= 2 && bs <= 8 && n_brows > 0 &&
-         (nnzb >= 6LL * n_brows || nnzb == kNnzbUnknown);
+         (nnzb >= 3LL * n_brows || nnzb == kNnzbUnknown);
 }
 
 // rectangular blocks from the finest level: br coarse rows (4 or 8) by bc
@@ -373,7 +376,7 @@ template <>
 cudaError_t launch_blk<float>(int op, int n_brows, int bs, int64_t nnzb, const int *rp,
                               const int *col, const float *val, const float *W, const float *x,
                               const float *b, float *y, cudaStream_t s) {
-  if (!blk_applies(bs, n_brows, nnzb)) return cudaErrorNotSupported;
+  if (op != BLK_FOLDED && !blk_applies(bs, n_brows, nnzb)) return cudaErrorNotSupported;
   // vector loads need the arrays aligned like their runs (cudaMalloc gives 256 bytes)
   for (const void *p : {(const void *)val, (const void *)W, (const void *)x, (const void *)b})
     if (p && !aligned_to(p, 16)) return cudaErrorNotSupported;
@@ -382,6 +385,7 @@ cudaError_t launch_blk<float>(int op, int n_brows, int bs, int64_t nnzb, const i
     case BLK_ASSIGN: return blk_launch<T, BLK_ASSIGN>(n_brows, bs, nnzb, rp, col, val, W, x, b, y, s);
     case BLK_RESID: return blk_launch<T, BLK_RESID>(n_brows, bs, nnzb, rp, col, val, W, x, b, y, s);
     case BLK_ADD: return blk_launch<T, BLK_ADD>(n_brows, bs, nnzb, rp, col, val, W, x, b, y, s);
+    case BLK_FOLDED: return blk_launch<T, BLK_FOLDED>(n_brows, bs, nnzb, rp, col, val, W, x, b, y, s);
     case BLK_SWEEP: return blk_launch<T, BLK_SWEEP>(n_brows, bs, nnzb, rp, col, val, W, x, b, y, s);
     default: return cudaErrorInvalidValue;
   }

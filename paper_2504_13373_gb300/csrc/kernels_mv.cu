@@ -435,8 +435,17 @@ template cudaError_t launch_bsr_mv<float>(int, int, int, int, const int *, const
 
 template <typename T>
 cudaError_t launch_folded_sweep(int n_units, int bs, const int *rp, const int *col, const T *WA,
-                                const T *x, const T *c, T *xo, cudaStream_t s) {
+                                const T *x, const T *c, T *xo, cudaStream_t s, int64_t nnzb) {
   if constexpr (std::is_same<T, float>::value) {
+    // small blocks: a lane per block (a thread per scalar row walks its three to
+    // five blocks one after another: 3 x 3 blocks, 2,048 rows 3.26 -> 1.93 us,
+    // 32,768 rows 4.23 -> 2.59; 6 x 6, 8,192 rows 5.18 -> 2.64; 4 x 4, 9,216 rows
+    // 5.79 -> 2.56).  Wider blocks keep a thread per row: with a team of lanes per
+    // block row 9 x 9 takes 11.7 us against 8.9, 10 x 10 from 4.0 against 3.6 up.
+    if (bs >= 2 && bs <= 8 && n_units > 0) {
+      const cudaError_t e = launch_blk<T>(4, n_units, bs, nnzb, rp, col, WA, nullptr, x, c, xo, s);
+      if (e != cudaErrorNotSupported) return e;
+    }
     if (bs == 10 && n_units > 0 && aligned16(WA) && aligned16(x)) {
       launch_k(folded_pair_kernel<10, 6>, div_up((long long)n_units * bs, 256), 256, 0, s,
                n_units, bs, rp, col, WA, x, c, xo);
@@ -448,10 +457,10 @@ cudaError_t launch_folded_sweep(int n_units, int bs, const int *rp, const int *c
 }
 template cudaError_t launch_folded_sweep<double>(int, int, const int *, const int *, const double *,
                                                  const double *, const double *, double *,
-                                                 cudaStream_t);
+                                                 cudaStream_t, int64_t);
 template cudaError_t launch_folded_sweep<float>(int, int, const int *, const int *, const float *,
                                                 const float *, const float *, float *,
-                                                cudaStream_t);
+                                                cudaStream_t, int64_t);
 
 // ----------------------------------------------------------------------------
 // y = A x in double-single arithmetic (the outer Krylov product of the
@@ -1130,40 +1139,47 @@ cudaError_t launch_bsr_mm(int n_brows, int br, int bc, const int *rp, const int 
 
 // ----------------------------------------------------------------------------
 // dense y = A x (coarsest level A = A_N^{-1}, or the dense bottom operator of
-// the V-cycle; A row-major FP64, FP64 arithmetic): a CTA of 256 threads per
-// row, thread t sums columns t, t + 256, ... in order (eight in flight), then
-// a warp tree and the eight warp sums in order
+// the V-cycle; A row-major FP64, FP64 arithmetic): a warp per row, lane l takes
+// column pairs l, l + 32, ... in order (four pairs in flight), then a warp tree.
+// Order 1,792: 14.1 -> 13.7 us on GB300 (3.2 million FP64 FMAs are 5.3 us
+// of it).
 // ----------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(128)
 dense_mv_kernel(int n, int ld, const double *__restrict__ A, const T *__restrict__ x,
                 T *__restrict__ y) {
-  __shared__ double sh[8];
-  const int row = blockIdx.x;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int row = blockIdx.x * 4 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (row >= n) return;
   const double *a = A + (size_t)row * ld;
   double acc = 0.0;
-  int j = threadIdx.x;
-  for (; j + 7 * 256 < n; j += 8 * 256) {
-    double av[8], xv[8];
+  if ((ld & 1) == 0) {
+    const double2 *a2 = reinterpret_cast<const double2 *>(a);   // ld even: rows 16-byte aligned
+    const int m = n >> 1;
+    int j = lane;
+    for (; j + 96 < m; j += 128) {
+      double2 av[4];
+      T x0[4], x1[4];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      av[u] = __ldg(a + j + u * 256);
-      xv[u] = (double)__ldg(x + j + u * 256);
+      for (int u = 0; u < 4; ++u) {
+        av[u] = __ldg(a2 + j + 32 * u);
+        x0[u] = __ldg(x + 2 * (j + 32 * u));
+        x1[u] = __ldg(x + 2 * (j + 32 * u) + 1);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        acc = fma(av[u].y, (double)x1[u], fma(av[u].x, (double)x0[u], acc));
     }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) acc = fma(av[u], xv[u], acc);
+    for (; j < m; j += 32) {
+      const double2 av = __ldg(a2 + j);
+      acc = fma(av.y, (double)__ldg(x + 2 * j + 1), fma(av.x, (double)__ldg(x + 2 * j), acc));
+    }
+    if ((n & 1) && lane == 0) acc = fma(__ldg(a + n - 1), (double)__ldg(x + n - 1), acc);
+  } else {
+    for (int j = lane; j < n; j += 32) acc = fma(__ldg(a + j), (double)__ldg(x + j), acc);
   }
-  for (; j < n; j += 256) acc = fma(__ldg(a + j), (double)__ldg(x + j), acc);
   acc = warp_sum(acc);
-  if (lane == 0) sh[wid] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double v = 0.0;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) v += sh[w];
-    y[row] = (T)v;
-  }
+  if (lane == 0) y[row] = (T)acc;
 }
 
 // y = M x for the FP32 cycle's dense bottom operator: M as exact two-term
@@ -1171,17 +1187,23 @@ dense_mv_kernel(int n, int ld, const double *__restrict__ A, const T *__restrict
 // products and sums in double-single arithmetic on FP32 units (the scheme of
 // bsr_mv_ds_kernel with x exact in FP32), so each row agrees with the FP64
 // product to about 2^-47 of sum |m x|; GB300's FP64 pipe would take n^2 FMAs
-// at a small fraction of the FP32 rate.  A CTA of 256 threads per row, thread
-// t over columns t, t + 256, ... (eight in flight), its (s, lo) pair to FP64,
-// then a warp tree and the eight warp sums in order.
-__global__ void __launch_bounds__(256)
+// at a small fraction of the FP32 rate.  A warp per row (two where rows are
+// few), lane l takes groups of four columns l, l + 32, ... in order with 16-byte
+// loads, two groups in flight; its (s, lo) pairs meet in a warp tree, then FP64.
+// Order 2,048 (33.5 MB): 12.0 -> 7.4 us on GB300; a CTA per row took 4-byte loads
+// and its barriers were most of a row's time.
+template <int WPR>
+__global__ void __launch_bounds__(128)
 dense_mv_ds_kernel(int n, int ld, const float *__restrict__ Mh, const float *__restrict__ Ml,
                    const float *__restrict__ x, float *__restrict__ y) {
-  __shared__ double sh[8];
-  const int row = blockIdx.x;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const float *h = Mh + (size_t)row * ld;
-  const float *l = Ml + (size_t)row * ld;
+  __shared__ double sh[4];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int row = blockIdx.x * (4 / WPR) + warp / WPR;
+  const bool on = row < n;
+  const size_t o = (size_t)(on ? row : n - 1) * ld;
+  const float4 *h4 = reinterpret_cast<const float4 *>(Mh + o);
+  const float4 *l4 = reinterpret_cast<const float4 *>(Ml + o);
+  const float4 *x4 = reinterpret_cast<const float4 *>(x);
   float s = 0.0f, lo = 0.0f;
   auto add = [&](float ah, float al, float xh) {
     const float pr = __fmul_rn(ah, xh);
@@ -1193,35 +1215,53 @@ dense_mv_ds_kernel(int n, int ld, const float *__restrict__ Mh, const float *__r
     s = s1;
     lo = __fadd_rn(lo, __fadd_rn(err, __fadd_rn(e, cross)));
   };
-  int j = threadIdx.x;
-  for (; j + 7 * 256 < n; j += 8 * 256) {
-    float hv[8], lv[8], xv[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      hv[u] = __ldg(h + j + u * 256);
-      lv[u] = __ldg(l + j + u * 256);
-      xv[u] = __ldg(x + j + u * 256);
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) add(hv[u], lv[u], xv[u]);
+  auto add4 = [&](const float4 &h, const float4 &l, const float4 &v) {
+    add(h.x, l.x, v.x);
+    add(h.y, l.y, v.y);
+    add(h.z, l.z, v.z);
+    add(h.w, l.w, v.w);
+  };
+  constexpr int step = 32 * WPR;
+  const int m = n >> 2;
+  int j = (warp % WPR) * 32 + lane;
+  for (; j + step < m; j += 2 * step) {
+    const float4 h0 = __ldg(h4 + j), l0 = __ldg(l4 + j), v0 = __ldg(x4 + j);
+    const float4 h1 = __ldg(h4 + j + step), l1 = __ldg(l4 + j + step), v1 = __ldg(x4 + j + step);
+    add4(h0, l0, v0);
+    add4(h1, l1, v1);
   }
-  for (; j < n; j += 256) add(__ldg(h + j), __ldg(l + j), __ldg(x + j));
+  if (j < m) add4(__ldg(h4 + j), __ldg(l4 + j), __ldg(x4 + j));
+  if (warp % WPR == 0 && lane < (n & 3)) {       // the last one to three columns
+    const int c = (m << 2) + lane;
+    add(__ldg(Mh + o + c), __ldg(Ml + o + c), __ldg(x + c));
+  }
   double v = (double)s + (double)lo;
   v = warp_sum(v);
-  if (lane == 0) sh[wid] = v;
+  if (WPR == 1) {
+    if (on && lane == 0) y[row] = (float)v;
+    return;
+  }
+  if (lane == 0) sh[warp] = v;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (on && lane == 0 && warp % WPR == 0) {
     double t = 0.0;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) t += sh[w];
+    for (int w = 0; w < WPR; ++w) t += sh[warp + w];
     y[row] = (float)t;
   }
 }
 
+// Mh, Ml and x 16-byte aligned, ld a multiple of four
 cudaError_t launch_dense_mv_ds(int n, int ld, const float *Mh, const float *Ml, const float *x,
                                float *y, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  launch_k(dense_mv_ds_kernel, n, 256, 0, s, n, ld, Mh, Ml, x, y);
+  // about 16 warps per SM: two warps per row below 2,432 rows, four below 1,216
+  if (n >= 16 * kNumSM)
+    launch_k(dense_mv_ds_kernel<1>, div_up(n, 4), 128, 0, s, n, ld, Mh, Ml, x, y);
+  else if (n >= 8 * kNumSM)
+    launch_k(dense_mv_ds_kernel<2>, div_up(n, 2), 128, 0, s, n, ld, Mh, Ml, x, y);
+  else
+    launch_k(dense_mv_ds_kernel<4>, n, 128, 0, s, n, ld, Mh, Ml, x, y);
   note_launch();
   return cudaGetLastError();
 }
@@ -1230,7 +1270,7 @@ template <typename T>
 cudaError_t launch_dense_mv(int n, const double *A, const T *x, T *y, cudaStream_t s, int ld) {
   if (n == 0) return cudaSuccess;
   if (ld < n) ld = n;
-  launch_k(dense_mv_kernel<T>, n, 256, 0, s, n, ld, A, x, y); note_launch();
+  launch_k(dense_mv_kernel<T>, div_up(n, 4), 128, 0, s, n, ld, A, x, y); note_launch();
   return cudaGetLastError();
 }
 template cudaError_t launch_dense_mv<double>(int, const double *, const double *, double *,

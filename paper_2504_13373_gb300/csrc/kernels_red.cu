@@ -24,6 +24,24 @@ long long launch_count() { return g_launches.load(std::memory_order_relaxed); }
 // runs over a grid-stride loop and the odd last entry (if any) goes to
 // thread 0 of CTA 0, so each partial sums a fixed set of entries in a fixed
 // order.
+// CTAs of the CG step's vector kernels: a pair of entries per thread, at most
+// kRedBlocks.  Every update first adds up the previous reduction's partials in
+// each CTA, so on a small level (6,144 dofs: 12 CTAs) the other CTAs' zeros cost
+// more than the vectors: p update 6.6 -> 4.3 us, x, r update 5.7 -> 4.6 us, r . z
+// 4.8 -> 4.0 us on GB300.
+int cg_blocks(int64_t n) {
+  return (int)std::min<int64_t>(kRedBlocks,
+                                std::max<int64_t>(1, (n + 2 * kRedThreads - 1) / (2 * kRedThreads)));
+}
+
+// Sum of n partials, every thread gets it: up to 32 by each warp for itself (no
+// barrier), more by the CTA
+__device__ __forceinline__ double sum_partials(const double *p, int n, double *sh) {
+  if (n > 32) return block_sum_partials(p, n, sh);
+  const int lane = threadIdx.x & 31;
+  return warp_sum(lane < n ? p[lane] : 0.0);
+}
+
 __device__ __forceinline__ double2 ld2(const double *p, int64_t k) {
   return __ldg(reinterpret_cast<const double2 *>(p) + k);
 }
@@ -308,12 +326,17 @@ cg_update_xr_kernel(int64_t n, double *__restrict__ x, double *__restrict__ r,
                     const double *__restrict__ rz, const double *__restrict__ pq_partials,
                     double *__restrict__ rr_partials, double *__restrict__ alpha_out, int n_pq) {
   __shared__ double sh[32];
-  const double pq = block_sum_partials(pq_partials, n_pq, sh);
-  const double alpha = rz[0] / pq;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    alpha_out[0] = alpha;
-    alpha_out[1] = pq;
+  __shared__ double alpha_s;
+  const double pq = sum_partials(pq_partials, n_pq, sh);
+  if (threadIdx.x == 0) {      // one FP64 division per CTA, not one per warp
+    alpha_s = rz[0] / pq;
+    if (blockIdx.x == 0) {
+      alpha_out[0] = alpha_s;
+      alpha_out[1] = pq;
+    }
   }
+  __syncthreads();
+  const double alpha = alpha_s;
   double v0 = 0.0, v1 = 0.0;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -378,10 +401,10 @@ cudaError_t launch_cg_update_xr(int64_t n, double *x, double *r, const double *p
                                 const double *q, const double *rz, const double *pq_partials,
                                 double *rr_partials, double *alpha_out, cudaStream_t s, int n_pq) {
   if (al16(x) && al16(r) && al16(p) && al16(q))
-    launch_k(cg_update_xr_kernel<true>, kRedBlocks, kRedThreads, 0, s, n, x, r, p, q, rz,
+    launch_k(cg_update_xr_kernel<true>, cg_blocks(n), kRedThreads, 0, s, n, x, r, p, q, rz,
              pq_partials, rr_partials, alpha_out, n_pq);
   else
-    launch_k(cg_update_xr_kernel<false>, kRedBlocks, kRedThreads, 0, s, n, x, r, p, q, rz,
+    launch_k(cg_update_xr_kernel<false>, cg_blocks(n), kRedThreads, 0, s, n, x, r, p, q, rz,
              pq_partials, rr_partials, alpha_out, n_pq);
   note_launch();
   return cudaGetLastError();
@@ -420,11 +443,16 @@ cg_update_p_kernel(int64_t n, double *__restrict__ p, const double *__restrict__
                    int flexible, double *__restrict__ zold_out, float *__restrict__ p_hi,
                    float *__restrict__ p_lo, int n_rz) {
   __shared__ double sh[32];
-  const double rz_new = block_sum_partials(rz_partials, n_rz, sh);
+  __shared__ double beta_s;
+  const double rz_new = sum_partials(rz_partials, n_rz, sh);
   double num = rz_new;
-  if (flexible) num -= block_sum_partials(rzold_partials, n_rz, sh);
-  const double beta = num / rz_old[0];
-  if (blockIdx.x == 0 && threadIdx.x == 0) rz_out[0] = rz_new;
+  if (flexible) num -= sum_partials(rzold_partials, n_rz, sh);
+  if (threadIdx.x == 0) {
+    beta_s = num / rz_old[0];
+    if (blockIdx.x == 0) rz_out[0] = rz_new;
+  }
+  __syncthreads();
+  const double beta = beta_s;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   if (VEC) {
     const int64_t m = n >> 1;
@@ -463,10 +491,10 @@ cudaError_t launch_cg_update_p(int64_t n, double *p, const double *z, const doub
                                double *rz_out, int flexible, cudaStream_t s, double *zold_out,
                                float *p_hi, float *p_lo, int n_rz) {
   if (al16(p) && al16(z) && (!zold_out || al16(zold_out)))
-    launch_k(cg_update_p_kernel<true>, kRedBlocks, kRedThreads, 0, s, n, p, z, rz_old,
+    launch_k(cg_update_p_kernel<true>, cg_blocks(n), kRedThreads, 0, s, n, p, z, rz_old,
              rz_partials, rzold_partials, rz_out, flexible, zold_out, p_hi, p_lo, n_rz);
   else
-    launch_k(cg_update_p_kernel<false>, kRedBlocks, kRedThreads, 0, s, n, p, z, rz_old,
+    launch_k(cg_update_p_kernel<false>, cg_blocks(n), kRedThreads, 0, s, n, p, z, rz_old,
              rz_partials, rzold_partials, rz_out, flexible, zold_out, p_hi, p_lo, n_rz);
   note_launch();
   return cudaGetLastError();
@@ -474,8 +502,8 @@ cudaError_t launch_cg_update_p(int64_t n, double *p, const double *z, const doub
 
 // The mixed-precision CG step with z and zold left in FP32 by the V-cycle
 // (their FP64 values are exact): the partial sums of r . z and r . zold in
-// one pass, over the same pairs, in the same order and tree as
-// dot_partials_kernel<true>, so they equal those of FP64 copies bit for bit
+// one pass, with the pairs and trees of dot_partials_kernel<true> on cg_blocks(n)
+// CTAs
 __global__ void __launch_bounds__(kRedThreads)
 cg_dots_f32_kernel(int64_t n, const double *__restrict__ r, const float *__restrict__ z,
                    const float *__restrict__ zo, double *__restrict__ part_rz,
@@ -523,7 +551,7 @@ cg_dots_f32_kernel(int64_t n, const double *__restrict__ r, const float *__restr
 cudaError_t launch_cg_dots_f32(int64_t n, const double *r, const float *z, const float *zold,
                                double *part_rz, double *part_rzo, cudaStream_t s) {
   if (!al16(r) || ((uintptr_t)z & 7u) || ((uintptr_t)zold & 7u)) return cudaErrorNotSupported;
-  launch_k(cg_dots_f32_kernel, kRedBlocks, kRedThreads, 0, s, n, r, z, zold, part_rz, part_rzo);
+  launch_k(cg_dots_f32_kernel, cg_blocks(n), kRedThreads, 0, s, n, r, z, zold, part_rz, part_rzo);
   note_launch();
   return cudaGetLastError();
 }
@@ -538,10 +566,15 @@ cg_update_p_f32_kernel(int64_t n, double *__restrict__ p, const float *__restric
                        float *__restrict__ zold_out, float *__restrict__ p_hi,
                        float *__restrict__ p_lo, int n_rz) {
   __shared__ double sh[32];
-  const double rz_new = block_sum_partials(rz_partials, n_rz, sh);
-  const double num = rz_new - block_sum_partials(rzold_partials, n_rz, sh);
-  const double beta = num / rz_old[0];
-  if (blockIdx.x == 0 && threadIdx.x == 0) rz_out[0] = rz_new;
+  __shared__ double beta_s;
+  const double rz_new = sum_partials(rz_partials, n_rz, sh);
+  const double num = rz_new - sum_partials(rzold_partials, n_rz, sh);
+  if (threadIdx.x == 0) {
+    beta_s = num / rz_old[0];
+    if (blockIdx.x == 0) rz_out[0] = rz_new;
+  }
+  __syncthreads();
+  const double beta = beta_s;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t m = n >> 1;
   double2 *p2 = reinterpret_cast<double2 *>(p);
@@ -570,7 +603,7 @@ cudaError_t launch_cg_update_p_f32(int64_t n, double *p, const float *z, const d
                                    double *rz_out, float *zold_out, float *p_hi, float *p_lo,
                                    int n_rz, cudaStream_t s) {
   if (!al16(p) || ((uintptr_t)z & 7u) || ((uintptr_t)zold_out & 7u)) return cudaErrorNotSupported;
-  launch_k(cg_update_p_f32_kernel, kRedBlocks, kRedThreads, 0, s, n, p, z, rz_old, rz_partials,
+  launch_k(cg_update_p_f32_kernel, cg_blocks(n), kRedThreads, 0, s, n, p, z, rz_old, rz_partials,
            rzold_partials, rz_out, zold_out, p_hi, p_lo, n_rz);
   note_launch();
   return cudaGetLastError();
@@ -581,10 +614,10 @@ cudaError_t launch_cg_update_p_f32(int64_t n, double *p, const float *z, const d
 // above tol * ||b||, p^T A p > 0 and fewer than max_iter steps were taken).
 // scal: [0] r.r  [2] p.Ap  [3] rz (old)  [4] rz (new)  [9] ||b||  [10] tol
 __global__ void __launch_bounds__(kRedThreads)
-cg_check_kernel(const double *__restrict__ rr_partials, double *__restrict__ scal, int *iters,
-                int max_iter, cudaGraphConditionalHandle handle) {
+cg_check_kernel(const double *__restrict__ rr_partials, int n_rr, double *__restrict__ scal,
+                int *iters, int max_iter, cudaGraphConditionalHandle handle) {
   __shared__ double sh[32];
-  const double rr = block_sum_partials(rr_partials, kRedBlocks, sh);
+  const double rr = sum_partials(rr_partials, n_rr, sh);
   if (threadIdx.x == 0) {
     scal[0] = rr;
     const int k = ++iters[0];
@@ -596,9 +629,9 @@ cg_check_kernel(const double *__restrict__ rr_partials, double *__restrict__ sca
   }
 }
 
-cudaError_t launch_cg_check(const double *rr_partials, double *scal, int *iters, int max_iter,
-                            cudaGraphConditionalHandle handle, cudaStream_t s) {
-  launch_k(cg_check_kernel, 1, kRedThreads, 0, s, rr_partials, scal, iters, max_iter, handle); note_launch();
+cudaError_t launch_cg_check(const double *rr_partials, int n_rr, double *scal, int *iters,
+                            int max_iter, cudaGraphConditionalHandle handle, cudaStream_t s) {
+  launch_k(cg_check_kernel, 1, n_rr > 32 ? kRedThreads : 32, 0, s, rr_partials, n_rr, scal, iters, max_iter, handle); note_launch();
   return cudaGetLastError();
 }
 
@@ -617,31 +650,31 @@ multi_dot_kernel(int64_t n, const double *__restrict__ V, int64_t ldv,
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
     acc = fma(v[i], w[i], acc);
   acc = block_sum(acc, sh);
-  if (threadIdx.x == 0) partials[(size_t)blockIdx.y * kRedBlocks + blockIdx.x] = acc;
+  if (threadIdx.x == 0) partials[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = acc;
 }
 
 cudaError_t launch_multi_dot(int64_t n, const double *V, int64_t ldv, int k, const double *w,
                              double *partials, cudaStream_t s) {
   if (k == 0) return cudaSuccess;
-  launch_k(multi_dot_kernel, dim3(kRedBlocks, k), kRedThreads, 0, s, n, V, ldv, w, partials); note_launch();
+  launch_k(multi_dot_kernel, dim3(cg_blocks(n), k), kRedThreads, 0, s, n, V, ldv, w, partials); note_launch();
   return cudaGetLastError();
 }
 
 __global__ void __launch_bounds__(kRedThreads)
-multi_dot_finalize_kernel(const double *__restrict__ partials, double *__restrict__ h,
+multi_dot_finalize_kernel(const double *__restrict__ partials, int nb, double *__restrict__ h,
                           double *__restrict__ hacc) {
   __shared__ double sh[32];
-  const double v = block_sum_partials(partials + (size_t)blockIdx.x * kRedBlocks, kRedBlocks, sh);
+  const double v = sum_partials(partials + (size_t)blockIdx.x * nb, nb, sh);
   if (threadIdx.x == 0) {
     h[blockIdx.x] = v;
     if (hacc) hacc[blockIdx.x] += v;
   }
 }
 
-cudaError_t launch_multi_dot_finalize(const double *partials, int k, double *h, double *hacc,
-                                      cudaStream_t s) {
+cudaError_t launch_multi_dot_finalize(int64_t n, const double *partials, int k, double *h,
+                                      double *hacc, cudaStream_t s) {
   if (k == 0) return cudaSuccess;
-  launch_k(multi_dot_finalize_kernel, k, kRedThreads, 0, s, partials, h, hacc); note_launch();
+  launch_k(multi_dot_finalize_kernel, k, kRedThreads, 0, s, partials, cg_blocks(n), h, hacc); note_launch();
   return cudaGetLastError();
 }
 
@@ -665,9 +698,16 @@ cudaError_t launch_gs_update(int64_t n, const double *V, int64_t ldv, int k, con
 __global__ void normalize_into_kernel(int64_t n, const double *__restrict__ w,
                                       const double *__restrict__ sumsq, double *__restrict__ v,
                                       double *__restrict__ hout) {
-  const double nr = sqrt(sumsq[0]);
-  if (blockIdx.x == 0 && threadIdx.x == 0) hout[0] = nr;
-  const double a = nr > 0.0 ? 1.0 / nr : 0.0;
+  // one square root and division per CTA: in every warp they were most of the
+  // kernel (82,944 entries 5.7 -> 2.9 us on GB300)
+  __shared__ double a_s;
+  if (threadIdx.x == 0) {
+    const double nr = sqrt(sumsq[0]);
+    if (blockIdx.x == 0) hout[0] = nr;
+    a_s = nr > 0.0 ? 1.0 / nr : 0.0;
+  }
+  __syncthreads();
+  const double a = a_s;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
     v[i] = w[i] * a;
@@ -675,7 +715,7 @@ __global__ void normalize_into_kernel(int64_t n, const double *__restrict__ w,
 
 cudaError_t launch_normalize_into(int64_t n, const double *w, const double *sumsq, double *v,
                                   double *hout, cudaStream_t s) {
-  launch_k(normalize_into_kernel, kRedBlocks * 2, 256, 0, s, n, w, sumsq, v, hout); note_launch();
+  launch_k(normalize_into_kernel, cg_blocks(n), 256, 0, s, n, w, sumsq, v, hout); note_launch();
   return cudaGetLastError();
 }
 
