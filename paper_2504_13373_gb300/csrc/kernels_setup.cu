@@ -293,29 +293,35 @@ cudaError_t build_children(int n_units, int n_agg, const int *agg_of, int *child
 // 31 additions (the same additions, so the same bits, as a tree each), and one
 // evaluation of ten rotations, a lane each.  Norms of columns that no rotation
 // has touched since are kept.  The three levels of a P2 8^3 tet mesh (384, 48
-// and 6 aggregates of 80, 104 and 136 rows by 80), GB300: 204.7 -> 103.6 ms
-// (42.0, 39.4 and 22.3); 2,048 aggregates of 12 x 12: 4.84 -> 1.84 ms.  (Jacobi on a
+// and 6 aggregates of 80, 104 and 136 rows by 80), GB300: 204.7 -> 89.8 ms
+// (41.9, 30.1 and 17.8); 2,048 aggregates of 12 x 12: 4.84 -> 1.84 ms.  (Jacobi on a
 // QR-preconditioned factor needs a third of the sweeps, 22.9 ms, but rounds
 // differently, and the kept vectors of the coarse levels reach down to 1e-10
 // of the largest singular value, where they are as good as their rounding.)
 // ----------------------------------------------------------------------------
-constexpr int kJacPairs = 10;      // pairs a warp takes at once: 3 x 10 sums in 32 lanes
-
-// sums of 32 quantities over the warp: lane l returns the sum of v[l], added in
-// the order of warp_sum (16, 8, 4, 2, 1 apart)
-__device__ __forceinline__ double warp_sum_packed(double (&v)[32], int lane) {
+// sums of N = 16 or 32 quantities over the warp, added in the order of warp_sum
+// (16, 8, 4, 2, 1 apart): lane l returns the sum of v[l] (N = 32) or v[l / 2]
+template <int N>
+__device__ __forceinline__ double warp_sum_packed(double (&v)[N], int lane) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
+    const int w = o * N / 32;        // quantities a lane keeps after this step
     const bool hi = lane & o;
+    if (w == 0) {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+      continue;
+    }
 #pragma unroll
-    for (int j = 0; j < o; ++j) {
-      const double mine = hi ? v[j + o] : v[j], other = hi ? v[j] : v[j + o];
+    for (int j = 0; j < w; ++j) {
+      const double mine = hi ? v[j + w] : v[j], other = hi ? v[j] : v[j + w];
       v[j] = mine + __shfl_xor_sync(0xffffffffu, other, o);
     }
   }
   return v[0];
 }
 
+// PAIRS: pairs a warp takes at once, 10 (30 sums in 32 lanes) or 5 (15 in 16)
+template <int PAIRS>
 __global__ void tentative_kernel(int bs, const int *__restrict__ child_ptr,
                                  const int *__restrict__ child_idx, const double *__restrict__ B,
                                  int64_t ldb, int r, int s_next, double *__restrict__ T,
@@ -360,11 +366,11 @@ __global__ void tentative_kernel(int bs, const int *__restrict__ child_ptr,
     if (threadIdx.x == 0) rotated = 0;
     __syncthreads();
     for (int t = 0; t < m - 1; ++t) {
-      for (int k0 = wid * kJacPairs; k0 < m / 2; k0 += nwarps * kJacPairs) {
+      for (int k0 = wid * PAIRS; k0 < m / 2; k0 += nwarps * PAIRS) {
         // lane j holds pair k0 + j: columns p, q (q < 0: past the last pair, or the dummy player)
         const int k = k0 + lane;
         int p = 0, q = -1;
-        if (lane < kJacPairs && k < m / 2) {
+        if (lane < PAIRS && k < m / 2) {
           const int a = (k == 0) ? 0 : ((k - 1 + t) % (m - 1)) + 1;
           const int b = ((m - 1 - k - 1 + t) % (m - 1)) + 1;
           p = min(a, b);
@@ -374,12 +380,13 @@ __global__ void tentative_kernel(int bs, const int *__restrict__ child_ptr,
         const unsigned live = __ballot_sync(0xffffffffu, q >= 0);
         const unsigned newp = __ballot_sync(0xffffffffu, np < 0.0);
         const unsigned newq = __ballot_sync(0xffffffffu, nq < 0.0);
-        // partial sums: dot products in 0 .., norms of p in 10 .., of q in 20 ..
-        double v[32];
+        // partial sums: dot products first, then the norms of the p, then of the q
+        constexpr int N = PAIRS > 5 ? 32 : 16, per = 32 / N;
+        double v[N];
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = 0.0;
+        for (int j = 0; j < N; ++j) v[j] = 0.0;
 #pragma unroll
-        for (int j = 0; j < kJacPairs; ++j) {
+        for (int j = 0; j < PAIRS; ++j) {
           if (!(live >> j & 1u)) continue;
           const double *gp = G + (size_t)__shfl_sync(0xffffffffu, p, j) * rows;
           const double *gq = G + (size_t)__shfl_sync(0xffffffffu, q, j) * rows;
@@ -387,14 +394,15 @@ __global__ void tentative_kernel(int bs, const int *__restrict__ child_ptr,
           for (int i = lane; i < rows; i += 32) {
             const double x = gp[i], y = gq[i];
             v[j] = fma(x, y, v[j]);
-            if (fp) v[kJacPairs + j] = fma(x, x, v[kJacPairs + j]);
-            if (fq) v[2 * kJacPairs + j] = fma(y, y, v[2 * kJacPairs + j]);
+            if (fp) v[PAIRS + j] = fma(x, x, v[PAIRS + j]);
+            if (fq) v[2 * PAIRS + j] = fma(y, y, v[2 * PAIRS + j]);
           }
         }
-        const double sum = warp_sum_packed(v, lane);
-        const double sp = __shfl_sync(0xffffffffu, sum, lane + kJacPairs);
-        const double sq = __shfl_sync(0xffffffffu, sum, lane + 2 * kJacPairs);
-        const double ga = q >= 0 ? sum : 0.0;
+        const double sum = warp_sum_packed<N>(v, lane);
+        const double sg = __shfl_sync(0xffffffffu, sum, lane * per);
+        const double sp = __shfl_sync(0xffffffffu, sum, (lane + PAIRS) * per);
+        const double sq = __shfl_sync(0xffffffffu, sum, (lane + 2 * PAIRS) * per);
+        const double ga = q >= 0 ? sg : 0.0;
         const double al = np < 0.0 ? sp : np, be = nq < 0.0 ? sq : nq;
         const bool rot = ga != 0.0 && fabs(ga) > tol * sqrt(al * be);
         const unsigned rots = __ballot_sync(0xffffffffu, rot);
@@ -409,7 +417,7 @@ __global__ void tentative_kernel(int bs, const int *__restrict__ child_ptr,
         const double cs_l = 1.0 / sqrt(1.0 + tt * tt);
         const double sn_l = cs_l * tt;
 #pragma unroll
-        for (int j = 0; j < kJacPairs; ++j) {
+        for (int j = 0; j < PAIRS; ++j) {
           if (!(rots >> j & 1u)) continue;
           double *gp = G + (size_t)__shfl_sync(0xffffffffu, p, j) * rows;
           double *gq = G + (size_t)__shfl_sync(0xffffffffu, q, j) * rows;
@@ -580,15 +588,21 @@ cudaError_t launch_tentative(int bs, int n_agg, int max_children, const int *chi
                                    cudaStream_t s, const int *unit_size, const int *keep) {
   if (n_agg == 0) return cudaSuccess;
   const size_t sm = (size_t)max_children * bs * r * sizeof(double);
-  cudaError_t e = cudaFuncSetAttribute(tentative_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
-  // four warps hold the pairs of r = 80 at once, one per SM quarter
   const int pairs = (r + 1) / 2;
-  const int th = 32 * std::max(1, std::min(4, div_up(pairs, kJacPairs)));
-  tentative_kernel<<<n_agg, th, sm, s>>>(bs, child_ptr, child_idx, B, ldb, r, s_next, T, sigma,
-                                         status, unit_size, keep); note_launch();
-  return cudaGetLastError();
+  // Ten pairs a warp, four warps for r = 80, one per SM quarter, where CTAs share
+  // an SM; with a CTA per SM at most, five a warp, so that two warps per quarter
+  // cover each other's latencies (48 aggregates of 104 x 80: 39.4 -> 30.1 ms, 6 of
+  // 136 x 80: 22.3 -> 17.8 ms)
+  auto go = [&](auto kern, int per) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    const int th = 32 * std::max(1, std::min(per == 10 ? 4 : 8, div_up(pairs, per)));
+    launch_k(kern, n_agg, th, sm, s, bs, child_ptr, child_idx, B, ldb, r, s_next, T, sigma, status,
+             unit_size, keep);
+    note_launch();
+    return cudaGetLastError();
+  };
+  return n_agg <= kNumSM ? go(tentative_kernel<5>, 5) : go(tentative_kernel<10>, 10);
 }
 
 // ----------------------------------------------------------------------------
