@@ -687,8 +687,10 @@ cudaError_t launch_bsr_mv_ds(int n_brows, int br, int bc, const int *rp, const i
 // the block row's residual meets in shared memory, then thread (li, r)
 // applies row r of W_i.
 // ----------------------------------------------------------------------------
-template <typename T, int BS, int MODE>
-__global__ void __launch_bounds__(256)
+// PAIR: the blocks of a row two at a time under a register cap, as in
+// folded_pair_kernel (same bits)
+template <typename T, int BS, int MODE, bool PAIR = false>
+__global__ void __launch_bounds__(256, PAIR ? 5 : 0)
 jacobi_kernel(int n_units, const int *__restrict__ rp, const int *__restrict__ col,
               const T *__restrict__ val, const T *__restrict__ Wm, const T *__restrict__ x,
               const T *__restrict__ b, T *__restrict__ xo, int lim) {
@@ -712,7 +714,25 @@ jacobi_kernel(int n_units, const int *__restrict__ rp, const int *__restrict__ c
         end = beg;
       }
       T acc = T(0);
-      for (int k = beg; k < end; ++k) {
+      int k = beg;
+      for (; PAIR && k + 2 <= end; k += 2) {
+        const int j0 = __ldg(col + k), j1 = __ldg(col + k + 1);
+        const T *a0 = val + ((size_t)k * BS + r) * BS, *a1 = a0 + BS * BS;
+        T av0[BS], av1[BS], xv0[BS], xv1[BS];
+#pragma unroll
+        for (int c = 0; c < BS; c += W) load_vec_stream<T, W>(a0 + c, av0 + c);
+#pragma unroll
+        for (int c = 0; c < BS; c += W) load_vec_stream<T, W>(a1 + c, av1 + c);
+#pragma unroll
+        for (int c = 0; c < BS; c += W) load_vec<T, W>(x + (size_t)j0 * BS + c, xv0 + c);
+#pragma unroll
+        for (int c = 0; c < BS; c += W) load_vec<T, W>(x + (size_t)j1 * BS + c, xv1 + c);
+#pragma unroll
+        for (int c = 0; c < BS; ++c) acc = fma(av0[c], xv0[c], acc);
+#pragma unroll
+        for (int c = 0; c < BS; ++c) acc = fma(av1[c], xv1[c], acc);
+      }
+      for (; k < end; ++k) {
         const int j = __ldg(col + k);
         const T *a = val + ((size_t)k * BS + r) * BS;
         const T *xj = x + (size_t)j * BS;
@@ -956,6 +976,14 @@ static cudaError_t jac_dispatch(int n_units, int bs, const int *rp, const int *c
   if (n_units == 0) return cudaSuccess;
   const bool al = aligned16(val) && aligned16(W) && (MODE == JAC_FIRST || aligned16(x));
   if (lim != INT_MAX && (!al || bs > 16)) return cudaErrorNotSupported;
+  if constexpr (std::is_same<T, float>::value && MODE == JAC_SWEEP) {
+    if (al && bs == 10) {
+      launch_k(jacobi_kernel<T, 10, MODE, true>, div_up(n_units, 25), 256, 0, s, n_units, rp, col,
+               val, W, x, b, xo, lim);
+      note_launch();
+      return cudaGetLastError();
+    }
+  }
 #define GASA_JAC_CASE(BS)                                                                   \
   case BS: {                                                                                \
     constexpr int rpb = 256 / BS;                                                           \

@@ -106,8 +106,8 @@ __device__ __forceinline__ void team_blocks(int k0, int end, int step, int br, i
 // smoothing step x2o = Wm y.  blockDim = 32 * ES * BS * teams; dynamic shared
 // memory: 32 * RPL floats per warp and 40 per team.
 // LONG: only the block rows of at least min_len blocks, the others being
-// left to the thread-per-row kernels.  A CTA then looks through 32 rows at a
-// time and its teams take the long ones among them.
+// left to the thread-per-row kernels.  A CTA then looks through 32 rows a warp
+// at a time and its teams take the long ones among them.
 // 64 registers (32 warps an SM) wherever the two blocks in flight fit them: at 80,
 // which the compiler took when left alone, the steps of 16 x 16 blocks went from
 // 8.8 to 11.6 us
@@ -206,22 +206,23 @@ bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, const int *
     const int u = blockIdx.x * teams + team;
     block_row(u, u < n_brows);
   } else {
-    __shared__ unsigned longs;
-    for (int base = blockIdx.x * 32; base < n_brows; base += gridDim.x * 32) {
-      if (warp == 0) {
-        const int i = base + lane;
-        const unsigned m =
-            __ballot_sync(0xffffffffu, i < n_brows && __ldg(rp + i + 1) - __ldg(rp + i) >= min_len);
-        if (lane == 0) longs = m;
-      }
-      __syncthreads();
-      unsigned m = longs;
-      while (m) {                       // uniform over the CTA: `teams` long rows per turn
-        unsigned t = m;
-        for (int q = 0; q < team && t; ++q) t &= t - 1u;
-        block_row(base + (t ? __ffs(t) - 1 : 0), t != 0);
-        for (int q = 0; q < teams && m; ++q) m &= m - 1u;
-        __syncthreads();
+    // every warp looks through 32 rows; then the CTA goes through the words
+    __shared__ unsigned longs[kTeamWarps];
+    for (int base = blockIdx.x * warps * 32; base < n_brows; base += gridDim.x * warps * 32) {
+      const int i = base + warp * 32 + lane;
+      const unsigned mine =
+          __ballot_sync(0xffffffffu, i < n_brows && __ldg(rp + i + 1) - __ldg(rp + i) >= min_len);
+      if (lane == 0) longs[warp] = mine;
+      if (!__syncthreads_or(mine != 0)) continue;
+      for (int w = 0; w < warps; ++w) {
+        unsigned m = longs[w];
+        while (m) {                       // uniform over the CTA: `teams` long rows per turn
+          unsigned t = m;
+          for (int q = 0; q < team && t; ++q) t &= t - 1u;
+          block_row(base + w * 32 + (t ? __ffs(t) - 1 : 0), t != 0);
+          for (int q = 0; q < teams && m; ++q) m &= m - 1u;
+          __syncthreads();
+        }
       }
       __syncthreads();
     }
@@ -257,7 +258,8 @@ cudaError_t team_go(int op, int n_brows, int br, int bc, double avg, const int *
   if (min_len == 0 && avg > 1e8) BS = std::min(BS, 4);   // rows of unknown length
   const int nw = ES * BS, teams = nw >= 8 ? 1 : 8 / nw, warps = nw * teams;
   const size_t smem = ((size_t)warps * 32 * RPL + teams * kWideMaxRows) * sizeof(float);
-  const int grid = min_len > 0 ? std::min(div_up(n_brows, 32), 8 * kNumSM) : div_up(n_brows, teams);
+  const int grid = min_len > 0 ? std::min(div_up(n_brows, 32 * warps), 4 * kNumSM)
+                               : div_up(n_brows, teams);
   auto go = [&](auto kern) {
     launch_k(kern, grid, 32 * warps, smem, s, op, n_brows, br, bc, ES, BS, rp, col, val, W, x, b, y,
              rp2, col2, val2, x2o, min_len);
