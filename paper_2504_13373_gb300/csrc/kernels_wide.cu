@@ -27,9 +27,12 @@
 //
 // GB300, FP32: level 1 of a P2 16^3 tet hierarchy (3,072 rows of about 25 blocks
 // of 13 x 13, 53 MB): product 16.0 -> 14.8 us, smoothing step 20.4 -> 17.0 us;
-// level 2 (384 rows of about 275 blocks of 17 x 17, 122 MB): step 35.6 ->
-// 24.4 us; fused restriction of level 1 92.4 -> 60.3 us.  GMRES on Q2 96^2:
-// 5.97 -> 4.75 ms.
+// level 2 (384 rows of about 98 blocks of 17 x 17, 44 MB): step 35.6 ->
+// 19.0 us; fused restriction of level 1 92.4 -> 23.7 us (the last two with a
+// cluster of CTAs per block row; 22.5 and 64.7 us without).  GMRES on Q2 96^2:
+// 5.97 -> 4.38 ms.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "common.cuh"
@@ -37,11 +40,14 @@
 
 namespace gasa {
 
+namespace cg = cooperative_groups;
+
 namespace {
 
+constexpr int kTeamCluster = 8;     // CTAs sharing a block row at most
 constexpr int kWideMaxRows = 40;    // rows and columns of a block at most
 constexpr int kTeamRows = 8;        // rows per lane at most
-constexpr int kTeamWarps = 16;      // warps per team at most
+constexpr int kTeamWarps = 8;       // warps per team in a CTA at most
 
 enum { WIDE_ASSIGN = 0, WIDE_RESID = 1, WIDE_ADD = 2, WIDE_SWEEP = 3, WIDE_RFUSED = 4 };
 
@@ -112,14 +118,18 @@ __device__ __forceinline__ void team_blocks(int k0, int end, int step, int br, i
 // which the compiler took when left alone, the steps of 16 x 16 blocks went from
 // 8.8 to 11.6 us
 template <int VW, int RPL, bool LONG>
-__global__ void __launch_bounds__(32 * kTeamWarps, (LONG || VW * RPL <= 16) ? 2 : 0)
-bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, const int *__restrict__ rp,
+__global__ void __launch_bounds__(32 * kTeamWarps, (LONG || VW * RPL <= 16) ? 4 : 0)
+bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, int CS,
+                const int *__restrict__ rp,
                 const int *__restrict__ col, const float *__restrict__ val,
                 const float *__restrict__ Wm, const float *__restrict__ x,
                 const float *__restrict__ b, float *__restrict__ y, const int *__restrict__ rp2,
                 const int *__restrict__ col2, const float *__restrict__ val2,
                 float *__restrict__ x2o, int min_len) {
   extern __shared__ float sm[];
+  __shared__ float gathered[kTeamCluster][kWideMaxRows];   // rank 0: the CTAs' row sums
+  const int rank = CS > 1 ? (int)cg::this_cluster().block_rank() : 0;
+  if (CS > 1) cg::this_cluster().barrier_arrive();         // waited for before the first remote write
   const int nw = ES * BS, warps = blockDim.x >> 5, teams = warps / nw;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int team = warp / nw, wt = warp - team * nw;
@@ -129,6 +139,18 @@ bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, const int *
   float *part = sm + (size_t)team * nw * 32 * RPL;            // [nw][RPL][32]
   float *res = sm + (size_t)warps * 32 * RPL + team * kWideMaxRows;
   const bool smooth = op == WIDE_SWEEP || (op == WIDE_RFUSED && Wm);
+  auto finish_row = [&](int u, int r, float v) {
+    const size_t t = (size_t)u * br + r;
+    if (op == WIDE_ASSIGN) y[t] = v;
+    else if (op == WIDE_RESID) y[t] = b[t] - v;
+    else if (op == WIDE_ADD) y[t] = y[t] + v;
+    else if (op == WIDE_RFUSED) {
+      y[t] = v;
+      res[r] = v;
+    } else {
+      res[r] = b[t] - v;
+    }
+  };
   auto block_row = [&](int u, bool on) {
     if (smooth && on) {
       // the block of Wm is needed last: bring it into L2 meanwhile
@@ -143,18 +165,20 @@ bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, const int *
     for (int m = 0; m < RPL; ++m) acc[m] = 0.f;
     if (on && g < G) {
       const int r0 = es * G + g, rs = ES * G;
+      const int first = rank * BS + bs, step = BS * CS;
       const int beg = __ldg(rp + u), end = __ldg(rp + u + 1);
       if (op == WIDE_RFUSED) {
         const int beg2 = __ldg(rp2 + u), end2 = __ldg(rp2 + u + 1);
-        team_blocks<VW, RPL>(beg + bs, end, BS, br, bc, r0, rs, cl * VW, col, val, b, 1.f, acc);
-        team_blocks<VW, RPL>(beg2 + bs, end2, BS, br, bc, r0, rs, cl * VW, col2, val2, x, -1.f, acc);
+        team_blocks<VW, RPL>(beg + first, end, step, br, bc, r0, rs, cl * VW, col, val, b, 1.f, acc);
+        team_blocks<VW, RPL>(beg2 + first, end2, step, br, bc, r0, rs, cl * VW, col2, val2, x, -1.f, acc);
       } else {
-        team_blocks<VW, RPL>(beg + bs, end, BS, br, bc, r0, rs, cl * VW, col, val, x, 1.f, acc);
+        team_blocks<VW, RPL>(beg + first, end, step, br, bc, r0, rs, cl * VW, col, val, x, 1.f, acc);
       }
     }
   #pragma unroll
     for (int m = 0; m < RPL; ++m) part[(wt * RPL + m) * 32 + lane] = acc[m];
     __syncthreads();
+    if (CS > 1) cg::this_cluster().barrier_wait();         // every CTA of the cluster runs
     // four lanes per row add the row's BS * LC partial sums: blocks' warps in
     // order, columns sub, sub + 4, ... in order, then the four
     const int sub = lane & 3;
@@ -171,16 +195,17 @@ bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, const int *
       v += __shfl_xor_sync(0xffffffffu, v, 1);
       v += __shfl_xor_sync(0xffffffffu, v, 2);
       if (on && r < br && sub == 0) {
-        const size_t t = (size_t)u * br + r;
-        if (op == WIDE_ASSIGN) y[t] = v;
-        else if (op == WIDE_RESID) y[t] = b[t] - v;
-        else if (op == WIDE_ADD) y[t] = y[t] + v;
-        else if (op == WIDE_RFUSED) {
-          y[t] = v;
-          res[r] = v;
-        } else {
-          res[r] = b[t] - v;
-        }
+        if (CS == 1) finish_row(u, r, v);
+        else cg::this_cluster().map_shared_rank(&gathered[0][0], 0)[rank * kWideMaxRows + r] = v;
+      }
+    }
+    if (CS > 1) {
+      cg::this_cluster().sync();
+      if (rank != 0) return;
+      for (int r = wt * 32 + lane; on && r < br; r += nw * 32) {
+        float v = 0.f;
+        for (int c = 0; c < CS; ++c) v += gathered[c][r];
+        finish_row(u, r, v);
       }
     }
     if (!smooth) return;
@@ -203,7 +228,7 @@ bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, const int *
     }
   };
   if constexpr (!LONG) {
-    const int u = blockIdx.x * teams + team;
+    const int u = CS > 1 ? (int)blockIdx.x / CS : (int)blockIdx.x * teams + team;
     block_row(u, u < n_brows);
   } else {
     // every warp looks through 32 rows; then the CTA goes through the words
@@ -256,12 +281,21 @@ cudaError_t team_go(int op, int n_brows, int br, int bc, double avg, const int *
          (long long)n_brows * ES * BS < 40LL * kNumSM)
     BS *= 2;
   if (min_len == 0 && avg > 1e8) BS = std::min(BS, 4);   // rows of unknown length
-  const int nw = ES * BS, teams = nw >= 8 ? 1 : 8 / nw, warps = nw * teams;
+  // Few long rows: a cluster of CTAs per block row, each with a share of its
+  // blocks, while it keeps the GPU within one wave (32 warps an SM) and every
+  // warp eight blocks; rank 0 adds up the CTAs' sums and finishes the row.  384
+  // rows of 98 blocks of 17 x 17: step 22.5 -> 19.0 us; the fused restriction to
+  // them 64.7 -> 23.7 us; 64 rows of 28 x 21 blocks 29.4 -> 12.5 us.
+  int CS = 1;
+  while (min_len == 0 && CS < kTeamCluster && avg < 1e8 && avg >= 16.0 * BS * CS &&
+         (long long)n_brows * ES * BS * CS * 2 <= 32LL * kNumSM)
+    CS *= 2;
+  const int nw = ES * BS, teams = CS > 1 || nw >= 8 ? 1 : 8 / nw, warps = nw * teams;
   const size_t smem = ((size_t)warps * 32 * RPL + teams * kWideMaxRows) * sizeof(float);
   const int grid = min_len > 0 ? std::min(div_up(n_brows, 32 * warps), 4 * kNumSM)
-                               : div_up(n_brows, teams);
+                               : CS * div_up(n_brows, teams);
   auto go = [&](auto kern) {
-    launch_k(kern, grid, 32 * warps, smem, s, op, n_brows, br, bc, ES, BS, rp, col, val, W, x, b, y,
+    launch_kc(kern, grid, 32 * warps, smem, s, CS, op, n_brows, br, bc, ES, BS, CS, rp, col, val, W, x, b, y,
              rp2, col2, val2, x2o, min_len);
   };
 #define GASA_TEAM(N)                              \

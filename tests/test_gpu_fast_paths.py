@@ -2,7 +2,7 @@
 import numpy as np
 import pytest
 
-from tests.helpers import gpu_setup, problem, to_dev
+from tests.helpers import gpu_setup, problem, rel_err, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -205,3 +205,39 @@ def test_fp64_team_products(br, bc, n, lo, hi):
         wtol = np.einsum("nij,nj->ni", np.abs(W),
                          (tol + np.abs(r).ravel() * br * 2.0 ** -52).reshape(n, br)).ravel()
         assert np.all(np.abs(out.cpu().numpy() - ref) <= wtol + 2.0 ** -52 * (np.abs(x) + np.abs(ref)))
+
+
+@pytest.mark.parametrize("n,b", [(160, 13), (64, 21), (35, 36), (40, 12), (16, 40)])
+def test_vcycle_few_long_rows(n, b):
+    """Few block rows of many blocks, each shared by a cluster of CTAs: the V-cycle on a
+    random SPD operator, ragged rows, against the oracle's (FP64 to the conditioning of the
+    kept vectors, FP32 to 1e-4, the bounds of the solver's V-cycle tests)."""
+    from oracle import gasa_oracle as O
+    from tests.test_gpu_solver import level_tolerances
+    gasa = _gasa()
+    rng = np.random.default_rng(n * 100 + b)
+    keep = rng.random((n, n)) < 0.8
+    keep = keep | keep.T | np.eye(n, dtype=bool)
+    A = rng.standard_normal((n, b, n, b)) * keep[:, None, :, None]
+    A = A.reshape(n * b, n * b)
+    A = (A + A.T) / np.sqrt(8.0 * n * b) + 4.0 * np.eye(n * b)
+    rp = np.concatenate([[0], np.cumsum(keep.sum(1))]).astype(np.int32)
+    row, col = np.nonzero(keep)
+    val = np.ascontiguousarray(A.reshape(n, b, n, b)[row, :, col, :])
+    agg = [np.arange(n, dtype=np.int32) // 8]
+    B0 = rng.standard_normal((n * b, 2 * b))
+    H = O.setup(rp, col.astype(np.int32), val, agg, B0=B0, r=2 * b, dim=2)
+    ctx = gasa.gasa_create(0)
+    try:
+        gasa.gasa_setup(ctx, rp, col.astype(np.int32), val.ravel(), b, agg,
+                        gasa.gasa_default_options(dim=2, n_cand=2 * b, dense_tail_dofs=0),
+                        init_candidates=B0)
+        f = rng.standard_normal(n * b)
+        want = O.make_vcycle(H)(f)
+        z = to_dev(np.zeros(n * b))
+        gasa.gasa_vcycle(ctx, to_dev(f), z)
+        assert rel_err(z.cpu().numpy(), want) <= 0.1 * level_tolerances(H)[-1]
+        gasa.gasa_vcycle(ctx, to_dev(f), z, gasa.GASA_PREC_MIXED32)
+        assert rel_err(z.cpu().numpy(), want) <= 1e-4
+    finally:
+        gasa.gasa_destroy(ctx)
