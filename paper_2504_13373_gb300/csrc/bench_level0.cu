@@ -159,7 +159,9 @@ int main(int argc, char **argv) {
   cudaStream_t s;
   CK(cudaStreamCreate(&s));
 
-  auto folded = [&] { return launch_folded_sweep<float>(nb, kB, d_rp, d_col, d_wa, d_x, d_c, d_xo, s); };
+  auto folded = [&] {
+    return launch_folded_sweep<float>(nb, kB, d_rp, d_col, d_wa, d_x, d_c, d_xo, s, (int64_t)nnzb);
+  };
   auto outer = [&] {
     return launch_bsr_mv_ds(nb, kB, kB, d_rp, d_col, d_ahi, d_alo, d_phi, d_plo, d_q, s, d_pd,
                             d_part);
