@@ -39,16 +39,15 @@ FALLBACK_HBM_GBS = 6800.0
 
 # DRAM bytes (read + write) per launch of the level-0 FP32 smoothing sweep
 # from one ncu capture each, valid while the kernel's source file hashes to
-# `src_sha`: the plain kernel and the bulk-copy staged one.
+# `src_sha`: the plain kernel, the bulk-copy staged one and the folded one.
 # kernel classes of gasa_profile_read, timed by CUDA events in the host-driven loop
 PROFILE_CLASSES = ["level0_step", "level0_residual_restriction", "outer_Ap", "level0_first_step",
                    "level0_prolongation"]
 
 NCU_TRAFFIC = {
     # captured on the 224x224 case of the same recipe (100,352 elements, 210.40 MB read +
-    # 2.19 MB written per launch, two launches) and scaled to 131,072 elements; both
-    # kernels below are unchanged since their captures (the hash is of the file, in
-    # which other kernels changed)
+    # 2.19 MB written per launch, two launches) and scaled to 131,072 elements; of the
+    # kernel that took one block at a time, so the record no longer holds
     "plain": {"kernel": "jacobi_kernel<float,10,0>", "file": "kernels_mv.cu",
               "src_sha": "e49eeb68f4ccb194",
               "bytes_per_launch": (210.40e6 + 2.19e6) * 131072 / 100352},
@@ -56,9 +55,10 @@ NCU_TRAFFIC = {
             "src_sha": "24cbc7a902631ea2", "bytes_per_launch": 274.87e6 + 6.52e6},
     # folded step x + c - (wD^-1 A) x, two blocks of a row in flight: captured at full
     # size on the benchmark's block pattern (csrc/bench_level0.cu, 131,072 block rows;
-    # 222.42 MB read + 3.81 MB written per launch)
+    # 222.42 MB read + 3.81 MB written per launch); unchanged since (the hash is of the
+    # file, in which other kernels changed)
     "folded": {"kernel": "folded_pair_kernel<10,6>", "file": "kernels_mv.cu",
-               "src_sha": "e49eeb68f4ccb194",
+               "src_sha": "621f29f6107b3a8d",
                "bytes_per_launch": 222.42e6 + 3.81e6},
 }
 
