@@ -609,16 +609,19 @@ bsr_mv_ds_pair_kernel(int n_brows, int br, const int *__restrict__ rp, const int
   }
 }
 
+// blocks wider than 16 (or unaligned operands); DOT as above
+template <bool DOT>
 __global__ void __launch_bounds__(256)
 bsr_mv_ds_generic(int n_brows, int br, int bc, const int *__restrict__ rp,
                   const int *__restrict__ col, const float *__restrict__ ahi,
                   const float *__restrict__ alo, const float *__restrict__ xhi,
-                  const float *__restrict__ xlo, double *__restrict__ y) {
+                  const float *__restrict__ xlo, double *__restrict__ y,
+                  const double *__restrict__ xd, double *__restrict__ partials) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)n_brows * br) return;
-  const int i = (int)(t / br);
-  const int r = (int)(t - (long long)i * br);
-  const int beg = __ldg(rp + i), end = __ldg(rp + i + 1);
+  const bool act = t < (long long)n_brows * br;
+  const int i = act ? (int)(t / br) : 0;
+  const int r = act ? (int)(t - (long long)i * br) : 0;
+  const int beg = act ? __ldg(rp + i) : 0, end = act ? __ldg(rp + i + 1) : 0;
   float s = 0.0f, lo = 0.0f;
   for (int k = beg; k < end; ++k) {
     const int j = __ldg(col + k);
@@ -629,7 +632,13 @@ bsr_mv_ds_generic(int n_brows, int br, int bc, const int *__restrict__ rp,
       ds_product_add(ah, al, xh, xl, s, lo);
     }
   }
-  y[t] = (double)s + (double)lo;
+  const double yt = (double)s + (double)lo;
+  if (act) y[t] = yt;
+  if (DOT) {
+    __shared__ double sh[32];
+    const double v = block_sum(act ? xd[t] * yt : 0.0, sh);
+    if (threadIdx.x == 0) partials[blockIdx.x] = v;
+  }
 }
 
 int bsr_mv_ds_grid(int n_brows, int br) { return div_up((long long)n_brows * br, 256); }
@@ -674,7 +683,12 @@ cudaError_t launch_bsr_mv_ds(int n_brows, int br, int bc, const int *rp, const i
     }
   }
 #undef GASA_DS_CASE
-  launch_k(bsr_mv_ds_generic, grid, 256, 0, s, n_brows, br, bc, rp, col, ahi, alo, xhi, xlo, y);
+  if (dot)
+    launch_k(bsr_mv_ds_generic<true>, grid, 256, 0, s, n_brows, br, bc, rp, col, ahi, alo, xhi, xlo,
+             y, xd, partials);
+  else
+    launch_k(bsr_mv_ds_generic<false>, grid, 256, 0, s, n_brows, br, bc, rp, col, ahi, alo, xhi, xlo,
+             y, xd, partials);
   note_launch();
   return cudaGetLastError();
 }

@@ -241,3 +241,30 @@ def test_vcycle_few_long_rows(n, b):
         assert rel_err(z.cpu().numpy(), want) <= 1e-4
     finally:
         gasa.gasa_destroy(ctx)
+
+
+@pytest.mark.parametrize("prec", ["mixed32", "mixed16"])
+def test_mixed_cg_level0_blocks_wider_than_16(prec):
+    """P3 tetrahedra (20 x 20 blocks): the double-single product of the Krylov step and its
+    p . q partial sums, graph-resident and host-driven, against the oracle's mixed solve."""
+    from oracle import gasa_oracle as O
+    from synth import configs
+    gasa = _gasa()
+    pr = configs.poisson3d(3, 3, r=80)
+    A = pr.A
+    H = O.setup(A.row_ptr, A.col, A.val, pr.agg_of, B0=pr.B0, r=pr.r, dim=3)
+    want = O.solve(H, pr.rhs, 1e-10, "cg", precision=prec, max_iter=500)
+    P = gasa.GASA_PREC_MIXED32 if prec == "mixed32" else gasa.GASA_PREC_MIXED16
+    ctx = gasa.gasa_create(0)
+    try:
+        gasa.gasa_setup(ctx, A.row_ptr, A.col, A.val.ravel(), A.b, pr.agg_of,
+                        gasa.gasa_default_options(dim=3, n_cand=pr.r), adj_ptr=pr.adj_ptr,
+                        adj_idx=pr.adj_idx, centroids=pr.centroids, init_candidates=pr.B0)
+        for host_driven in (False, True):
+            gasa.gasa_profile_enable(ctx, host_driven)
+            x = np.zeros_like(pr.rhs)
+            info = gasa.gasa_solve(ctx, pr.rhs, x, 1e-10, P)
+            assert info.converged and info.rel_residual <= 1e-10
+            assert abs(info.iterations - want.iterations) <= 1, (info.iterations, want.iterations)
+    finally:
+        gasa.gasa_destroy(ctx)
