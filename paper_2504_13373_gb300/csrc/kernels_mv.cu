@@ -298,12 +298,23 @@ static inline bool maybe_short(int br, int bc, int64_t nnzb) {
   return nnzb == kNnzbUnknown && br * bc < 32;
 }
 
-// FP64: the team kernel of kernels_team64.cu instead of these, for blocks that
-// fill a warp's lanes at least (smaller ones leave them idle, which FP64
-// instructions do not forgive) or rows long enough to be worth it anyway;
-// without the average, blocks of 32 values on
-static inline bool team64_rows(int n_brows, int br, int bc, int64_t nnzb) {
+// FP64: the team kernel of kernels_team64.cu instead of these for blocks that fill a
+// warp's lanes, or rows long enough to be worth it anyway; without the average, blocks
+// of 32 values on.  It idles the lanes that a smaller block leaves, which FP64
+// instructions do not forgive, so blocks whose rows are a power of two keep the lane
+// groups and the CTA kernel there (GB300, 8,192 rows of 31 blocks of 4 x 4: smoothing
+// step 14.8 us with lane groups, 25.4 with teams; 2,048 of 75: 17.7 and 15.3, but 19.8
+// and 30.7 from HBM); other small blocks do not fit lane groups (3,000 rows of 16 blocks
+// of 5 x 5: 19.9 and 8.2).  With more than 4,096 rows lane groups also win on 4-row
+// blocks of any width (8,192 rows of 40 blocks of 4 x 10: 36.7 and 53.4) and on 8-row
+// ones in rows of fewer than 64 blocks (6,000 rows of 20 blocks of 8 x 12: 25.5 and
+// 30.6; 8 x 8, 13 blocks: 17.4 and 15.9; 20,000 rows of 70: 195 and 163).
+bool team64_rows(int n_brows, int br, int bc, int64_t nnzb) {
   if (!warp_rows(n_brows, br, nnzb)) return false;
+  if (pow2_le32(br)) {
+    if (br * bc < 32) return false;
+    if (n_brows > 4096 && (br == 4 || (br == 8 && nnzb < 64LL * n_brows))) return false;
+  }
   return br * bc >= 32 || nnzb >= 16LL * n_brows;
 }
 
