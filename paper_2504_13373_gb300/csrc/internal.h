@@ -85,6 +85,7 @@ bool wide_shape(int br, int bc, const float *val, const float *x);
 // ---- kernels_team64.cu: FP64, a team of warps per block row ------------------
 // whether these products and smoothing steps take it (kernels_mv.cu)
 bool team64_rows(int n_brows, int br, int bc, int64_t nnzb);
+void team64_split(int n_brows, int br, int bc, int64_t nnzb, int *es, int *epl, int *bs, int *cs);
 // op as launch_wide, blocks up to 64 x 64; cudaErrorNotSupported for others
 cudaError_t launch_team64(int op, int n_brows, int br, int bc, int64_t nnzb, const int *rp,
                           const int *col, const double *val, const double *W, const double *x,

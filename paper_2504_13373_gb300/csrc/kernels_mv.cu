@@ -298,6 +298,21 @@ static inline bool maybe_short(int br, int bc, int64_t nnzb) {
   return nnzb == kNnzbUnknown && br * bc < 32;
 }
 
+// FP64, narrow blocks (a thread reads 12 values of a row or fewer) in few rows (one wave
+// of eight CTAs an SM): the CTA kernel's threads take a whole row's blocks in one or two
+// rounds, and where those fill 60 % of its lanes it has less to add up than a team
+// (smoothing step, GB300: 256 rows of 17 blocks of 12 x 12 5.5 us, teams 6.5; 1,024 rows
+// 10.0 and 11.4; 1,000 rows of 26 of 9 x 9 10.1 and 10.9; product with 256 rows of 45 of
+// 12 x 9 6.8 and 7.2; but 11.4 and 10.1 for 800 rows of 22 of 11 x 11; 2,304 rows of 17
+// of 12 x 12 19.2 and 17.2; 13 x 13, 128 rows of 53 11.9 and 8.6; a third full, 1,296
+// rows of 4 of 10 x 10 9.0 and 7.1).
+static inline bool cta_filled(int n_brows, int br, int bc, int64_t nnzb) {
+  if (nnzb < 0 || bc > 12 || br > 64 || n_brows > 8 * kNumSM) return false;
+  const int64_t per_round = (int64_t)n_brows * (256 / br);     // blocks
+  const int64_t rounds = (nnzb + per_round - 1) / per_round;
+  return (double)nnzb * br >= 0.6 * 256.0 * (double)rounds * n_brows;
+}
+
 // FP64: the team kernel of kernels_team64.cu instead of these for blocks that fill a
 // warp's lanes, or rows long enough to be worth it anyway; without the average, blocks
 // of 32 values on.  It idles the lanes that a smaller block leaves, which FP64
@@ -310,7 +325,7 @@ static inline bool maybe_short(int br, int bc, int64_t nnzb) {
 // ones in rows of fewer than 64 blocks (6,000 rows of 20 blocks of 8 x 12: 25.5 and
 // 30.6; 8 x 8, 13 blocks: 17.4 and 15.9; 20,000 rows of 70: 195 and 163).
 bool team64_rows(int n_brows, int br, int bc, int64_t nnzb) {
-  if (!warp_rows(n_brows, br, nnzb)) return false;
+  if (!warp_rows(n_brows, br, nnzb) || cta_filled(n_brows, br, bc, nnzb)) return false;
   if (pow2_le32(br)) {
     if (br * bc < 32) return false;
     if (n_brows > 4096 && (br == 4 || (br == 8 && nnzb < 64LL * n_brows))) return false;

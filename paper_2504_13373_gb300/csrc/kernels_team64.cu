@@ -188,18 +188,24 @@ team64_kernel(int op, int n_brows, int br, int bc, int ES, int BS, int CS, int L
 
 }  // namespace
 
-cudaError_t launch_team64(int op, int n_brows, int br, int bc, int64_t nnzb, const int *rp,
-                          const int *col, const double *val, const double *W, const double *x,
-                          const double *b, double *y, cudaStream_t s) {
-  if (n_brows == 0) return cudaSuccess;
-  if (br > 64 || bc > 64 || (op == 3 && br != bc)) return cudaErrorNotSupported;
+// Warps over a block's positions (ES), over a row's blocks (BS) and CTAs over a row (CS),
+// and the values per lane (EPL).
+void team64_split(int n_brows, int br, int bc, int64_t nnzb, int *es, int *epl, int *bs, int *cs) {
   const int per = div_up(br * bc, 32);
   const int ES = div_up(per, kT64Values), EPL = div_up(per, ES);
-  // blocks shared out over warps while each keeps eight or more (its sums cost
-  // about as much as one) and the GPU has fewer than 16 warps an SM
   const double avg = nnzb >= 0 ? (double)nnzb / (double)n_brows : 1e9;
+  // Blocks shared out over warps while each keeps eight or more and the GPU has fewer
+  // than 16 warps an SM; beyond that down to one or two blocks a warp as long as the
+  // GPU stays within 16 warps an SM, where a warp's own chain of blocks is all there is
+  // (smoothing step, GB300, 256 rows of 17 blocks of 12 x 12: two warps 9.3 us, eight
+  // 6.5; 256 rows of 27 blocks of 16 x 16: 12.5 and 9.9, four 9.5; 384 rows of 4 blocks
+  // of 10 x 10: one 6.7, four 5.2).  Twice as many at 16 an SM cost more in the teams'
+  // sums than they hide (1,024 rows of 17 of 12 x 12: 11.4, four 11.8).
+  const long long most = 16LL * kNumSM;
   int BS = 1;
-  while (ES * BS * 2 <= kT64Warps && avg >= 16.0 * BS && (long long)n_brows * ES * BS < 16LL * kNumSM)
+  while (ES * BS * 2 <= kT64Warps &&
+         ((avg >= 16.0 * BS && (long long)n_brows * ES * BS < most) ||
+          (avg >= 2.0 * BS && (long long)n_brows * ES * BS * 2 <= most)))
     BS *= 2;
   if (nnzb < 0 && BS > 4) BS = 4;
   // few long rows: a cluster of CTAs per block row, each with a share of its
@@ -210,6 +216,19 @@ cudaError_t launch_team64(int op, int n_brows, int br, int bc, int64_t nnzb, con
   while (nnzb >= 0 && CS < kT64Cluster && avg >= 16.0 * BS * CS &&
          (long long)n_brows * ES * BS * CS * 2 <= 24LL * kNumSM)
     CS *= 2;
+  *es = ES;
+  *epl = EPL;
+  *bs = BS;
+  *cs = CS;
+}
+
+cudaError_t launch_team64(int op, int n_brows, int br, int bc, int64_t nnzb, const int *rp,
+                          const int *col, const double *val, const double *W, const double *x,
+                          const double *b, double *y, cudaStream_t s) {
+  if (n_brows == 0) return cudaSuccess;
+  if (br > 64 || bc > 64 || (op == 3 && br != bc)) return cudaErrorNotSupported;
+  int ES, EPL, BS, CS;
+  team64_split(n_brows, br, bc, nnzb, &ES, &EPL, &BS, &CS);
   const int nw = ES * BS, teams = CS > 1 || nw >= 4 ? 1 : 4 / nw, warps = nw * teams;
   // lanes that add up a row: two where one warp does it (fewest instructions), up
   // to sixteen where the team's warps share them (shortest chain)
