@@ -53,13 +53,28 @@ enum { WIDE_ASSIGN = 0, WIDE_RESID = 1, WIDE_ADD = 2, WIDE_SWEEP = 3, WIDE_RFUSE
 
 // adds sign * (rows r0, r0 + rstep, ... of the blocks k0, k0 + BS, ... < end,
 // columns c .. c + VW) . x to acc; two blocks in flight, and the column indices
-// of the next two
+// of the next two.
+// Rounding: one FP32 sum over a whole row's blocks lost up to half a bit against
+// summing block by block (25 blocks of 12 x 12, random values: rms error 1.4e-7 of
+// the sums' rms, block by block 8.8e-8).  So a pair of blocks is summed by itself
+// before it joins the row's sum, alternately one of two sums where blocks are narrow
+// and rows therefore short (8.3e-8); the widest blocks, where those additions would
+// take a tenth of the time and the registers another warp (3,000 rows of 12 blocks of
+// 24 x 24: 16.5 us, with pairs 20.4), keep a sum for the first and one for the second
+// block of the pairs (12 blocks of 24 x 24: 1.0e-7 -> 8.7e-8, block by block 8.8e-8).
+template <int VW, int RPL>
+struct TeamSums {
+  static constexpr bool pairs = VW < 4 || RPL <= 4;
+  static constexpr int n = !pairs || (VW > 1 && VW * RPL <= 8) ? 2 : 1;
+};
+
 template <int VW, int RPL>
 __device__ __forceinline__ void team_blocks(int k0, int end, int step, int br, int bc, int r0,
                                             int rstep, int c, const int *__restrict__ col,
                                             const float *__restrict__ val,
                                             const float *__restrict__ x, float sign,
-                                            float (&acc)[RPL]) {
+                                            float (&acc)[TeamSums<VW, RPL>::n][RPL]) {
+  constexpr int NA = TeamSums<VW, RPL>::n;
   const float *vp = val + (size_t)r0 * bc + c;
   const size_t bb = (size_t)br * bc;
   const float *xc = x + c;
@@ -83,10 +98,31 @@ __device__ __forceinline__ void team_blocks(int k0, int end, int step, int br, i
 #pragma unroll
     for (int m = 0; m < RPL; ++m) {
       if (!row[m]) continue;
+      if constexpr (!TeamSums<VW, RPL>::pairs) {
 #pragma unroll
-      for (int v = 0; v < VW; ++v) {
-        acc[m] = fmaf(sign * a0[m][v], x0[v], acc[m]);
-        acc[m] = fmaf(sign * a1[m][v], x1[v], acc[m]);
+        for (int v = 0; v < VW; ++v) {
+          acc[0][m] = fmaf(sign * a0[m][v], x0[v], acc[0][m]);
+          acc[1][m] = fmaf(sign * a1[m][v], x1[v], acc[1][m]);
+        }
+      } else {
+        float t0 = sign * a0[m][0] * x0[0];
+        if (NA == 1) {
+#pragma unroll
+          for (int v = 1; v < VW; ++v) t0 = fmaf(sign * a0[m][v], x0[v], t0);
+#pragma unroll
+          for (int v = 0; v < VW; ++v) t0 = fmaf(sign * a1[m][v], x1[v], t0);
+        } else {
+          float t1 = sign * a1[m][0] * x1[0];
+#pragma unroll
+          for (int v = 1; v < VW; ++v) {
+            t0 = fmaf(sign * a0[m][v], x0[v], t0);
+            t1 = fmaf(sign * a1[m][v], x1[v], t1);
+          }
+          t0 += t1;
+        }
+        const float other = acc[NA - 1][m];
+        acc[NA - 1][m] = acc[0][m] + t0;
+        if (NA == 2) acc[0][m] = other;
       }
     }
   }
@@ -100,8 +136,10 @@ __device__ __forceinline__ void team_blocks(int k0, int end, int step, int br, i
 #pragma unroll
     for (int m = 0; m < RPL; ++m) {
       if (!row[m]) continue;
+      float t0 = sign * a0[m][0] * x0[0];
 #pragma unroll
-      for (int v = 0; v < VW; ++v) acc[m] = fmaf(sign * a0[m][v], x0[v], acc[m]);
+      for (int v = 1; v < VW; ++v) t0 = fmaf(sign * a0[m][v], x0[v], t0);
+      acc[0][m] += t0;
     }
   }
 }
@@ -118,7 +156,8 @@ __device__ __forceinline__ void team_blocks(int k0, int end, int step, int br, i
 // which the compiler took when left alone, the steps of 16 x 16 blocks went from
 // 8.8 to 11.6 us
 template <int VW, int RPL, bool LONG>
-__global__ void __launch_bounds__(32 * kTeamWarps, (LONG || VW * RPL <= 16) ? 4 : 0)
+__global__ void __launch_bounds__(32 * kTeamWarps, LONG || VW * RPL < 14 || VW == 2 && RPL == 8 ? 4
+                                                 : VW * RPL <= 20 ? 3 : 2)
 bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, int CS,
                 const int *__restrict__ rp,
                 const int *__restrict__ col, const float *__restrict__ val,
@@ -160,9 +199,10 @@ bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, int CS,
         asm volatile("prefetch.global.L2 [%0];" ::"l"(Wm + (size_t)u * br * br + o));
       }
     }
-    float acc[RPL];
+    constexpr int NA = TeamSums<VW, RPL>::n;
+    float acc[NA][RPL];
   #pragma unroll
-    for (int m = 0; m < RPL; ++m) acc[m] = 0.f;
+    for (int m = 0; m < RPL; ++m) acc[0][m] = acc[NA - 1][m] = 0.f;
     if (on && g < G) {
       const int r0 = es * G + g, rs = ES * G;
       const int first = rank * BS + bs, step = BS * CS;
@@ -176,11 +216,11 @@ bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, int CS,
       }
     }
   #pragma unroll
-    for (int m = 0; m < RPL; ++m) part[(wt * RPL + m) * 32 + lane] = acc[m];
+    for (int m = 0; m < RPL; ++m) part[(wt * RPL + m) * 32 + lane] = NA == 2 ? acc[0][m] + acc[NA - 1][m] : acc[0][m];
     __syncthreads();
     if (CS > 1) cg::this_cluster().barrier_wait();         // every CTA of the cluster runs
-    // four lanes per row add the row's BS * LC partial sums: blocks' warps in
-    // order, columns sub, sub + 4, ... in order, then the four
+    // four lanes per row add the row's BS * LC partial sums: a warp's columns sub,
+    // sub + 4, ... in order, the warps in order, then the four
     const int sub = lane & 3;
     const int rounds = (br * 4 + nw * 32 - 1) / (nw * 32);
     for (int it = 0; it < rounds; ++it) {
@@ -189,8 +229,11 @@ bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, int CS,
       if (r < br) {
         const int m = r / (ES * G), q = r - m * ES * G;
         const float *p = part + ((size_t)(q / G) * RPL + m) * 32 + (q % G) * LC;
-        for (int s = 0; s < BS; ++s)
-          for (int c = sub; c < LC; c += 4) v += p[(size_t)s * ES * RPL * 32 + c];
+        for (int s = 0; s < BS; ++s) {
+          float w = 0.f;
+          for (int c = sub; c < LC; c += 4) w += p[(size_t)s * ES * RPL * 32 + c];
+          v += w;
+        }
       }
       v += __shfl_xor_sync(0xffffffffu, v, 1);
       v += __shfl_xor_sync(0xffffffffu, v, 2);

@@ -268,3 +268,25 @@ def test_mixed_cg_level0_blocks_wider_than_16(prec):
             assert abs(info.iterations - want.iterations) <= 1, (info.iterations, want.iterations)
     finally:
         gasa.gasa_destroy(ctx)
+
+
+@pytest.mark.parametrize("n,b,per_row,limit", [
+    (3000, 12, 25, 9.5e-8), (5400, 12, 17, 9.5e-8), (8000, 10, 15, 9.0e-8), (200, 36, 50, 1.2e-7),
+    (4000, 13, 25, 9.5e-8), (3000, 16, 27, 9.8e-8)])
+def test_wide_team_rounding(n, b, per_row, limit):
+    """FP32 sums of wide blocks round like sums taken block by block in several groups: the
+    rms error over the rows of random values, in units of the sums' rms, to that of eight
+    groups of blocks (8.4e-8, 8.4e-8, 7.9e-8, 1.1e-7, 8.8e-8, 9.1e-8) and about 8 %."""
+    gasa = _gasa()
+    rng = np.random.default_rng(n + b)
+    rp = (per_row * np.arange(n + 1)).astype(np.int32)
+    col = np.sort(np.argsort(rng.random((n, max(2 * per_row, 60))), axis=1)[:, :per_row], axis=1)
+    col = ((col + 7 * np.arange(n)[:, None]) % n).astype(np.int32).ravel()
+    val = rng.standard_normal((n * per_row, b, b)).astype(np.float32)
+    x = rng.standard_normal(n * b).astype(np.float32)
+    want = np.einsum("nkij,nkj->ni", val.astype(np.float64).reshape(n, per_row, b, b),
+                     x.astype(np.float64).reshape(n, b)[col].reshape(n, per_row, b)).ravel()
+    y = to_dev(np.zeros(n * b, np.float32))
+    gasa.gasa_bsr_mv_f32(0, n, b, b, to_dev(rp), to_dev(col), to_dev(val.ravel()), to_dev(x), y, y)
+    err = np.sqrt(np.mean((y.cpu().numpy() - want) ** 2) / np.mean(want ** 2))
+    assert err <= limit, err
