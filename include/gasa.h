@@ -146,8 +146,11 @@ typedef struct {
                                 k .. N-1 and the coarsest solve, started from u_k = 0, form a fixed
                                 linear map b_k -> u_k.  Setup forms it (FP64, n_k x n_k) by running
                                 those steps on the unit vectors, and the V-cycle applies it as one
-                                dense FP64 product (FP32 vectors in the FP32 cycle).  Results agree
-                                with the per-step cycle to rounding.  Not built when tail_kib or
+                                dense product: FP64 multiply-adds in the FP64 cycle; in the FP32
+                                cycle, on FP32 vectors, sums of two FP32 words on a two-word split of
+                                the operator (a row to about 2^-47 of its sum of |m b|), or for a
+                                server's batches three words of both, no less accurate than FP64
+                                multiply-adds.  Results agree with the per-step cycle to rounding.  Not built when tail_kib or
                                 grid_tail is set.  0: off; default 2048; at most 8192. */
   int32_t folded_smoother;   /* 1 (default): level 0 also stores w D_0^{-1} A_0 in FP32 (block row i
                                 multiplied by its block inverse, in A_0's pattern, formed in FP64),

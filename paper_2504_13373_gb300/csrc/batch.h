@@ -53,9 +53,9 @@ template <typename T>
 cudaError_t launch_bdense(int nc, const double *Ainv, const T *B, T *X, int K, cudaStream_t s,
                           int ld = 0);
 
-// X = M B from the exact two-term FP32 split of M (row pitch ld), double-single arithmetic
-cudaError_t launch_bdense_ds(int n, int ld, const float *Mh, const float *Ml, const float *B,
-                             float *X, int K, cudaStream_t s);
+// X = M B for FP32 B and X on FP32 units, as accurate as FP64 FMAs (row pitch ld)
+cudaError_t launch_bdense_split(int n, int ld, const double *M, const float *B, float *X, int K,
+                                cudaStream_t s);
 
 // partial sums of x . y (y null: x . x) and, with Z, of x . z; the launchers
 // that add partials up take the n of the dot product

@@ -57,6 +57,15 @@ __device__ __forceinline__ double block_sum_partials(const double *p, int n, dou
   return block_sum(v, sh);
 }
 
+// a + b = returned sum + err exactly (Knuth); the intrinsics keep the compiler from
+// contracting it
+__device__ __forceinline__ float two_sum(float a, float b, float &err) {
+  const float s = __fadd_rn(a, b);
+  const float bp = __fsub_rn(s, a);
+  err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bp)), __fsub_rn(b, bp));
+  return s;
+}
+
 // ----------------------------------------------------------------------------
 // vector load helpers
 // ----------------------------------------------------------------------------

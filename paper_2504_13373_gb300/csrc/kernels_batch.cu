@@ -987,109 +987,117 @@ bdense_warp_kernel(int n, int ld, const double *__restrict__ A, const T *__restr
   }
 }
 
-// X = M B for the FP32 cycle's dense bottom operator on K columns: M as its exact
-// two-term FP32 split (Mh the FP32 rounding of M, Ml that of M - Mh, row pitch
-// ld), FP32 B and X, double-single arithmetic as in the single solve's
-// dense_mv_ds_kernel, so a row agrees with the FP64 product to about 2^-47 of
-// sum |m b|.  FP64 FMAs took 123 us for order 2,048 and eight columns (33.5
-// million FMAs at 0.6 per ns, and a conversion each); this takes 15.8 us.
-// A CTA owns four rows, so B is read once per four rows; thread t takes columns
-// t, t + 256, ... in order, then the (s, lo) pairs meet in a packed warp tree
-// and the warps in order.  A column's sum does not depend on K.
-constexpr int kDsRows = 4;
+// X = M B for the FP32 cycle's dense bottom operator on K columns: FP64 M (row pitch
+// ld), FP32 B and X, no less accurate than FP64 FMAs would be (order 2,048, random
+// values: rms error 73 x 2^-53 of an entry's, a warp's FP64 chain 117), on FP32 units.
+// FP64 FMAs take 152 us for order 2,048 and eight columns (33.5 million of them at
+// 0.6 per ns, and a conversion each), 20 for one; this takes 48.6 and 14.5, 33 FP32
+// operations a product, which is what bounds it.
+// An entry of M is cut into three FP32 words that hold all of its 53 bits, each
+// product of the first two words and x is exact in two words, and a row's sum is
+// three words (s, lo, u), every rounding error of s and lo carried into the next.  (Two
+// words of M and of the sum took 15.8 us but lost four bits against FP64.)
+// A CTA owns a row (two took 58.8 us: 114 registers, half the warps); thread t takes
+// columns t, t + 256, ... in order, then the sums meet in a packed warp tree and the warps
+// in order.  A column's sum does not depend on K.
 
-__device__ __forceinline__ void ds_add_product(float ah, float al, float x, float &s, float &lo) {
-  const float pr = __fmul_rn(ah, x);
-  const float e = __fmaf_rn(ah, x, -pr);
-  const float cross = __fmul_rn(al, x);
-  const float s1 = __fadd_rn(s, pr);
-  const float bp = __fsub_rn(s1, s);
-  const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(s1, bp)), __fsub_rn(pr, bp));
-  s = s1;
-  lo = __fadd_rn(lo, __fadd_rn(err, __fadd_rn(e, cross)));
+// the rare entry beyond 2^-80 .. 2^127, whose last words meet the end of the FP32 range; a
+// call, so that its FP64 instructions are not run for every entry and their result dropped
+__device__ __noinline__ float3 three_words_by_rounding(double m) {
+  const float h = __double2float_rn(m);
+  const double r = m - (double)h;
+  const float l = __double2float_rn(r);
+  return make_float3(h, l, __double2float_rn(r - (double)l));
 }
-// (s, lo) += (s2, lo2), the same either way round
-__device__ __forceinline__ void ds_add_pair(float &s, float &lo, float s2, float lo2) {
-  const float s1 = __fadd_rn(s, s2);
-  const float bp = __fsub_rn(s1, s);
-  const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(s1, bp)), __fsub_rn(s2, bp));
-  s = s1;
-  lo = __fadd_rn(__fadd_rn(lo, lo2), err);
+
+// m = h + l + t exactly (24, 23 and 6 bits, truncated)
+__device__ __forceinline__ void three_words(double m, float &h, float &l, float &t) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(m);
+  const int e = (int)(b >> 52) & 0x7ff;
+  if (e >= 943 && e <= 1150) {
+    const unsigned sign = (unsigned)(b >> 32) & 0x80000000u, low = (unsigned)b & 0x1fffffffu;
+    // 2^k with the bits in its fraction, less 2^k
+    const unsigned bl = sign | (unsigned)(e - 919) << 23, bt = sign | (unsigned)(e - 942) << 23;
+    h = __uint_as_float(sign | (unsigned)(e - 896) << 23 | ((unsigned)(b >> 29) & 0x7fffffu));
+    l = __fsub_rn(__uint_as_float(bl | low >> 6), __uint_as_float(bl));
+    t = __fsub_rn(__uint_as_float(bt | (low & 63u) << 17), __uint_as_float(bt));
+  } else {
+    const float3 w = three_words_by_rounding(m);
+    h = w.x;
+    l = w.y;
+    t = w.z;
+  }
+}
+
+__device__ __forceinline__ void split_add_product(float ah, float al, float at, float x, float &s,
+                                                  float &lo, float &u) {
+  const float p = __fmul_rn(ah, x), pe = __fmaf_rn(ah, x, -p);
+  const float c = __fmul_rn(al, x), ce = __fmaf_rn(al, x, -c);
+  float es, r1, r2, r3;
+  s = two_sum(s, p, es);
+  lo = two_sum(lo, two_sum(two_sum(pe, c, r1), es, r2), r3);
+  u = __fadd_rn(u, __fadd_rn(__fadd_rn(r1, r2), __fadd_rn(r3, __fmaf_rn(at, x, ce))));
+}
+// (s, lo, u) += (s2, lo2, u2), the same either way round
+__device__ __forceinline__ void split_add_sum(float &s, float &lo, float &u, float s2, float lo2,
+                                              float u2) {
+  float es, r1, r2;
+  s = two_sum(s, s2, es);
+  lo = two_sum(two_sum(lo, lo2, r1), es, r2);
+  u = __fadd_rn(__fadd_rn(u, u2), __fadd_rn(r1, r2));
 }
 
 template <int K>
 __global__ void __launch_bounds__(kThreads)
-bdense_ds_kernel(int n, int ld, const float *__restrict__ Mh, const float *__restrict__ Ml,
-                 const float *__restrict__ B, float *__restrict__ X) {
-  constexpr int Q = kDsRows * K;                    // sums of a CTA, at most 32
-  __shared__ float sh[kThreads / 32][Q], sl[kThreads / 32][Q];
-  const int r0 = blockIdx.x * kDsRows;
+bdense_split_kernel(int n, int ld, const double *__restrict__ M, const float *__restrict__ B,
+                    float *__restrict__ X) {
+  __shared__ float sh[3][kThreads / 32][K];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const float *hp[kDsRows], *lp[kDsRows];
+  const double *m = M + (size_t)blockIdx.x * ld;
+  float s[K], lo[K], u[K];
 #pragma unroll
-  for (int r = 0; r < kDsRows; ++r) {               // rows past the last repeat it
-    const size_t o = (size_t)min(r0 + r, n - 1) * ld;
-    hp[r] = Mh + o;
-    lp[r] = Ml + o;
-  }
-  float s[Q], lo[Q];
-#pragma unroll
-  for (int q = 0; q < Q; ++q) s[q] = lo[q] = 0.f;
+  for (int c = 0; c < K; ++c) s[c] = lo[c] = u[c] = 0.f;
 #pragma unroll 2
   for (int j = threadIdx.x; j < n; j += kThreads) {
-    float b[K], h[kDsRows], l[kDsRows];
+    float b[K], h, l, t;
     load_k<float, K>(B + (size_t)j * K, b);
+    three_words(__ldg(m + j), h, l, t);
 #pragma unroll
-    for (int r = 0; r < kDsRows; ++r) {
-      h[r] = __ldg(hp[r] + j);
-      l[r] = __ldg(lp[r] + j);
-    }
-#pragma unroll
-    for (int r = 0; r < kDsRows; ++r)
-#pragma unroll
-      for (int c = 0; c < K; ++c) ds_add_product(h[r], l[r], b[c], s[r * K + c], lo[r * K + c]);
+    for (int c = 0; c < K; ++c) split_add_product(h, l, t, b[c], s[c], lo[c], u[c]);
   }
-  int width = Q;
+  int width = K;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    if (width > 1) {
-      width >>= 1;
-      const bool hi = lane & o;
+    if (width > 1) width >>= 1;
+    const bool packed = K >> (__ffs(16 / o) - 1) > 1;   // half of the sums each, while there are two
+    const bool hi = lane & o;
 #pragma unroll
-      for (int j = 0; j < Q / 2; ++j) {
-        if (j >= width) continue;
-        const float ms = hi ? s[j + width] : s[j], os = hi ? s[j] : s[j + width];
-        const float ml = hi ? lo[j + width] : lo[j], ol = hi ? lo[j] : lo[j + width];
-        // the lower lane's pair first in both lanes
-        const float ps = __shfl_xor_sync(0xffffffffu, os, o);
-        const float pl = __shfl_xor_sync(0xffffffffu, ol, o);
-        s[j] = hi ? ps : ms;
-        lo[j] = hi ? pl : ml;
-        ds_add_pair(s[j], lo[j], hi ? ms : ps, hi ? ml : pl);
-      }
-    } else {
-      const bool hi = lane & o;
-      const float ps = __shfl_xor_sync(0xffffffffu, s[0], o);
-      const float pl = __shfl_xor_sync(0xffffffffu, lo[0], o);
-      const float ms = s[0], ml = lo[0];
-      s[0] = hi ? ps : ms;
-      lo[0] = hi ? pl : ml;
-      ds_add_pair(s[0], lo[0], hi ? ms : ps, hi ? ml : pl);
+    for (int j = 0; j < (K > 1 ? K / 2 : 1); ++j) {
+      if (j >= width) continue;
+      const int jo = packed ? j + width : j;
+      const float ms = hi ? s[jo] : s[j], ml = hi ? lo[jo] : lo[j], mu = hi ? u[jo] : u[j];
+      const float os = hi ? s[j] : s[jo], ol = hi ? lo[j] : lo[jo], ou = hi ? u[j] : u[jo];
+      s[j] = ms;
+      lo[j] = ml;
+      u[j] = mu;
+      split_add_sum(s[j], lo[j], u[j], __shfl_xor_sync(0xffffffffu, os, o),
+                    __shfl_xor_sync(0xffffffffu, ol, o), __shfl_xor_sync(0xffffffffu, ou, o));
     }
   }
-  constexpr int per = 32 / Q;
+  constexpr int per = 32 / K;
   if (lane % per == 0) {
-    sh[wid][lane / per] = s[0];
-    sl[wid][lane / per] = lo[0];
+    sh[0][wid][lane / per] = s[0];
+    sh[1][wid][lane / per] = lo[0];
+    sh[2][wid][lane / per] = u[0];
   }
   __syncthreads();
-  if (threadIdx.x < Q) {
+  if (threadIdx.x < K) {
     double v = 0.0;
 #pragma unroll
     for (int w = 0; w < kThreads / 32; ++w)
-      v += (double)sh[w][threadIdx.x] + (double)sl[w][threadIdx.x];
-    const int r = r0 + threadIdx.x / K;
-    if (r < n) X[(size_t)r * K + threadIdx.x % K] = (float)v;
+      v += (double)sh[0][w][threadIdx.x] +
+           ((double)sh[1][w][threadIdx.x] + (double)sh[2][w][threadIdx.x]);
+    X[(size_t)blockIdx.x * K + threadIdx.x] = (float)v;
   }
 }
 
@@ -1209,11 +1217,10 @@ cudaError_t launch_bdense(int nc, const double *Ainv, const T *B, T *X, int K, c
   return cudaGetLastError();
 }
 
-cudaError_t launch_bdense_ds(int n, int ld, const float *Mh, const float *Ml, const float *B,
-                             float *X, int K, cudaStream_t s) {
+cudaError_t launch_bdense_split(int n, int ld, const double *M, const float *B, float *X, int K,
+                                cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  GASA_KSWITCH(K, launch_k(bdense_ds_kernel<KK>, div_up(n, kDsRows), kThreads, 0, s, n, ld, Mh, Ml,
-                           B, X));
+  GASA_KSWITCH(K, launch_k(bdense_split_kernel<KK>, n, kThreads, 0, s, n, ld, M, B, X));
   note_launch();
   return cudaGetLastError();
 }

@@ -329,8 +329,8 @@ cudaError_t vcycle_b(Engine &e, const T *rhs, T *out) {
   }
   if (kt < N) {
     if constexpr (std::is_same<T, float>::value)
-      ECU(launch_bdense_ds(ctx->dtail_n, ctx->dtail_ld, ctx->dtail_Mh, ctx->dtail_Ml,
-                           P::b(e.lv[kt]), P::x(e.lv[kt]), K, s));
+      ECU(launch_bdense_split(ctx->dtail_n, ctx->dtail_ld, ctx->dtail_M, P::b(e.lv[kt]),
+                              P::x(e.lv[kt]), K, s));
     else
       ECU(launch_bdense<T>(ctx->dtail_n, ctx->dtail_M, P::b(e.lv[kt]), P::x(e.lv[kt]), K, s,
                            ctx->dtail_ld));
