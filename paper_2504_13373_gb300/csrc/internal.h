@@ -79,6 +79,9 @@ cudaError_t launch_wide_restrict(int n_brows, int br, int bc, int64_t nnzb, cons
 cudaError_t launch_wide(int op, int n_brows, int br, int bc, int64_t nnzb, const int *rp,
                         const int *col, const float *val, const float *W, const float *x,
                         const float *b, float *y, cudaStream_t s, int min_len = 0);
+// whether launch_wide and launch_wide_restrict (op 4) put a lane on a row of a block, not a
+// team on a block row; vw: columns per load
+bool wide_by_rows(int op, int n_brows, int br, int bc, int64_t nnzb, int vw);
 // whether launch_wide takes these blocks, whatever the row lengths
 bool wide_shape(int br, int bc, const float *val, const float *x);
 

@@ -297,6 +297,132 @@ bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, int CS,
   }
 }
 
+// ---------------------------------------------------------------------------
+// Narrow or low blocks: a lane per row of a block (two rows a lane beyond 32).  The
+// lanes of a warp form G = 32 / br groups of br lanes and group g of warp w takes the
+// blocks beg + w G + g, beg + (w + nw) G + g, ...; lane r of a group reads row r of its
+// block and the block's bc entries of x, even and odd columns in sums of their own.
+// The partial sums of the team's nw warps meet in shared memory and its first warp adds
+// them, warps in order, then groups.  Several short blocks per instruction and next to
+// nothing per block row: the team kernel above brings a block in fewer L1 lines, but
+// half-fills its lanes with low blocks, and a row's sums cost it as much as ten blocks.
+// ---------------------------------------------------------------------------
+// one lane's rows (r0 and, with two, r0 + 32) over the blocks kbeg, kbeg + step, ... < end
+// of one block row: adds sign * (row . x_col) to a0, a1
+template <int VW>
+__device__ __forceinline__ void lane_rows(int kbeg, int end, int step, int br, int bc, int r0,
+                                          bool two, const int *__restrict__ col,
+                                          const float *__restrict__ val,
+                                          const float *__restrict__ x, float sign, float &a0,
+                                          float &a1) {
+  for (int k = kbeg; k < end; k += step) {
+    const int j = __ldg(col + k);
+    const float *ar0 = val + ((size_t)k * br + r0) * bc;
+    const float *ar1 = ar0 + (size_t)32 * bc;
+    const float *xj = x + (size_t)j * bc;
+    constexpr int W = VW == 1 ? 2 : VW;          // columns per turn: at least an even and an odd one
+    float s[2] = {0.f, 0.f}, t[2] = {0.f, 0.f};
+    int c = 0;
+    for (; c + W <= bc; c += W) {
+      float xv[W], av[W];
+#pragma unroll
+      for (int q = 0; q < W; q += VW) load_vec<float, VW>(xj + c + q, xv + q);
+#pragma unroll
+      for (int q = 0; q < W; q += VW) load_vec<float, VW>(ar0 + c + q, av + q);
+#pragma unroll
+      for (int q = 0; q < W; ++q) s[q & 1] = fmaf(av[q], xv[q], s[q & 1]);
+      if (two) {
+#pragma unroll
+        for (int q = 0; q < W; q += VW) load_vec<float, VW>(ar1 + c + q, av + q);
+#pragma unroll
+        for (int q = 0; q < W; ++q) t[q & 1] = fmaf(av[q], xv[q], t[q & 1]);
+      }
+    }
+    if (VW == 1 && c < bc) {
+      const float xc = __ldg(xj + c);
+      s[0] = fmaf(__ldg(ar0 + c), xc, s[0]);
+      if (two) t[0] = fmaf(__ldg(ar1 + c), xc, t[0]);
+    }
+    a0 += sign * (s[0] + s[1]);
+    a1 += sign * (t[0] + t[1]);
+  }
+}
+
+template <int OP, int VW>
+__global__ void __launch_bounds__(32 * kTeamWarps)
+bsr_rows_kernel(int n_brows, int br, int bc, int nw, const int *__restrict__ rp,
+                const int *__restrict__ col, const float *__restrict__ val,
+                const float *__restrict__ Wm, const float *__restrict__ x,
+                const float *__restrict__ b, float *__restrict__ y, const int *__restrict__ rp2,
+                const int *__restrict__ col2, const float *__restrict__ val2,
+                float *__restrict__ x2o) {
+  // red[warp][slot]: each lane's partial row sums (slot = lane, lane + 32)
+  __shared__ float red[kTeamWarps][kWideMaxRows];
+  __shared__ float res[kTeamWarps][kWideMaxRows];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int team = warp / nw, wt = warp - team * nw;
+  const int u = blockIdx.x * (kTeamWarps / nw) + team;
+  const int G = br <= 32 ? 32 / br : 1;          // block groups per warp
+  const int g = br <= 32 ? lane / br : 0;
+  const int r0 = br <= 32 ? lane - g * br : lane;
+  const bool lane_on = g < G && r0 < br;
+  const bool two = br > 32 && lane + 32 < br;    // second row of this lane
+  float a0 = 0.f, a1 = 0.f;
+  if (u < n_brows && lane_on) {
+    const int step = nw * G, off = wt * G + g;
+    if (OP == WIDE_RFUSED) {
+      lane_rows<VW>(__ldg(rp + u) + off, __ldg(rp + u + 1), step, br, bc, r0, two, col, val, b,
+                    1.f, a0, a1);
+      lane_rows<VW>(__ldg(rp2 + u) + off, __ldg(rp2 + u + 1), step, br, bc, r0, two, col2, val2, x,
+                    -1.f, a0, a1);
+    } else {
+      lane_rows<VW>(__ldg(rp + u) + off, __ldg(rp + u + 1), step, br, bc, r0, two, col, val, x,
+                    1.f, a0, a1);
+    }
+  }
+  if (lane_on) red[warp][br <= 32 ? g * br + r0 : r0] = a0;
+  if (two) red[warp][lane + 32] = a1;
+  __syncthreads();
+  if (u >= n_brows || wt != 0) return;
+  const int w0 = team * nw;
+  for (int r = lane; r < br; r += 32) {
+    float v = 0.f;
+    for (int w = 0; w < nw; ++w) {
+      if (br <= 32) {
+        for (int q = 0; q < G; ++q) v += red[w0 + w][q * br + r];
+      } else {
+        v += red[w0 + w][r];
+      }
+    }
+    const size_t t = (size_t)u * br + r;
+    if (OP == WIDE_ASSIGN) y[t] = v;
+    else if (OP == WIDE_RESID) y[t] = b[t] - v;
+    else if (OP == WIDE_ADD) y[t] = y[t] + v;
+    else if (OP == WIDE_RFUSED) {
+      y[t] = v;
+      res[w0][r] = v;
+    } else {
+      res[w0][r] = b[t] - v;
+    }
+  }
+  if (OP != WIDE_SWEEP && (OP != WIDE_RFUSED || !Wm)) return;
+  __syncwarp();
+  // SWEEP: x_out = x + W (b - A x); RFUSED: x2o = Wm y (W row r against res)
+  for (int r = lane; r < br; r += 32) {
+    const float *w = Wm + ((size_t)u * br + r) * br;
+    float o[2] = {0.f, 0.f};
+    int c = 0;
+    for (; c + 1 < br; c += 2) {
+      o[0] = fmaf(__ldg(w + c), res[w0][c], o[0]);
+      o[1] = fmaf(__ldg(w + c + 1), res[w0][c + 1], o[1]);
+    }
+    if (c < br) o[0] = fmaf(__ldg(w + c), res[w0][c], o[0]);
+    const size_t t = (size_t)u * br + r;
+    if (OP == WIDE_SWEEP) y[t] = x[t] + (o[0] + o[1]);
+    else x2o[t] = o[0] + o[1];
+  }
+}
+
 bool al(const void *p, size_t a) { return p == nullptr || ((uintptr_t)p % a) == 0; }
 
 // widest run the block width and every pointer allow
@@ -355,6 +481,23 @@ cudaError_t team_go(int op, int n_brows, int br, int bc, double avg, const int *
   return cudaGetLastError();
 }
 
+template <int OP, int VW>
+cudaError_t rows_go(int n_brows, int br, int bc, double avg, const int *rp, const int *col,
+                    const float *val, const float *W, const float *x, const float *b, float *y,
+                    const int *rp2, const int *col2, const float *val2, float *x2o,
+                    cudaStream_t s) {
+  // warps per block row: about four blocks per group, at most a CTA; without the average
+  // as many as give an SM 16
+  const int G = br <= 32 ? 32 / br : 1;
+  int nw = 1;
+  while (nw < kTeamWarps && (avg < 1e8 ? nw * G * 4 < avg : (long long)n_brows * nw < 16LL * kNumSM))
+    nw *= 2;
+  launch_k(bsr_rows_kernel<OP, VW>, div_up(n_brows, kTeamWarps / nw), 32 * kTeamWarps, 0, s, n_brows,
+           br, bc, nw, rp, col, val, W, x, b, y, rp2, col2, val2, x2o);
+  note_launch();
+  return cudaGetLastError();
+}
+
 cudaError_t team_launch(int op, int n_brows, int br, int bc, int64_t nnzb, const int *rp,
                         const int *col, const float *val, const float *W, const float *x,
                         const float *b, float *y, const int *rp2, const int *col2,
@@ -364,6 +507,21 @@ cudaError_t team_launch(int op, int n_brows, int br, int bc, int64_t nnzb, const
   // RFUSED multiplies val with b and val2 with x
   const int vw = op == WIDE_RFUSED ? wide_vec(bc, val, b, val2, x)
                                    : wide_vec(bc, val, x, nullptr, nullptr);
+  if (min_len == 0 && wide_by_rows(op, n_brows, br, bc, nnzb, vw)) {
+#define GASA_ROWS(OP)                                                                             \
+  case OP:                                                                                        \
+    return vw == 4 ? rows_go<OP, 4>(n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2,     \
+                                    val2, x2o, s)                                                 \
+           : vw == 2 ? rows_go<OP, 2>(n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2,   \
+                                      val2, x2o, s)                                               \
+                     : rows_go<OP, 1>(n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2,   \
+                                      val2, x2o, s);
+    switch (op) {
+      GASA_ROWS(WIDE_ASSIGN) GASA_ROWS(WIDE_RESID) GASA_ROWS(WIDE_ADD) GASA_ROWS(WIDE_SWEEP)
+      GASA_ROWS(WIDE_RFUSED)
+    }
+#undef GASA_ROWS
+  }
   if (bc / vw > 32) return cudaErrorNotSupported;
   if (vw == 4)
     return team_go<4>(op, n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2, val2, x2o, min_len, s);
@@ -373,6 +531,34 @@ cudaError_t team_launch(int op, int n_brows, int br, int bc, int64_t nnzb, const
 }
 
 }  // namespace
+
+// Lanes on rows of blocks instead of teams (GB300, us with lanes on rows / with teams):
+//  - low blocks, at most 8 rows by 16 columns: 32,768 rows of 16 blocks of 4 x 10
+//    24.6 / 42.1, 4,000 rows 4.7 / 7.6, 20,000 rows of 10 of 8 x 12 16.8 / 20.6 (wider
+//    ones: 4,000 rows of 16 of 4 x 31 17.6 / 10.1);
+//  - blocks up to 15 x 15 where the GPU has blocks enough to be busy but rows are short or
+//    the blocks few enough to come from L2: smoothing step, 1,000 rows of 40 blocks of
+//    9 x 9 6.4 / 10.5, 8,000 of 12 12.2 / 14.7, 2,000 of 12 of 12 x 12 5.9 / 6.8, 1,000 of
+//    28 of 14 x 14 7.2 / 8.5 (256 of 20 of 12 x 12 5.1 / 4.8, 4,000 of 20 16.6 / 12.7,
+//    2,000 of 40 of 13 x 13 20.4 / 16.2);
+//  - the fused restriction likewise: 1,024 rows of 45 blocks of 10 x 8 5.7 / 9.9, of
+//    12 x 12 10.1 / 11.5 (4,096 rows of 36 of 12 x 12 30.7 / 18.1); and with odd widths
+//    of 17 to 20, which leave a third of a team's lanes idle, on tall blocks: 2,500 rows
+//    of 36 of 22 x 17 41.3 / 57.3 (64 rows of 90 13.4 / 8.6, a cluster a row).
+bool wide_by_rows(int op, int n_brows, int br, int bc, int64_t nnzb, int vw) {
+  if (br <= 8 && bc <= 16) return true;
+  if (nnzb < 0) return false;
+  const int b = std::max(br, bc);
+  const int64_t k = 1000;
+  if (op == WIDE_RFUSED) {
+    if (vw == 1 && bc >= 17 && bc <= 20 && br >= 20) return n_brows > 128;
+    return br <= 16 && bc <= 12 && nnzb >= 14 * k && nnzb <= (br <= 10 && bc <= 10 ? 100 : 60) * k;
+  }
+  if (b > 15 || nnzb < 14 * k) return false;
+  const int short_row = b <= 10 ? 24 : b <= 12 ? 14 : 10;
+  const int64_t few = (b <= 10 ? 72 : b <= 12 ? 60 : 30) * k;
+  return nnzb < (int64_t)short_row * n_brows || nnzb <= few;
+}
 
 bool wide_applies(int br, int bc, int n_brows, int64_t nnzb) {
   return (br > 8 || bc > 8) && br <= kWideMaxRows && bc <= kWideMaxRows && n_brows > 0 &&

@@ -65,3 +65,26 @@ def test_fp64_filled_ctas_keep_few_narrow_rows():
     for n, br, bc, per_row in ((2304, 12, 12, 17), (128, 13, 13, 53), (1296, 10, 10, 4),
                                (256, 16, 16, 27), (256, 12, 12, None)):
         assert _team64_rows(n, br, bc, per_row)
+
+
+def test_fp32_low_and_short_rows_keep_a_lane_per_row():
+    """FP32 blocks wider than 8: lanes on rows of blocks for low blocks and for short or few
+    rows of blocks up to 15 x 15, teams on block rows elsewhere."""
+    f = _lib()["_ZN4gasa12wide_by_rowsEiiiili"]
+    f.restype = ctypes.c_bool
+
+    def by_rows(op, n, br, bc, per_row):
+        vw = 4 if bc % 4 == 0 else 2 if bc % 2 == 0 else 1
+        return f(op, n, br, bc, ctypes.c_int64(-2 if per_row is None else per_row * n), vw)
+
+    for op in (0, 1, 2, 4):
+        for n in (64, 500, 32768):
+            assert by_rows(op, n, 4, 10, 16) and by_rows(op, n, 8, 12, 10)
+            assert by_rows(op, n, 1, 16, 9) and not by_rows(op, n, 4, 31, 16)
+    assert by_rows(0, 500, 4, 10, None) and not by_rows(0, 500, 10, 10, None)
+    for n, b, per_row in ((1000, 9, 40), (8000, 9, 12), (2000, 12, 12), (1000, 14, 28), (9000, 10, 9)):
+        assert by_rows(3, n, b, b, per_row), (n, b, per_row)
+    for n, b, per_row in ((256, 12, 20), (4000, 12, 20), (2000, 13, 40), (3072, 13, 25), (4000, 16, 16)):
+        assert not by_rows(3, n, b, b, per_row), (n, b, per_row)
+    assert by_rows(4, 1024, 10, 8, 45) and by_rows(4, 2500, 22, 17, 36)
+    assert not by_rows(4, 4096, 12, 12, 36) and not by_rows(4, 64, 22, 17, 90)
