@@ -149,14 +149,11 @@ __device__ __forceinline__ void team_blocks(int k0, int end, int step, int br, i
 // R A = (rp2, col2, val2), and, with Wm (the next level's w D^{-1}), its first
 // smoothing step x2o = Wm y.  blockDim = 32 * ES * BS * teams; dynamic shared
 // memory: 32 * RPL floats per warp and 40 per team.
-// LONG: only the block rows of at least min_len blocks, the others being
-// left to the thread-per-row kernels.  A CTA then looks through 32 rows a warp
-// at a time and its teams take the long ones among them.
 // 64 registers (32 warps an SM) wherever the two blocks in flight fit them: at 80,
 // which the compiler took when left alone, the steps of 16 x 16 blocks went from
 // 8.8 to 11.6 us
-template <int VW, int RPL, bool LONG>
-__global__ void __launch_bounds__(32 * kTeamWarps, LONG || VW * RPL < 14 || VW == 2 && RPL == 8 ? 4
+template <int VW, int RPL>
+__global__ void __launch_bounds__(32 * kTeamWarps, VW * RPL < 14 || VW == 2 && RPL == 8 ? 4
                                                  : VW * RPL <= 20 ? 3 : 2)
 bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, int CS,
                 const int *__restrict__ rp,
@@ -164,7 +161,7 @@ bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, int CS,
                 const float *__restrict__ Wm, const float *__restrict__ x,
                 const float *__restrict__ b, float *__restrict__ y, const int *__restrict__ rp2,
                 const int *__restrict__ col2, const float *__restrict__ val2,
-                float *__restrict__ x2o, int min_len) {
+                float *__restrict__ x2o) {
   extern __shared__ float sm[];
   __shared__ float gathered[kTeamCluster][kWideMaxRows];   // rank 0: the CTAs' row sums
   const int rank = CS > 1 ? (int)cg::this_cluster().block_rank() : 0;
@@ -178,7 +175,9 @@ bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, int CS,
   float *part = sm + (size_t)team * nw * 32 * RPL;            // [nw][RPL][32]
   float *res = sm + (size_t)warps * 32 * RPL + team * kWideMaxRows;
   const bool smooth = op == WIDE_SWEEP || (op == WIDE_RFUSED && Wm);
-  auto finish_row = [&](int u, int r, float v) {
+  const int u = CS > 1 ? (int)blockIdx.x / CS : (int)blockIdx.x * teams + team;
+  const bool on = u < n_brows;
+  auto finish_row = [&](int r, float v) {
     const size_t t = (size_t)u * br + r;
     if (op == WIDE_ASSIGN) y[t] = v;
     else if (op == WIDE_RESID) y[t] = b[t] - v;
@@ -190,109 +189,82 @@ bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, int CS,
       res[r] = b[t] - v;
     }
   };
-  auto block_row = [&](int u, bool on) {
-    if (smooth && on) {
-      // the block of Wm is needed last: bring it into L2 meanwhile
-      const int lines = (br * br * 4 + 127) / 128 + 1;
-      for (int q = wt * 32 + lane; q < lines; q += nw * 32) {
-        const int o = min(q * 32, br * br - 1);
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(Wm + (size_t)u * br * br + o));
+  if (smooth && on) {
+    // the block of Wm is needed last: bring it into L2 meanwhile
+    const int lines = (br * br * 4 + 127) / 128 + 1;
+    for (int q = wt * 32 + lane; q < lines; q += nw * 32) {
+      const int o = min(q * 32, br * br - 1);
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(Wm + (size_t)u * br * br + o));
+    }
+  }
+  constexpr int NA = TeamSums<VW, RPL>::n;
+  float acc[NA][RPL];
+#pragma unroll
+  for (int m = 0; m < RPL; ++m) acc[0][m] = acc[NA - 1][m] = 0.f;
+  if (on && g < G) {
+    const int r0 = es * G + g, rs = ES * G;
+    const int first = rank * BS + bs, step = BS * CS;
+    const int beg = __ldg(rp + u), end = __ldg(rp + u + 1);
+    if (op == WIDE_RFUSED) {
+      const int beg2 = __ldg(rp2 + u), end2 = __ldg(rp2 + u + 1);
+      team_blocks<VW, RPL>(beg + first, end, step, br, bc, r0, rs, cl * VW, col, val, b, 1.f, acc);
+      team_blocks<VW, RPL>(beg2 + first, end2, step, br, bc, r0, rs, cl * VW, col2, val2, x, -1.f, acc);
+    } else {
+      team_blocks<VW, RPL>(beg + first, end, step, br, bc, r0, rs, cl * VW, col, val, x, 1.f, acc);
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < RPL; ++m) part[(wt * RPL + m) * 32 + lane] = NA == 2 ? acc[0][m] + acc[NA - 1][m] : acc[0][m];
+  __syncthreads();
+  if (CS > 1) cg::this_cluster().barrier_wait();         // every CTA of the cluster runs
+  // four lanes per row add the row's BS * LC partial sums: a warp's columns sub,
+  // sub + 4, ... in order, the warps in order, then the four
+  const int sub = lane & 3;
+  const int rounds = (br * 4 + nw * 32 - 1) / (nw * 32);
+  for (int it = 0; it < rounds; ++it) {
+    const int r = (it * nw * 32 + wt * 32 + lane) >> 2;
+    float v = 0.f;
+    if (r < br) {
+      const int m = r / (ES * G), q = r - m * ES * G;
+      const float *p = part + ((size_t)(q / G) * RPL + m) * 32 + (q % G) * LC;
+      for (int s = 0; s < BS; ++s) {
+        float w = 0.f;
+        for (int c = sub; c < LC; c += 4) w += p[(size_t)s * ES * RPL * 32 + c];
+        v += w;
       }
     }
-    constexpr int NA = TeamSums<VW, RPL>::n;
-    float acc[NA][RPL];
-  #pragma unroll
-    for (int m = 0; m < RPL; ++m) acc[0][m] = acc[NA - 1][m] = 0.f;
-    if (on && g < G) {
-      const int r0 = es * G + g, rs = ES * G;
-      const int first = rank * BS + bs, step = BS * CS;
-      const int beg = __ldg(rp + u), end = __ldg(rp + u + 1);
-      if (op == WIDE_RFUSED) {
-        const int beg2 = __ldg(rp2 + u), end2 = __ldg(rp2 + u + 1);
-        team_blocks<VW, RPL>(beg + first, end, step, br, bc, r0, rs, cl * VW, col, val, b, 1.f, acc);
-        team_blocks<VW, RPL>(beg2 + first, end2, step, br, bc, r0, rs, cl * VW, col2, val2, x, -1.f, acc);
-      } else {
-        team_blocks<VW, RPL>(beg + first, end, step, br, bc, r0, rs, cl * VW, col, val, x, 1.f, acc);
-      }
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    if (on && r < br && sub == 0) {
+      if (CS == 1) finish_row(r, v);
+      else cg::this_cluster().map_shared_rank(&gathered[0][0], 0)[rank * kWideMaxRows + r] = v;
     }
-  #pragma unroll
-    for (int m = 0; m < RPL; ++m) part[(wt * RPL + m) * 32 + lane] = NA == 2 ? acc[0][m] + acc[NA - 1][m] : acc[0][m];
-    __syncthreads();
-    if (CS > 1) cg::this_cluster().barrier_wait();         // every CTA of the cluster runs
-    // four lanes per row add the row's BS * LC partial sums: a warp's columns sub,
-    // sub + 4, ... in order, the warps in order, then the four
-    const int sub = lane & 3;
-    const int rounds = (br * 4 + nw * 32 - 1) / (nw * 32);
-    for (int it = 0; it < rounds; ++it) {
-      const int r = (it * nw * 32 + wt * 32 + lane) >> 2;
+  }
+  if (CS > 1) {
+    cg::this_cluster().sync();
+    if (rank != 0) return;
+    for (int r = wt * 32 + lane; on && r < br; r += nw * 32) {
       float v = 0.f;
-      if (r < br) {
-        const int m = r / (ES * G), q = r - m * ES * G;
-        const float *p = part + ((size_t)(q / G) * RPL + m) * 32 + (q % G) * LC;
-        for (int s = 0; s < BS; ++s) {
-          float w = 0.f;
-          for (int c = sub; c < LC; c += 4) w += p[(size_t)s * ES * RPL * 32 + c];
-          v += w;
-        }
-      }
-      v += __shfl_xor_sync(0xffffffffu, v, 1);
-      v += __shfl_xor_sync(0xffffffffu, v, 2);
-      if (on && r < br && sub == 0) {
-        if (CS == 1) finish_row(u, r, v);
-        else cg::this_cluster().map_shared_rank(&gathered[0][0], 0)[rank * kWideMaxRows + r] = v;
-      }
+      for (int c = 0; c < CS; ++c) v += gathered[c][r];
+      finish_row(r, v);
     }
-    if (CS > 1) {
-      cg::this_cluster().sync();
-      if (rank != 0) return;
-      for (int r = wt * 32 + lane; on && r < br; r += nw * 32) {
-        float v = 0.f;
-        for (int c = 0; c < CS; ++c) v += gathered[c][r];
-        finish_row(u, r, v);
-      }
+  }
+  if (!smooth) return;
+  __syncthreads();
+  // SWEEP: x_out = x + W (b - A x); RFUSED: x2o = Wm y, four lanes per row
+  for (int it = 0; it < rounds; ++it) {
+    const int r = (it * nw * 32 + wt * 32 + lane) >> 2;
+    float v = 0.f;
+    if (on && r < br) {
+      const float *w = Wm + ((size_t)u * br + r) * br;
+      for (int c = sub; c < br; c += 4) v = fmaf(__ldg(w + c), res[c], v);
     }
-    if (!smooth) return;
-    __syncthreads();
-    // SWEEP: x_out = x + W (b - A x); RFUSED: x2o = Wm y, four lanes per row
-    for (int it = 0; it < rounds; ++it) {
-      const int r = (it * nw * 32 + wt * 32 + lane) >> 2;
-      float v = 0.f;
-      if (on && r < br) {
-        const float *w = Wm + ((size_t)u * br + r) * br;
-        for (int c = sub; c < br; c += 4) v = fmaf(__ldg(w + c), res[c], v);
-      }
-      v += __shfl_xor_sync(0xffffffffu, v, 1);
-      v += __shfl_xor_sync(0xffffffffu, v, 2);
-      if (on && r < br && sub == 0) {
-        const size_t t = (size_t)u * br + r;
-        if (op == WIDE_SWEEP) y[t] = x[t] + v;
-        else x2o[t] = v;
-      }
-    }
-  };
-  if constexpr (!LONG) {
-    const int u = CS > 1 ? (int)blockIdx.x / CS : (int)blockIdx.x * teams + team;
-    block_row(u, u < n_brows);
-  } else {
-    // every warp looks through 32 rows; then the CTA goes through the words
-    __shared__ unsigned longs[kTeamWarps];
-    for (int base = blockIdx.x * warps * 32; base < n_brows; base += gridDim.x * warps * 32) {
-      const int i = base + warp * 32 + lane;
-      const unsigned mine =
-          __ballot_sync(0xffffffffu, i < n_brows && __ldg(rp + i + 1) - __ldg(rp + i) >= min_len);
-      if (lane == 0) longs[warp] = mine;
-      if (!__syncthreads_or(mine != 0)) continue;
-      for (int w = 0; w < warps; ++w) {
-        unsigned m = longs[w];
-        while (m) {                       // uniform over the CTA: `teams` long rows per turn
-          unsigned t = m;
-          for (int q = 0; q < team && t; ++q) t &= t - 1u;
-          block_row(base + w * 32 + (t ? __ffs(t) - 1 : 0), t != 0);
-          for (int q = 0; q < teams && m; ++q) m &= m - 1u;
-          __syncthreads();
-        }
-      }
-      __syncthreads();
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    if (on && r < br && sub == 0) {
+      const size_t t = (size_t)u * br + r;
+      if (op == WIDE_SWEEP) y[t] = x[t] + v;
+      else x2o[t] = v;
     }
   }
 }
@@ -303,9 +275,14 @@ bsr_team_kernel(int op, int n_brows, int br, int bc, int ES, int BS, int CS,
 // blocks beg + w G + g, beg + (w + nw) G + g, ...; lane r of a group reads row r of its
 // block and the block's bc entries of x, even and odd columns in sums of their own.
 // The partial sums of the team's nw warps meet in shared memory and its first warp adds
-// them, warps in order, then groups.  Several short blocks per instruction and next to
-// nothing per block row: the team kernel above brings a block in fewer L1 lines, but
-// half-fills its lanes with low blocks, and a row's sums cost it as much as ten blocks.
+// them, warps in order, then groups.
+// LONG: only the block rows of at least min_len blocks, the others being the
+// thread-per-row kernels': a CTA looks through `chunk` rows at once and its warps take the
+// long ones among them in turn, a warp each (8,000 rows of 15 blocks of 10 x 10: with 256
+// rows a CTA and their long ones one team after another 170 us; so 18.8).
+// Several short blocks per instruction and next to nothing per block row: the team kernel
+// above brings a block in fewer L1 lines, but half-fills its lanes with low blocks, and a
+// row's sums cost it as much as ten blocks.
 // ---------------------------------------------------------------------------
 // one lane's rows (r0 and, with two, r0 + 32) over the blocks kbeg, kbeg + step, ... < end
 // of one block row: adds sign * (row . x_col) to a0, a1
@@ -323,7 +300,7 @@ __device__ __forceinline__ void lane_rows(int kbeg, int end, int step, int br, i
     constexpr int W = VW == 1 ? 2 : VW;          // columns per turn: at least an even and an odd one
     float s[2] = {0.f, 0.f}, t[2] = {0.f, 0.f};
     int c = 0;
-    for (; c + W <= bc; c += W) {
+    for (; VW == 1 ? c + 1 < bc : c < bc; c += W) {
       float xv[W], av[W];
 #pragma unroll
       for (int q = 0; q < W; q += VW) load_vec<float, VW>(xj + c + q, xv + q);
@@ -348,9 +325,10 @@ __device__ __forceinline__ void lane_rows(int kbeg, int end, int step, int br, i
   }
 }
 
-template <int OP, int VW>
+template <int OP, int VW, bool LONG>
 __global__ void __launch_bounds__(32 * kTeamWarps)
-bsr_rows_kernel(int n_brows, int br, int bc, int nw, const int *__restrict__ rp,
+bsr_rows_kernel(int n_brows, int br, int bc, int nw, int chunk, int min_len,
+                const int *__restrict__ rp,
                 const int *__restrict__ col, const float *__restrict__ val,
                 const float *__restrict__ Wm, const float *__restrict__ x,
                 const float *__restrict__ b, float *__restrict__ y, const int *__restrict__ rp2,
@@ -360,66 +338,87 @@ bsr_rows_kernel(int n_brows, int br, int bc, int nw, const int *__restrict__ rp,
   __shared__ float red[kTeamWarps][kWideMaxRows];
   __shared__ float res[kTeamWarps][kWideMaxRows];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int team = warp / nw, wt = warp - team * nw;
-  const int u = blockIdx.x * (kTeamWarps / nw) + team;
   const int G = br <= 32 ? 32 / br : 1;          // block groups per warp
   const int g = br <= 32 ? lane / br : 0;
   const int r0 = br <= 32 ? lane - g * br : lane;
   const bool lane_on = g < G && r0 < br;
   const bool two = br > 32 && lane + 32 < br;    // second row of this lane
-  float a0 = 0.f, a1 = 0.f;
-  if (u < n_brows && lane_on) {
-    const int step = nw * G, off = wt * G + g;
-    if (OP == WIDE_RFUSED) {
-      lane_rows<VW>(__ldg(rp + u) + off, __ldg(rp + u + 1), step, br, bc, r0, two, col, val, b,
-                    1.f, a0, a1);
-      lane_rows<VW>(__ldg(rp2 + u) + off, __ldg(rp2 + u + 1), step, br, bc, r0, two, col2, val2, x,
-                    -1.f, a0, a1);
-    } else {
-      lane_rows<VW>(__ldg(rp + u) + off, __ldg(rp + u + 1), step, br, bc, r0, two, col, val, x,
-                    1.f, a0, a1);
-    }
-  }
-  if (lane_on) red[warp][br <= 32 ? g * br + r0 : r0] = a0;
-  if (two) red[warp][lane + 32] = a1;
-  __syncthreads();
-  if (u >= n_brows || wt != 0) return;
-  const int w0 = team * nw;
-  for (int r = lane; r < br; r += 32) {
-    float v = 0.f;
-    for (int w = 0; w < nw; ++w) {
-      if (br <= 32) {
-        for (int q = 0; q < G; ++q) v += red[w0 + w][q * br + r];
+  // block row u by warp wt of nw of a team
+  auto block_row = [&](int u, bool on, int wt, int nw) {
+    float a0 = 0.f, a1 = 0.f;
+    if (on && lane_on) {
+      const int step = nw * G, off = wt * G + g;
+      if (OP == WIDE_RFUSED) {
+        lane_rows<VW>(__ldg(rp + u) + off, __ldg(rp + u + 1), step, br, bc, r0, two, col, val, b,
+                      1.f, a0, a1);
+        lane_rows<VW>(__ldg(rp2 + u) + off, __ldg(rp2 + u + 1), step, br, bc, r0, two, col2, val2, x,
+                      -1.f, a0, a1);
       } else {
-        v += red[w0 + w][r];
+        lane_rows<VW>(__ldg(rp + u) + off, __ldg(rp + u + 1), step, br, bc, r0, two, col, val, x,
+                      1.f, a0, a1);
       }
     }
-    const size_t t = (size_t)u * br + r;
-    if (OP == WIDE_ASSIGN) y[t] = v;
-    else if (OP == WIDE_RESID) y[t] = b[t] - v;
-    else if (OP == WIDE_ADD) y[t] = y[t] + v;
-    else if (OP == WIDE_RFUSED) {
-      y[t] = v;
-      res[w0][r] = v;
-    } else {
-      res[w0][r] = b[t] - v;
+    if (lane_on) red[warp][br <= 32 ? g * br + r0 : r0] = a0;
+    if (two) red[warp][lane + 32] = a1;
+    if (LONG) __syncwarp();
+    else __syncthreads();
+    if (!on || wt != 0) return;
+    const int w0 = warp;                         // the team's first warp
+    for (int r = lane; r < br; r += 32) {
+      float v = 0.f;
+      for (int w = 0; w < nw; ++w) {
+        if (br <= 32) {
+          for (int q = 0; q < G; ++q) v += red[w0 + w][q * br + r];
+        } else {
+          v += red[w0 + w][r];
+        }
+      }
+      const size_t t = (size_t)u * br + r;
+      if (OP == WIDE_ASSIGN) y[t] = v;
+      else if (OP == WIDE_RESID) y[t] = b[t] - v;
+      else if (OP == WIDE_ADD) y[t] = y[t] + v;
+      else if (OP == WIDE_RFUSED) {
+        y[t] = v;
+        res[w0][r] = v;
+      } else {
+        res[w0][r] = b[t] - v;
+      }
     }
-  }
-  if (OP != WIDE_SWEEP && (OP != WIDE_RFUSED || !Wm)) return;
-  __syncwarp();
-  // SWEEP: x_out = x + W (b - A x); RFUSED: x2o = Wm y (W row r against res)
-  for (int r = lane; r < br; r += 32) {
-    const float *w = Wm + ((size_t)u * br + r) * br;
-    float o[2] = {0.f, 0.f};
-    int c = 0;
-    for (; c + 1 < br; c += 2) {
-      o[0] = fmaf(__ldg(w + c), res[w0][c], o[0]);
-      o[1] = fmaf(__ldg(w + c + 1), res[w0][c + 1], o[1]);
+    if (OP != WIDE_SWEEP && (OP != WIDE_RFUSED || !Wm)) return;
+    __syncwarp();
+    // SWEEP: x_out = x + W (b - A x); RFUSED: x2o = Wm y (W row r against res)
+    for (int r = lane; r < br; r += 32) {
+      const float *w = Wm + ((size_t)u * br + r) * br;
+      float o[2] = {0.f, 0.f};
+      int c = 0;
+      for (; c + 1 < br; c += 2) {
+        o[0] = fmaf(__ldg(w + c), res[w0][c], o[0]);
+        o[1] = fmaf(__ldg(w + c + 1), res[w0][c + 1], o[1]);
+      }
+      if (c < br) o[0] = fmaf(__ldg(w + c), res[w0][c], o[0]);
+      const size_t t = (size_t)u * br + r;
+      if (OP == WIDE_SWEEP) y[t] = x[t] + (o[0] + o[1]);
+      else x2o[t] = o[0] + o[1];
     }
-    if (c < br) o[0] = fmaf(__ldg(w + c), res[w0][c], o[0]);
-    const size_t t = (size_t)u * br + r;
-    if (OP == WIDE_SWEEP) y[t] = x[t] + (o[0] + o[1]);
-    else x2o[t] = o[0] + o[1];
+  };
+  if constexpr (LONG) {
+    __shared__ unsigned longs[kTeamWarps];
+    const int base = blockIdx.x * chunk, i = base + threadIdx.x;
+    const unsigned mine =
+        __ballot_sync(0xffffffffu, (int)threadIdx.x < chunk && i < n_brows &&
+                                       __ldg(rp + i + 1) - __ldg(rp + i) >= min_len);
+    if (lane == 0) longs[warp] = mine;
+    if (!__syncthreads_or(mine != 0)) return;
+    int turn = 0;
+    for (int w = 0; w < kTeamWarps; ++w)
+      for (unsigned m = longs[w]; m; m &= m - 1u)
+        if (turn++ % kTeamWarps == warp) {
+          block_row(base + w * 32 + __ffs(m) - 1, true, 0, 1);
+          __syncwarp();                          // red and res serve the next row
+        }
+  } else {
+    const int team = warp / nw, u = blockIdx.x * (kTeamWarps / nw) + team;
+    block_row(u, u < n_brows, warp - team * nw, nw);
   }
 }
 
@@ -436,7 +435,7 @@ template <int VW>
 cudaError_t team_go(int op, int n_brows, int br, int bc, double avg, const int *rp, const int *col,
                     const float *val, const float *W, const float *x, const float *b, float *y,
                     const int *rp2, const int *col2, const float *val2, float *x2o,
-                    int min_len, cudaStream_t s) {
+                    cudaStream_t s) {
   const int LC = bc / VW, G = 32 / LC;
   const int rows = div_up(br, G);                  // row steps of one warp over a block
   const int ES = div_up(rows, kTeamRows);
@@ -449,29 +448,25 @@ cudaError_t team_go(int op, int n_brows, int br, int bc, double avg, const int *
   while (ES * BS * 2 <= kTeamWarps && avg >= 8.0 * BS &&
          (long long)n_brows * ES * BS < 40LL * kNumSM)
     BS *= 2;
-  if (min_len == 0 && avg > 1e8) BS = std::min(BS, 4);   // rows of unknown length
+  if (avg > 1e8) BS = std::min(BS, 4);   // rows of unknown length
   // Few long rows: a cluster of CTAs per block row, each with a share of its
   // blocks, while it keeps the GPU within one wave (32 warps an SM) and every
   // warp eight blocks; rank 0 adds up the CTAs' sums and finishes the row.  384
   // rows of 98 blocks of 17 x 17: step 22.5 -> 19.0 us; the fused restriction to
   // them 64.7 -> 23.7 us; 64 rows of 28 x 21 blocks 29.4 -> 12.5 us.
   int CS = 1;
-  while (min_len == 0 && CS < kTeamCluster && avg < 1e8 && avg >= 16.0 * BS * CS &&
+  while (CS < kTeamCluster && avg < 1e8 && avg >= 16.0 * BS * CS &&
          (long long)n_brows * ES * BS * CS * 2 <= 32LL * kNumSM)
     CS *= 2;
   const int nw = ES * BS, teams = CS > 1 || nw >= 8 ? 1 : 8 / nw, warps = nw * teams;
   const size_t smem = ((size_t)warps * 32 * RPL + teams * kWideMaxRows) * sizeof(float);
-  const int grid = min_len > 0 ? std::min(div_up(n_brows, 32 * warps), 4 * kNumSM)
-                               : CS * div_up(n_brows, teams);
+  const int grid = CS * div_up(n_brows, teams);
   auto go = [&](auto kern) {
     launch_kc(kern, grid, 32 * warps, smem, s, CS, op, n_brows, br, bc, ES, BS, CS, rp, col, val, W, x, b, y,
-             rp2, col2, val2, x2o, min_len);
+             rp2, col2, val2, x2o);
   };
-#define GASA_TEAM(N)                              \
-  case N:                                         \
-    if (min_len > 0) go(bsr_team_kernel<VW, N, true>); \
-    else go(bsr_team_kernel<VW, N, false>);       \
-    break;
+#define GASA_TEAM(N) \
+  case N: go(bsr_team_kernel<VW, N>); break;
   switch (RPL) {
     GASA_TEAM(1) GASA_TEAM(2) GASA_TEAM(3) GASA_TEAM(4) GASA_TEAM(5) GASA_TEAM(6) GASA_TEAM(7)
     GASA_TEAM(8)
@@ -484,18 +479,28 @@ cudaError_t team_go(int op, int n_brows, int br, int bc, double avg, const int *
 template <int OP, int VW>
 cudaError_t rows_go(int n_brows, int br, int bc, double avg, const int *rp, const int *col,
                     const float *val, const float *W, const float *x, const float *b, float *y,
-                    const int *rp2, const int *col2, const float *val2, float *x2o,
+                    const int *rp2, const int *col2, const float *val2, float *x2o, int min_len,
                     cudaStream_t s) {
+  auto go = [&](auto kern, int grid, int nw, int chunk) {
+    launch_k(kern, grid, 32 * kTeamWarps, 0, s, n_brows, br, bc, nw, chunk, min_len, rp, col, val, W,
+             x, b, y, rp2, col2, val2, x2o);
+    note_launch();
+    return cudaGetLastError();
+  };
+  if constexpr (OP != WIDE_RFUSED) {
+    if (min_len > 0) {
+      // as many rows a CTA as give an SM eight CTAs, a row a warp at least
+      const int chunk = std::min(32 * kTeamWarps, div_up(div_up(n_brows, 8 * kNumSM), kTeamWarps) * kTeamWarps);
+      return go(bsr_rows_kernel<OP, VW, true>, div_up(n_brows, chunk), 1, chunk);
+    }
+  }
   // warps per block row: about four blocks per group, at most a CTA; without the average
   // as many as give an SM 16
   const int G = br <= 32 ? 32 / br : 1;
   int nw = 1;
   while (nw < kTeamWarps && (avg < 1e8 ? nw * G * 4 < avg : (long long)n_brows * nw < 16LL * kNumSM))
     nw *= 2;
-  launch_k(bsr_rows_kernel<OP, VW>, div_up(n_brows, kTeamWarps / nw), 32 * kTeamWarps, 0, s, n_brows,
-           br, bc, nw, rp, col, val, W, x, b, y, rp2, col2, val2, x2o);
-  note_launch();
-  return cudaGetLastError();
+  return go(bsr_rows_kernel<OP, VW, false>, div_up(n_brows, kTeamWarps / nw), nw, 0);
 }
 
 cudaError_t team_launch(int op, int n_brows, int br, int bc, int64_t nnzb, const int *rp,
@@ -507,15 +512,15 @@ cudaError_t team_launch(int op, int n_brows, int br, int bc, int64_t nnzb, const
   // RFUSED multiplies val with b and val2 with x
   const int vw = op == WIDE_RFUSED ? wide_vec(bc, val, b, val2, x)
                                    : wide_vec(bc, val, x, nullptr, nullptr);
-  if (min_len == 0 && wide_by_rows(op, n_brows, br, bc, nnzb, vw)) {
+  if (min_len > 0 || wide_by_rows(op, n_brows, br, bc, nnzb, vw)) {
 #define GASA_ROWS(OP)                                                                             \
   case OP:                                                                                        \
     return vw == 4 ? rows_go<OP, 4>(n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2,     \
-                                    val2, x2o, s)                                                 \
+                                    val2, x2o, min_len, s)                                        \
            : vw == 2 ? rows_go<OP, 2>(n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2,   \
-                                      val2, x2o, s)                                               \
+                                      val2, x2o, min_len, s)                                      \
                      : rows_go<OP, 1>(n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2,   \
-                                      val2, x2o, s);
+                                      val2, x2o, min_len, s);
     switch (op) {
       GASA_ROWS(WIDE_ASSIGN) GASA_ROWS(WIDE_RESID) GASA_ROWS(WIDE_ADD) GASA_ROWS(WIDE_SWEEP)
       GASA_ROWS(WIDE_RFUSED)
@@ -524,10 +529,10 @@ cudaError_t team_launch(int op, int n_brows, int br, int bc, int64_t nnzb, const
   }
   if (bc / vw > 32) return cudaErrorNotSupported;
   if (vw == 4)
-    return team_go<4>(op, n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2, val2, x2o, min_len, s);
+    return team_go<4>(op, n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2, val2, x2o, s);
   if (vw == 2)
-    return team_go<2>(op, n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2, val2, x2o, min_len, s);
-  return team_go<1>(op, n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2, val2, x2o, min_len, s);
+    return team_go<2>(op, n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2, val2, x2o, s);
+  return team_go<1>(op, n_brows, br, bc, avg, rp, col, val, W, x, b, y, rp2, col2, val2, x2o, s);
 }
 
 }  // namespace

@@ -290,3 +290,49 @@ def test_wide_team_rounding(n, b, per_row, limit):
     gasa.gasa_bsr_mv_f32(0, n, b, b, to_dev(rp), to_dev(col), to_dev(val.ravel()), to_dev(x), y, y)
     err = np.sqrt(np.mean((y.cpu().numpy() - want) ** 2) / np.mean(want ** 2))
     assert err <= limit, err
+
+
+@pytest.mark.parametrize("n,br,bc,per_row", [(8000, 10, 10, 15), (4300, 16, 16, 20), (9000, 8, 12, 9)])
+def test_many_long_rows_of_unknown_length(n, br, bc, per_row):
+    """Many rows, all of them long, in one call: no slower than four times the same rows in
+    two calls that are few rows each (and take teams or lanes for all of them)."""
+    import torch
+    gasa = _gasa()
+    rng = np.random.default_rng(n)
+    rp = (per_row * np.arange(n + 1)).astype(np.int32)
+    col = ((np.arange(per_row)[None, :] * 3 + np.arange(n)[:, None]) % n)
+    col = np.sort(col, axis=1).astype(np.int32).ravel()
+    val = rng.standard_normal((n * per_row, br, bc)).astype(np.float32)
+    x = rng.standard_normal(n * bc).astype(np.float32)
+    dv, dx, dc = to_dev(val.ravel()), to_dev(x), to_dev(col)
+    y, y2 = to_dev(np.zeros(n * br, np.float32)), to_dev(np.zeros(n * br, np.float32))
+    h = n // 2
+    drp, drp1, drp2 = to_dev(rp), to_dev(rp[:h + 1]), to_dev(rp[h:] - rp[h])
+    k = int(rp[h])
+
+    def whole():
+        gasa.gasa_bsr_mv_f32(0, n, br, bc, drp, dc, dv, dx, y, y)
+
+    def halves():
+        gasa.gasa_bsr_mv_f32(0, h, br, bc, drp1, dc, dv, dx, y2, y2)
+        gasa.gasa_bsr_mv_f32(0, n - h, br, bc, drp2, dc[k:], dv[k * br * bc:], dx, y2[h * br:], y2[h * br:])
+
+    def ms(f):
+        best = np.inf
+        for _ in range(5):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            for _ in range(20):
+                f()
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b) / 20)
+        return best
+
+    whole()
+    halves()
+    ref = _bsr_apply(rp, col, val.astype(np.float64), x.astype(np.float64))
+    mag = _bsr_apply(rp, col, np.abs(val).astype(np.float64), np.abs(x).astype(np.float64))
+    for got in (y, y2):
+        assert np.all(np.abs(got.cpu().numpy() - ref) <= (per_row * bc + 4) * 2.0 ** -23 * mag)
+    assert ms(whole) <= 4 * ms(halves)
