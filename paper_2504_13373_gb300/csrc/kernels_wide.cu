@@ -20,8 +20,8 @@
 // and the team.
 //
 // Operations: y = A x, y = b - A x, y += A x for any br x bc blocks (at most
-// 40 x 40, bc <= 32 where it is odd), the block-Jacobi step
-// x_out = x + W (b - A x) of Alg. 1 (W = w D^{-1}, square blocks), and the fused
+// 40 x 40), the block-Jacobi step x_out = x + W (b - A x) of Alg. 1 (W = w D^{-1},
+// square blocks, at most 32 wide where read an entry at a time), and the fused
 // residual and restriction y = R b - (R A) x of Alg. 2 with the next level's
 // first step W y.
 //
@@ -538,6 +538,9 @@ cudaError_t team_launch(int op, int n_brows, int br, int bc, int64_t nnzb, const
 }  // namespace
 
 // Lanes on rows of blocks instead of teams (GB300, us with lanes on rows / with teams):
+//  - products with widths of 33 to 40 that have to be read an entry at a time, more than
+//    a team's lanes (300 rows of 30 blocks of 37 x 37 18.3, with the general kernels, which
+//    they fell to, 35.2); smoothing steps stay there (300 rows of 10 11.0 / 16.0);
 //  - low blocks, at most 8 rows by 16 columns: 32,768 rows of 16 blocks of 4 x 10
 //    24.6 / 42.1, 4,000 rows 4.7 / 7.6, 20,000 rows of 10 of 8 x 12 16.8 / 20.6 (wider
 //    ones: 4,000 rows of 16 of 4 x 31 17.6 / 10.1);
@@ -551,6 +554,7 @@ cudaError_t team_launch(int op, int n_brows, int br, int bc, int64_t nnzb, const
 //    of 17 to 20, which leave a third of a team's lanes idle, on tall blocks: 2,500 rows
 //    of 36 of 22 x 17 41.3 / 57.3 (64 rows of 90 13.4 / 8.6, a cluster a row).
 bool wide_by_rows(int op, int n_brows, int br, int bc, int64_t nnzb, int vw) {
+  if (bc / vw > 32) return op != WIDE_SWEEP;
   if (br <= 8 && bc <= 16) return true;
   if (nnzb < 0) return false;
   const int b = std::max(br, bc);
@@ -570,6 +574,8 @@ bool wide_applies(int br, int bc, int n_brows, int64_t nnzb) {
          nnzb >= (long long)kLongRow * n_brows;
 }
 
+// widths beyond a team's lanes: the general kernels when the row length is unknown, too
+// (1,000 rows of 12 of 37 x 37: product 32.9 us, lanes on rows 28.8; step 28.7 and 32.8)
 bool wide_shape(int br, int bc, const float *val, const float *x) {
   return (br > 8 || bc > 8) && br <= kWideMaxRows && bc <= kWideMaxRows &&
          bc / wide_vec(bc, val, x, nullptr, nullptr) <= 32;

@@ -86,5 +86,9 @@ def test_fp32_low_and_short_rows_keep_a_lane_per_row():
         assert by_rows(3, n, b, b, per_row), (n, b, per_row)
     for n, b, per_row in ((256, 12, 20), (4000, 12, 20), (2000, 13, 40), (3072, 13, 25), (4000, 16, 16)):
         assert not by_rows(3, n, b, b, per_row), (n, b, per_row)
+    # products of every width up to 40 have a kernel here, odd ones beyond a team's lanes too
+    for bc in range(33, 41):
+        for op in (0, 1, 2, 4):
+            assert by_rows(op, 1000, bc, bc, 12) == (bc % 2 == 1)
     assert by_rows(4, 1024, 10, 8, 45) and by_rows(4, 2500, 22, 17, 36)
     assert not by_rows(4, 4096, 12, 12, 36) and not by_rows(4, 64, 22, 17, 90)

@@ -336,3 +336,9 @@ def test_many_long_rows_of_unknown_length(n, br, bc, per_row):
     for got in (y, y2):
         assert np.all(np.abs(got.cpu().numpy() - ref) <= (per_row * bc + 4) * 2.0 ** -23 * mag)
     assert ms(whole) <= 4 * ms(halves)
+
+
+@pytest.mark.parametrize("n,b", [(48, 37), (30, 33)])
+def test_vcycle_odd_widths_beyond_a_warp(n, b):
+    """Blocks wider than a warp that are read an entry at a time, in a hierarchy."""
+    test_vcycle_few_long_rows(n, b)
