@@ -1250,15 +1250,18 @@ dense_mv_kernel(int n, int ld, const double *__restrict__ A, const T *__restrict
   if (lane == 0) y[row] = (T)acc;
 }
 
-// y = M x for the FP32 cycle's dense bottom operator: M as exact two-term
-// FP32 splits (Mh the FP32 rounding of M, Ml that of M - Mh), FP32 x,
+// y = M x for the FP32 cycle's dense bottom operator: M as two FP32 words (Mh the
+// FP32 rounding of M, Ml that of M - Mh, together 48 of its 53 bits) and FP32 x,
 // products and sums in double-single arithmetic on FP32 units (the scheme of
 // bsr_mv_ds_kernel with x exact in FP32), so each row agrees with the FP64
 // product to about 2^-47 of sum |m x|; GB300's FP64 pipe would take n^2 FMAs
 // at a small fraction of the FP32 rate.  A warp per row (two where rows are
 // few), lane l takes groups of four columns l, l + 32, ... in order with 16-byte
-// loads, two groups in flight; its (s, lo) pairs meet in a warp tree, then FP64.
-// Order 2,048 (33.5 MB): 12.0 -> 7.4 us on GB300; a CTA per row took 4-byte loads
+// loads, two groups in flight; its sum goes to FP64, then a warp tree.  The rounding
+// errors of the low word are carried in a third, so that a lane's 16 to 64 columns
+// round like a few (order 2,048, rms error in 2^-53 of an entry: 4,510 without, 430
+// with it, 1,609 for a CTA a row with 8 columns a thread).
+// Order 2,048 (33.5 MB): 12.0 -> 7.3 us on GB300 (7.0 without the third word); a CTA per row took 4-byte loads
 // and its barriers were most of a row's time.
 template <int WPR>
 __global__ void __launch_bounds__(128)
@@ -1272,16 +1275,14 @@ dense_mv_ds_kernel(int n, int ld, const float *__restrict__ Mh, const float *__r
   const float4 *h4 = reinterpret_cast<const float4 *>(Mh + o);
   const float4 *l4 = reinterpret_cast<const float4 *>(Ml + o);
   const float4 *x4 = reinterpret_cast<const float4 *>(x);
-  float s = 0.0f, lo = 0.0f;
+  float s = 0.0f, lo = 0.0f, u = 0.0f;
   auto add = [&](float ah, float al, float xh) {
     const float pr = __fmul_rn(ah, xh);
     const float e = __fmaf_rn(ah, xh, -pr);
-    const float cross = __fmul_rn(al, xh);
-    const float s1 = __fadd_rn(s, pr);
-    const float bp = __fsub_rn(s1, s);
-    const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(s1, bp)), __fsub_rn(pr, bp));
-    s = s1;
-    lo = __fadd_rn(lo, __fadd_rn(err, __fadd_rn(e, cross)));
+    float es, r1, r2;
+    s = two_sum(s, pr, es);
+    lo = two_sum(lo, two_sum(__fmaf_rn(al, xh, e), es, r1), r2);
+    u = __fadd_rn(u, __fadd_rn(r1, r2));
   };
   auto add4 = [&](const float4 &h, const float4 &l, const float4 &v) {
     add(h.x, l.x, v.x);
@@ -1303,7 +1304,7 @@ dense_mv_ds_kernel(int n, int ld, const float *__restrict__ Mh, const float *__r
     const int c = (m << 2) + lane;
     add(__ldg(Mh + o + c), __ldg(Ml + o + c), __ldg(x + c));
   }
-  double v = (double)s + (double)lo;
+  double v = (double)s + ((double)lo + (double)u);
   v = warp_sum(v);
   if (WPR == 1) {
     if (on && lane == 0) y[row] = (float)v;

@@ -22,7 +22,8 @@ def _ptr(t):
 
 def _exact_rows(M, x):
     """sum_j M_ij x_j rounded once (products of 26-bit halves of M and FP32 x are exact)"""
-    hi = np.ldexp(np.round(np.ldexp(M, 25 - np.frexp(M)[1])), np.frexp(M)[1] - 25)
+    e = np.frexp(M)[1]
+    hi = np.ldexp(np.round(np.ldexp(M, 25 - e)), e - 25)
     x = x.astype(np.float64)
     return np.array([math.fsum(np.concatenate([h * x, l * x])) for h, l in zip(hi, M - hi)])
 
@@ -75,3 +76,33 @@ def test_batched_bottom_operator(n, spread):
         if first is None:
             first = got[:, c].copy()
         assert np.array_equal(got[:, c], first)
+
+
+@pytest.mark.parametrize("n", [1, 5, 31, 33, 130, 515, 816, 1217, 2048, 2435])
+def test_bottom_operator(n):
+    """On one vector, orders on both sides of every split: with two FP32 words of the operator
+    within 12 x 2^-53 of the products' norm (rms over the rows) of those words' exact sums;
+    with FP64 multiply-adds to a warp's chain."""
+    rng = np.random.default_rng(n)
+    M, x = _cancelling(rng, n, 2.0)
+    Mp, ld = _pitched(M)
+    hi = Mp.astype(np.float32)
+    lo = (Mp - hi).astype(np.float32)
+    words = (hi.astype(np.float64) + lo)[:, :n]
+    norm = np.sqrt(((M * x.astype(np.float64)) ** 2).sum(1))
+
+    def rms(y, op):
+        return np.sqrt(np.mean(((to_host(y).astype(np.float64) - _exact_rows(op, x)) / norm) ** 2))
+
+    dM, dx = to_dev(Mp), to_dev(x)
+    y = to_dev(np.zeros(n, np.float32))
+    f = _fn("_ZN4gasa18launch_dense_mv_dsEiiPKfS1_S1_PfP11CUstream_st")
+    dh, dl = to_dev(hi), to_dev(lo)
+    one = 2.0 ** -24 if n == 1 else 0.0
+    assert f(n, ld, _ptr(dh), _ptr(dl), _ptr(dx), _ptr(y), None) == 0
+    assert rms(y, words) <= 12 * 2.0 ** -53 + one
+    for t, m, v in ((np.float32, "If", dx), (np.float64, "Id", to_dev(x.astype(np.float64)))):
+        y = to_dev(np.zeros(n, t))
+        g = _fn("_ZN4gasa15launch_dense_mv%sEE9cudaErroriPKdPKT_PS4_P11CUstream_sti" % m)
+        assert g(n, _ptr(dM), _ptr(v), _ptr(y), None, ld) == 0
+        assert rms(y, M) <= 3 * 2.0 ** -53 + one
