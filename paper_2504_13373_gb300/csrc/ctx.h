@@ -83,6 +83,8 @@ struct gasa_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
+  cudaStream_t capture_stream = nullptr;   // graphs are captured here (the context's own stream, or
+                                           // one beside the caller's)
   std::string err;
   bool ready = false;
   gasa_options opt{};
@@ -116,7 +118,7 @@ struct gasa_ctx {
   long long cg_kernels[6] = {};
   int cg_max_iter[6] = {};
   // one V-cycle per precision as an instantiated graph (host-driven callers,
-  // from their second V-cycle on); vc_calls < 0: the stream cannot be captured
+  // from their second V-cycle on); vc_calls < 0: the graph could not be built
   cudaGraphExec_t vc_exec[3] = {};
   int vc_calls[3] = {};
   long long vc_kernels[3] = {};

@@ -95,6 +95,27 @@ void free_graphs(gasa_ctx *ctx) {
   }
 }
 
+// While one lives, the context's launches go to its capture stream and carry no event
+// records.  A stream that the caller gave is never captured: what
+// another thread enqueues on it meanwhile would go into the graph instead of running.
+struct CaptureScope {
+  gasa_ctx *ctx;
+  cudaStream_t stream;
+  bool prof;
+  long long before;
+  explicit CaptureScope(gasa_ctx *c) : ctx(c), stream(c->stream), prof(c->prof) {
+    ctx->stream = ctx->capture_stream;
+    ctx->prof = false;
+    before = launch_count();
+  }
+  long long kernels() const { return launch_count() - before; }
+  ~CaptureScope() {
+    ctx->stream = stream;
+    ctx->prof = prof;
+    note_launches(-kernels());   // recorded, not launched
+  }
+};
+
 void free_all(gasa_ctx *ctx) {
   cudaStreamSynchronize(ctx->stream);
   free_graphs(ctx);
@@ -884,32 +905,25 @@ gasa_status vcycle_body(gasa_ctx *ctx, int precision) {
                             first_step_reads_f64(ctx, precision));
 }
 
-// Capture vcycle_body into ctx->vc_exec[precision]; a stream that cannot be
-// captured leaves vc_calls negative and every V-cycle as separate launches.
-gasa_status build_vcycle_graph(gasa_ctx *ctx, int precision) {
-  cudaStream_t s = ctx->stream;
-  if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-    (void)cudaGetLastError();
-    ctx->vc_calls[precision] = -1;
-    return GASA_OK;
-  }
-  const long long k0 = launch_count();
-  const gasa_status st = vcycle_body(ctx, precision);
-  const long long captured = launch_count() - k0;
-  note_launches(-captured);   // recorded, not launched
+// Capture vcycle_body into ctx->vc_exec[precision]; where that fails, vc_calls is left
+// negative and every V-cycle stays separate launches.
+void build_vcycle_graph(gasa_ctx *ctx, int precision) {
+  CaptureScope cap(ctx);
   cudaGraph_t g = nullptr;
-  const cudaError_t e = cudaStreamEndCapture(s, &g);
-  if (st != GASA_OK || e != cudaSuccess) {
-    if (g) cudaGraphDestroy(g);
-    ST(st);
-    CU(e);
+  cudaError_t e = cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal);
+  if (e == cudaSuccess) {
+    const gasa_status st = vcycle_body(ctx, precision);
+    e = cudaStreamEndCapture(ctx->stream, &g);
+    if (st != GASA_OK && e == cudaSuccess) e = cudaErrorStreamCaptureInvalidated;
   }
-  const cudaError_t ei = cudaGraphInstantiate(&ctx->vc_exec[precision], g, 0);
-  cudaGraphDestroy(g);
-  if (ei != cudaSuccess) ctx->vc_exec[precision] = nullptr;
-  CU(ei);
-  ctx->vc_kernels[precision] = captured;
-  return GASA_OK;
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&ctx->vc_exec[precision], g, 0);
+  if (g) cudaGraphDestroy(g);
+  if (e != cudaSuccess) {
+    (void)cudaGetLastError();
+    ctx->vc_exec[precision] = nullptr;
+    ctx->vc_calls[precision] = -1;
+  }
+  ctx->vc_kernels[precision] = cap.kernels();
 }
 
 // z = M r for host-driven callers (gasa_vcycle, GMRES).  A V-cycle is 30 to 40
@@ -928,7 +942,7 @@ gasa_status apply_M_host(gasa_ctx *ctx, const double *rr, double *z, int precisi
     return apply_M(ctx, rr, z, precision);
   }
   if (!ctx->vc_exec[precision]) {
-    ST(build_vcycle_graph(ctx, precision));
+    build_vcycle_graph(ctx, precision);
     if (!ctx->vc_exec[precision]) return apply_M(ctx, rr, z, precision);
   }
   cudaStream_t s = ctx->stream;
@@ -1146,6 +1160,7 @@ gasa_status build_cg_graph(gasa_ctx *ctx, int precision) {
   if (ctx->cg_graph[pi]) cudaGraphDestroy(ctx->cg_graph[pi]);
   ctx->cg_exec[pi] = nullptr;
   ctx->cg_graph[pi] = nullptr;
+  CaptureScope cap(ctx);
   cudaStream_t s = ctx->stream;
   const int64_t n = ctx->L[0].ndof;
   const bool flex = precision != GASA_PREC_FP64;
@@ -1163,9 +1178,6 @@ gasa_status build_cg_graph(gasa_ctx *ctx, int precision) {
   cudaGraph_t body = cp.conditional.phGraph_out[0];
   double *x = ctx->kx, *r = ctx->kr, *z = ctx->kz, *p = ctx->kp, *q = ctx->kq;
   double *pq_part = ctx->part, *rr_part = ctx->part + kRedBlocks;
-  const bool prof = ctx->prof;
-  ctx->prof = false;   // no event records inside a graph body
-  const long long k0 = launch_count();
   CU(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
   int np = flex ? cg_blocks(n) : kRedBlocks;
   gasa_status st = GASA_OK;
@@ -1203,8 +1215,7 @@ gasa_status build_cg_graph(gasa_ctx *ctx, int precision) {
   }
   cudaGraph_t captured = nullptr;
   cudaError_t e2 = cudaStreamEndCapture(s, &captured);
-  ctx->prof = prof;
-  ctx->cg_kernels[pi] = launch_count() - k0;
+  ctx->cg_kernels[pi] = cap.kernels();
   if (st != GASA_OK) return st;
   CU(e);
   CU(e2);
@@ -1420,6 +1431,7 @@ gasa_status build_st_graph(gasa_ctx *ctx, int precision) {
   if (ctx->cg_graph[pi]) cudaGraphDestroy(ctx->cg_graph[pi]);
   ctx->cg_exec[pi] = nullptr;
   ctx->cg_graph[pi] = nullptr;
+  CaptureScope cap(ctx);
   cudaStream_t s = ctx->stream;
   cudaGraph_t g = nullptr;
   CU(cudaGraphCreate(&g, 0));
@@ -1433,15 +1445,11 @@ gasa_status build_st_graph(gasa_ctx *ctx, int precision) {
   cudaGraphNode_t node;
   CU(cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &cp));
   cudaGraph_t body = cp.conditional.phGraph_out[0];
-  const bool prof = ctx->prof;
-  ctx->prof = false;
-  const long long k0 = launch_count();
   CU(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
   gasa_status st = stationary_step(ctx, precision, max_iter, h, true);
   cudaGraph_t captured = nullptr;
   cudaError_t e2 = cudaStreamEndCapture(s, &captured);
-  ctx->prof = prof;
-  ctx->cg_kernels[pi] = launch_count() - k0;
+  ctx->cg_kernels[pi] = cap.kernels();
   if (st != GASA_OK) return st;
   CU(e2);
   CU(cudaGraphInstantiate(&ctx->cg_exec[pi], g, 0));
@@ -2300,15 +2308,12 @@ gasa_status gasa_create(gasa_ctx **out, int32_t device, void *stream) {
   if (cudaSetDevice(device) != cudaSuccess) return GASA_ERR_CUDA;
   gasa_ctx *c = new gasa_ctx();
   c->device = device;
-  if (stream) {
-    c->stream = (cudaStream_t)stream;
-  } else {
-    if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) {
-      delete c;
-      return GASA_ERR_CUDA;
-    }
-    c->own_stream = true;
+  if (cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
+    delete c;
+    return GASA_ERR_CUDA;
   }
+  c->own_stream = stream == nullptr;
+  c->stream = c->own_stream ? c->capture_stream : (cudaStream_t)stream;
   gasa_default_options(&c->opt);
   // look up the allocation-free entry point's scratch on this device now, so
   // that its module is loaded here rather than inside an allocation-free call
@@ -2546,7 +2551,7 @@ gasa_status gasa_destroy(gasa_ctx *ctx) {
   free_all(ctx);
   for (auto &p : ctx->pc)
     for (auto e : p.ev) cudaEventDestroy(e);
-  if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
+  cudaStreamDestroy(ctx->capture_stream);   // the context's own stream where none was given
   delete ctx;
   return GASA_OK;
 }

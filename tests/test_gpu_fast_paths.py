@@ -342,3 +342,57 @@ def test_many_long_rows_of_unknown_length(n, br, bc, per_row):
 def test_vcycle_odd_widths_beyond_a_warp(n, b):
     """Blocks wider than a warp that are read an entry at a time, in a hierarchy."""
     test_vcycle_few_long_rows(n, b)
+
+
+@pytest.mark.parametrize("call", ["vcycle", "solve"])
+def test_graphs_are_not_captured_on_the_callers_stream(call):
+    """What another thread enqueues on the stream that the caller gave, while a graph is being
+    built, runs once and does not become part of the graph."""
+    import threading
+    import torch
+    gasa = _gasa()
+    pr = problem("p3_16")
+    A = pr.A
+    stream = torch.cuda.Stream()
+    ctx = gasa.gasa_create(0, stream)
+    try:
+        gasa.gasa_setup(ctx, A.row_ptr, A.col, A.val.ravel(), A.b, pr.agg_of,
+                        gasa.gasa_default_options(dim=2, n_cand=pr.r), adj_ptr=pr.adj_ptr,
+                        adj_idx=pr.adj_idx, centroids=pr.centroids, init_candidates=pr.B0)
+        r = to_dev(pr.rhs)
+        z, z2, x = torch.empty_like(r), torch.empty_like(r), torch.empty_like(r)
+        count = torch.zeros(1, dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        gasa.gasa_vcycle(ctx, r, z, 1)
+        added, stop, started, errors = [0], threading.Event(), threading.Event(), []
+
+        def other():
+            try:
+                with torch.cuda.stream(stream):
+                    while not stop.is_set():
+                        count.add_(1.0)
+                        added[0] += 1
+                        started.set()
+            except Exception as e:      # a launch refused because of the capture
+                errors.append(e)
+                started.set()
+
+        t = threading.Thread(target=other)
+        t.start()
+        started.wait()
+        try:
+            if call == "vcycle":
+                gasa.gasa_vcycle(ctx, r, z2, 1)                       # builds its graph
+            else:
+                gasa.gasa_solve(ctx, r, x, 1e-8, 1, on_device=True)   # builds the CG graph
+        finally:
+            stop.set()
+            t.join()
+        for _ in range(3):
+            gasa.gasa_vcycle(ctx, r, z2, 1)
+        torch.cuda.synchronize()
+        assert not errors and count.item() == added[0]
+        assert torch.equal(z, z2)
+    finally:
+        gasa.gasa_destroy(ctx)
+
