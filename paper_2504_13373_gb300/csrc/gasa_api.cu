@@ -95,24 +95,23 @@ void free_graphs(gasa_ctx *ctx) {
   }
 }
 
-// While one lives, the context's launches go to its capture stream and carry no event
-// records.  A stream that the caller gave is never captured: what
+// While one lives, the context's launches go to its capture stream, count into `kernels` and
+// carry no event records.  A stream that the caller gave is never captured: what
 // another thread enqueues on it meanwhile would go into the graph instead of running.
 struct CaptureScope {
   gasa_ctx *ctx;
   cudaStream_t stream;
   bool prof;
-  long long before;
+  long long kernels = 0;
   explicit CaptureScope(gasa_ctx *c) : ctx(c), stream(c->stream), prof(c->prof) {
     ctx->stream = ctx->capture_stream;
     ctx->prof = false;
-    before = launch_count();
+    record_launches(&kernels);
   }
-  long long kernels() const { return launch_count() - before; }
   ~CaptureScope() {
     ctx->stream = stream;
     ctx->prof = prof;
-    note_launches(-kernels());   // recorded, not launched
+    record_launches(nullptr);
   }
 };
 
@@ -923,7 +922,7 @@ void build_vcycle_graph(gasa_ctx *ctx, int precision) {
     ctx->vc_exec[precision] = nullptr;
     ctx->vc_calls[precision] = -1;
   }
-  ctx->vc_kernels[precision] = cap.kernels();
+  ctx->vc_kernels[precision] = cap.kernels;
 }
 
 // z = M r for host-driven callers (gasa_vcycle, GMRES).  A V-cycle is 30 to 40
@@ -1215,7 +1214,7 @@ gasa_status build_cg_graph(gasa_ctx *ctx, int precision) {
   }
   cudaGraph_t captured = nullptr;
   cudaError_t e2 = cudaStreamEndCapture(s, &captured);
-  ctx->cg_kernels[pi] = cap.kernels();
+  ctx->cg_kernels[pi] = cap.kernels;
   if (st != GASA_OK) return st;
   CU(e);
   CU(e2);
@@ -1449,7 +1448,7 @@ gasa_status build_st_graph(gasa_ctx *ctx, int precision) {
   gasa_status st = stationary_step(ctx, precision, max_iter, h, true);
   cudaGraph_t captured = nullptr;
   cudaError_t e2 = cudaStreamEndCapture(s, &captured);
-  ctx->cg_kernels[pi] = cap.kernels();
+  ctx->cg_kernels[pi] = cap.kernels;
   if (st != GASA_OK) return st;
   CU(e2);
   CU(cudaGraphInstantiate(&ctx->cg_exec[pi], g, 0));

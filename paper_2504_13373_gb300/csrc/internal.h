@@ -52,6 +52,9 @@ cudaError_t noalloc_scratch_on_current_device(double **out);
 // kernel launches issued by this library (process-wide counter)
 void note_launch();
 long long launch_count();
+// this thread's launches from here on count into *into (a graph's kernels) and not as
+// launched; null: as launched again
+void record_launches(long long *into);
 
 enum JacobiMode { JAC_SWEEP = 0, JAC_FIRST = 1, JAC_APPLY = 2, JAC_RELAX = 3 };
 

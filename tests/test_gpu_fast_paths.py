@@ -396,3 +396,47 @@ def test_graphs_are_not_captured_on_the_callers_stream(call):
     finally:
         gasa.gasa_destroy(ctx)
 
+
+def test_launch_count_of_graphs_is_this_threads():
+    """Launches of other threads while a V-cycle's graph is built are not counted as its own:
+    every later V-cycle counts what a hierarchy built alone does."""
+    import threading
+    import torch
+    gasa = _gasa()
+    pr = problem("p3_16")
+
+    def per_cycle(busy):
+        ctx, _ = gpu_setup("p3_16", keep=False)
+        stop = threading.Event()
+        n = 4096
+        x, y = (torch.zeros(n, dtype=torch.float64, device="cuda") for _ in range(2))
+        rp, col = to_dev(np.arange(n + 1, dtype=np.int32)), to_dev(np.arange(n, dtype=np.int32))
+
+        def other():
+            s = torch.cuda.Stream()
+            while not stop.is_set():
+                gasa.gasa_bsr_mv(0, n, 1, 1, rp, col, x, x, x, y, s)
+
+        t = threading.Thread(target=other)
+        try:
+            r = to_dev(pr.rhs)
+            z = torch.empty_like(r)
+            gasa.gasa_vcycle(ctx, r, z, 1)
+            if busy:
+                t.start()
+            gasa.gasa_vcycle(ctx, r, z, 1)
+            if busy:
+                stop.set()
+                t.join()
+            torch.cuda.synchronize()
+            k = gasa.gasa_kernel_launches()
+            for _ in range(5):
+                gasa.gasa_vcycle(ctx, r, z, 1)
+            return (gasa.gasa_kernel_launches() - k) / 5
+        finally:
+            stop.set()
+            gasa.gasa_destroy(ctx)
+
+    alone = per_cycle(False)
+    for _ in range(3):
+        assert per_cycle(True) == alone
