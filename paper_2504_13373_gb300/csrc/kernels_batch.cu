@@ -9,6 +9,7 @@
 // gives the same bits whether it runs alone or in a batch, in any slot and at
 // any batch width K.
 #include <algorithm>
+#include <type_traits>
 
 #include "batch.h"
 #include "common.cuh"
@@ -54,7 +55,7 @@ __device__ __forceinline__ void row_dot_k(int beg, int end, int r, int br, int b
 }
 
 // ---------------------------------------------------------------------------
-// Served meshes of a few thousand rows: eight slices per scalar row.  A thread
+// Served meshes of a few thousand rows (sliced_rows below): eight slices per scalar row.  A thread
 // per row leaves most SMs empty and walks its 40 to 700 values one dependent
 // load after another; here the row's values are dealt to eight lanes (slice q
 // takes entries q, q + 8, ... of the row), each for two of the K columns, so a
@@ -73,32 +74,38 @@ struct Slices {
 };
 
 // Sum over `len` entries dealt to the slices: entry f of the row is a(f) and
-// x(f) points at its K columns.  Returns the sum of column column_of(sub).  A slice
-// adds its entries eight at a time, the eights in order: in one chain rows of hundreds
-// of values rounded up to 1.8 times as much as lanes that take whole blocks each (98
-// blocks of 17 x 17, random values, rms error in units of the rounding 4.4 and 2.4; so 2.0).
-template <typename T, int K, typename FA, typename FX>
+// x(f) points at its K columns.  Returns the sum of column column_of(sub).  A slice adds
+// its entries in CH chains: in one, long rows rounded up to 1.8 times as much as with lanes
+// that take whole blocks each (98 blocks of 17 x 17 in FP32, random values, rms error
+// 2.6e-7 and 1.4e-7 of the sums' rms), in four no more than they (1.4e-7).
+template <typename T, int K, int CH, typename FA, typename FX>
 __device__ __forceinline__ T sliced_sum(int sub, int len, FA a, FX x) {
   using S = Slices<K>;
   const int sl = sub / S::CG, cg = sub % S::CG;
-  T acc[S::C], t[S::C];
-  // the slice's entries f .. end, one after another
-  auto chain = [&](int f, int end, T (&sum)[S::C]) {
+  T t[CH][S::C];
 #pragma unroll
-    for (int c = 0; c < S::C; ++c) sum[c] = T(0);
-#pragma unroll 4
-    for (; f < end; f += 8) {
-      const T av = a(f);
-      const T *xp = x(f) + cg * S::C;
+  for (int q = 0; q < CH; ++q)
 #pragma unroll
-      for (int c = 0; c < S::C; ++c) sum[c] = fma(av, xp[c], sum[c]);
-    }
+    for (int c = 0; c < S::C; ++c) t[q][c] = T(0);
+  auto add = [&](int f, T (&sum)[S::C]) {
+    const T av = a(f);
+    const T *xp = x(f) + cg * S::C;
+#pragma unroll
+    for (int c = 0; c < S::C; ++c) sum[c] = fma(av, xp[c], sum[c]);
   };
-  chain(sl, min(len, 64), acc);
-  for (int f0 = 64; f0 < len; f0 += 64) {
-    chain(f0 + sl, min(len, f0 + 64), t);
+  int f = sl;
+  if constexpr (CH > 1) {
+    for (; f + 8 * (CH - 1) < len; f += 8 * CH)
 #pragma unroll
-    for (int c = 0; c < S::C; ++c) acc[c] += t[c];
+      for (int q = 0; q < CH; ++q) add(f + 8 * q, t[q]);
+  }
+#pragma unroll 4
+  for (; f < len; f += 8) add(f, t[0]);
+  T acc[S::C];
+#pragma unroll
+  for (int c = 0; c < S::C; ++c) {
+    if constexpr (CH == 4) acc[c] = (t[0][c] + t[1][c]) + (t[2][c] + t[3][c]);
+    else acc[c] = t[0][c];
   }
   T v;
   if constexpr (S::C == 2) {
@@ -124,13 +131,13 @@ __device__ __forceinline__ bool stores(int sub) {
 }
 
 // sliced sum of scalar row r of block row [beg, end)
-template <typename T, int K>
+template <typename T, int K, int CH>
 __device__ __forceinline__ T sliced_row(int sub, int beg, int end, int r, int br, int bc,
                                         const int *__restrict__ col, const T *__restrict__ val,
                                         const T *__restrict__ X) {
   const T *a0 = val + ((size_t)beg * br + r) * bc;
   const size_t bstep = (size_t)(br - 1) * bc;     // skip of one block beyond its row r
-  return sliced_sum<T, K>(
+  return sliced_sum<T, K, CH>(
       sub, (end - beg) * bc,
       [&](int f) { return __ldg(a0 + f + (f / bc) * bstep); },
       [&](int f) {
@@ -139,7 +146,8 @@ __device__ __forceinline__ T sliced_row(int sub, int beg, int end, int r, int br
       });
 }
 
-template <typename T, int K>
+// CH: 4 for matrices of long rows, else 1
+template <typename T, int K, int CH>
 __global__ void __launch_bounds__(kThreads)
 bmv_sliced_kernel(int mode, int64_t n_rows, int br, int bc, const int *__restrict__ rp,
                   const int *__restrict__ col, const T *__restrict__ val, const T *__restrict__ X,
@@ -151,7 +159,7 @@ bmv_sliced_kernel(int mode, int64_t n_rows, int br, int bc, const int *__restric
   const int64_t row = on ? t / L : n_rows - 1;
   const int i = (int)(row / br);
   const int r = (int)(row - (int64_t)i * br);
-  const T v = sliced_row<T, K>(sub, __ldg(rp + i), __ldg(rp + i + 1), r, br, bc, col, val, X);
+  const T v = sliced_row<T, K, CH>(sub, __ldg(rp + i), __ldg(rp + i + 1), r, br, bc, col, val, X);
   if (!on || !stores<K>(sub)) return;
   const size_t e = (size_t)row * K + column_of<K>(sub);
   Y[e] = mode == GASA_MV_RESIDUAL ? B[e] - v : mode == GASA_MV_ADD ? Y[e] + v : v;
@@ -159,7 +167,7 @@ bmv_sliced_kernel(int mode, int64_t n_rows, int br, int bc, const int *__restric
 
 // block-Jacobi step, `units` whole block rows per CTA (blockDim = units * bs rows' lanes,
 // rounded up to warps)
-template <typename T, int K>
+template <typename T, int K, int CH>
 __global__ void __launch_bounds__(1024)
 bjacobi_sliced_kernel(int mode, int n, int bs, int units, const int *__restrict__ rp,
                       const int *__restrict__ col, const T *__restrict__ A,
@@ -180,7 +188,7 @@ bjacobi_sliced_kernel(int mode, int n, int bs, int units, const int *__restrict_
     const int i = u0 + tr / bs, r = tr % bs;
     T v = T(0);
     if (mode == JAC_SWEEP)
-      v = sliced_row<T, K>(sub, __ldg(rp + i), __ldg(rp + i + 1), r, bs, bs, col, A, X);
+      v = sliced_row<T, K, CH>(sub, __ldg(rp + i), __ldg(rp + i + 1), r, bs, bs, col, A, X);
     if (on && stores<K>(sub)) {
       const int c = column_of<K>(sub);
       const T b = B[((size_t)u0 * bs + t) * K + c];
@@ -194,7 +202,7 @@ bjacobi_sliced_kernel(int mode, int n, int bs, int units, const int *__restrict_
     const int tr = on ? t : nrow - 1;
     const T *w = W + ((size_t)u0 * bs + tr) * bs;
     const T *rl = res + (size_t)(tr / bs) * bs * K;
-    const T v = sliced_sum<T, K>(sub, bs, [&](int f) { return __ldg(w + f); },
+    const T v = sliced_sum<T, K, 1>(sub, bs, [&](int f) { return __ldg(w + f); },
                                  [&](int f) { return rl + f * K; });
     if (on && stores<K>(sub)) {
       const size_t g = ((size_t)u0 * bs + t) * K + column_of<K>(sub);
@@ -1132,10 +1140,31 @@ bdense_split_kernel(int n, int ld, const double *__restrict__ M, const float *__
 // column's bits do not depend on the batch width
 static bool long_rows(int n_brows, int64_t nnzb) { return nnzb >= 16 * (int64_t)n_brows; }
 
-// Rows in eight slices while a thread per row would leave SMs without their
-// 1,024 threads; long rows on such a mesh too (their warp variant gives every
-// lane whole blocks).  By the matrix only, as above.
-static bool few_rows(int64_t rows) { return rows < (int64_t)kNumSM * 1024; }
+// Rows in eight slices while that is the faster way, by the matrix and the type only, as
+// above (GB300, eight columns, us sliced / a thread a row, from 16 blocks on a warp a row):
+//  - short rows, FP32: products below 16,384 scalar rows (rows of 4 blocks of 10 x 10:
+//    5,000 rows 4.1 / 9.3, 20,000 10.3 / 9.3, 150,000 62 / 15), steps below 10,240
+//    (6.2 / 8.5, 15.5 / 8.7, 100 / 18);
+//  - short rows, FP64: bound by FP64 instructions, of which slices spend 5 more a row than
+//    a thread a row (14 in a step) next to a quarter of its values, while a thread a row
+//    takes as long for 256 rows an SM as for a few (its CTAs of eight warps; 40 values:
+//    products 5,000 rows 6.5 / 23.0, 20,000 17.0 / 23.2, 40,000 31 / 43, 80,000 60 / 63,
+//    150,000 110 / 83; steps 5,000 11.2 / 29.9, 20,000 32.8 / 30.0; 169 values: products
+//    59,904 156 / 171, steps 26,624 94.6 / 96.9, 59,904 226 / 190);
+//  - long rows, FP32: where a row leaves a quarter of a warp's lanes without a block, below
+//    16,384 rows (5,000 rows of 17 blocks of 12 x 12 12.1 / 13.3, of 25 of 13 x 13
+//    18.2 / 11.0); FP64 below 1,024 rows an SM (5,000 22.9 / 47.6, 80,000 241 / 600).
+template <typename T>
+static bool sliced_rows(bool step, int n_brows, int br, int bc, int64_t nnzb) {
+  const int64_t rows = (int64_t)n_brows * br;
+  if (std::is_same<T, float>::value)
+    return long_rows(n_brows, nnzb) ? rows < 16384 && nnzb < 24 * (int64_t)n_brows
+                                    : rows < (step ? 10240 : 16384);
+  if (long_rows(n_brows, nnzb)) return rows < (int64_t)kNumSM * 1024;
+  const double v = std::max(1.0, (double)nnzb * bc / n_brows);     // values of a scalar row
+  const int64_t wave = (int64_t)kNumSM * kThreads;
+  return (double)rows * (1.0 + 4.0 * (step ? 14 : 5) / v) < (double)((rows + wave - 1) / wave * wave);
+}
 
 template <typename T>
 cudaError_t launch_bmv(int mode, int n_brows, int br, int bc, const int *rp, const int *col,
@@ -1143,9 +1172,11 @@ cudaError_t launch_bmv(int mode, int n_brows, int br, int bc, const int *rp, con
                        int64_t nnzb) {
   const int64_t rows = (int64_t)n_brows * br;
   if (rows == 0) return cudaSuccess;
-  if (few_rows(rows)) {
-    GASA_KSWITCH(K, launch_k(bmv_sliced_kernel<T, KK>, div_up(rows * Slices<KK>::lanes, kThreads),
-                             kThreads, 0, s, mode, rows, br, bc, rp, col, val, X, B, Y));
+  if (sliced_rows<T>(false, n_brows, br, bc, nnzb)) {
+    GASA_KSWITCH(K, launch_k(long_rows(n_brows, nnzb) ? bmv_sliced_kernel<T, KK, 4>
+                                                      : bmv_sliced_kernel<T, KK, 1>,
+                             div_up(rows * Slices<KK>::lanes, kThreads), kThreads, 0, s, mode, rows,
+                             br, bc, rp, col, val, X, B, Y));
   } else if (long_rows(n_brows, nnzb)) {
     GASA_KSWITCH(K, launch_k(bmv_warp_kernel<T, KK>, div_up(rows * 32, kThreads), kThreads, 0, s,
                              mode, rows, br, bc, rp, col, val, X, B, Y));
@@ -1162,7 +1193,8 @@ cudaError_t launch_bjacobi(int mode, int n, int bs, const int *rp, const int *co
                            const T *W, const T *X, const T *B, T *Xo, int K, cudaStream_t s,
                            int64_t nnzb) {
   if (n == 0) return cudaSuccess;
-  const bool few = few_rows((int64_t)n * bs);
+  // the first step from zero reads one block of W a row, whatever the row's length
+  const bool few = sliced_rows<T>(true, n, bs, bs, mode == JAC_SWEEP ? nnzb : n);
   const bool warp = !few && mode == JAC_SWEEP && long_rows(n, nnzb);
   int rows_cta = warp ? 1 : std::max(1, kThreads / bs);
   int th = kThreads;
@@ -1174,8 +1206,10 @@ cudaError_t launch_bjacobi(int mode, int n, int bs, const int *rp, const int *co
   const size_t smem = (size_t)rows_cta * bs * K * sizeof(T);
   if (smem > 48 * 1024) return cudaErrorInvalidValue;
   if (few) {
-    GASA_KSWITCH(K, launch_k(bjacobi_sliced_kernel<T, KK>, div_up(n, rows_cta), th, smem, s, mode,
-                             n, bs, rows_cta, rp, col, A, W, X, B, Xo));
+    GASA_KSWITCH(K, launch_k(long_rows(n, nnzb) ? bjacobi_sliced_kernel<T, KK, 4>
+                                                : bjacobi_sliced_kernel<T, KK, 1>,
+                             div_up(n, rows_cta), th, smem, s, mode, n, bs, rows_cta, rp, col, A, W,
+                             X, B, Xo));
   } else if (warp) {
     GASA_KSWITCH(K, launch_k(bjacobi_kernel<T, KK, true>, div_up(n, rows_cta), kThreads, smem, s,
                              mode, n, bs, rows_cta, rp, col, A, W, X, B, Xo));

@@ -47,11 +47,13 @@ def _apply(rp, col, val, X):
     return y
 
 
-# below 155,648 scalar rows a row is dealt to eight slices; above, a thread a row, or a warp
-# from 16 blocks a row on
+# few scalar rows are dealt to eight slices each (short rows by type, operation, number and
+# length); many take a thread a row, or a warp from 16 blocks a row on (FP32 from 24
+# blocks or 16,384 rows, FP64 from 155,648 rows)
 SHAPES = [(1, 3, 3, 1, 1), (37, 5, 5, 0, 9), (700, 13, 13, 3, 30), (120, 28, 21, 2, 12),
           (3, 1, 1, 0, 2), (15565, 10, 10, 1, 4), (15563, 10, 10, 1, 4), (40000, 4, 4, 14, 20),
-          (40000, 4, 9, 1, 3)]
+          (40000, 4, 9, 1, 3), (900, 10, 10, 20, 30), (2000, 10, 10, 14, 22), (1200, 10, 10, 0, 6),
+          (1700, 10, 10, 1, 5), (39000, 4, 4, 16, 20)]
 
 
 @pytest.mark.parametrize("t", ["f", "d"])
@@ -178,6 +180,34 @@ def test_folded_step(n, bs, lo, hi):
           np.int64(col.size))
     tol = (hi * bs + 4) * eps * (mag + np.abs(c) + np.abs(x))
     assert np.all(np.abs(to_host(out) - (x + (c - ax))) <= tol)
+
+
+def test_many_short_rows_are_not_sliced():
+    """150,000 scalar rows of four blocks and eight columns: no slower than six times the
+    15,000 that are dealt to slices (a thread a row takes about four times their time, slices
+    take ten)."""
+    import torch
+    rng = np.random.default_rng(0)
+
+    def ms(n):
+        rp, col, val = _bsr(rng, n, n, 10, 10, 4, 4)
+        X = to_dev(rng.standard_normal((n, 10, 8)).astype(np.float32))
+        Y = torch.empty_like(X)
+        d = [to_dev(a) for a in (rp, col, val.astype(np.float32).ravel())]
+        name = "_ZN4gasa10launch_bmvIfEE9cudaErroriiiiPKiS3_PKT_S6_S6_PS4_iP11CUstream_stl"
+        best = np.inf
+        for _ in range(6):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            torch.cuda.synchronize()
+            a.record()
+            for _ in range(50):
+                _call(name, 0, n, 10, 10, *d, X, Y, Y, 8, None, np.int64(col.size))
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b) / 50)
+        return best
+
+    assert ms(15000) <= 6 * ms(1500)
 
 
 @pytest.mark.parametrize("n,br,bc,per,limit", [(150, 17, 17, 98, 1.5e-7), (300, 13, 13, 25, 9.4e-8),
