@@ -729,7 +729,7 @@ cudaError_t launch_bsr_mv_ds(int n_brows, int br, int bc, const int *rp, const i
 // ----------------------------------------------------------------------------
 // PAIR: the blocks of a row two at a time under a register cap, as in
 // folded_pair_kernel (same bits)
-template <typename T, int BS, int MODE, bool PAIR = false>
+template <typename T, int BS, int MODE, bool PAIR>
 __global__ void __launch_bounds__(256, PAIR ? 5 : 0)
 jacobi_kernel(int n_units, const int *__restrict__ rp, const int *__restrict__ col,
               const T *__restrict__ val, const T *__restrict__ Wm, const T *__restrict__ x,
@@ -1016,19 +1016,17 @@ static cudaError_t jac_dispatch(int n_units, int bs, const int *rp, const int *c
   if (n_units == 0) return cudaSuccess;
   const bool al = aligned16(val) && aligned16(W) && (MODE == JAC_FIRST || aligned16(x));
   if (lim != INT_MAX && (!al || bs > 16)) return cudaErrorNotSupported;
-  if constexpr (std::is_same<T, float>::value && MODE == JAC_SWEEP) {
-    if (al && bs == 10) {
-      launch_k(jacobi_kernel<T, 10, MODE, true>, div_up(n_units, 25), 256, 0, s, n_units, rp, col,
-               val, W, x, b, xo, lim);
-      note_launch();
-      return cudaGetLastError();
-    }
-  }
+  // PAIR for the FP32 step at width 10, 131,072 rows of three to four blocks 54.1 -> 51.2 us on
+  // GB300.  Elsewhere it gives less or nothing (131,072 rows of four blocks, without and
+  // with: 9 49.5 and 49.4, 11 67.8 both, 12 65.8 and 65.0, 13 96.5 both, 14 89.9 and 86.2,
+  // 15 133.7 and 129.4, 16 106.0 and 106.1; 40,000 rows of 16 39.6 and 41.3)
 #define GASA_JAC_CASE(BS)                                                                   \
   case BS: {                                                                                \
     constexpr int rpb = 256 / BS;                                                           \
-    launch_k(jacobi_kernel<T, BS, MODE>, div_up(n_units, rpb), 256, 0, s, n_units, rp, col, val,  \
-                                                                    W, x, b, xo, lim); note_launch();      \
+    constexpr bool pair = std::is_same<T, float>::value && MODE == JAC_SWEEP && BS == 10;   \
+    launch_k(jacobi_kernel<T, BS, MODE, pair>, div_up(n_units, rpb), 256, 0, s, n_units, rp, col,  \
+             val, W, x, b, xo, lim);                                                        \
+    note_launch();                                                                          \
     return cudaGetLastError();                                                              \
   }
   if (al && bs <= 16) {

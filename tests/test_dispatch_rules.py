@@ -92,3 +92,16 @@ def test_fp32_low_and_short_rows_keep_a_lane_per_row():
             assert by_rows(op, 1000, bc, bc, 12) == (bc % 2 == 1)
     assert by_rows(4, 1024, 10, 8, 45) and by_rows(4, 2500, 22, 17, 36)
     assert not by_rows(4, 4096, 12, 12, 36) and not by_rows(4, 64, 22, 17, 90)
+
+
+def test_every_smoothing_kernel_compiled_is_reached():
+    """Thread-per-row smoothing kernels: the variant with two blocks in flight exists for the
+    FP32 step at width 10, and the plain one everywhere else and not there."""
+    import re
+    import subprocess
+    gasa = _lib()
+    out = subprocess.run(["nm", "-C", gasa._name], capture_output=True, text=True, check=True).stdout
+    found = {tuple(m.split(", ")) for m in re.findall(r"\bjacobi_kernel<([^>]*)>\(", out)}
+    want = {(t, str(bs), str(mode), "true" if (t, bs, mode) == ("float", 10, 0) else "false")
+            for t in ("float", "double") for bs in range(1, 17) for mode in range(4)}
+    assert found == want
