@@ -440,3 +440,14 @@ def test_launch_count_of_graphs_is_this_threads():
     alone = per_cycle(False)
     for _ in range(3):
         assert per_cycle(True) == alone
+
+
+@pytest.mark.parametrize("n_agg,bs,size,r,s_next", [
+    (160, 4, 3, 80, 6),       # many aggregates: ten pairs a warp, four warps
+    (154, 2, 3, 256, 6),      # the most candidates: several rounds of ten pairs
+    (170, 5, 4, 37, 5),       # an odd count, a short last chunk of pairs
+    (153, 1, 2, 1, 1), (155, 3, 2, 21, 3),
+])
+def test_tentative_many_aggregates(n_agg, bs, size, r, s_next):
+    """More aggregates than SMs, which share them: as the tests of few aggregates."""
+    test_tentative_packed_sums(n_agg * size, bs, size, r, s_next)
