@@ -307,7 +307,7 @@ gasa_status gasa_bsr_mv_f32(int32_t mode, int32_t n_brows, int32_t br, int32_t b
 
 /* y = A x (FP64 result) of the outer Krylov product of the mixed-precision
  * solve (the Alg. 2 preconditioner runs in FP32; the paper fixes no
- * precision), in double-single arithmetic from exact two-term FP32 splits:
+ * precision), in double-single arithmetic from two-term FP32 splits:
  * a = a_hi + a_lo per stored value and x = x_hi + x_lo per entry (hi the FP32
  * rounding, lo the FP32 rounding of the remainder).  Each product's leading
  * part is exact and joins the sum by an error-free two-sum; the low word

@@ -493,8 +493,8 @@ gasa_status grid_build(gasa_ctx *ctx, int pi) {
 // step, residual, restriction, prolongation and the coarsest solve is linear
 // in it.  On the coarse levels each of those steps is a launch whose cost is
 // latency rather than bytes, so setup runs exactly those steps (FP64, the
-// batched kernels of the request server) on the unit vectors, eight at a
-// time, and keeps the results as the columns of M_kt; the V-cycle then
+// many-column kernels of kernels_setup.cu) on the unit vectors, 64 or more at
+// a time, and keeps the results as the columns of M_kt; the V-cycle then
 // applies u_kt = M_kt b_kt as one dense product.  kt is the first level
 // k >= 1 from which every level holds at most dense_tail_dofs stored dofs
 // and is stored (not matrix-free).
@@ -520,7 +520,8 @@ gasa_status dense_tail_build(gasa_ctx *ctx) {
   // pitch that is no power of two)
   const int ld = ((n + 15) / 16) * 16 + 16;
   // columns per pass: as many as keep the scratch (x, x2, b, r per level
-  // kt .. N) within the size of M, whose FP32 split follows when it is freed
+  // kt .. N) within the size of M, whose FP32 split follows when it is freed, 64 at
+  // least (or all)
   size_t dofs = 0;
   for (int k = kt; k <= N; ++k) dofs += (size_t)ctx->L[k].ndof;
   const int C = std::min(n, std::max(64, (int)((size_t)n * ld / (4 * dofs)) / 32 * 32));
@@ -590,7 +591,7 @@ gasa_status dense_tail_build(gasa_ctx *ctx) {
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   dfree(ctx, scr);
   ctx->device_bytes -= (int64_t)(tot * sizeof(double));
-  // the FP32 cycle applies M from its exact two-term FP32 split
+  // the FP32 cycle applies M from its two-term FP32 split
   float *Mh = nullptr, *Ml = nullptr;
   if (st == GASA_OK) st = dalloc(ctx, &Mh, (size_t)n * ld);
   if (st == GASA_OK) st = dalloc(ctx, &Ml, (size_t)n * ld);
@@ -681,7 +682,6 @@ struct FusedEnds {
 };
 
 // first0: the caller has already launched level 0's first smoothing step
-//
 template <typename T>
 gasa_status vcycle_impl(gasa_ctx *ctx, const T *rhs, T *out, bool h16 = false,
                         const FusedEnds *fe = nullptr, bool first0 = false) {
@@ -825,8 +825,9 @@ gasa_status vcycle_impl(gasa_ctx *ctx, const T *rhs, T *out, bool h16 = false,
     xk[kt] = P::x(ctx->L[kt]);
   } else if (kt < N) {
     // levels kt .. N-1 and the coarsest solve as their dense operator: FP64
-    // arithmetic in the FP64 cycle, double-single arithmetic on FP32 units
-    // (the same to about 2^-47 of sum |m x| per row) in the FP32 cycle
+    // arithmetic in the FP64 cycle, on two FP32 words of the operator with
+    // double-single sums on FP32 units (the same to about 2^-47 of sum |m x| per
+    // row) in the FP32 cycle
     Level &ld = ctx->L[kt];
     if constexpr (std::is_same<T, float>::value)
       CU(launch_dense_mv_ds(ctx->dtail_n, ctx->dtail_ld, ctx->dtail_Mh, ctx->dtail_Ml, P::b(ld),
@@ -933,7 +934,9 @@ void build_vcycle_graph(gasa_ctx *ctx, int precision) {
 // written outside the graph, so it does not depend on their addresses: the
 // FP32 cycles convert at both ends anyway, the FP64 cycle takes two copies.
 // The first call launches directly: a hierarchy that is applied once pays for
-// no graph.
+// no graph and gains nothing from one (first P3 256^2 V-cycle 2 % faster than
+// without graphs); the second captures and instantiates it, so the gain is there
+// from the third on.
 gasa_status apply_M_host(gasa_ctx *ctx, const double *rr, double *z, int precision) {
   int &calls = ctx->vc_calls[precision];
   if (ctx->prof || calls < 1) {

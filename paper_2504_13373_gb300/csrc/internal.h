@@ -61,11 +61,12 @@ enum JacobiMode { JAC_SWEEP = 0, JAC_FIRST = 1, JAC_APPLY = 2, JAC_RELAX = 3 };
 // nnzb argument of the launchers below when the host does not know it (reading
 // it from the device would wait for the stream)
 constexpr int64_t kNnzbUnknown = -2;
-// rows of at least this many wide FP32 blocks take the team kernel when the
+// rows of at least this many wide FP32 blocks take the kernels of kernels_wide.cu when the
 // host does not know the matrix's average
 constexpr int kLongRow = 8;
 
-// ---- kernels_wide.cu: FP32 blocks wider than 8, a team of warps per block row
+// ---- kernels_wide.cu: FP32 blocks wider than 8, a team of warps per block row or
+// lanes on rows of blocks
 // true for blocks with more than 8 rows or columns (at most 40 of either) and
 // at least 8 blocks per block row on average
 bool wide_applies(int br, int bc, int n_brows, int64_t nnzb);
@@ -170,7 +171,7 @@ cudaError_t launch_bsr_mm(int n_brows, int br, int bc, const int *rp, const int 
                           const double *val, const double *X, int64_t ldx, double *Y,
                           int64_t ldy, int ncols, cudaStream_t s);
 
-// y = A x (FP64 out) in double-single arithmetic from exact two-term FP32
+// y = A x (FP64 out) in double-single arithmetic from two-term FP32
 // splits of A (hi, lo) and x (hi, lo); with xd and partials also the
 // bsr_mv_ds_grid(n_brows, br) partial sums of xd . y (16-byte aligned
 // operands only, else cudaErrorNotSupported)
@@ -183,7 +184,7 @@ int bsr_mv_ds_grid(int n_brows, int br);
 // y = A x for a dense row-major n x n matrix with row pitch ld (>= n; 0 = n)
 template <typename T>
 cudaError_t launch_dense_mv(int n, const double *A, const T *x, T *y, cudaStream_t s, int ld = 0);
-// the same in double-single arithmetic on FP32 units from the exact two-term
+// the same in double-single arithmetic on FP32 units from the two-term
 // FP32 split (Mh, Ml) of A (row pitch ld), FP32 x and y
 cudaError_t launch_dense_mv_ds(int n, int ld, const float *Mh, const float *Ml, const float *x,
                                float *y, cudaStream_t s);
@@ -239,7 +240,7 @@ cudaError_t launch_cg_update_p_f32(int64_t n, double *p, const float *z, const d
                                    const double *rz_partials, const double *rzold_partials,
                                    double *rz_out, float *zold_out, float *p_hi, float *p_lo,
                                    int n_rz, cudaStream_t s);
-// exact two-term FP32 split v = hi + lo of an FP64 vector
+// two-term FP32 split v = hi + lo of an FP64 vector
 cudaError_t launch_split(int64_t n, const double *v, float *hi, float *lo, cudaStream_t s);
 cudaError_t launch_cg_check(const double *rr_partials, int n_rr, double *scal, int *iters,
                             int max_iter, cudaGraphConditionalHandle handle, cudaStream_t s);

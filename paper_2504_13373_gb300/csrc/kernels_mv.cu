@@ -490,7 +490,7 @@ template cudaError_t launch_folded_sweep<float>(int, int, const int *, const int
 
 // ----------------------------------------------------------------------------
 // y = A x in double-single arithmetic (the outer Krylov product of the
-// mixed-precision solve).  A and x arrive as exact two-term FP32 splits,
+// mixed-precision solve).  A and x arrive as two-term FP32 splits,
 // a = a_hi + a_lo and x = x_hi + x_lo (a_hi the FP32 rounding of a, a_lo the
 // FP32 rounding of a - a_hi, so each pair holds a to 2^-48 relative).  Per
 // product: a_hi x_hi = p + e exactly (p rounded, e = fma(a_hi, x_hi, -p)),

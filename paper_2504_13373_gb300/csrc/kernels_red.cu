@@ -24,11 +24,6 @@ long long launch_count() { return g_launches.load(std::memory_order_relaxed); }
 // ----------------------------------------------------------------------------
 // reductions
 // ----------------------------------------------------------------------------
-// Streaming vector kernels read 16-byte pairs when both arrays are 16-byte
-// aligned (VEC), four pairs per array in flight per thread; the pair index
-// runs over a grid-stride loop and the odd last entry (if any) goes to
-// thread 0 of CTA 0, so each partial sums a fixed set of entries in a fixed
-// order.
 // CTAs of the CG step's vector kernels: a pair of entries per thread, at most
 // kRedBlocks.  Every update first adds up the previous reduction's partials in
 // each CTA, so on a small level (6,144 dofs: 12 CTAs) the other CTAs' zeros cost
@@ -47,6 +42,11 @@ __device__ __forceinline__ double sum_partials(const double *p, int n, double *s
   return warp_sum(lane < n ? p[lane] : 0.0);
 }
 
+// Streaming vector kernels read 16-byte pairs when both arrays are 16-byte
+// aligned (VEC), four pairs per array in flight per thread; the pair index
+// runs over a grid-stride loop and the odd last entry (if any) goes to
+// thread 0 of CTA 0, so each partial sums a fixed set of entries in a fixed
+// order.
 __device__ __forceinline__ double2 ld2(const double *p, int64_t k) {
   return __ldg(reinterpret_cast<const double2 *>(p) + k);
 }
@@ -415,7 +415,7 @@ cudaError_t launch_cg_update_xr(int64_t n, double *x, double *r, const double *p
   return cudaGetLastError();
 }
 
-// exact two-term FP32 split v = hi + lo (hi the FP32 rounding of v, lo the
+// two-term FP32 split v = hi + lo (hi the FP32 rounding of v, lo the
 // FP32 rounding of v - hi)
 __device__ __forceinline__ void split_f32(double v, float *hi, float *lo, int64_t i) {
   const float h = __double2float_rn(v);

@@ -10,9 +10,10 @@
 // divides bc) in RPL of its rows: LC = bc / VW lanes read one row of the block
 // side by side, G = 32 / LC rows at once, so every load instruction reads one
 // contiguous run of the block whatever its width, the entries of x are loaded
-// once per block, and the lane keeps one partial sum per row over all blocks.
-// (A lane per row, as this file had it before, read a 13-wide block with 4-byte
-// loads 52 bytes apart, eleven 128-byte lines each.)  A team of ES x BS warps
+// once per block, and the lane keeps one or two partial sums per row over all blocks.
+// (A lane per row reads a 13-wide block with 4-byte loads 52 bytes apart, eleven
+// 128-byte lines each; low blocks and short rows take it all the same, see
+// wide_by_rows.)  A team of ES x BS warps
 // owns a block row: ES of them share out the rows of a block (at most
 // kTeamRows each), BS the blocks (block beg + b, beg + b + BS, ...).  The
 // partial sums meet in shared memory and four lanes add up a row in a fixed
@@ -26,7 +27,8 @@
 // first step W y.
 //
 // GB300, FP32: level 1 of a P2 16^3 tet hierarchy (3,072 rows of about 25 blocks
-// of 13 x 13, 53 MB): product 16.0 -> 14.8 us, smoothing step 20.4 -> 17.0 us;
+// of 13 x 13, 53 MB), with a lane per row and with teams: product 16.0 -> 14.8 us,
+// smoothing step 20.4 -> 17.0 us;
 // level 2 (384 rows of about 98 blocks of 17 x 17, 44 MB): step 35.6 ->
 // 19.0 us; fused restriction of level 1 92.4 -> 23.7 us (the last two with a
 // cluster of CTAs per block row; 22.5 and 64.7 us without).  GMRES on Q2 96^2:
