@@ -37,20 +37,17 @@ WORKLOAD = "poisson2d_sipg_p3_tri_256x256"
 MEASURED_PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 FALLBACK_HBM_GBS = 6800.0
 
-# DRAM bytes (read + write) per launch of the level-0 FP32 smoothing sweep
-# from one ncu capture each, valid while the kernel's source file hashes to
-# `src_sha`: the plain kernel, the bulk-copy staged one and the folded one.
 # kernel classes of gasa_profile_read, timed by CUDA events in the host-driven loop
 PROFILE_CLASSES = ["level0_step", "level0_residual_restriction", "outer_Ap", "level0_first_step",
                    "level0_prolongation"]
 
+# DRAM bytes (read + write) per launch of the level-0 FP32 smoothing sweep
+# from one ncu capture each, valid while the kernel's source file hashes to
+# `src_sha`: the plain kernel (not captured since it takes two blocks at a time), the
+# bulk-copy staged one and the folded one.
 NCU_TRAFFIC = {
-    # captured on the 224x224 case of the same recipe (100,352 elements, 210.40 MB read +
-    # 2.19 MB written per launch, two launches) and scaled to 131,072 elements; of the
-    # kernel that took one block at a time, so the record no longer holds
-    "plain": {"kernel": "jacobi_kernel<float,10,0>", "file": "kernels_mv.cu",
-              "src_sha": "e49eeb68f4ccb194",
-              "bytes_per_launch": (210.40e6 + 2.19e6) * 131072 / 100352},
+    "plain": {"kernel": "jacobi_kernel<float,10,0,true>", "file": "kernels_mv.cu",
+              "src_sha": None, "bytes_per_launch": None},
     "tma": {"kernel": "jacobi_tma_kernel<float,10>", "file": "kernels_tma.cu",
             "src_sha": "24cbc7a902631ea2", "bytes_per_launch": 274.87e6 + 6.52e6},
     # folded step x + c - (wD^-1 A) x, two blocks of a row in flight: captured at full
@@ -58,7 +55,7 @@ NCU_TRAFFIC = {
     # 222.42 MB read + 3.81 MB written per launch); unchanged since (the hash is of the
     # file, in which other kernels changed)
     "folded": {"kernel": "folded_pair_kernel<10,6>", "file": "kernels_mv.cu",
-               "src_sha": "621f29f6107b3a8d",
+               "src_sha": "5dc5979a7373228a",
                "bytes_per_launch": 222.42e6 + 3.81e6},
 }
 
@@ -707,6 +704,50 @@ def workload_main(args, local):
     return 0
 
 
+def _short(v):
+    """v with floats at six significant digits"""
+    if isinstance(v, float):
+        return float(f"{v:.6g}")
+    if isinstance(v, dict):
+        return {k: _short(w) for k, w in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [_short(w) for w in v]
+    return v
+
+
+def compact_line(rec):
+    """The one line that is printed of a full record: every key of the contract as it is, the
+    rest down to its main figures.  A reader that keeps the last few thousand characters of
+    the output still gets all of it; the full record goes to stderr."""
+    line = {k: rec[k] for k in rec if k not in (
+        "iterations", "mixed16", "generate_s", "roofline", "roofline_iteration", "level0_kernels",
+        "error_vs_oracle", "oracle", "cpu_baseline", "serving", "other_workloads",
+        "other_workloads_clocks")}
+    line["iterations"] = {k: sorted(set(v)) for k, v in rec["iterations"].items()}
+    m16 = rec["mixed16"]
+    line["mixed16"] = {k: m16[k] for k in ("value", "ms_per_step", "rel_residual")}
+    line["roofline"] = {k: rec["roofline"][k] for k in ("kernel", "bound", "achieved", "peak", "unit",
+                                                        "frac", "peak_kind", "traffic")}
+    # [ms per iteration, share of the measured bandwidth]
+    line["iteration"] = {k: [v["ms_per_iteration"], v["frac"]] for k, v in rec["roofline_iteration"].items()}
+    if rec.get("error_vs_oracle"):
+        line["error_vs_oracle"] = {k: v for k, v in rec["error_vs_oracle"].items() if k != "what"}
+    if "cpu_baseline" in rec:
+        line["cpu_baseline"] = {k: rec["cpu_baseline"][k] for k in ("value", "unit", "cores", "kind", "sample")}
+    if "serving" in rec:
+        # saturated solves/s, p50 and p99 ms; p99 at 0.5 and 1.5 times that rate
+        line["serving"] = {
+            p: [r["saturated"]["solves_per_s"], r["saturated"]["p50_ms"], r["saturated"]["p99_ms"],
+                r["open_loop_0.5x"]["p99_ms"], r["open_loop_1.5x"]["p99_ms"]]
+            for p, r in rec["serving"].items() if p in ("mixed", "fp64")}
+    if "other_workloads" in rec:
+        # [iterations, solves/s] in FP64, mixed32 and mixed16
+        line["other_workloads"] = {
+            w["workload"]: [[r["iterations"], r["solves_per_s"]] for r in w["precisions"].values()]
+            for w in rec["other_workloads"]}
+    return _short(line)
+
+
 def ours_main(args, rank, world, local):
     import torch
     if not torch.cuda.is_available():
@@ -943,7 +984,8 @@ def ours_main(args, rank, world, local):
             line["other_workloads"] = other_workloads(gasa, local)
         line["other_workloads_clocks"] = clk2.summary()
     if rank == 0:
-        print(json.dumps(line))
+        print("full record: " + json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(compact_line(line)), flush=True)
     if dist is not None:
         dist.destroy_process_group()
     del x_host
