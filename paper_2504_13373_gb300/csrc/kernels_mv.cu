@@ -408,7 +408,7 @@ cudaError_t launch_bsr_mv(int mode, int n_brows, int br, int bc, const int *rp, 
     if (nnzb == kNnzbUnknown && wide_shape(br, bc, val, x)) {
       // few scalar rows: a team per block row whatever its length.  Many: each
       // row's own length decides on the device, short rows a thread per scalar
-      // row, long ones the team kernel's second launch, which looks through the
+      // row, long ones a warp per row in a second launch, which looks through the
       // row pointers for them (2 us for 131,072 rows; the read-back it replaces
       // cost the call 10 to 20 us and drained the stream)
       if (few_scalar_rows(n_brows, br))
@@ -1259,8 +1259,8 @@ dense_mv_kernel(int n, int ld, const double *__restrict__ A, const T *__restrict
 // errors of the low word are carried in a third, so that a lane's 16 to 64 columns
 // round like a few (order 2,048, rms error in 2^-53 of an entry: 4,510 without, 430
 // with it, 1,609 for a CTA a row with 8 columns a thread).
-// Order 2,048 (33.5 MB): 12.0 -> 7.3 us on GB300 (7.0 without the third word); a CTA per row took 4-byte loads
-// and its barriers were most of a row's time.
+// Order 2,048 (33.5 MB): 12.0 -> 7.3 us on GB300 (7.0 without the third word); a CTA per
+// row took 4-byte loads and its barriers were most of a row's time.
 template <int WPR>
 __global__ void __launch_bounds__(128)
 dense_mv_ds_kernel(int n, int ld, const float *__restrict__ Mh, const float *__restrict__ Ml,
