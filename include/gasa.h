@@ -195,7 +195,8 @@ typedef struct gasa_ctx gasa_ctx;
 void gasa_default_options(gasa_options *opt);
 
 /* Create a context on CUDA device `device`; `stream` (nullable) is used for
- * every launch of the context, else the context creates its own. */
+ * every launch of the context, else the context creates its own, which does not wait
+ * for the legacy default stream: what a call reads must be complete when it is made. */
 gasa_status gasa_create(gasa_ctx **ctx, int32_t device, void *stream);
 
 /* Alg. 5: build the hierarchy on the device.  A is copied; adj (element face
